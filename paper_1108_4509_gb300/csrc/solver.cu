@@ -1034,8 +1034,6 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
                              s_));
   else
     random_block(N_, m_, opt_.seed, C64_, s_);
-  for (void* p : {Gb_[0], Gb_[1], Pb_})
-    TRM_CUDA(cudaMemsetAsync(p, 0, nm * 8, s_));
 
   enum { PH_SP = 0, PH_MP2 = 1, PH_FP64 = 2 };
   const int prec = opt_.precision;
@@ -1366,8 +1364,7 @@ void Solver::energy_gradient(const double* C, double* E, double* HD,
 void Solver::set_block(const double* C_dev) {
   TRM_CUDA(cudaMemcpyAsync(C64_, C_dev, (size_t)N_ * m_ * 8,
                            cudaMemcpyDeviceToDevice, s_));
-  for (void* p : {Gb_[0], Gb_[1], Pb_})
-    TRM_CUDA(cudaMemsetAsync(p, 0, (size_t)N_ * m_ * 8, s_));
+  cg_fresh_ = true;
   set_restart();
   TRM_CUDA(cudaStreamSynchronize(s_));
 }
@@ -1381,11 +1378,10 @@ void Solver::get_block(double* C_dev) {
 void Solver::iterate(int mode, int restart, double* E, double* rms,
                      double* alpha) {
   const size_t nm = (size_t)N_ * m_;
-  if (restart) {
-    for (void* p : {Gb_[0], Gb_[1], Pb_})
-      TRM_CUDA(cudaMemsetAsync(p, 0, nm * 8, s_));
-    set_restart();
-  }
+  // a new CG sequence reads no value of G_prev or P (gamma = 0), whatever
+  // they hold: the flag is set here, last before the iteration
+  if (restart || cg_fresh_) set_restart();
+  cg_fresh_ = false;
   if (mode == TRM_FP64) {
     double* G = static_cast<double*>(Gb_[0]);
     double* Gp = static_cast<double*>(Gb_[1]);
@@ -1433,8 +1429,7 @@ void Solver::rayleigh_ritz(double* C_dev, double* lambda_host,
     TRM_CUDA(cudaMemcpyAsync(res_host, res_, m_ * 8, cudaMemcpyDeviceToHost,
                              s_));
   TRM_CUDA(cudaStreamSynchronize(s_));
-  for (void* p : {Gb_[0], Gb_[1], Pb_})
-    TRM_CUDA(cudaMemsetAsync(p, 0, (size_t)N_ * m_ * 8, s_));
+  cg_fresh_ = true;  // final_rr used G as scratch
   set_restart();
 }
 

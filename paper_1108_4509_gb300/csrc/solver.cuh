@@ -196,6 +196,7 @@ class Solver {
   IterScalars* ring_ = nullptr;  // pinned host ring of per-iteration scalars
   std::vector<cudaEvent_t> ev_;
   int state_ = 0;  // 0: C64 current, 1: C32 current
+  bool cg_fresh_ = true;  // G_prev and P hold nothing of this CG sequence
   std::vector<IterRecord> history_;
   int ring_phase_[kRingSize] = {};  // phase of each ring entry's iteration
   // generalized problem: S as an operator, Y = S C (and its swap buffer),

@@ -1,0 +1,123 @@
+"""Sequences of calls and sizes at the edges of the dispatch rules, through the
+C ABI."""
+import numpy as np
+import pytest
+
+import trm_inputs as ti
+from oracle import operator as op
+from oracle import trm as otrm
+
+from . import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def trm():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1108_4509_gb300 as mod
+    return mod
+
+
+def _near(H, m, seed):
+    """An orthonormal block near the m lowest eigenvectors (its line search
+    has positive curvature: the step does not depend on earlier ones)."""
+    w, v = np.linalg.eigh(H.toarray())
+    return np.linalg.qr(v[:, :m] + 0.01 * ti.random_block(len(w), m, seed))[0]
+
+
+@pytest.mark.parametrize("mode", ["TRM_FP64", "TRM_FULL_SP", "TRM_MP2"])
+@pytest.mark.parametrize("shape,m", [((13, 11, 9), 7), ((8, 8, 10), 32)])
+def test_new_sequence_ignores_the_last(trm, mode, shape, m):
+    """After trm_set_block or trm_rayleigh_ritz the first iteration starts a
+    new CG sequence whatever G_prev and P hold: the same bytes as on a fresh
+    handle, also with trm_energy_gradient in between."""
+    V = ti.gaussian_wells(shape, 4, seed=2)
+    N = V.size
+    H = op.grid_hamiltonian(shape, 4, 1.0, V)
+    cd = gu.to_dev(_near(H, m, 3))
+
+    def first(h):
+        trm.trm_set_block(h, cd.data_ptr())
+        return first_iteration(h)
+
+    def first_iteration(h):
+        r = trm.trm_iterate(h, getattr(trm, mode))
+        out = gu.empty(N, m, np.float64)
+        trm.trm_get_block(h, out.data_ptr())
+        return r, gu.from_dev(out)
+
+    opt = trm.trm_default_options(stream=gu.stream(), precond=1)
+    fresh = trm.trm_create_stencil(*shape, 4, 1.0, V, m, 1e-10, opt)
+    used = trm.trm_create_stencil(*shape, 4, 1.0, V, m, 1e-10, opt)
+    try:
+        ref = first(fresh)
+        first(used)
+        trm.trm_iterate(used, getattr(trm, mode))
+        again = first(used)
+        assert again[0] == ref[0] and np.array_equal(again[1], ref[1])
+        trm.trm_set_block(used, cd.data_ptr())
+        g = gu.empty(N, m, np.float64)
+        trm.trm_energy_gradient(used, cd.data_ptr(), 0, 0, g.data_ptr(),
+                                trm.TRM_F64, True)
+        between = first_iteration(used)
+        assert between[0] == ref[0] and np.array_equal(between[1], ref[1])
+        trm.trm_set_block(used, cd.data_ptr())
+        other = gu.to_dev(_near(H, m, 5))
+        trm.trm_rayleigh_ritz(used, other.data_ptr(), m)
+        after = first_iteration(used)
+        assert after[0] == ref[0] and np.array_equal(after[1], ref[1])
+    finally:
+        trm.trm_destroy(fresh)
+        trm.trm_destroy(used)
+
+
+@pytest.mark.parametrize("mode", ["TRM_FULL_SP", "TRM_MP2"])
+@pytest.mark.parametrize("m", [1, 5, 31, 32, 33, 64, 65, 96, 127, 128, 129, 200,
+                               255, 256, 257])
+def test_step_factorisation_edges(trm, mode, m):
+    """One step against (C + a G) L^{-T} element by element, at the edges of
+    the 32-column panels and of the one-CTA factorisation (m = 256). The
+    bound: the FP32-class gradient (dG), the FP32-class Grams of the overlap
+    (dS, twice for the factor's first-order change) and the product's
+    rounding, each at 2^-19 of the magnitudes multiplied, C stored in FP32 in
+    full SP."""
+    shape, order = (16, 12, 11), 4
+    V = ti.gaussian_wells(shape, 4, seed=6)
+    H = op.grid_hamiltonian(shape, order, 1.0, V)
+    N = V.size
+    C = otrm.orthonormalize(ti.random_block(N, m, seed=3))
+    X = op.apply_h(H, C)
+    Xp = X - C * np.sum(C * X, axis=0)
+    Hp = C.T @ Xp
+    np.fill_diagonal(Hp, 0.0)
+    G = -2.0 * (Xp - C @ Hp)
+    u = 2.0 ** -19
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_stencil(*shape, order, 1.0, V, m, 1e-10, opt)
+    try:
+        cd = gu.to_dev(C)
+        trm.trm_set_block(h, cd.data_ptr())
+        _, _, a = trm.trm_iterate(h, getattr(trm, mode), restart=True)
+        out = gu.empty(N, m, np.float64)
+        trm.trm_get_block(h, out.data_ptr())
+        C1 = gu.from_dev(out)
+    finally:
+        trm.trm_destroy(h)
+    Y = C + a * G
+    R = np.linalg.inv(np.linalg.cholesky(Y.T @ Y)).T
+    f32 = 2.0 ** -24 * (np.abs(X) + np.abs(C) * np.abs(np.sum(C * X, axis=0)))
+    dG = 2.0 * (f32 * (1 if mode == "TRM_FULL_SP" else 0)
+                + 2.0 ** -24 * np.abs(Xp) + u * np.abs(C) @ np.abs(Hp)
+                + np.abs(C) @ (u * np.abs(C).T @ np.abs(Xp)))
+    cp = np.abs(C).T @ np.abs(G)
+    dS = u * (a * a * np.abs(G).T @ np.abs(G) + a * (cp + cp.T))
+    off = np.abs(R - np.diag(np.diag(R)))
+    prod = u * np.abs(Y) @ off
+    if mode == "TRM_FULL_SP":
+        prod = u * np.abs(Y) @ np.abs(R)
+        dS = dS + 2.0 ** -23 * np.eye(m)
+    bound = (a * np.linalg.norm(dG) + 2 * np.linalg.norm(dS)
+             + np.linalg.norm(prod) + 1e-12)
+    assert np.linalg.norm(C1 - Y @ R) <= bound
