@@ -695,12 +695,16 @@ void update_p(int64_t N, int m, const T* G, T* P, const T* minv,
   TRM_CHECK_LAUNCH();
 }
 
+bool rotate_on_tc(int64_t N, int m, const float* C, const float* P,
+                  const TcWork* tw) {
+  return mul_tc_eligible(N, m, m, tw) && aligned16(C) && aligned16(P);
+}
+
 template <typename T, typename TP>
 void rotate(int64_t N, int m, const T* C, const TP* P, const double* R, T* Cn,
             const IterScalars* sc, cudaStream_t s, const TcWork* tw) {
   if constexpr (sizeof(T) == 4 && sizeof(TP) == 4) {
-    if (mul_tc_eligible(N, m, m, tw) && aligned16(C) &&
-        (P == nullptr || (sc && aligned16(P)))) {
+    if (rotate_on_tc(N, m, C, P, tw) && (P == nullptr || sc)) {
       mul_tc_store(N, m, m, C, P, sc, R, Cn, *tw, s);
       return;
     }
@@ -725,7 +729,7 @@ void rotate_split(int64_t N, int m, const double* C, const float* P,
 void rotate_split_df(int64_t N, int m, const float* Ch, const float* Cl,
                      const float* P, const double* R, float* Cnh, float* Cnl,
                      const IterScalars* sc, cudaStream_t s, const TcWork* tw) {
-  if (mul_tc_eligible(N, m, m, tw) && aligned16(Ch) && aligned16(P)) {
+  if (rotate_on_tc(N, m, Ch, P, tw)) {
     mul_tc_splitdf(N, m, Ch, Cl, P, sc, R, Cnh, Cnl, *tw, s);
     return;
   }

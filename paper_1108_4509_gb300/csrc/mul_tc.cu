@@ -627,9 +627,11 @@ void launch(const MulArgs& a0, const float* A, const float* P,
   float* lo = ws + (size_t)ldm * a.n;
   float* diag2 = MODE == kSplitDf ? lo + (size_t)ldm * a.n : nullptr;
   if (diag2) a.rdiag = diag2;
-  k_split_small<<<ceil_div((int64_t)ldm * a.n, 256), 256, 0, s>>>(
-      a.k, a.n, ldm, M, hi, lo, zero_diag, diag2);
-  TRM_CHECK_LAUNCH();
+  if (M) {  // (null: the terms are there already, from the factorisation)
+    k_split_small<<<ceil_div((int64_t)ldm * a.n, 256), 256, 0, s>>>(
+        a.k, a.n, ldm, M, hi, lo, zero_diag, diag2);
+    TRM_CHECK_LAUNCH();
+  }
   CUtensorMap mA = f32_map(A, a.N, a.k, a.N, 32, BK);
   CUtensorMap mP = f32_map(P ? P : A, a.N, a.k, a.N, 32, BK);
   CUtensorMap mBh = f32_map(hi, a.k, a.n, ldm, BK, NC);
@@ -662,6 +664,8 @@ void launch(const MulArgs& a0, const float* A, const float* P,
 }
 
 }  // namespace
+
+int mul_tc_ldm(int k) { return ldm_of(k); }
 
 bool mul_tc_eligible(int64_t N, int k, int n, const TcWork* tw) {
   if (!tw || !tw->msplit || !tw->err) return false;

@@ -188,6 +188,7 @@ struct TcWork {
   int* err = nullptr;
 };
 size_t mul_tc_work_floats(int k, int n);
+int mul_tc_ldm(int k);  // leading dimension of the split small matrix
 // Y: N x k FP32 block, M: k x n; N % 4 == 0, N >= 128, k, n >= 32, 16-byte
 // aligned blocks (checked by the callers).
 bool mul_tc_eligible(int64_t N, int k, int n, const TcWork* tw);
@@ -229,6 +230,10 @@ void gradient(int64_t N, int m, const T* C, const T* Xp, const double* Hp,
 template <typename T>
 void update_p(int64_t N, int m, const T* G, T* P, const T* minv,
               const IterScalars* sc, cudaStream_t s);
+// Do rotate<float, float> and rotate_split_df run on the tensor cores for
+// these blocks? Their R may then be null: the split factor is in tw.msplit.
+bool rotate_on_tc(int64_t N, int m, const float* C, const float* P,
+                  const TcWork* tw);
 // Cn = (C + alpha P) R, R upper triangular m x m FP64 (alpha from sc, or 0
 // when P is null)
 template <typename T, typename TP>
@@ -296,12 +301,17 @@ void line_factor(int m, const double* Hp, const double* HD, const double* Bm,
                  const double* tr_parts, int n_tr_parts, const double* W,
                  double* Linv, double* R, IterScalars* sc, double* gwork,
                  double* part, bool dev, cudaStream_t s);
-// line_factor<float> with the m x m inputs given in FP32 (Gram copies)
-void line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
+// line_factor<float> with the m x m inputs given in FP32 (Gram copies). With
+// split (mul_tc_work_floats(m, m) floats) and m small enough for one CTA the
+// factor goes out as the TF32 terms the tensor-core rotations read (leading
+// dimension split_ldm; split_diag: the diagonal left out, as pairs) instead of
+// R, and the call returns true: the rotation then takes a null R.
+bool line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
                    const float* Q, const double* hpd, int hpd_stride,
                    const double* tr_parts, int n_tr_parts, const float* W,
-                   double* Linv, double* R, IterScalars* sc, double* gwork,
-                   double* part, cudaStream_t s);
+                   double* R, IterScalars* sc, double* gwork, double* part,
+                   cudaStream_t s, float* split = nullptr, int split_ldm = 0,
+                   bool split_diag = false);
 // Elements (of the arithmetic type) of the factorisation workspace gwork.
 size_t chol_work_elems(int m);
 // S = L L^T (lower); writes Linv = L^{-1} (unless null) and R = L^{-T}. Non-PD sets

@@ -7,7 +7,9 @@
 #include <atomic>
 #include <cstdlib>
 
+#include "dfmath.cuh"
 #include "ops.cuh"
+#include "tc.cuh"
 
 namespace trm {
 
@@ -79,6 +81,27 @@ __global__ void k_make_A0(int m, const double* __restrict__ Hp,
 // The step along P: minimiser of the parabola a tr(D1) + a^2 (tr(D2) -
 // tr(S1 D1)), bounded so that the RMS column change a ||P||_F / sqrt(m)
 // stays below 1; a restart is requested when P is not a descent direction.
+__device__ __forceinline__ void line_alpha(int m, const double* v,
+                                           IterScalars* sc) {
+  const double g0 = v[0];
+  const double c2 = v[1] - v[2];
+  const double qn = v[3];
+  double alpha = 0.0;
+  const double cap = qn > 0.0 ? sqrt((double)m / qn) : 0.0;
+  if (g0 < 0.0 && qn > 0.0) {
+    if (c2 > 0.0)
+      alpha = -g0 / (2.0 * c2);
+    else
+      alpha = sc->alpha_prev > 0.0 ? 2.0 * sc->alpha_prev : 0.5 * cap;
+    if (alpha > cap) alpha = cap;
+  } else {
+    sc->restart = 1;  // not a descent direction: restart CG next time
+  }
+  sc->alpha = alpha;
+  sc->alpha_prev = alpha > 0.0 ? alpha : sc->alpha_prev;
+  sc->c2 = c2;
+  sc->dE = alpha * g0 + alpha * alpha * c2;
+}
 __device__ void line_alpha_block(int m, const double* __restrict__ part,
                                  int nparts, IterScalars* sc, double* red) {
   double v[4] = {0, 0, 0, 0};
@@ -86,26 +109,7 @@ __device__ void line_alpha_block(int m, const double* __restrict__ part,
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] += part[(size_t)p * 4 + q];
   block_sum<4>(v, red);
-  if (threadIdx.x == 0) {
-    const double g0 = v[0];
-    const double c2 = v[1] - v[2];
-    const double qn = v[3];
-    double alpha = 0.0;
-    const double cap = qn > 0.0 ? sqrt((double)m / qn) : 0.0;
-    if (g0 < 0.0 && qn > 0.0) {
-      if (c2 > 0.0)
-        alpha = -g0 / (2.0 * c2);
-      else
-        alpha = sc->alpha_prev > 0.0 ? 2.0 * sc->alpha_prev : 0.5 * cap;
-      if (alpha > cap) alpha = cap;
-    } else {
-      sc->restart = 1;  // not a descent direction: restart CG next time
-    }
-    sc->alpha = alpha;
-    sc->alpha_prev = alpha > 0.0 ? alpha : sc->alpha_prev;
-    sc->c2 = c2;
-    sc->dE = alpha * g0 + alpha * alpha * c2;
-  }
+  if (threadIdx.x == 0) line_alpha(m, v, sc);
 }
 
 // ---------------------------------------------------------------------------
@@ -541,6 +545,419 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
         }
       }
   }
+  if (tid == 0 && isbad && sc) sc->status |= 1;
+}
+
+// ---------------------------------------------------------------------------
+// The FP32 factorisation for m <= 256: S = L L^T and X = L^{-1} in one CTA of
+// 16 warps, by block elimination on [S | I] with 32-column panels. The working
+// copy M holds the lower 32 x 32 blocks (row-major, leading dimension 36) in
+// shared memory; block (i, j) starts as A_ij and turns, once panel j has been
+// eliminated, into the block W_ij of the growing inverse, so no other copy of
+// either triangle exists. Panel p:
+//   (1) warp 0 factors the diagonal block, one row per lane in registers;
+//       warp 1 follows one group of four columns behind and forms
+//       X_pp = L_pp^{-1}, one column per lane;
+//   (2) Z (32 x mp) takes what this panel contributes to every block column:
+//       X_pj = X_pp W_pj for j < p, X_pp, and L_ip = A_ip X_pp^T for i > p;
+//   (3) every block (i, j), i > p, j <= i, takes M_ij -= L_ip Z_j, with M_ip
+//       starting from zero: the Cholesky update for j > p and the inverse's
+//       for j <= p are the same product, 8 x 4 register tiles. Warp 0 updates
+//       the next diagonal block first and goes on with (1) for it, so the
+//       pivot chain runs beside the updates.
+// What bounds it is that chain (one dependent rsqrt, multiply, shuffle per
+// column, about 110 cycles) and one SM's FP32 rate. In deviation form (dev,
+// S = I + E, see above) only the diagonal needs care: it holds the deviation
+// d of the pivot from 1, and y_cc = -f_cc / L_cc is kept apart (ydiag).
+// With `split` the inverse goes out as the two TF32 terms the product kernels
+// read (hi, lo, leading dimension ldm; split_diag: the diagonal left out and
+// written as FP32 pairs after them), else as FP64 R = L^{-T}.
+// ---------------------------------------------------------------------------
+constexpr int PLD = 36, PSZ = 32 * PLD;  // block row stride, block size
+constexpr int kPanelMax = 256;
+constexpr int kPanelThreads = 512;
+
+__host__ __device__ constexpr int panel_blocks(int P) { return P * (P + 1) / 2; }
+inline size_t panel_smem(int m) {
+  const int P = (m + 31) >> 5;
+  return ((size_t)panel_blocks(P) * PSZ + (size_t)32 * (32 * P + 4) +
+          33 * 32 + 32) * sizeof(float);
+}
+
+// Factor the diagonal block D (warp 0; the updated block in shared memory).
+// lcol[c][r] = L_rc (0 for r <= c), rd[c] = 1 / L_cc, ydg[c] = y_cc. Four
+// columns a round, the row shifted by four registers after each, so that every
+// index is static and the code is short. thr: pivot floor of column `lane`.
+template <bool dev>
+__device__ __forceinline__ bool panel_factor(const float* D, float thr,
+                                             float* lcol, float* rd,
+                                             float* ydg) {
+  const int lane = threadIdx.x & 31;
+  float w[36];
+#pragma unroll
+  for (int j = 0; j < 32; j += 4) {
+    const float4 t = *reinterpret_cast<const float4*>(D + lane * PLD + j);
+    w[j] = t.x; w[j + 1] = t.y; w[j + 2] = t.z; w[j + 3] = t.w;
+  }
+  w[32] = w[33] = w[34] = w[35] = 0.f;
+  bool bad = false;
+#pragma unroll 1
+  for (int g = 0; g < 8; ++g) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = 4 * g + u;
+      float d = __shfl_sync(0xffffffffu, w[u], c);
+      float rl;
+      if (dev) {
+        if (!(d > -0.999f)) {  // pivot 1 + d not positive
+          bad = true;
+          d = 0.f;
+        }
+        rl = piv_rsqrt(1.f + d);
+      } else {
+        if (!(d > __shfl_sync(0xffffffffu, thr, c))) {
+          bad = true;
+          d = 1.f;
+        }
+        rl = piv_rsqrt(d);
+      }
+      const float l = lane > c ? w[u] * rl : 0.f;
+      // the next pivot column first: it is the chain's next link
+      const float ln = __shfl_sync(0xffffffffu, l, (c + 1) & 31);
+      w[u + 1] -= l * ln;
+      float* lc = lcol + 32 * c;
+      lc[lane] = l;
+      if (lane == c) {
+        rd[c] = rl;
+        if (dev) ydg[c] = -(d * piv_rcp(1.f + (1.f + d) * rl)) * rl;
+      }
+      __syncwarp();
+      const float4* lv = reinterpret_cast<const float4*>(lc + 4 * g);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {  // (past the block: never used again)
+        const float4 b = lv[t];
+        if (4 * t + 0 > u + 1) w[4 * t + 0] -= l * b.x;
+        if (4 * t + 1 > u + 1) w[4 * t + 1] -= l * b.y;
+        if (4 * t + 2 > u + 1) w[4 * t + 2] -= l * b.z;
+        if (4 * t + 3 > u + 1) w[4 * t + 3] -= l * b.w;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) w[j] = w[j + 4];
+    // columns 4 g .. 4 g + 3 are out: warp 1 may use them
+    asm volatile("bar.arrive %0, 64;" ::"r"(1 + g) : "memory");
+  }
+  return bad;
+}
+
+// X = L^{-1} of the diagonal block into D (warp 1, a group behind warp 0):
+// lane j runs column j of the forward substitution, right-looking.
+__device__ __forceinline__ void panel_invert(float* D, const float* lcol,
+                                             const float* rd) {
+  const int lane = threadIdx.x & 31;
+  float a[36];
+#pragma unroll
+  for (int i = 0; i < 36; ++i) a[i] = i == lane ? 1.f : 0.f;
+#pragma unroll 1
+  for (int g = 0; g < 8; ++g) {
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + g) : "memory");
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int c = 4 * g + u;
+      const float x = a[u] * rd[c];
+      D[c * PLD + lane] = x;
+      const float4* lv = reinterpret_cast<const float4*>(lcol + 32 * c + 4 * g);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const float4 b = lv[t];
+        if (4 * t + 0 > u) a[4 * t + 0] -= b.x * x;
+        if (4 * t + 1 > u) a[4 * t + 1] -= b.y * x;
+        if (4 * t + 2 > u) a[4 * t + 2] -= b.z * x;
+        if (4 * t + 3 > u) a[4 * t + 3] -= b.w * x;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) a[j] = a[j + 4];
+  }
+}
+
+// M_ij -= L_ip Z_j on one warp (zero: M_ij starts from 0): lane (ti, tj) owns
+// rows 8 ti .. +7 and columns 4 tj .. +3, so each quarter of the warp reads
+// and writes 128 contiguous bytes.
+__device__ __forceinline__ void panel_update(float* B, const float* Z, int ldz,
+                                             int i0, int j0, bool zero) {
+  const int lane = threadIdx.x & 31, ti = lane >> 3, tj = lane & 7;
+  float4 acc[8];
+  float4* row = reinterpret_cast<float4*>(B + 8 * ti * PLD + 4 * tj);
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    acc[u] = zero ? make_float4(0.f, 0.f, 0.f, 0.f) : row[u * (PLD / 4)];
+  const float* zi = Z + i0 + 8 * ti;
+  const float* zj = Z + j0 + 4 * tj;
+#pragma unroll 4
+  for (int k = 0; k < 32; ++k) {
+    const float4 p = *reinterpret_cast<const float4*>(zi + k * ldz);
+    const float4 q = *reinterpret_cast<const float4*>(zi + k * ldz + 4);
+    const float4 b = *reinterpret_cast<const float4*>(zj + k * ldz);
+    const float l[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      acc[u].x -= l[u] * b.x;
+      acc[u].y -= l[u] * b.y;
+      acc[u].z -= l[u] * b.z;
+      acc[u].w -= l[u] * b.w;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) row[u * (PLD / 4)] = acc[u];
+}
+
+struct PanelOut {
+  double* Linv = nullptr;  // may be null
+  double* R = nullptr;     // FP64 L^{-T} (when split is null)
+  float* split = nullptr;  // TF32 hi and lo of L^{-T}
+  int ldm = 0;
+  int split_diag = 0;      // leave the diagonal out, written as pairs
+};
+
+template <bool dev>
+__global__ void __launch_bounds__(kPanelThreads, 1)
+    k_chol_panel(int m, const double* __restrict__ S,
+                 const float* __restrict__ Bf, const float* __restrict__ Qf,
+                 PanelOut out, IterScalars* sc,
+                 const double* __restrict__ lpart, int nlpart) {
+  extern __shared__ __align__(16) float psm[];
+  __shared__ int bad;
+  __shared__ float ydg[kPanelMax];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int nw = kPanelThreads / 32;
+  const int P = (m + 31) >> 5, mp = 32 * P, ldz = mp + 4;
+  float* M = psm;
+  float* Z = M + panel_blocks(P) * PSZ;
+  float* lcol = Z + 32 * ldz;   // 32 x 32, and a line read past its end
+  float* rd = lcol + 33 * 32;
+  auto blk = [&](int i, int j) { return M + (panel_blocks(i) + j) * PSZ; };
+  if (tid == 0) bad = 0;
+  if (lpart) {  // the line step first (it sets sc->alpha)
+    __shared__ double lq[4];
+    if (warp < 4) {
+      double v = 0.0;
+      for (int k = lane; k < nlpart; k += 32) v += lpart[4 * (size_t)k + warp];
+      v = warp_sum(v);
+      if (lane == 0) lq[warp] = v;
+    }
+    __syncthreads();
+    if (tid == 0) line_alpha(m, lq, sc);
+    __syncthreads();
+  }
+  // S (or S(a)) into the blocks, minus I in deviation form; the padding is the
+  // identity. Both orientations of B and Q are read along their columns, the
+  // second one added after a barrier. A unit is eight columns of a block.
+  const int units = 4 * panel_blocks(P);
+  const float al = Bf ? (float)sc->alpha : 0.f;
+  const float hq = Bf ? (float)(0.5 * sc->alpha * sc->alpha) : 0.f;
+  for (int pass = 0; pass < (Bf ? 2 : 1); ++pass) {
+    for (int u = warp; u < units; u += nw) {
+      int bi = 0;
+      while (panel_blocks(bi + 1) <= (u >> 2)) ++bi;
+      const int bj = (u >> 2) - panel_blocks(bi), g = 8 * (u & 3);
+      float* D = blk(bi, bj);
+      // pass 0: column 32 bj + g + q, row 32 bi + lane of the matrix;
+      // pass 1: its mirror, column 32 bi + g + q, row 32 bj + lane
+      const int row = 32 * (pass ? bj : bi) + lane;
+      const int col = 32 * (pass ? bi : bj) + g;
+      float v[8];
+      if (Bf) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          v[q] = row < m && col + q < m
+                     ? al * Bf[row + (col + q) * m] + hq * Qf[row + (col + q) * m]
+                     : 0.f;
+      } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          v[q] = row < m && col + q < m
+                     ? (float)(S[row + (col + q) * m] -
+                               (dev && row == col + q ? 1.0 : 0.0))
+                     : 0.f;
+      }
+      if (pass == 0) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (!dev && row == col + q && (Bf || row >= m)) v[q] += 1.f;
+          D[lane * PLD + g + q] = v[q];
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) D[(g + q) * PLD + lane] += v[q];
+      }
+    }
+    __syncthreads();
+  }
+  auto diag = [&](int p) {  // warps 0 and 1
+    if (warp == 0) {
+      float thr = 0.f;
+      if (!dev) {
+        // a pivot that has lost all but 4m roundings of its original diagonal
+        // entry marks a (numerically) singular S
+        const int c = 32 * p + lane;
+        const double sjj = (Bf || c >= m) ? 1.0 : fabs(S[c + c * m]);
+        thr = (float)(4 * m) * 1.2e-7f * (float)sjj;
+      }
+      const bool b = panel_factor<dev>(blk(p, p), thr, lcol, rd, ydg + 32 * p);
+      if (lane == 0 && b) bad = 1;
+    } else {
+      panel_invert(blk(p, p), lcol, rd);
+    }
+  };
+  if (warp < 2) diag(0);
+  __syncthreads();
+  for (int p = 0; p < P && P > 1; ++p) {
+    // (2) the panel Z: warp units are (block column, half of the 32 rows)
+    const float* X = blk(p, p);
+    const int xq = lane & 7;
+    for (int u = warp; u < 2 * P; u += nw) {
+      const int b = u >> 1, k0 = 16 * (u & 1) + 4 * (lane >> 3);
+      float acc[4][4] = {};
+      const int kend = 16 * (u & 1) + 16;  // X_pp is lower triangular
+      if (b > p) {  // L_bp(x, k) = sum_q A_bp(x, q) X_pp(k, q), x = xq + 8 v
+        const float* A = blk(b, p);
+        for (int q = 0; q < kend; q += 4) {
+          float4 a[4], x[4];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            a[v] = *reinterpret_cast<const float4*>(A + (xq + 8 * v) * PLD + q);
+            x[v] = *reinterpret_cast<const float4*>(X + (k0 + v) * PLD + q);
+          }
+#pragma unroll
+          for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+              acc[s][v] += x[s].x * a[v].x + x[s].y * a[v].y +
+                           x[s].z * a[v].z + x[s].w * a[v].w;
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            Z[(k0 + s) * ldz + 32 * b + xq + 8 * v] = acc[s][v];
+      } else if (b < p) {  // X_pb(k, x) = sum_q X_pp(k, q) W_pb(q, x)
+        const float* W = blk(p, b);
+        for (int q = 0; q < kend; q += 4) {
+          float4 x[4];
+#pragma unroll
+          for (int s = 0; s < 4; ++s)
+            x[s] = *reinterpret_cast<const float4*>(X + (k0 + s) * PLD + q);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float4 t =
+                *reinterpret_cast<const float4*>(W + (q + e) * PLD + 4 * xq);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+              const float xe = e == 0 ? x[s].x : e == 1 ? x[s].y
+                             : e == 2 ? x[s].z : x[s].w;
+              acc[s][0] += xe * t.x;
+              acc[s][1] += xe * t.y;
+              acc[s][2] += xe * t.z;
+              acc[s][3] += xe * t.w;
+            }
+          }
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+          *reinterpret_cast<float4*>(Z + (k0 + s) * ldz + 32 * b + 4 * xq) =
+              make_float4(acc[s][0], acc[s][1], acc[s][2], acc[s][3]);
+      } else {
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+          *reinterpret_cast<float4*>(Z + (k0 + s) * ldz + 32 * b + 4 * xq) =
+              *reinterpret_cast<const float4*>(X + (k0 + s) * PLD + 4 * xq);
+      }
+    }
+    __syncthreads();
+    // (3) block updates; row p takes its final values X_pj from Z
+    const int nupd = panel_blocks(P) - panel_blocks(p + 1);
+    const bool more = p + 1 < P;
+    if (more && warp == 0) {
+      panel_update(blk(p + 1, p + 1), Z, ldz, 32 * (p + 1), 32 * (p + 1), false);
+      __syncwarp();
+    }
+    if (more && warp < 2) {
+      diag(p + 1);
+    } else {
+      const int w0 = more ? warp - 2 : warp, wn = more ? nw - 2 : nw;
+      for (int u = w0; u < nupd + p; u += wn) {
+        if (u < nupd) {
+          const int b = panel_blocks(p + 1) + u;
+          int bi = p + 1;
+          while (panel_blocks(bi + 1) <= b) ++bi;
+          const int bj = b - panel_blocks(bi);
+          if (bi == p + 1 && bj == p + 1) continue;  // warp 0 has it
+          panel_update(blk(bi, bj), Z, ldz, 32 * bi, 32 * bj, bj == p);
+        } else {
+          const int bj = u - nupd;
+          float* D = blk(p, bj);
+#pragma unroll
+          for (int k = 0; k < 32; k += 4) {
+            const int r = k + (lane >> 3);
+            *reinterpret_cast<float4*>(D + r * PLD + 4 * xq) =
+                *reinterpret_cast<const float4*>(Z + r * ldz + 32 * bj + 4 * xq);
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  const bool isbad = bad != 0;
+  // column i of R = L^{-T} is row i of X: contiguous in its block row
+  auto entry = [&](int k, int i) -> float {  // off the diagonal, k < i
+    return isbad ? 0.f : blk(i >> 5, k >> 5)[(i & 31) * PLD + (k & 31)];
+  };
+  auto dfull = [&](int i) -> float {  // deviation form: y_ii, else x_ii
+    return isbad ? (dev ? 0.f : 1.f)
+                 : (dev ? ydg[i] : blk(i >> 5, i >> 5)[(i & 31) * (PLD + 1)]);
+  };
+  if (out.split) {
+    float* hi = out.split;
+    float* lo = hi + (size_t)out.ldm * m;
+    float* dg = lo + (size_t)out.ldm * m;
+    for (int i = warp; i < m; i += nw)
+      for (int k = lane; k < out.ldm; k += 32) {
+        float h = 0.f, l = 0.f;
+        if (k < i) {
+          const float x = entry(k, i);
+          h = tc::tf32_rna(x);
+          l = tc::tf32_rna(x - h);
+        } else if (k == i) {
+          const float y = dfull(i);
+          if (out.split_diag) {
+            const F2 d = dev ? two_sum(1.f, y) : F2{y, 0.f};
+            dg[i] = d.h;
+            dg[m + i] = d.l;
+          } else if (dev) {
+            h = tc::tf32_rna(1.f + y);
+            l = tc::tf32_rna(y - (h - 1.f));
+          } else {
+            h = tc::tf32_rna(y);
+            l = tc::tf32_rna(y - h);
+          }
+        }
+        hi[k + (size_t)i * out.ldm] = h;
+        lo[k + (size_t)i * out.ldm] = l;
+      }
+  } else {
+    for (int i = warp; i < m; i += nw)
+      for (int k = lane; k < m; k += 32)
+        out.R[k + i * m] = k < i ? to_f64(entry(k, i))
+                         : k > i ? 0.0
+                                 : (dev ? 1.0 : 0.0) + (double)dfull(i);
+  }
+  if (out.Linv)
+    for (int k = warp; k < m; k += nw)
+      for (int i = lane; i < m; i += 32)
+        out.Linv[i + k * m] = i > k ? to_f64(entry(k, i))
+                            : i < k ? 0.0
+                                    : (dev ? 1.0 : 0.0) + (double)dfull(i);
   if (tid == 0 && isbad && sc) sc->status |= 1;
 }
 
@@ -1131,7 +1548,7 @@ static int chol_blocked_from() {
 // CTA), or of W, L, X, T and the failure flag (blocked)
 size_t chol_work_elems(int m) {
   const size_t mp = (size_t)((m + 31) & ~31);
-  if (m >= chol_blocked_from()) return 4 * mp * mp + 8;
+  if (m >= chol_blocked_from() || m >= kPanelMax) return 4 * mp * mp + 8;
   return mp * (mp + 1) + 33 * mp;
 }
 
@@ -1177,6 +1594,32 @@ static void chol_blocked(int m, const double* S, const double* Bm,
   TRM_CHECK_LAUNCH();
 }
 
+// FP32, m <= kPanelMax: one CTA with everything in shared memory.
+template <bool dev>
+static void panel_launch(int m, const double* S, const float* Bf,
+                         const float* Qf, const PanelOut& out, IterScalars* sc,
+                         cudaStream_t s, const double* lpart, int nlpart) {
+  static std::atomic<int> done[64] = {};  // per device; any thread may launch
+  int dv = 0;
+  cudaGetDevice(&dv);
+  if (dv < 0 || dv >= 64 || !done[dv].load(std::memory_order_relaxed)) {
+    TRM_CUDA(cudaFuncSetAttribute(k_chol_panel<dev>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)panel_smem(kPanelMax)));
+    if (dv >= 0 && dv < 64) done[dv].store(1, std::memory_order_relaxed);
+  }
+  k_chol_panel<dev><<<1, kPanelThreads, panel_smem(m), s>>>(
+      m, S, Bf, Qf, out, sc, lpart, nlpart);
+  TRM_CHECK_LAUNCH();
+}
+
+// FP32 up to this m runs on one CTA out of shared memory (k_chol_panel): at
+// m = 256 that is the largest packed copy that fits, and still faster than
+// the blocked launches.
+static bool panel_fits(int m) {
+  return m <= kPanelMax && (m < chol_blocked_from() || m == kPanelMax);
+}
+
 template <typename Tm, bool dev>
 static void chol_launch(int m, const double* S, const double* Bm,
                         const double* Q, const float* Bf, const float* Qf,
@@ -1184,32 +1627,44 @@ static void chol_launch(int m, const double* S, const double* Bm,
                         double* gwork, cudaStream_t s,
                         const double* lpart = nullptr, int nlpart = 0) {
   if (m > 1024) throw Error(-1, "chol_inv: m > 1024");
-  if (m >= chol_blocked_from()) {
+  if constexpr (sizeof(Tm) == 4) {
+    if (panel_fits(m)) {
+      PanelOut out;
+      out.Linv = Linv;
+      out.R = R;
+      panel_launch<dev>(m, S, Bf, Qf, out, sc, s, lpart, nlpart);
+      return;
+    }
     chol_blocked<Tm, dev>(m, S, Bm, Q, Bf, Qf, Linv, R, sc, gwork, s, lpart,
                           nlpart);
-    return;
-  }
-  const size_t bytes = chol_work_elems(m) * sizeof(Tm);
-  const bool smem = bytes <= 200 * 1024;
-  if (smem) {
-    static std::atomic<int> done[64] = {};  // per device; any thread may launch
-    int dv = 0;
-    cudaGetDevice(&dv);
-    if (dv < 0 || dv >= 64 || !done[dv].load(std::memory_order_relaxed)) {
-      TRM_CUDA(cudaFuncSetAttribute(k_chol_inv<Tm, dev, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    200 * 1024));
-      if (dv >= 0 && dv < 64) done[dv].store(1, std::memory_order_relaxed);
+  } else {
+    if (m >= chol_blocked_from()) {
+      chol_blocked<Tm, dev>(m, S, Bm, Q, Bf, Qf, Linv, R, sc, gwork, s, lpart,
+                            nlpart);
+      return;
     }
+    const size_t bytes = chol_work_elems(m) * sizeof(Tm);
+    const bool smem = bytes <= 200 * 1024;
+    if (smem) {
+      static std::atomic<int> done[64] = {};  // per device; any thread may launch
+      int dv = 0;
+      cudaGetDevice(&dv);
+      if (dv < 0 || dv >= 64 || !done[dv].load(std::memory_order_relaxed)) {
+        TRM_CUDA(cudaFuncSetAttribute(k_chol_inv<Tm, dev, true>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      200 * 1024));
+        if (dv >= 0 && dv < 64) done[dv].store(1, std::memory_order_relaxed);
+      }
+    }
+    if (smem)
+      k_chol_inv<Tm, dev, true><<<1, chol_threads<Tm>(), bytes, s>>>(
+          m, S, Bm, Q, Bf, Qf, Linv, R, sc, nullptr, lpart, nlpart);
+    else
+      k_chol_inv<Tm, dev, false><<<1, chol_threads<Tm>(), 0, s>>>(
+          m, S, Bm, Q, Bf, Qf, Linv, R, sc, reinterpret_cast<Tm*>(gwork), lpart,
+          nlpart);
+    TRM_CHECK_LAUNCH();
   }
-  if (smem)
-    k_chol_inv<Tm, dev, true><<<1, chol_threads<Tm>(), bytes, s>>>(
-        m, S, Bm, Q, Bf, Qf, Linv, R, sc, nullptr, lpart, nlpart);
-  else
-    k_chol_inv<Tm, dev, false><<<1, chol_threads<Tm>(), 0, s>>>(
-        m, S, Bm, Q, Bf, Qf, Linv, R, sc, reinterpret_cast<Tm*>(gwork), lpart,
-        nlpart);
-  TRM_CHECK_LAUNCH();
 }
 
 template <typename Tm>
@@ -1266,19 +1721,29 @@ void line_factor(int m, const double* Hp, const double* HD, const double* Bm,
 
 // The FP32 path with the m x m inputs already in FP32 (copies the Gram sums
 // write): no FP64 conversion in the line terms or the factorisation.
-void line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
+bool line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
                    const float* Q, const double* hpd, int hpd_stride,
                    const double* tr_parts, int n_tr_parts, const float* W,
-                   double* Linv, double* R, IterScalars* sc, double* gwork,
-                   double* part, cudaStream_t s) {
+                   double* R, IterScalars* sc, double* gwork, double* part,
+                   cudaStream_t s, float* split, int split_ldm,
+                   bool split_diag) {
   const int t = ceil_div(m, 32);
   const int ksplit = line_ksplit(m);
   k_line_terms<float, float><<<dim3(t, t, ksplit), 1024, 0, s>>>(
       m, Hp, HD, Bm, Q, hpd, hpd_stride, tr_parts, n_tr_parts, W, part,
       nullptr, nullptr);
   TRM_CHECK_LAUNCH();
-  chol_launch<float, true>(m, nullptr, nullptr, nullptr, Bm, Q, Linv, R, sc,
+  if (split && panel_fits(m)) {
+    PanelOut out;
+    out.split = split;
+    out.ldm = split_ldm;
+    out.split_diag = split_diag ? 1 : 0;
+    panel_launch<true>(m, nullptr, Bm, Q, out, sc, s, part, t * t * ksplit);
+    return true;
+  }
+  chol_launch<float, true>(m, nullptr, nullptr, nullptr, Bm, Q, nullptr, R, sc,
                            gwork, s, part, t * t * ksplit);
+  return false;
 }
 
 template void chol_inv_dev<float>(int, const double*, double*, double*,

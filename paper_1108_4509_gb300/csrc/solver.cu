@@ -675,17 +675,23 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
   }
   const double m3 = md * md * md;
   prof.begin(KC_SMALL, s_);
-  if constexpr (sizeof(T) == 4 && sizeof(Tm) == 4)
-    line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
-                  PG32_ + woff, nullptr, R_, sc_, mmw_, T1_,
-                  s_);  // alpha, Fig. ONFIG
-  else
+  const double* R = R_;
+  if constexpr (sizeof(T) == 4 && sizeof(Tm) == 4) {
+    // alpha, Fig. ONFIG; for the tensor-core rotations the factor goes
+    // straight into their operand format
+    const bool tc = rotate_on_tc(N_, m_, C, P, &tw_) &&
+                    (!gen || rotate_on_tc(N_, m_, Yc, SPt, &tw_));
+    if (line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
+                      PG32_ + woff, R_, sc_, mmw_, T1_, s_,
+                      tc ? tw_.msplit : nullptr, mul_tc_ldm(m_)))
+      R = nullptr;
+  } else
     line_factor<Tm>(m_, Hp_, HD_, Bm_, PG_, hpd, m_ + 1, trp, ntrp,
                     PG_ + woff, nullptr, R_, sc_, mmw_, T1_,
                     sizeof(Tm) == 4, s_);
   prof.end(KC_SMALL, 4 * m3 + 2 * m3 / 3, 0.0, s_);
   TRM_PROF(krt, m2N, 3 * es * nm,
-           (rotate<T, T>(N_, m_, C, P, R_, Cn, sc_, s_, &tw_)));  // (C+aP)L^-T
+           (rotate<T, T>(N_, m_, C, P, R, Cn, sc_, s_, &tw_)));  // (C+aP)L^-T
   if (gen) {  // S (C + aP) L^-T = (Y + a S P) L^-T
     if constexpr (sizeof(T) == 8) {
       TRM_PROF(krt, m2N, 3 * es * nm,
@@ -694,7 +700,7 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
       std::swap(Y64_, Y64n_);
     } else {
       TRM_PROF(krt, m2N, 3 * es * nm,
-               (rotate<float, float>(N_, m_, Y32_, SP32_, R_, Y32n_, sc_, s_,
+               (rotate<float, float>(N_, m_, Y32_, SP32_, R, Y32n_, sc_, s_,
                                      &tw_)));
       std::swap(Y32_, Y32n_);
     }
@@ -789,11 +795,16 @@ void Solver::iter_mp2() {
                          &sc_->status, PG32_));
   }
   prof.begin(KC_SMALL, s_);
-  line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
-                PG32_ + woff, nullptr, R_, sc_, mmw_, T1_, s_);
+  const bool tc = rotate_on_tc(N_, m_, Ch, P, &tw_);
+  const double* R = R_;
+  if (line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
+                    PG32_ + woff, R_, sc_, mmw_, T1_, s_,
+                    tc ? tw_.msplit : nullptr, mul_tc_ldm(m_),
+                    /*split_diag=*/true))
+    R = nullptr;
   prof.end(KC_SMALL, 4 * m3 + 2 * m3 / 3, 0.0, s_);
   TRM_PROF(KC_ROTDF, m2N, 24 * dnm,
-           rotate_split_df(N_, m_, Ch, Cl, P, R_, Cdfn_, Cdfn_ + nm, sc_, s_,
+           rotate_split_df(N_, m_, Ch, Cl, P, R, Cdfn_, Cdfn_ + nm, sc_, s_,
                            &tw_));
   std::swap(Cdf_, Cdfn_);
   std::swap(Gb_[0], Gb_[1]);
