@@ -92,8 +92,12 @@ struct TcSmem {
 // lo = rna_tf32(x - trunc_tf32(x)) for half of a 128-byte line (16 values)
 // of a raw stage, at the same offsets of the lo buffer. Chunks are visited
 // in a bank-spread order.
+// The rounding is an integer add of half a TF32 ulp: the MMA ignores the 13
+// bits below, so this is rna_tf32 without its conversion instruction (an
+// infinity or NaN is in hi already).
 __device__ __forceinline__ float tf32_lo(float x) {
-  return tf32_rna(x - __uint_as_float(__float_as_uint(x) & 0xFFFFE000u));
+  const float d = x - __uint_as_float(__float_as_uint(x) & 0xFFFFE000u);
+  return __uint_as_float(__float_as_uint(d) + 0x1000u);
 }
 __device__ __forceinline__ void split_line_half(const float* raw, float* lo,
                                                 int line, int half) {

@@ -355,10 +355,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int j = 0; j < 8; ++j) {
           const int q = j ^ (i & 7);  // 128-byte swizzle
           float4 a, o;
-          a.x = tf32_rna(v[4 * j + 0]); o.x = tf32_rna(v[4 * j + 0] - a.x);
-          a.y = tf32_rna(v[4 * j + 1]); o.y = tf32_rna(v[4 * j + 1] - a.y);
-          a.z = tf32_rna(v[4 * j + 2]); o.z = tf32_rna(v[4 * j + 2] - a.z);
-          a.w = tf32_rna(v[4 * j + 3]); o.w = tf32_rna(v[4 * j + 3] - a.w);
+          tf32_split(v[4 * j + 0], a.x, o.x);
+          tf32_split(v[4 * j + 1], a.y, o.y);
+          tf32_split(v[4 * j + 2], a.z, o.z);
+          tf32_split(v[4 * j + 3], a.w, o.w);
           hi[q] = a;
           lo[q] = o;
         }

@@ -221,37 +221,14 @@ __device__ __forceinline__ float tf32_rna(float x) {
   return __uint_as_float(r);
 }
 
-// Form and split half of a 128-byte line (16 values) of a staged tile, in
-// place: y = a (+ alpha p, with p read from l), then hi -> a and lo -> l at
-// the same offsets. Chunks are visited in a bank-spread order.
-__device__ __forceinline__ void split_half(float* a, float* l, int line,
-                                           int half, bool axpy, float alpha) {
-  float4* pa = reinterpret_cast<float4*>(a + line * 32);
-  float4* pl = reinterpret_cast<float4*>(l + line * 32);
-  float4 v[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) v[j] = pa[(half * 4 + j) ^ (line & 7)];
-  if (axpy) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float4 p = pl[(half * 4 + j) ^ (line & 7)];
-      v[j].x = fmaf(alpha, p.x, v[j].x);
-      v[j].y = fmaf(alpha, p.y, v[j].y);
-      v[j].z = fmaf(alpha, p.z, v[j].z);
-      v[j].w = fmaf(alpha, p.w, v[j].w);
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int q = (half * 4 + j) ^ (line & 7);
-    float4 h, o;
-    h.x = tf32_rna(v[j].x); o.x = tf32_rna(v[j].x - h.x);
-    h.y = tf32_rna(v[j].y); o.y = tf32_rna(v[j].y - h.y);
-    h.z = tf32_rna(v[j].z); o.z = tf32_rna(v[j].z - h.z);
-    h.w = tf32_rna(v[j].w); o.w = tf32_rna(v[j].w - h.w);
-    pa[q] = h;
-    pl[q] = o;
-  }
+// The same two-term split on the integer pipe, for operands of a TF32 MMA:
+// hi = rna_tf32(x), and lo the bits whose TF32 part (the MMA ignores the 13
+// below) is rna_tf32(x - hi). Infinities and NaN stay in hi.
+__device__ __forceinline__ void tf32_split(float x, float& hi, float& lo) {
+  const uint32_t u = __float_as_uint(x);
+  const uint32_t r = (u + 0x1000u) & 0xFFFFE000u;
+  hi = __uint_as_float((u & 0x7F800000u) == 0x7F800000u ? u : r);
+  lo = __uint_as_float(__float_as_uint(x - hi) + 0x1000u);
 }
 
 // Host side: cuTensorMapEncodeTiled through the runtime's driver entry point
