@@ -3,6 +3,8 @@
 // the direction update of Fig. TMFIG; the rotation C (+ alpha P) L^{-T} of
 // Fig. ONFIG step (4), including the split form C L_D + C L' of Sec. 2.2
 // (MP1 (ii)); column residual norms; the random initial block.
+#include <algorithm>
+
 #include "dfmath.cuh"
 #include "ops.cuh"
 
@@ -32,42 +34,63 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) part[(size_t)blockIdx.x * m + j] = v[0];
 }
 
-// out[j] = sum_chunks part[chunk*m + j]; optional total into *tot (one CTA)
-// out[j] = sum_c part[c m + j] (then sqrt when do_sqrt), *tot = sum_j out[j];
-// one CTA of 1024 threads, m <= 1024: warp w takes the 32 columns of group
-// w % G (G = ceil(m / 32); loads coalesced across columns) and the chunks
-// c = w / G (mod 32 / G); the slices are added in a fixed order.
-__global__ void __launch_bounds__(1024)
+// out[j] = sum_c part[c m + j] (then sqrt when do_sqrt), 32 columns a CTA: warp
+// w adds the chunks w, w + warps, ... (loads coalesced across columns, four in
+// flight), then the warps' sums are added in a fixed order. With sc the CTA
+// that finishes last adds up E = sum_j out[j]. One CTA for all columns was
+// bound by one SM's two FP64 lanes.
+__global__ void __launch_bounds__(512)
     k_colsum(const double* __restrict__ part, int chunks, int m,
-             double* __restrict__ out, double* tot, int do_sqrt) {
-  __shared__ double sl_sum[1024];  // [slice][column], S m <= 1024
-  __shared__ double red[32];
+             double* out, IterScalars* sc, int do_sqrt) {
+  __shared__ double red[16][33];
+  __shared__ int last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int G = (m + 31) >> 5, S = 32 / G;
-  const int cg = warp % G, sl = warp / G;
-  const int j = 32 * cg + lane;
-  if (sl < S && j < m) {
-    double s0 = 0.0, s1 = 0.0;
-    int c = sl;
-    for (; c + S < chunks; c += 2 * S) {
-      s0 += part[(size_t)c * m + j];
-      s1 += part[(size_t)(c + S) * m + j];
+  const int nw = blockDim.x >> 5;
+  const int j = 32 * blockIdx.x + lane;
+  double s0 = 0.0;
+  if (j < m) {
+    double s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    int c = warp;
+    for (; c + 3 * nw < chunks; c += 4 * nw) {
+      const double* p = part + (size_t)c * m + j;
+      const size_t d = (size_t)nw * m;
+      const double a0 = p[0], a1 = p[d], a2 = p[2 * d], a3 = p[3 * d];
+      s0 += a0;
+      s1 += a1;
+      s2 += a2;
+      s3 += a3;
     }
-    if (c < chunks) s0 += part[(size_t)c * m + j];
-    sl_sum[sl * m + j] = s0 + s1;
+    for (; c < chunks; c += nw) s0 += part[(size_t)c * m + j];
+    s0 = (s0 + s1) + (s2 + s3);
+  }
+  red[warp][lane] = s0;
+  __syncthreads();
+  if (warp == 0) {
+    double a = red[0][lane], b = nw > 1 ? red[1][lane] : 0.0;
+    for (int w = 2; w < nw; w += 2) {
+      a += red[w][lane];
+      if (w + 1 < nw) b += red[w + 1][lane];
+    }
+    a += b;
+    if (do_sqrt) a = sqrt(a);
+    if (j < m) out[j] = a;
+  }
+  if (!sc) return;
+  if (threadIdx.x == 0) {
+    // (this CTA's sums, written by its first warp, before its count)
+    __threadfence();
+    last = atomicAdd(&sc->sum_done, 1u) == gridDim.x - 1;
   }
   __syncthreads();
+  if (!last || warp != 0) return;
+  __threadfence();
   double t = 0.0;
-  for (int jj = threadIdx.x; jj < m; jj += blockDim.x) {
-    double s = sl_sum[jj];
-    for (int q = 1; q < S; ++q) s += sl_sum[q * m + jj];
-    if (do_sqrt) s = sqrt(s);
-    out[jj] = s;
-    t += s;
+  for (int k = lane; k < m; k += 32) t += __ldcg(out + k);
+  t = warp_sum(t);
+  if (lane == 0) {
+    sc->E = t;
+    sc->sum_done = 0u;
   }
-  double v[1] = {t};
-  block_sum<1>(v, red);
-  if (threadIdx.x == 0 && tot) *tot = v[0];
 }
 
 // ---------------------------------------------------------------------------
@@ -262,7 +285,7 @@ __global__ void __launch_bounds__(256)
     }
   }
   double v[4] = {(double)s_gg, (double)s_gmg, (double)s_pmg, (double)s_gpp};
-  block_sum<4>(v, red);
+  block_sum4(v, red);
   if (threadIdx.x == 0) {
     const size_t b = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
 #pragma unroll
@@ -278,7 +301,7 @@ __global__ void k_cg_scalars(const double* __restrict__ part, int nparts,
   for (int p = threadIdx.x; p < nparts; p += blockDim.x)
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] += part[(size_t)p * 4 + q];
-  block_sum<4>(v, red);
+  block_sum4(v, red);
   if (threadIdx.x == 0) cg_scalars(v, m, sc);
 }
 
@@ -610,21 +633,27 @@ int elem_grid_x(int64_t N) {
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+static void colsum(const double* part, int chunks, int m, double* out,
+                   IterScalars* sc, int do_sqrt, cudaStream_t s) {
+  // a warp per eight chunks: few chunks leave little for more warps to add
+  const int warps = std::max(1, std::min(16, ceil_div(chunks, 8)));
+  k_colsum<<<ceil_div(m, 32), 32 * warps, 0, s>>>(part, chunks, m, out, sc,
+                                                  do_sqrt);
+  TRM_CHECK_LAUNCH();
+}
+
+void energy_from_dots(const double* dots, int chunks, int m, double* HD,
+                      IterScalars* sc, cudaStream_t s) {
+  colsum(dots, chunks, m, HD, sc, 0, s);
+}
+
 template <typename T>
 void energy_diag(int64_t N, int m, const T* C, const T* X, double* HD,
                  IterScalars* sc, double* partials, cudaStream_t s) {
   const int chunks = ceil_div(N, RCHUNK);
   k_coldot<T><<<dim3(chunks, m), 256, 0, s>>>(N, m, C, X, partials);
   TRM_CHECK_LAUNCH();
-  k_colsum<<<1, 1024, 0, s>>>(partials, chunks, m, HD, sc ? &sc->E : nullptr,
-                              0);
-  TRM_CHECK_LAUNCH();
-}
-
-void energy_from_dots(const double* dots, int chunks, int m, double* HD,
-                      IterScalars* sc, cudaStream_t s) {
-  k_colsum<<<1, 1024, 0, s>>>(dots, chunks, m, HD, sc ? &sc->E : nullptr, 0);
-  TRM_CHECK_LAUNCH();
+  energy_from_dots(partials, chunks, m, HD, sc, s);
 }
 
 template <typename T>
@@ -654,7 +683,7 @@ template <typename T>
 void gradient(int64_t N, int m, const T* C, const T* Xp, const double* Hp,
               T* G, const T* Gprev, const T* Pprev, const T* minv,
               IterScalars* sc, double* partials, size_t cap, cudaStream_t s,
-              const TcWork* tw) {
+              const TcWork* tw, bool split) {
   if constexpr (sizeof(T) == 4) {
     // TMA reads C and the epilogue operands X', G_prev, P_prev
     if (mul_tc_eligible(N, m, m, tw) && aligned16(C) && aligned16(Xp) &&
@@ -662,8 +691,8 @@ void gradient(int64_t N, int m, const T* C, const T* Xp, const double* Hp,
       if ((size_t)mul_tc_parts(N, m) * 4 > cap)
         throw Error(-2, "gradient: partials buffer too small");
       // the kernel's last CTA forms the CG scalars from the per-CTA sums
-      mul_tc_grad(N, m, C, Hp, Xp, G, Gprev, Pprev, minv, partials, sc, *tw,
-                  s);
+      mul_tc_grad(N, m, C, split ? nullptr : Hp, Xp, G, Gprev, Pprev, minv,
+                  partials, sc, *tw, s);
       return;
     }
   }
@@ -673,7 +702,9 @@ void gradient(int64_t N, int m, const T* C, const T* Xp, const double* Hp,
   k_gradient<T><<<grid, 256, 0, s>>>(N, m, C, Xp, Hp, G, Gprev, Pprev, minv,
                                      partials);
   TRM_CHECK_LAUNCH();
-  k_cg_scalars<<<1, 1024, 0, s>>>(partials, (int)nparts, m, sc);
+  // (one SM adds them two a cycle: more threads than records only wait)
+  const int ct = nparts <= 256 ? 128 : nparts <= 1024 ? 256 : 512;
+  k_cg_scalars<<<1, ct, 0, s>>>(partials, (int)nparts, m, sc);
   TRM_CHECK_LAUNCH();
 }
 
@@ -758,8 +789,7 @@ void column_residuals(int64_t N, int m, const double* X, const double* C,
   const int chunks = ceil_div(N, RCHUNK);
   k_resid<<<dim3(chunks, m), 256, 0, s>>>(N, m, X, C, lam, partials);
   TRM_CHECK_LAUNCH();
-  k_colsum<<<1, 1024, 0, s>>>(partials, chunks, m, res, nullptr, 1);
-  TRM_CHECK_LAUNCH();
+  colsum(partials, chunks, m, res, nullptr, 1, s);
 }
 
 void fix_signs(int64_t N, int m, double* C, double* X, double* work,
@@ -798,7 +828,8 @@ void random_block(int64_t N, int m, uint64_t seed, double* C, cudaStream_t s) {
                           float*, cudaStream_t, bool);                       \
   template void gradient<T>(int64_t, int, const T*, const T*, const double*, \
                             T*, const T*, const T*, const T*, IterScalars*,  \
-                            double*, size_t, cudaStream_t, const TcWork*);   \
+                            double*, size_t, cudaStream_t, const TcWork*,    \
+                            bool);                                           \
   template void update_p<T>(int64_t, int, const T*, T*, const T*,            \
                             const IterScalars*, cudaStream_t);
 TRM_INST(float)

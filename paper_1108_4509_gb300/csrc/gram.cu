@@ -8,6 +8,7 @@
 // order, so the result is bitwise reproducible.
 #include "dfmath.cuh"
 #include "ops.cuh"
+#include "tc.cuh"
 
 namespace trm {
 
@@ -204,13 +205,13 @@ __global__ void __launch_bounds__(256)
 // partials) and the 8 sums are added in a fixed order.
 __global__ void __launch_bounds__(256)
     k_sum_splits(const double* __restrict__ part, int splits, size_t count,
-                 double* __restrict__ out, float* __restrict__ out32) {
+                 double* __restrict__ out, int m, GramOut also) {
   __shared__ double red[8][33];
   const int el = threadIdx.x & 31, g = threadIdx.x >> 5;
   const size_t e = (size_t)blockIdx.x * 32 + el;
   double s = 0.0;
   if (e < count) {
-#pragma unroll 4
+#pragma unroll 8
     for (int k = g; k < splits; k += 8) s += part[(size_t)k * count + e];
   }
   red[g][el] = s;
@@ -219,8 +220,9 @@ __global__ void __launch_bounds__(256)
     double t = red[0][el];
 #pragma unroll
     for (int q = 1; q < 8; ++q) t += red[q][el];
+    if (also.zero_diag && e % (m + 1) == 0) t = 0.0;
     out[e] = t;
-    if (out32) out32[e] = (float)t;
+    if (also.f32) also.f32[e] = (float)t;
   }
 }
 
@@ -229,8 +231,8 @@ __global__ void __launch_bounds__(256)
 // is converted to FP64 once.
 __global__ void __launch_bounds__(256)
     k_sum_splits_pairs(const float* __restrict__ part, int splits,
-                       size_t count, double* __restrict__ out,
-                       float* __restrict__ out32, SymSeg sym) {
+                       size_t count, double* __restrict__ out, int m,
+                       GramOut also, SymSeg sym) {
   __shared__ float rh[8][33], rl[8][33];
   const int el = threadIdx.x & 31, g = threadIdx.x >> 5;
   const size_t e = (size_t)blockIdx.x * 32 + el;
@@ -255,8 +257,16 @@ __global__ void __launch_bounds__(256)
     F2 t = {rh[0][el], rl[0][el]};
 #pragma unroll
     for (int q = 1; q < 8; ++q) t = df_add(t, F2{rh[q][el], rl[q][el]});
+    if (also.zero_diag && e % (m + 1) == 0) t = F2{0.f, 0.f};
     out[e] = (double)t.h + (double)t.l;
-    if (out32) out32[e] = t.h;  // the sum rounded to FP32
+    if (also.f32) also.f32[e] = t.h;  // the sum rounded to FP32
+    if (also.split) {
+      const int j = (int)(e / m), i = (int)(e - (size_t)j * m);
+      const float h = tc::tf32_rna(t.h);
+      float* o = also.split + i + (size_t)j * also.split_ldm;
+      o[0] = h;
+      o[(size_t)also.split_ldm * (count / m)] = tc::tf32_rna((t.h - h) + t.l);
+    }
   }
 }
 
@@ -286,29 +296,30 @@ size_t gram_partials_doubles(int64_t N, int m, int n) {
 }
 
 void sum_splits_pairs(const float* part, int splits, size_t count,
-                      double* out, cudaStream_t s, float* out32, SymSeg sym) {
+                      double* out, cudaStream_t s, int m, const GramOut& also,
+                      SymSeg sym) {
   k_sum_splits_pairs<<<ceil_div(count, 32), 256, 0, s>>>(part, splits, count,
-                                                         out, out32, sym);
+                                                         out, m, also, sym);
   TRM_CHECK_LAUNCH();
 }
 
 void sum_splits(const double* part, int splits, size_t count, double* out,
                 cudaStream_t s) {
   k_sum_splits<<<ceil_div(count, 32), 256, 0, s>>>(part, splits, count, out,
-                                                   nullptr);
+                                                   1, GramOut{});
   TRM_CHECK_LAUNCH();
 }
 
 template <typename T>
-void gram(int64_t N, int m, const T* A, const Blocks<T>& B, double* out,
+bool gram(int64_t N, int m, const T* A, const Blocks<T>& B, double* out,
           double* partials, size_t partials_cap, cudaStream_t s, int* err,
-          float* out32) {
+          const GramOut& also) {
   const int n = B.total();
-  if (m <= 0 || n <= 0) return;
+  if (m <= 0 || n <= 0) return false;
   if constexpr (sizeof(T) == 4) {
     if (gram_tc_eligible(N, m, A, B)) {  // tensor cores, FP32-class accuracy
-      gram_tc(N, m, A, B, out, partials, partials_cap, err, s, out32);
-      return;
+      gram_tc(N, m, A, B, out, partials, partials_cap, err, s, also);
+      return true;
     }
   }
   int splits;
@@ -322,8 +333,9 @@ void gram(int64_t N, int m, const T* A, const Blocks<T>& B, double* out,
   TRM_CHECK_LAUNCH();
   const size_t count = (size_t)m * n;
   k_sum_splits<<<ceil_div(count, 32), 256, 0, s>>>(partials, splits, count,
-                                                   out, out32);
+                                                   out, m, also);
   TRM_CHECK_LAUNCH();
+  return false;
 }
 
 template <typename T>
@@ -349,7 +361,7 @@ void gram_in_scratch(int64_t N, int m, const T* A, const Blocks<T>& B,
   TRM_CHECK_LAUNCH();
   const size_t count = (size_t)m * n;
   k_sum_splits<<<ceil_div(count, 32), 256, 0, s>>>(scratch, splits, count,
-                                                   out, nullptr);
+                                                   out, m, GramOut{});
   TRM_CHECK_LAUNCH();
 }
 
@@ -376,15 +388,15 @@ void gram_df(int64_t N, int m, const double* A, const Blocks<double>& B,
   TRM_CHECK_LAUNCH();
   const size_t count = (size_t)m * n;
   k_sum_splits<<<ceil_div(count, 32), 256, 0, s>>>(partials, splits, count,
-                                                   out, nullptr);
+                                                   out, m, GramOut{});
   TRM_CHECK_LAUNCH();
 }
 
-template void gram<float>(int64_t, int, const float*, const Blocks<float>&,
+template bool gram<float>(int64_t, int, const float*, const Blocks<float>&,
                           double*, double*, size_t, cudaStream_t, int*,
-                          float*);
-template void gram<double>(int64_t, int, const double*, const Blocks<double>&,
+                          const GramOut&);
+template bool gram<double>(int64_t, int, const double*, const Blocks<double>&,
                            double*, double*, size_t, cudaStream_t, int*,
-                           float*);
+                           const GramOut&);
 
 }  // namespace trm

@@ -67,7 +67,7 @@ int gram_noalloc(int64_t N, int m, int n, int dtype, const void* A,
       int* err = reinterpret_cast<int*>(scratch + cap);
       int herr = 0;
       TRM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-      gram_tc(N, m, a, b, out, scratch, cap, err, s, nullptr,
+      gram_tc(N, m, a, b, out, scratch, cap, err, s, trm::GramOut{},
               (int)(cap / ((size_t)m * n)));
       TRM_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
       TRM_CUDA(cudaStreamSynchronize(s));

@@ -496,18 +496,18 @@ size_t gram_tc_partials_doubles(int64_t N, int m, int n, int skipped_tiles) {
 
 void gram_tc(int64_t N, int m, const float* A, const Blocks<float>& B,
              double* out, double* partials, size_t cap, int* err,
-             cudaStream_t s, float* out32, int max_splits) {
+             cudaStream_t s, const GramOut& also, int max_splits) {
   Blocks<float> a;
   a.p[0] = A;
   a.cols = m;
   a.count = 1;
-  gram_tc_pairs(N, m, a, B, out, partials, cap, err, s, out32, -1,
+  gram_tc_pairs(N, m, a, B, out, partials, cap, err, s, also, -1,
                 max_splits);
 }
 
 void gram_tc_pairs(int64_t N, int m, const Blocks<float>& A,
                    const Blocks<float>& B, double* out, double* partials,
-                   size_t cap, int* err, cudaStream_t s, float* out32,
+                   size_t cap, int* err, cudaStream_t s, const GramOut& also,
                    int sym_seg, int max_splits) {
   const int n = B.total();
   const int tiles_m = ceil_div(m, BM);
@@ -572,7 +572,7 @@ void gram_tc_pairs(int64_t N, int m, const Blocks<float>& A,
     k_gram_tc<<<dim3(splits, tiles), THREADS, smem, s>>>(maps, a);
     TRM_CHECK_LAUNCH();
     sum_splits_pairs(reinterpret_cast<const float*>(partials), splits, count,
-                     out, s, out32, SymSeg{sym_seg, m, segcols, BM});
+                     out, s, m, also, SymSeg{sym_seg, m, segcols, BM});
   };
   run(tuned_splits(N, m, n, tiles, sym_seg, smax, s, run));
 }

@@ -106,13 +106,23 @@ struct Blocks {
 };
 
 size_t gram_partials_doubles(int64_t N, int m, int n);
+// What the split sum of a Gram writes besides its FP64 result: the result
+// rounded to FP32, its two TF32 terms for the product kernels (hi, then lo
+// split_ldm * n floats on; tensor-core Grams only), and whether entries (i, i)
+// are zero instead of the sum.
+struct GramOut {
+  float* f32 = nullptr;
+  float* split = nullptr;
+  int split_ldm = 0;
+  int zero_diag = 0;
+};
 // FP32 inputs go to the tensor-core kernel when gram_tc_eligible; err (device
-// int, may be null) receives bit 2 if one of its bounded waits gave up;
-// out32 (may be null) receives the result rounded to FP32 as well.
+// int, may be null) receives bit 2 if one of its bounded waits gave up.
+// Returns whether that kernel ran (and GramOut::split was written).
 template <typename T>
-void gram(int64_t N, int m, const T* A, const Blocks<T>& B, double* out,
+bool gram(int64_t N, int m, const T* A, const Blocks<T>& B, double* out,
           double* partials, size_t partials_cap, cudaStream_t s,
-          int* err = nullptr, float* out32 = nullptr);
+          int* err = nullptr, const GramOut& also = GramOut{});
 void sum_splits(const double* part, int splits, size_t count, double* out,
                 cudaStream_t s);
 // A^T B of FP64 blocks in double-float on the FP32 pipe (about 2^-46
@@ -131,8 +141,8 @@ struct SymSeg {
 };
 // the same for partials stored as FP32 pairs (hi, then lo, per split)
 void sum_splits_pairs(const float* part, int splits, size_t count,
-                      double* out, cudaStream_t s, float* out32 = nullptr,
-                      SymSeg sym = SymSeg{});
+                      double* out, cudaStream_t s, int m,
+                      const GramOut& also = GramOut{}, SymSeg sym = SymSeg{});
 // tcgen05 Gram of FP32 blocks (two-term TF32 split, three products, FP32
 // accumulation in tensor memory): needs N % 4 == 0, m >= 32, A and every B
 // segment 16-byte aligned (TMA), at most 4 B segments (each padded to whole
@@ -151,11 +161,12 @@ size_t gram_tc_partials_doubles(int64_t N, int m, int n, int skipped_tiles = 0);
 void gram_tc_pairs(int64_t N, int m, const Blocks<float>& A,
                    const Blocks<float>& B, double* out, double* partials,
                    size_t cap, int* err, cudaStream_t s,
-                   float* out32 = nullptr, int sym_seg = -1,
+                   const GramOut& also = GramOut{}, int sym_seg = -1,
                    int max_splits = 0);
 void gram_tc(int64_t N, int m, const float* A, const Blocks<float>& B,
              double* out, double* partials, size_t cap, int* err,
-             cudaStream_t s, float* out32 = nullptr, int max_splits = 0);
+             cudaStream_t s, const GramOut& also = GramOut{},
+             int max_splits = 0);
 
 // Same product with the split partials in a caller-given scratch of
 // scratch_doubles doubles (fewer row slices when it is small); m*n must fit.
@@ -220,12 +231,13 @@ void mul_tc_splitdf(int64_t N, int m, const float* Ch, const float* Cl,
 
 // G = -2 (X' - C H') with the Polak-Ribiere partial sums; G_prev/P_prev may
 // be null (first iteration). Then the device scalar update of gamma, r.
-// FP32 blocks use the tensor cores when tw allows.
+// FP32 blocks use the tensor cores when tw allows (split: H's TF32 terms are
+// in tw.msplit already).
 template <typename T>
 void gradient(int64_t N, int m, const T* C, const T* Xp, const double* Hp,
               T* G, const T* Gprev, const T* Pprev, const T* minv,
               IterScalars* sc, double* partials, size_t partials_cap,
-              cudaStream_t s, const TcWork* tw = nullptr);
+              cudaStream_t s, const TcWork* tw = nullptr, bool split = false);
 // P = M G + gamma P (gamma from sc)
 template <typename T>
 void update_p(int64_t N, int m, const T* G, T* P, const T* minv,
@@ -302,7 +314,7 @@ void line_factor(int m, const double* Hp, const double* HD, const double* Bm,
                  double* Linv, double* R, IterScalars* sc, double* gwork,
                  double* part, bool dev, cudaStream_t s);
 // line_factor<float> with the m x m inputs given in FP32 (Gram copies). With
-// split (mul_tc_work_floats(m, m) floats) and m small enough for one CTA the
+// split (mul_tc_work_floats(m, m) floats, zero when first used) and m small enough for one CTA the
 // factor goes out as the TF32 terms the tensor-core rotations read (leading
 // dimension split_ldm; split_diag: the diagonal left out, as pairs) instead of
 // R, and the call returns true: the rotation then takes a null R.
@@ -325,9 +337,6 @@ void chol_inv(int m, const double* S, double* Linv, double* R,
 template <typename Tm>
 void chol_inv_dev(int m, const double* S, double* Linv, double* R,
                   IterScalars* sc, double* gwork, cudaStream_t s);
-// set diagonal of an m x m matrix (and of its FP32 copy A32, may be null)
-// to zero
-void zero_diag(int m, double* A, cudaStream_t s, float* A32 = nullptr);
 // symmetric eigenproblem A = Z diag(w) Z^T to FP64 accuracy (FP32 cyclic
 // Jacobi, FP64 refinement of the eigenvectors, FP64 Jacobi on the refined
 // projection), w ascending; work: sym_eig_work_doubles(m); info (device

@@ -48,14 +48,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-__global__ void k_zero_diag(int m, double* A, float* A32) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) {
-    A[i + (int64_t)i * m] = 0.0;
-    if (A32) A32[i + (int64_t)i * m] = 0.f;
-  }
-}
-
 // A0 = sym(H') + diag(H_D): the projected matrix C^T H C when C^T C = I
 // (H_D may be null: plain symmetrisation).
 __global__ void k_make_A0(int m, const double* __restrict__ Hp,
@@ -78,27 +70,63 @@ __global__ void k_make_A0(int m, const double* __restrict__ Hp,
 //   E(a) - E(0) = a tr(D1) + a^2 (tr(D2) - tr(S1 D1)).
 // ---------------------------------------------------------------------------
 
+// Reciprocal square root and reciprocal of the pivot chain by Newton's
+// method from the hardware approximations (rsqrt, reciprocal): one step in
+// FP32, two from the FP32 seed in FP64. Arguments are positive normal numbers (the pivot
+// tests come first); the results are within a few ulp, and the chain stays
+// free of the slow-path calls of the IEEE operations.
+__device__ __forceinline__ float piv_rcp(float t) {
+  const float r = __fdividef(1.0f, t);
+  return fmaf(r, fmaf(-t, r, 1.0f), r);
+}
+__device__ __forceinline__ double piv_rcp(double t) {
+  double r = (double)__fdividef(1.0f, (float)t);
+  r = fma(r, fma(-t, r, 1.0), r);
+  return fma(r, fma(-t, r, 1.0), r);
+}
+// 1 / sqrt(t): the hardware reciprocal square root refined by Newton's step
+// r <- r (3 - t r^2) / 2, once in FP32, twice (from the FP32 seed) in FP64.
+__device__ __forceinline__ float piv_rsqrt(float t) {
+  const float r = rsqrtf(t);
+  return r * fmaf(-0.5f * t * r, r, 1.5f);
+}
+__device__ __forceinline__ double piv_rsqrt(double t) {
+  double r = (double)rsqrtf((float)t);
+  r = r * fma(-0.5 * t * r, r, 1.5);
+  return r * fma(-0.5 * t * r, r, 1.5);
+}
+
 // The step along P: minimiser of the parabola a tr(D1) + a^2 (tr(D2) -
 // tr(S1 D1)), bounded so that the RMS column change a ||P||_F / sqrt(m)
 // stays below 1; a restart is requested when P is not a descent direction.
-__device__ __forceinline__ void line_alpha(int m, const double* v,
-                                           IterScalars* sc) {
+// (One division by Newton's method where the FP32 seed is in range, and the
+// cap's square root only where the cap binds: the FP64 library calls of this
+// chain cost more than the sums before it.)
+__device__ __forceinline__ double line_alpha(int m, const double* v,
+                                             const IterScalars* sc) {
   const double g0 = v[0];
   const double c2 = v[1] - v[2];
   const double qn = v[3];
-  double alpha = 0.0;
-  const double cap = qn > 0.0 ? sqrt((double)m / qn) : 0.0;
-  if (g0 < 0.0 && qn > 0.0) {
-    if (c2 > 0.0)
-      alpha = -g0 / (2.0 * c2);
-    else
-      alpha = sc->alpha_prev > 0.0 ? 2.0 * sc->alpha_prev : 0.5 * cap;
-    if (alpha > cap) alpha = cap;
-  } else {
+  if (!(g0 < 0.0 && qn > 0.0)) return 0.0;
+  double alpha;
+  if (c2 > 1e-30 && c2 < 1e30)
+    alpha = -0.5 * g0 * piv_rcp(c2);
+  else if (c2 > 0.0)
+    alpha = -g0 / (2.0 * c2);
+  else
+    alpha = sc->alpha_prev > 0.0 ? 2.0 * sc->alpha_prev
+                                 : 0.5 * sqrt((double)m / qn);
+  if (!(alpha * alpha * qn <= (double)m)) alpha = sqrt((double)m / qn);
+  return alpha;
+}
+// What the step leaves in sc (after every reader of alpha_prev).
+__device__ __forceinline__ void line_store(const double* v, double alpha,
+                                           IterScalars* sc) {
+  const double g0 = v[0], c2 = v[1] - v[2];
+  if (!(g0 < 0.0 && v[3] > 0.0))
     sc->restart = 1;  // not a descent direction: restart CG next time
-  }
   sc->alpha = alpha;
-  sc->alpha_prev = alpha > 0.0 ? alpha : sc->alpha_prev;
+  if (alpha > 0.0) sc->alpha_prev = alpha;
   sc->c2 = c2;
   sc->dE = alpha * g0 + alpha * alpha * c2;
 }
@@ -108,8 +136,8 @@ __device__ void line_alpha_block(int m, const double* __restrict__ part,
   for (int p = threadIdx.x; p < nparts; p += blockDim.x)
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] += part[(size_t)p * 4 + q];
-  block_sum<4>(v, red);
-  if (threadIdx.x == 0) line_alpha(m, v, sc);
+  block_sum4(v, red);
+  if (threadIdx.x == 0) line_store(v, line_alpha(m, v, sc), sc);
 }
 
 // ---------------------------------------------------------------------------
@@ -141,32 +169,6 @@ __device__ void line_alpha_block(int m, const double* __restrict__ part,
 // diagonal y_cc = -f_cc / (1 + f_cc). When S - I is small, FP32 arithmetic
 // here yields L to FP64 accuracy relative to I.
 // ---------------------------------------------------------------------------
-// Reciprocal square root and reciprocal of the pivot chain by Newton's
-// method from the hardware approximations (rsqrt, reciprocal): one step in
-// FP32, two from the FP32 seed in FP64. Arguments are positive normal numbers (the pivot
-// tests come first); the results are within a few ulp, and the chain stays
-// free of the slow-path calls of the IEEE operations.
-__device__ __forceinline__ float piv_rcp(float t) {
-  const float r = __fdividef(1.0f, t);
-  return fmaf(r, fmaf(-t, r, 1.0f), r);
-}
-__device__ __forceinline__ double piv_rcp(double t) {
-  double r = (double)__fdividef(1.0f, (float)t);
-  r = fma(r, fma(-t, r, 1.0), r);
-  return fma(r, fma(-t, r, 1.0), r);
-}
-// 1 / sqrt(t): the hardware reciprocal square root refined by Newton's step
-// r <- r (3 - t r^2) / 2, once in FP32, twice (from the FP32 seed) in FP64.
-__device__ __forceinline__ float piv_rsqrt(float t) {
-  const float r = rsqrtf(t);
-  return r * fmaf(-0.5f * t * r, r, 1.5f);
-}
-__device__ __forceinline__ double piv_rsqrt(double t) {
-  double r = (double)rsqrtf((float)t);
-  r = r * fma(-0.5 * t * r, r, 1.5);
-  return r * fma(-0.5 * t * r, r, 1.5);
-}
-
 // Cholesky of a 32 x 32 diagonal block on one warp (Fig. ONFIG step (2)
 // restricted to the block). Lane r holds row r of the block in w (w[j] =
 // entry (r, j), meaningful for j <= r) and ends with row r of L (of F in
@@ -562,16 +564,17 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
 //       X_pj = X_pp W_pj for j < p, X_pp, and L_ip = A_ip X_pp^T for i > p;
 //   (3) every block (i, j), i > p, j <= i, takes M_ij -= L_ip Z_j, with M_ip
 //       starting from zero: the Cholesky update for j > p and the inverse's
-//       for j <= p are the same product, 8 x 4 register tiles. Warp 0 updates
-//       the next diagonal block first and goes on with (1) for it, so the
-//       pivot chain runs beside the updates.
+//       for j <= p are the same product, 8 x 4 register tiles. Four warps
+//       update the next diagonal block first and two go on with (1) for it,
+//       so the pivot chain runs beside the updates.
 // What bounds it is that chain (one dependent rsqrt, multiply, shuffle per
 // column, about 110 cycles) and one SM's FP32 rate. In deviation form (dev,
 // S = I + E, see above) only the diagonal needs care: it holds the deviation
 // d of the pivot from 1, and y_cc = -f_cc / L_cc is kept apart (ydiag).
 // With `split` the inverse goes out as the two TF32 terms the product kernels
-// read (hi, lo, leading dimension ldm; split_diag: the diagonal left out and
-// written as FP32 pairs after them), else as FP64 R = L^{-T}.
+// read (hi, lo, leading dimension ldm, the part below the diagonal left as it
+// is; split_diag: the diagonal zero and written as FP32 pairs after them), else
+// as FP64 R = L^{-T}.
 // ---------------------------------------------------------------------------
 constexpr int PLD = 36, PSZ = 32 * PLD;  // block row stride, block size
 constexpr int kPanelMax = 256;
@@ -584,100 +587,149 @@ inline size_t panel_smem(int m) {
           33 * 32 + 32) * sizeof(float);
 }
 
+// 1 / sqrt(t), t a positive normal number: one instruction and a Newton step
+// (piv_rsqrt without the library call's subnormal path).
+__device__ __forceinline__ float panel_rsqrt(float t) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
+  return r * fmaf(-0.5f * t * r, r, 1.5f);
+}
+
 // Factor the diagonal block D (warp 0; the updated block in shared memory).
 // lcol[c][r] = L_rc (0 for r <= c), rd[c] = 1 / L_cc, ydg[c] = y_cc. Four
-// columns a round, the row shifted by four registers after each, so that every
-// index is static and the code is short. thr: pivot floor of column `lane`.
+// columns a round: within it only the round's own columns are updated, by
+// shuffles; the other columns take the round's rank-4 update from shared memory
+// during the next one, in the shadow of its pivot chain (shuffle, rsqrt with a
+// Newton step, two multiplies: about 100 of the 180 cycles a column takes). The
+// row moves down by four registers a round, so that every index is static and
+// the code is short. thr: pivot floor of column `lane`.
 template <bool dev>
 __device__ __forceinline__ bool panel_factor(const float* D, float thr,
                                              float* lcol, float* rd,
                                              float* ydg) {
   const int lane = threadIdx.x & 31;
-  float w[36];
+  float w[32];
 #pragma unroll
   for (int j = 0; j < 32; j += 4) {
     const float4 t = *reinterpret_cast<const float4*>(D + lane * PLD + j);
     w[j] = t.x; w[j + 1] = t.y; w[j + 2] = t.z; w[j + 3] = t.w;
   }
-  w[32] = w[33] = w[34] = w[35] = 0.f;
   bool bad = false;
+  float dk = 0.f, rk = 1.f;  // pivot and 1 / L_cc of this lane's column
+  float lp[4] = {0.f, 0.f, 0.f, 0.f};  // the round before: its column entries
+  float dn = w[0];  // in lane c: the pivot of column c
 #pragma unroll 1
   for (int g = 0; g < 8; ++g) {
+    float l[4];
+    const float* lv = lcol + 132 * g;   // column 4 g from row 4 g on
+    const float* pv = g ? lv - 128 : lv;  // the round before, from row 4 g on
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int c = 4 * g + u;
-      float d = __shfl_sync(0xffffffffu, w[u], c);
-      float rl;
-      if (dev) {
-        if (!(d > -0.999f)) {  // pivot 1 + d not positive
-          bad = true;
-          d = 0.f;
-        }
-        rl = piv_rsqrt(1.f + d);
+      // (a pivot that is not positive makes everything after it meaningless;
+      // the caller then writes the identity)
+      const float d = __shfl_sync(0xffffffffu, dn, c);
+      const float t = dev ? 1.f + d : d;  // the pivot
+      bad |= !(d > (dev ? -0.999f : __shfl_sync(0xffffffffu, thr, c)));
+      const float rl = panel_rsqrt(t);
+      l[u] = lane > c ? w[u] * rl : 0.f;
+      // the next pivot: its lane has the row's entries itself, so the chain
+      // does not wait for the column's broadcast
+      if (u < 3) {
+        dn = w[u + 1] - l[u] * l[u];
       } else {
-        if (!(d > __shfl_sync(0xffffffffu, thr, c))) {
-          bad = true;
-          d = 1.f;
-        }
-        rl = piv_rsqrt(d);
+        dn = w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) dn -= l[e] * l[e];
       }
-      const float l = lane > c ? w[u] * rl : 0.f;
-      // the next pivot column first: it is the chain's next link
-      const float ln = __shfl_sync(0xffffffffu, l, (c + 1) & 31);
-      w[u + 1] -= l * ln;
-      float* lc = lcol + 32 * c;
-      lc[lane] = l;
+#pragma unroll
+      for (int v = u + 1; v < 4; ++v)
+        w[v] -= l[u] * __shfl_sync(0xffffffffu, l[u], 4 * g + v);
       if (lane == c) {
-        rd[c] = rl;
-        if (dev) ydg[c] = -(d * piv_rcp(1.f + (1.f + d) * rl)) * rl;
+        dk = d;
+        rk = rl;
       }
-      __syncwarp();
-      const float4* lv = reinterpret_cast<const float4*>(lc + 4 * g);
+      // the update by the round before, a quarter of it in each column's
+      // shadow (lp = 0 in the first round, where pv reads unwritten entries)
+      if (g) {
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {  // (past the block: never used again)
-        const float4 b = lv[t];
-        if (4 * t + 0 > u + 1) w[4 * t + 0] -= l * b.x;
-        if (4 * t + 1 > u + 1) w[4 * t + 1] -= l * b.y;
-        if (4 * t + 2 > u + 1) w[4 * t + 2] -= l * b.z;
-        if (4 * t + 3 > u + 1) w[4 * t + 3] -= l * b.w;
+        for (int q = 1 + 2 * u; q < 3 + 2 * u && q < 8; ++q)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float4 b =
+                *reinterpret_cast<const float4*>(pv + 32 * e + 4 * q);
+            w[4 * q + 0] -= lp[e] * b.x;
+            w[4 * q + 1] -= lp[e] * b.y;
+            w[4 * q + 2] -= lp[e] * b.z;
+            w[4 * q + 3] -= lp[e] * b.w;
+          }
       }
+      lcol[32 * c + lane] = l[u];
+      if (lane == 0) rd[c] = rl;
     }
-#pragma unroll
-    for (int j = 0; j < 32; ++j) w[j] = w[j + 4];
+    __syncwarp();
     // columns 4 g .. 4 g + 3 are out: warp 1 may use them
     asm volatile("bar.arrive %0, 64;" ::"r"(1 + g) : "memory");
+    // the next round's own columns now, the others in its shadow
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float4 b = *reinterpret_cast<const float4*>(lv + 32 * e + 4);
+      w[4] -= l[e] * b.x;
+      w[5] -= l[e] * b.y;
+      w[6] -= l[e] * b.z;
+      w[7] -= l[e] * b.w;
+      lp[e] = l[e];
+    }
+#pragma unroll
+    for (int j = 0; j < 28; ++j) w[j] = w[j + 4];
   }
+  // L_cc - 1 = d / (1 + sqrt(1 + d)) with sqrt(1 + d) = (1 + d) rl
+  if (dev) ydg[lane] = -(dk * piv_rcp(1.f + (1.f + dk) * rk)) * rk;
   return bad;
 }
 
-// X = L^{-1} of the diagonal block into D (warp 1, a group behind warp 0):
+// X = L^{-1} of the diagonal block into D (warp 1, a round behind warp 0):
 // lane j runs column j of the forward substitution, right-looking.
 __device__ __forceinline__ void panel_invert(float* D, const float* lcol,
                                              const float* rd) {
   const int lane = threadIdx.x & 31;
-  float a[36];
+  float a[32];
 #pragma unroll
-  for (int i = 0; i < 36; ++i) a[i] = i == lane ? 1.f : 0.f;
+  for (int i = 0; i < 32; ++i) a[i] = i == lane ? 1.f : 0.f;
 #pragma unroll 1
   for (int g = 0; g < 8; ++g) {
     asm volatile("bar.sync %0, 64;" ::"r"(1 + g) : "memory");
+    const float* lv = lcol + 132 * g;
+    const float4 r4 = *reinterpret_cast<const float4*>(rd + 4 * g);
+    const float4 l0 = *reinterpret_cast<const float4*>(lv);
+    const float4 l1 = *reinterpret_cast<const float4*>(lv + 32);
+    const float4 l2 = *reinterpret_cast<const float4*>(lv + 64);
+    float x[4];
+    x[0] = a[0] * r4.x;
+    x[1] = (a[1] - l0.y * x[0]) * r4.y;
+    x[2] = (a[2] - l0.z * x[0] - l1.z * x[1]) * r4.z;
+    x[3] = (a[3] - l0.w * x[0] - l1.w * x[1] - l2.w * x[2]) * r4.w;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = 4 * g + u;
-      const float x = a[u] * rd[c];
-      D[c * PLD + lane] = x;
-      const float4* lv = reinterpret_cast<const float4*>(lcol + 32 * c + 4 * g);
+    for (int u = 0; u < 4; ++u) D[(4 * g + u) * PLD + lane] = x[u];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const float4 b = lv[t];
-        if (4 * t + 0 > u) a[4 * t + 0] -= b.x * x;
-        if (4 * t + 1 > u) a[4 * t + 1] -= b.y * x;
-        if (4 * t + 2 > u) a[4 * t + 2] -= b.z * x;
-        if (4 * t + 3 > u) a[4 * t + 3] -= b.w * x;
+    for (int q = 1; q < 8; ++q) {
+      float4 b[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        b[u] = *reinterpret_cast<const float4*>(lv + 32 * u + 4 * q);
+      const int o = 4 * q - 4;
+      a[o + 0] = a[o + 4];
+      a[o + 1] = a[o + 5];
+      a[o + 2] = a[o + 6];
+      a[o + 3] = a[o + 7];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        a[o + 0] -= b[u].x * x[u];
+        a[o + 1] -= b[u].y * x[u];
+        a[o + 2] -= b[u].z * x[u];
+        a[o + 3] -= b[u].w * x[u];
       }
     }
-#pragma unroll
-    for (int j = 0; j < 32; ++j) a[j] = a[j + 4];
   }
 }
 
@@ -712,6 +764,26 @@ __device__ __forceinline__ void panel_update(float* B, const float* Z, int ldz,
   for (int u = 0; u < 8; ++u) row[u * (PLD / 4)] = acc[u];
 }
 
+// The update of the next diagonal block, rows 8 h .. +7 on this warp (lane
+// (ti, tj): two rows, four columns): the pivot chain waits for it, so four
+// warps share it.
+__device__ __forceinline__ void panel_update_quarter(float* B, const float* Zd,
+                                                     int ldz, int h) {
+  const int lane = threadIdx.x & 31, ti = lane >> 3, tj = lane & 7;
+  const int r = 8 * h + 2 * ti;
+  float4* row = reinterpret_cast<float4*>(B + r * PLD + 4 * tj);
+  float4 a0 = row[0], a1 = row[PLD / 4];
+#pragma unroll 8
+  for (int k = 0; k < 32; ++k) {
+    const float2 l = *reinterpret_cast<const float2*>(Zd + k * ldz + r);
+    const float4 b = *reinterpret_cast<const float4*>(Zd + k * ldz + 4 * tj);
+    a0.x -= l.x * b.x; a0.y -= l.x * b.y; a0.z -= l.x * b.z; a0.w -= l.x * b.w;
+    a1.x -= l.y * b.x; a1.y -= l.y * b.y; a1.z -= l.y * b.z; a1.w -= l.y * b.w;
+  }
+  row[0] = a0;
+  row[PLD / 4] = a1;
+}
+
 struct PanelOut {
   double* Linv = nullptr;  // may be null
   double* R = nullptr;     // FP64 L^{-T} (when split is null)
@@ -738,62 +810,107 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
   float* rd = lcol + 33 * 32;
   auto blk = [&](int i, int j) { return M + (panel_blocks(i) + j) * PSZ; };
   if (tid == 0) bad = 0;
-  if (lpart) {  // the line step first (it sets sc->alpha)
-    __shared__ double lq[4];
-    if (warp < 4) {
-      double v = 0.0;
-      for (int k = lane; k < nlpart; k += 32) v += lpart[4 * (size_t)k + warp];
-      v = warp_sum(v);
-      if (lane == 0) lq[warp] = v;
-    }
-    __syncthreads();
-    if (tid == 0) line_alpha(m, lq, sc);
-    __syncthreads();
-  }
-  // S (or S(a)) into the blocks, minus I in deviation form; the padding is the
-  // identity. Both orientations of B and Q are read along their columns, the
-  // second one added after a barrier. A unit is eight columns of a block.
+  // S (or S(a) from B and Q) into the blocks, minus I in deviation form; the
+  // padding is the identity. A unit is eight columns of a block, read along
+  // its columns; with B and Q the mirrored unit is added after a barrier.
   const int units = 4 * panel_blocks(P);
-  const float al = Bf ? (float)sc->alpha : 0.f;
-  const float hq = Bf ? (float)(0.5 * sc->alpha * sc->alpha) : 0.f;
-  for (int pass = 0; pass < (Bf ? 2 : 1); ++pass) {
-    for (int u = warp; u < units; u += nw) {
-      int bi = 0;
-      while (panel_blocks(bi + 1) <= (u >> 2)) ++bi;
-      const int bj = (u >> 2) - panel_blocks(bi), g = 8 * (u & 3);
-      float* D = blk(bi, bj);
-      // pass 0: column 32 bj + g + q, row 32 bi + lane of the matrix;
-      // pass 1: its mirror, column 32 bi + g + q, row 32 bj + lane
-      const int row = 32 * (pass ? bj : bi) + lane;
-      const int col = 32 * (pass ? bi : bj) + g;
-      float v[8];
-      if (Bf) {
+  struct Unit {
+    int bi, bj, g;
+  };
+  auto unit = [&](int u) {
+    int bi = 0;
+    while (panel_blocks(bi + 1) <= (u >> 2)) ++bi;
+    return Unit{bi, (u >> 2) - panel_blocks(bi), 8 * (u & 3)};
+  };
+  auto load = [&](int u, bool mirror, float (&b)[8], float (&q)[8]) {
+    const Unit t = unit(u);
+    const int row = 32 * (mirror ? t.bj : t.bi) + lane;
+    const int col = 32 * (mirror ? t.bi : t.bj) + t.g;
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          v[q] = row < m && col + q < m
-                     ? al * Bf[row + (col + q) * m] + hq * Qf[row + (col + q) * m]
-                     : 0.f;
-      } else {
+    for (int e = 0; e < 8; ++e) {
+      const bool in = row < m && col + e < m;
+      b[e] = in ? Bf[row + (col + e) * m] : 0.f;
+      q[e] = in ? Qf[row + (col + e) * m] : 0.f;
+    }
+  };
+  if (Bf) {
+    // (the loads of three units are in flight while the line step is formed)
+    constexpr int NU = 3;
+    float b[NU][8], q[NU][8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          v[q] = row < m && col + q < m
-                     ? (float)(S[row + (col + q) * m] -
-                               (dev && row == col + q ? 1.0 : 0.0))
-                     : 0.f;
+    for (int k = 0; k < NU; ++k)
+      if (warp + k * nw < units) load(warp + k * nw, false, b[k], q[k]);
+    float al, hq;
+    if (lpart) {  // the line step (it sets sc->alpha)
+      __shared__ double lq[4], la;
+      if (warp < 4) {
+        double v = lane < nlpart ? lpart[4 * (size_t)lane + warp] : 0.0;
+        for (int k = lane + 32; k < nlpart; k += 32)
+          v += lpart[4 * (size_t)k + warp];
+        v = warp_sum(v);
+        if (lane == 0) lq[warp] = v;
       }
-      if (pass == 0) {
+      __syncthreads();
+      if (tid == 0) la = line_alpha(m, lq, sc);
+      __syncthreads();
+      al = (float)la;
+      hq = (float)(0.5 * la * la);
+      if (tid == kPanelThreads - 1) line_store(lq, la, sc);
+    } else {
+      al = (float)sc->alpha;
+      hq = (float)(0.5 * sc->alpha * sc->alpha);
+    }
+    for (int base = warp; base < units; base += NU * nw) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          if (!dev && row == col + q && (Bf || row >= m)) v[q] += 1.f;
-          D[lane * PLD + g + q] = v[q];
-        }
-      } else {
+      for (int k = 0; k < NU; ++k) {
+        const int u = base + k * nw;
+        if (u >= units) break;
+        if (base != warp) load(u, false, b[k], q[k]);
+        const Unit t = unit(u);
+        const int row = 32 * t.bi + lane, col = 32 * t.bj + t.g;
+        float v[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) D[(g + q) * PLD + lane] += v[q];
+        for (int e = 0; e < 8; ++e)
+          v[e] = al * b[k][e] + hq * q[k][e] +
+                 (!dev && row == col + e ? 1.f : 0.f);
+        float4* D =
+            reinterpret_cast<float4*>(blk(t.bi, t.bj) + lane * PLD + t.g);
+        D[0] = make_float4(v[0], v[1], v[2], v[3]);
+        D[1] = make_float4(v[4], v[5], v[6], v[7]);
       }
     }
+#pragma unroll
+    for (int k = 0; k < NU; ++k)
+      if (warp + k * nw < units) load(warp + k * nw, true, b[k], q[k]);
     __syncthreads();
+    for (int base = warp; base < units; base += NU * nw) {
+#pragma unroll
+      for (int k = 0; k < NU; ++k) {
+        const int u = base + k * nw;
+        if (u >= units) break;
+        if (base != warp) load(u, true, b[k], q[k]);
+        const Unit t = unit(u);
+        float* D = blk(t.bi, t.bj) + t.g * PLD + lane;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) D[e * PLD] += al * b[k][e] + hq * q[k][e];
+      }
+    }
+  } else {
+    for (int u = warp; u < units; u += nw) {
+      const Unit t = unit(u);
+      const int row = 32 * t.bi + lane, col = 32 * t.bj + t.g;
+      float* D = blk(t.bi, t.bj) + lane * PLD + t.g;
+      double v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        v[e] = row < m && col + e < m
+                   ? S[row + (col + e) * m] - (dev && row == col + e ? 1.0 : 0.0)
+                   : (!dev && row == col + e ? 1.0 : 0.0);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) D[e] = (float)v[e];
+    }
   }
+  __syncthreads();
   auto diag = [&](int p) {  // warps 0 and 1
     if (warp == 0) {
       float thr = 0.f;
@@ -878,9 +995,9 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
     // (3) block updates; row p takes its final values X_pj from Z
     const int nupd = panel_blocks(P) - panel_blocks(p + 1);
     const bool more = p + 1 < P;
-    if (more && warp == 0) {
-      panel_update(blk(p + 1, p + 1), Z, ldz, 32 * (p + 1), 32 * (p + 1), false);
-      __syncwarp();
+    if (more && warp < 4) {
+      panel_update_quarter(blk(p + 1, p + 1), Z + 32 * (p + 1), ldz, warp);
+      asm volatile("bar.sync 9, 128;" ::: "memory");
     }
     if (more && warp < 2) {
       diag(p + 1);
@@ -892,7 +1009,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
           int bi = p + 1;
           while (panel_blocks(bi + 1) <= b) ++bi;
           const int bj = b - panel_blocks(bi);
-          if (bi == p + 1 && bj == p + 1) continue;  // warp 0 has it
+          if (bi == p + 1 && bj == p + 1) continue;  // done above
           panel_update(blk(bi, bj), Z, ldz, 32 * bi, 32 * bj, bj == p);
         } else {
           const int bj = u - nupd;
@@ -921,30 +1038,48 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
     float* hi = out.split;
     float* lo = hi + (size_t)out.ldm * m;
     float* dg = lo + (size_t)out.ldm * m;
-    for (int i = warp; i < m; i += nw)
-      for (int k = lane; k < out.ldm; k += 32) {
-        float h = 0.f, l = 0.f;
-        if (k < i) {
-          const float x = entry(k, i);
-          h = tc::tf32_rna(x);
-          l = tc::tf32_rna(x - h);
-        } else if (k == i) {
-          const float y = dfull(i);
-          if (out.split_diag) {
-            const F2 d = dev ? two_sum(1.f, y) : F2{y, 0.f};
-            dg[i] = d.h;
-            dg[m + i] = d.l;
-          } else if (dev) {
-            h = tc::tf32_rna(1.f + y);
-            l = tc::tf32_rna(y - (h - 1.f));
-          } else {
-            h = tc::tf32_rna(y);
-            l = tc::tf32_rna(y - h);
+    // Four entries of a column per lane at a time. Only the triangle: the zeros
+    // below it stay from the buffer's allocation (one SM's stores, not the
+    // arithmetic, are what this phase takes).
+    for (int i = warp; i < m; i += nw) {
+      const float* X = blk(i >> 5, 0) + (i & 31) * PLD + lane;
+      float* ph = hi + (size_t)i * out.ldm;
+      float* pl = lo + (size_t)i * out.ldm;
+      for (int k0 = 0; k0 < i; k0 += 128) {
+        float x[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int k = k0 + 32 * e + lane;
+          x[e] = k < i && !isbad ? X[((k0 >> 5) + e) * PSZ] : 0.f;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int k = k0 + 32 * e + lane;
+          if (k < i) {
+            const float h = tc::tf32_rna(x[e]);
+            ph[k] = h;
+            pl[k] = tc::tf32_rna(x[e] - h);
           }
         }
-        hi[k + (size_t)i * out.ldm] = h;
-        lo[k + (size_t)i * out.ldm] = l;
       }
+    }
+    for (int i = tid; i < m; i += kPanelThreads) {  // the diagonal
+      const float y = dfull(i);
+      float h = 0.f, l = 0.f;
+      if (out.split_diag) {
+        const F2 d = dev ? two_sum(1.f, y) : F2{y, 0.f};
+        dg[i] = d.h;
+        dg[m + i] = d.l;
+      } else if (dev) {
+        h = tc::tf32_rna(1.f + y);
+        l = tc::tf32_rna(y - (h - 1.f));
+      } else {
+        h = tc::tf32_rna(y);
+        l = tc::tf32_rna(y - h);
+      }
+      hi[i + (size_t)i * out.ldm] = h;
+      lo[i + (size_t)i * out.ldm] = l;
+    }
   } else {
     for (int i = warp; i < m; i += nw)
       for (int k = lane; k < m; k += 32)
@@ -1276,17 +1411,39 @@ __global__ void __launch_bounds__(1024)
       }
     }
   }
-  double v[4] = {(double)v0, (double)v1, (double)v2, (double)v3};
-  if (tr_parts && ks == 0) {
-    // tr(P^T H P) as the sum of the stencil's partial column dots, each
-    // first-split CTA adding a fixed share
-    const int cta = blockIdx.y * gridDim.x + blockIdx.x;
-    const int ncta = gridDim.x * gridDim.y;
-    for (int k = cta * blockDim.x + threadIdx.x; k < n_tr_parts;
-         k += ncta * blockDim.x)
-      v[1] += tr_parts[k];
+  // the sums over the CTA: FP64, or for FP32 terms double-float pairs within
+  // each warp (an FP64 add of every thread would take most of the kernel)
+  double v[4];
+  const int cta = blockIdx.y * gridDim.x + blockIdx.x;
+  const int ncta = gridDim.x * gridDim.y;
+  if constexpr (sizeof(Tm) == 4) {
+    F2 p[4] = {{v0, 0.f}, {v1, 0.f}, {v2, 0.f}, {v3, 0.f}};
+    if (tr_parts && ks == 0)
+      // tr(P^T H P) as the sum of the stencil's partial column dots, each
+      // first-split CTA adding a fixed share
+      for (int k = cta * blockDim.x + threadIdx.x; k < n_tr_parts;
+           k += ncta * blockDim.x)
+        p[1] = df_add(p[1], df_of_bits(tr_parts[k]));
+    const F2 t = warp_sum4(
+        p,
+        [](F2 x, int o) {
+          return F2{__shfl_xor_sync(0xffffffffu, x.h, o),
+                    __shfl_xor_sync(0xffffffffu, x.l, o)};
+        },
+        [](F2 x, F2 y) { return df_add(x, y); });
+    if ((tx & 7) == 0) red[(tx >> 3) * 32 + ty] = to_f64(t.h) + to_f64(t.l);
+    block_sum4_finish(v, red, blockDim.x >> 5);
+  } else {
+    v[0] = v0;
+    v[1] = v1;
+    v[2] = v2;
+    v[3] = v3;
+    if (tr_parts && ks == 0)
+      for (int k = cta * blockDim.x + threadIdx.x; k < n_tr_parts;
+           k += ncta * blockDim.x)
+        v[1] += tr_parts[k];
+    block_sum4(v, red);
   }
-  block_sum<4>(v, red);
   if (threadIdx.x == 0) {
     const size_t b =
         ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -1515,11 +1672,6 @@ void mm_gemm(int m, const double* A, bool trA, const double* B, bool trB,
     k_mm_gemm<float><<<grid, 256, 0, s>>>(m, A, trA, B, trB, Cm, alpha, beta);
   else
     k_mm_gemm<double><<<grid, 256, 0, s>>>(m, A, trA, B, trB, Cm, alpha, beta);
-  TRM_CHECK_LAUNCH();
-}
-
-void zero_diag(int m, double* A, cudaStream_t s, float* A32) {
-  k_zero_diag<<<ceil_div(m, 256), 256, 0, s>>>(m, A, A32);
   TRM_CHECK_LAUNCH();
 }
 

@@ -245,7 +245,7 @@ size_t Solver::footprint(int64_t N, int m) {
   b += std::max<size_t>(1, (size_t)ceil_div(N, 256) * m) * 8;  // P's dots
   b += sym_eig_work_doubles(m) * 8 + 5 * mm * 4;
   b += part_capacity(N, m) * 8 + sizeof(IterScalars) + 16;
-  b += mul_tc_work_floats(m, m) * 4;
+  b += 2 * mul_tc_work_floats(m, m) * 4;
   b += (size_t)N * (8 + 4 + 4 + 8 + 4 + 8);  // diagonals, M, V
   return b + (64u << 10);                    // allocation granularity
 }
@@ -306,6 +306,9 @@ Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
   tw_.msplit_floats = mul_tc_work_floats(m, m);
   tw_.msplit = f(tw_.msplit_floats);
   tw_.err = &sc_->status;
+  rw_ = tw_;
+  rw_.msplit = f(rw_.msplit_floats);
+  TRM_CUDA(cudaMemsetAsync(rw_.msplit, 0, rw_.msplit_floats * 4, s_));
   diag64_ = d(N);
   diag32_ = f(N);
   diaglo_ = f(N);
@@ -547,6 +550,17 @@ bool Solver::line_grams_fusable(const T* C, const T* P, const T* G) const {
   }
 }
 
+// H' of an FP32 phase: its diagonal set to zero (Sec. 2.2), an FP32 copy for the
+// line model and, as far as the tensor cores run, the gradient's operand.
+GramOut Solver::hprime_out() const {
+  GramOut o;
+  o.f32 = Hp32_;
+  o.split = tw_.msplit;
+  o.split_ldm = mul_tc_ldm(m_);
+  o.zero_diag = 1;
+  return o;
+}
+
 template <typename T>
 void Solver::line_grams_fused(const T* C, const T* P, const T* G) {
   if constexpr (sizeof(T) == 4) {
@@ -558,10 +572,12 @@ void Solver::line_grams_fused(const T* C, const T* P, const T* G) {
     a.cols = b.cols = m_;
     a.count = b.count = 3;
     const double nm = (double)N_ * m_, m2N = nm * m_;
+    GramOut also;
+    also.f32 = Bm32_;
     // algorithmic: 2 m^2 N per product, m^2 N for the symmetric one
     TRM_PROF(KC_GRAM32, 5 * m2N, 12 * nm,
              gram_tc_pairs(N_, m_, a, b, Bm_, part_, part_cap_, &sc_->status,
-                           s_, Bm32_, /*sym_seg=*/1));
+                           s_, also, /*sym_seg=*/1));
   }
 }
 
@@ -619,16 +635,19 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
   bx.cols = m_;
   bx.count = 1;
   // FP32 phases also get FP32 copies of the m x m Gram results
-  float* const hp32 = sizeof(T) == 4 ? Hp32_ : nullptr;
-  float* const bm32 = sizeof(T) == 4 ? Bm32_ : nullptr;
-  float* const pg32 = sizeof(T) == 4 ? PG32_ : nullptr;
+  GramOut hp_also, bm_also, pg_also;
+  if (sizeof(T) == 4) {
+    hp_also = hprime_out();
+    bm_also.f32 = Bm32_;
+    pg_also.f32 = PG32_;
+  }
+  bool hsplit = false;  // H' is in tw_.msplit as the gradient reads it
   TRM_PROF(kgr, 2 * m2N, 2 * es * nm,
-           gram<T>(N_, m_, C, bx, Hp_, part_, part_cap_, s_, &sc_->status,
-                   hp32));                                            // (6)
-  if (sizeof(T) == 4) zero_diag(m_, Hp_, s_, hp32);
+           hsplit = gram<T>(N_, m_, C, bx, Hp_, part_, part_cap_, s_,
+                            &sc_->status, hp_also));                  // (6)
   TRM_PROF(kgd, 2 * m2N, 5 * es * nm,
            gradient<T>(N_, m_, Yc, X, Hp_, G, Gp, P, minv, sc_, part_,
-                       part_cap_, s_, &tw_));                         // (7)
+                       part_cap_, s_, &tw_, hsplit));                 // (7)
   TRM_PROF(KC_ROWOPS, 2 * nm, 3 * es * nm,
            update_p<T>(N_, m_, G, P, minv, sc_, s_));                 // P
   const bool fused = !gen && line_grams_fusable<T>(C, P, G);
@@ -662,7 +681,7 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
     bp.count = 1;
     TRM_PROF(kgr, 2 * m2N, 2 * es * nm,
              gram<T>(N_, m_, Yc, bp, Bm_, part_, part_cap_, s_, &sc_->status,
-                     bm32));                                     // C^T (S) P
+                     bm_also));                                  // C^T (S) P
     Blocks<T> b3;
     b3.p[0] = SPt;
     b3.p[1] = HP;
@@ -671,7 +690,7 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
     b3.count = 3;
     TRM_PROF(kgr, 6 * m2N, 4 * es * nm,
              gram<T>(N_, m_, P, b3, PG_, part_, part_cap_, s_, &sc_->status,
-                     pg32));                                          // P^T[P HP G]
+                     pg_also));                                       // P^T[P HP G]
   }
   const double m3 = md * md * md;
   prof.begin(KC_SMALL, s_);
@@ -683,7 +702,7 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
                     (!gen || rotate_on_tc(N_, m_, Yc, SPt, &tw_));
     if (line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
                       PG32_ + woff, R_, sc_, mmw_, T1_, s_,
-                      tc ? tw_.msplit : nullptr, mul_tc_ldm(m_)))
+                      tc ? rw_.msplit : nullptr, mul_tc_ldm(m_)))
       R = nullptr;
   } else
     line_factor<Tm>(m_, Hp_, HD_, Bm_, PG_, hpd, m_ + 1, trp, ntrp,
@@ -691,7 +710,8 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
                     sizeof(Tm) == 4, s_);
   prof.end(KC_SMALL, 4 * m3 + 2 * m3 / 3, 0.0, s_);
   TRM_PROF(krt, m2N, 3 * es * nm,
-           (rotate<T, T>(N_, m_, C, P, R, Cn, sc_, s_, &tw_)));  // (C+aP)L^-T
+           (rotate<T, T>(N_, m_, C, P, R, Cn, sc_, s_,
+                         R ? &tw_ : &rw_)));  // (C+aP)L^-T
   if (gen) {  // S (C + aP) L^-T = (Y + a S P) L^-T
     if constexpr (sizeof(T) == 8) {
       TRM_PROF(krt, m2N, 3 * es * nm,
@@ -701,7 +721,7 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
     } else {
       TRM_PROF(krt, m2N, 3 * es * nm,
                (rotate<float, float>(N_, m_, Y32_, SP32_, R, Y32n_, sc_, s_,
-                                     &tw_)));
+                                     R ? &tw_ : &rw_)));
       std::swap(Y32_, Y32n_);
     }
   }
@@ -752,13 +772,13 @@ void Solver::iter_mp2() {
   bx.p[0] = X32_;
   bx.cols = m_;
   bx.count = 1;
+  bool hsplit = false;
   TRM_PROF(KC_GRAM32, 2 * m2N, 8 * dnm,
-           gram<float>(N_, m_, Ch, bx, Hp_, part_, part_cap_, s_, &sc_->status,
-                       Hp32_));                                       // (6)
-  zero_diag(m_, Hp_, s_, Hp32_);
+           hsplit = gram<float>(N_, m_, Ch, bx, Hp_, part_, part_cap_, s_,
+                                &sc_->status, hprime_out()));         // (6)
   TRM_PROF(KC_GRAD32, 2 * m2N, 20 * dnm,
            gradient<float>(N_, m_, Ch, X32_, Hp_, G, Gp, P, minv, sc_,
-                           part_, part_cap_, s_, &tw_));      // (7)
+                           part_, part_cap_, s_, &tw_, hsplit));      // (7)
   TRM_PROF(KC_ROWOPS, 2 * dnm, 12 * dnm,
            update_p<float>(N_, m_, G, P, minv, sc_, s_));
   const bool fused = line_grams_fusable<float>(Ch, P, G);
@@ -774,6 +794,9 @@ void Solver::iter_mp2() {
     ntrp = chunks * m_;
     line_grams_fused<float>(Ch, P, G);
   } else {
+    GramOut bm_also, pg_also;
+    bm_also.f32 = Bm32_;
+    pg_also.f32 = PG32_;
     TRM_PROF(KC_SPMM32, f32, b32, apply_h(op_, P, HP, m_, s_));
     hpd = PG_ + mm;  // the diagonal of P^T H P, stride m + 1
     woff = 2 * mm;
@@ -783,7 +806,7 @@ void Solver::iter_mp2() {
     bp.count = 1;
     TRM_PROF(KC_GRAM32, 2 * m2N, 8 * dnm,
              gram<float>(N_, m_, Ch, bp, Bm_, part_, part_cap_, s_,
-                         &sc_->status, Bm32_));
+                         &sc_->status, bm_also));
     Blocks<float> b3;
     b3.p[0] = P;
     b3.p[1] = HP;
@@ -792,20 +815,20 @@ void Solver::iter_mp2() {
     b3.count = 3;
     TRM_PROF(KC_GRAM32, 6 * m2N, 16 * dnm,
              gram<float>(N_, m_, P, b3, PG_, part_, part_cap_, s_,
-                         &sc_->status, PG32_));
+                         &sc_->status, pg_also));
   }
   prof.begin(KC_SMALL, s_);
   const bool tc = rotate_on_tc(N_, m_, Ch, P, &tw_);
   const double* R = R_;
   if (line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
                     PG32_ + woff, R_, sc_, mmw_, T1_, s_,
-                    tc ? tw_.msplit : nullptr, mul_tc_ldm(m_),
+                    tc ? rw_.msplit : nullptr, mul_tc_ldm(m_),
                     /*split_diag=*/true))
     R = nullptr;
   prof.end(KC_SMALL, 4 * m3 + 2 * m3 / 3, 0.0, s_);
   TRM_PROF(KC_ROTDF, m2N, 24 * dnm,
            rotate_split_df(N_, m_, Ch, Cl, P, R, Cdfn_, Cdfn_ + nm, sc_, s_,
-                           &tw_));
+                           R ? &tw_ : &rw_));
   std::swap(Cdf_, Cdfn_);
   std::swap(Gb_[0], Gb_[1]);
 }
@@ -1338,14 +1361,15 @@ void Solver::energy_gradient(const double* C, double* E, double* HD,
   apply_h(op_, C, X64_, m_, s_);
   energy_diag<double>(N_, m_, C, X64_, HD_, sc_, part_, s_);
   set_restart();
+  GramOut also;
+  also.zero_diag = zdiag != 0;
   if (G_dtype == TRM_F64) {
     xprime<double>(N_, m_, C, X64_, HD_, nullptr, nullptr, s_);
     Blocks<double> b;
     b.p[0] = X64_;
     b.cols = m_;
     b.count = 1;
-    gram<double>(N_, m_, C, b, Hp_, part_, part_cap_, s_, &sc_->status);
-    if (zdiag) zero_diag(m_, Hp_, s_);
+    gram<double>(N_, m_, C, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
     gradient<double>(N_, m_, C, X64_, Hp_, static_cast<double*>(G), nullptr,
                      nullptr, nullptr, sc_, part_, part_cap_, s_);
   } else if (G_dtype == TRM_F32) {
@@ -1354,8 +1378,7 @@ void Solver::energy_gradient(const double* C, double* E, double* HD,
     b.p[0] = X32_;
     b.cols = m_;
     b.count = 1;
-    gram<float>(N_, m_, C32_, b, Hp_, part_, part_cap_, s_, &sc_->status);
-    if (zdiag) zero_diag(m_, Hp_, s_);
+    gram<float>(N_, m_, C32_, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
     gradient<float>(N_, m_, C32_, X32_, Hp_, static_cast<float*>(G), nullptr,
                     nullptr, nullptr, sc_, part_, part_cap_, s_, &tw_);
   } else {

@@ -132,6 +132,7 @@ class Solver {
   // the FP32 blocks are eligible.
   template <typename T>
   bool line_grams_fusable(const T* C, const T* P, const T* G) const;
+  GramOut hprime_out() const;
   template <typename T>
   void line_grams_fused(const T* C, const T* P, const T* G);
   // CUDA graphs of block iterations. An iteration is a fixed kernel
@@ -193,6 +194,8 @@ class Solver {
   size_t part_cap_;
   IterScalars* sc_;
   TcWork tw_;  // tensor-core product workspace (error word in sc_->status)
+  TcWork rw_;  // the same for the factor as line_factor32 writes it: upper
+               // triangle only, zero below since its allocation
   IterScalars* ring_ = nullptr;  // pinned host ring of per-iteration scalars
   std::vector<cudaEvent_t> ev_;
   int state_ = 0;  // 0: C64 current, 1: C32 current
