@@ -615,11 +615,36 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
   return z ^ (z >> 31);
 }
 
-__global__ void k_random(int64_t total, uint64_t seed, double* __restrict__ C) {
+__global__ void k_random(int64_t N, int64_t total, int64_t ld, uint64_t seed,
+                         double* __restrict__ C) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
     const uint64_t u = splitmix64(seed ^ splitmix64((uint64_t)i));
-    C[i] = (double)(u >> 11) * 0x1.0p-53 - 0.5;
+    const int64_t o = ld == N ? i : i + (i / N) * (ld - N);
+    C[o] = (double)(u >> 11) * 0x1.0p-53 - 0.5;
+  }
+}
+
+template <typename T>
+__global__ void k_copy_columns(int64_t N, const T* __restrict__ src,
+                               int64_t lds, T* __restrict__ dst, int64_t ldd) {
+  const T* a = src + (int64_t)blockIdx.y * lds;
+  T* b = dst + (int64_t)blockIdx.y * ldd;
+#pragma unroll 4
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
+       i += (int64_t)gridDim.x * blockDim.x)
+    b[i] = a[i];
+}
+
+__global__ void k_clear_pad(PadList l, int64_t N, int64_t ld, int m) {
+  const int w = (int)(ld - N), b = blockIdx.y;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < w * m;
+       e += gridDim.x * blockDim.x) {
+    const size_t o = (size_t)(e / w) * ld + N + e % w;
+    if (l.es[b] == 8)
+      static_cast<double*>(l.p[b])[o] = 0.0;
+    else
+      static_cast<float*>(l.p[b])[o] = 0.f;
   }
 }
 
@@ -807,6 +832,26 @@ void fix_signs(int64_t N, int m, double* C, double* X, double* work,
   TRM_CHECK_LAUNCH();
 }
 
+template <typename T>
+void copy_columns(int64_t N, int m, const T* src, int64_t lds, T* dst,
+                  int64_t ldd, cudaStream_t s) {
+  k_copy_columns<T><<<dim3(elem_grid_x(N), m), 256, 0, s>>>(N, src, lds, dst,
+                                                            ldd);
+  TRM_CHECK_LAUNCH();
+}
+template void copy_columns<float>(int64_t, int, const float*, int64_t, float*,
+                                  int64_t, cudaStream_t);
+template void copy_columns<double>(int64_t, int, const double*, int64_t,
+                                   double*, int64_t, cudaStream_t);
+
+void clear_pad_rows(const PadList& l, int64_t N, int64_t ld, int m,
+                    cudaStream_t s) {
+  if (ld == N || l.n == 0) return;
+  k_clear_pad<<<dim3(ceil_div((ld - N) * m, 256), l.n), 256, 0, s>>>(l, N, ld,
+                                                                    m);
+  TRM_CHECK_LAUNCH();
+}
+
 void to_f32(const double* x, float* y, int64_t n, cudaStream_t s) {
   k_to_f32<<<elem_grid_x(n), 256, 0, s>>>(x, y, n);
   TRM_CHECK_LAUNCH();
@@ -816,8 +861,9 @@ void to_f64(const float* x, double* y, int64_t n, cudaStream_t s) {
   TRM_CHECK_LAUNCH();
 }
 
-void random_block(int64_t N, int m, uint64_t seed, double* C, cudaStream_t s) {
-  k_random<<<elem_grid_x(N * m), 256, 0, s>>>(N * m, seed, C);
+void random_block(int64_t N, int m, uint64_t seed, double* C, cudaStream_t s,
+                  int64_t ld) {
+  k_random<<<elem_grid_x(N * m), 256, 0, s>>>(N, N * m, ld ? ld : N, seed, C);
   TRM_CHECK_LAUNCH();
 }
 

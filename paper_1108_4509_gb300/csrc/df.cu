@@ -87,7 +87,7 @@ constexpr int kCols = 4;  // columns per CTA (grid.y walks column groups)
 // X = H C for the stencil operator, one grid point per thread.
 template <int R>
 __global__ void __launch_bounds__(256)
-    k_stencil_df(StencilOp st, int64_t N, const float* __restrict__ dh,
+    k_stencil_df(StencilOp st, int64_t N, int64_t ld, const float* __restrict__ dh,
                  const float* __restrict__ dl, const float* __restrict__ Ch,
                  const float* __restrict__ Cl, float* __restrict__ Xh,
                  float* __restrict__ Xl, int ncols) {
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(256)
   for (int q = 0; q < kCols; ++q) {
     const int c = cb + q;
     if (c >= ncols) break;
-    const int64_t base = (int64_t)c * N + i;
+    const int64_t base = (int64_t)c * ld + i;
     const float* ph = Ch + base;
     const float* pl = Cl + base;
     Acc s1, s2;
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(256)
 
 // X = H C for a CSR operator (values split into hi + lo at creation).
 __global__ void __launch_bounds__(256)
-    k_csr_df(int64_t N, const int32_t* __restrict__ rowptr,
+    k_csr_df(int64_t N, int64_t ld, const int32_t* __restrict__ rowptr,
              const int32_t* __restrict__ cols, const float* __restrict__ vh,
              const float* __restrict__ vl, const float* __restrict__ Ch,
              const float* __restrict__ Cl, float* __restrict__ Xh,
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(256)
   for (int q = 0; q < kCols; ++q) {
     const int c = cb + q;
     if (c >= ncols) break;
-    const int64_t off = (int64_t)c * N;
+    const int64_t off = (int64_t)c * ld;
     F2 acc = {0.f, 0.f};
     for (int k = b; k < e; ++k) {
       const int64_t j = off + cols[k];
@@ -412,13 +412,13 @@ void apply_h_df(const Operator& op, const float* Ch, const float* Cl,
           op.st, op.N, op.diag32, op.diaglo, Ch, Cl, Xh, Xl, ncols, nullptr);
   } else if (op.kind == 0) {
     if (op.st.radius == 1)
-      k_stencil_df<1><<<grid, 256, 0, s>>>(op.st, op.N, op.diag32, op.diaglo,
+      k_stencil_df<1><<<grid, 256, 0, s>>>(op.st, op.N, op.ld, op.diag32, op.diaglo,
                                            Ch, Cl, Xh, Xl, ncols);
     else
-      k_stencil_df<2><<<grid, 256, 0, s>>>(op.st, op.N, op.diag32, op.diaglo,
+      k_stencil_df<2><<<grid, 256, 0, s>>>(op.st, op.N, op.ld, op.diag32, op.diaglo,
                                            Ch, Cl, Xh, Xl, ncols);
   } else {
-    k_csr_df<<<grid, 256, 0, s>>>(op.N, op.csr.rowptr, op.csr.cols,
+    k_csr_df<<<grid, 256, 0, s>>>(op.N, op.ld, op.csr.rowptr, op.csr.cols,
                                   op.csr.valshi, op.csr.valslo, Ch, Cl, Xh,
                                   Xl, ncols);
   }

@@ -28,6 +28,7 @@ struct CsrOp {
 struct Operator {
   int kind = 0;  // 0 stencil, 1 csr
   int64_t N = 0;
+  int64_t ld = 0;  // entries between the columns of a block
   StencilOp st;
   CsrOp csr;
   const double* diag64 = nullptr;  // H_ii
@@ -285,7 +286,27 @@ void fix_signs(int64_t N, int m, double* C, double* X, double* work,
                cudaStream_t s);
 void to_f32(const double* x, float* y, int64_t n, cudaStream_t s);
 void to_f64(const float* x, double* y, int64_t n, cudaStream_t s);
-void random_block(int64_t N, int m, uint64_t seed, double* C, cudaStream_t s);
+// N x m entries between blocks whose columns are lds and ldd entries apart
+template <typename T>
+void copy_columns(int64_t N, int m, const T* src, int64_t lds, T* dst,
+                  int64_t ldd, cudaStream_t s);
+// Blocks whose rows N .. ld - 1 clear_pad_rows sets to zero (element sizes 4
+// and 8; null pointers are skipped).
+struct PadList {
+  void* p[32];
+  int es[32];
+  int n = 0;
+  void add(void* q, int e) {
+    if (!q || n == 32) return;
+    p[n] = q;
+    es[n++] = e;
+  }
+};
+void clear_pad_rows(const PadList& l, int64_t N, int64_t ld, int m,
+                    cudaStream_t s);
+// (ld: entries between columns, 0 for N)
+void random_block(int64_t N, int m, uint64_t seed, double* C, cudaStream_t s,
+                  int64_t ld = 0);
 
 // ---------------------------------------------------------------------------
 // m x m FP64 matrices on the device

@@ -238,7 +238,8 @@ size_t Solver::part_capacity(int64_t N, int m) {
 
 // Device bytes the constructor (and a stencil's potential) allocates; used
 // to admit requests by footprint.
-size_t Solver::footprint(int64_t N, int m) {
+size_t Solver::footprint(int64_t n_rows, int m) {
+  const int64_t N = padded(n_rows);
   const size_t nm = (size_t)N * m, mm = (size_t)m * m;
   size_t b = nm * (3 * 8 + 3 * 4 + 3 * 8 + 4 * 8);  // blocks
   b += mm * 8 * 13 + std::max(2 * mm, chol_work_elems(m)) * 8 + 4 * m * 8;
@@ -251,10 +252,10 @@ size_t Solver::footprint(int64_t N, int m) {
 }
 
 Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
-    : N_(N), m_(m), tol_(tol), opt_(opt) {
+    : N_(N), ld_(padded(N)), m_(m), tol_(tol), opt_(opt) {
   s_ = reinterpret_cast<cudaStream_t>(opt.stream);
   mem_.set_stream(s_);
-  const size_t nm = (size_t)N * m;
+  const size_t nm = (size_t)ld_ * m;
   const size_t mm = (size_t)m * m;
   auto d = [&](size_t n) { return static_cast<double*>(mem_.alloc(n * 8)); };
   auto f = [&](size_t n) { return static_cast<float*>(mem_.alloc(n * 4)); };
@@ -273,6 +274,14 @@ Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
   HPb_ = d(nm);
   for (void* p : {Gb_[0], Gb_[1], Pb_, HPb_})
     TRM_CUDA(cudaMemsetAsync(p, 0, nm * 8, s_));
+  if (ld_ != N_) {  // the rows that pad a column stay zero
+    for (double* p : {C64_, C64n_, X64_})
+      TRM_CUDA(cudaMemsetAsync(p, 0, nm * 8, s_));
+    for (float* p : {C32_, C32n_, X32_})
+      TRM_CUDA(cudaMemsetAsync(p, 0, nm * 4, s_));
+    for (float* p : {Cdf_, Cdfn_, Xdf_})
+      TRM_CUDA(cudaMemsetAsync(p, 0, nm * 8, s_));
+  }
   HD_ = d(m);
   // partial column dots of the stencil applied to P (their sum is
   // tr(P^T H P)), kept apart from part_, which the Grams then reuse
@@ -298,7 +307,7 @@ Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
   lam_ = d(m);
   res_ = d(m);
   info_ = static_cast<int*>(mem_.alloc(16));
-  part_cap_ = part_capacity(N, m);
+  part_cap_ = part_capacity(ld_, m);
   part_ = d(part_cap_);
   sc_ = static_cast<IterScalars*>(mem_.alloc(sizeof(IterScalars)));
   TRM_CUDA(cudaMemsetAsync(sc_, 0, sizeof(IterScalars), s_));
@@ -312,8 +321,10 @@ Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
   diag64_ = d(N);
   diag32_ = f(N);
   diaglo_ = f(N);
-  minv64_ = d(N);
-  minv32_ = f(N);
+  minv64_ = d(ld_);
+  minv32_ = f(ld_);
+  TRM_CUDA(cudaMemsetAsync(minv64_, 0, ld_ * 8, s_));
+  TRM_CUDA(cudaMemsetAsync(minv32_, 0, ld_ * 4, s_));
   ring_ = ring_acquire();
   ev_.resize(kRing);
   for (auto& e : ev_) TRM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -342,6 +353,7 @@ void Solver::init_stencil(int nx, int ny, int nz, int order, double h,
   const int ndim = (nx > 1) + (ny > 1) + (nz > 1);
   op_.kind = 0;
   op_.N = N_;
+  op_.ld = ld_;
   op_.st.nx = nx;
   op_.st.ny = ny;
   op_.st.nz = nz;
@@ -382,6 +394,7 @@ void Solver::init_csr(const int32_t* rowptr, const int32_t* cols,
                            s_));
   op_.kind = 1;
   op_.N = N_;
+  op_.ld = ld_;
   op_.csr.rowptr = rp;
   op_.csr.cols = ci;
   int mx = 0;
@@ -436,6 +449,7 @@ void Solver::init_overlap(const int32_t* rowptr, const int32_t* cols,
   sop_ = Operator{};
   sop_.kind = 1;
   sop_.N = N_;
+  sop_.ld = ld_;
   sop_.csr.rowptr = rp;
   sop_.csr.cols = ci;
   sop_.csr.vals64 = v;
@@ -448,10 +462,12 @@ void Solver::init_overlap(const int32_t* rowptr, const int32_t* cols,
     TRM_CUDA(cudaStreamSynchronize(s_));  // v32 leaves scope
     sop_.csr.vals32 = vf;
     if (!Y32_) {
-      const size_t nm = (size_t)N_ * m_;
+      const size_t nm = (size_t)ld_ * m_;
       Y32_ = static_cast<float*>(mem_.alloc(nm * 4));
       Y32n_ = static_cast<float*>(mem_.alloc(nm * 4));
       SP32_ = static_cast<float*>(mem_.alloc(nm * 4));
+      for (float* p : {Y32_, Y32n_, SP32_})
+        TRM_CUDA(cudaMemsetAsync(p, 0, nm * 4, s_));
     }
   }
   int mx = 0;
@@ -459,10 +475,12 @@ void Solver::init_overlap(const int32_t* rowptr, const int32_t* cols,
   sop_.csr.max_row_nnz = mx;
   sop_.err = &sc_->status;
   if (!Y64_) {
-    const size_t nm = (size_t)N_ * m_;
+    const size_t nm = (size_t)ld_ * m_;
     Y64_ = static_cast<double*>(mem_.alloc(nm * 8));
     Y64n_ = static_cast<double*>(mem_.alloc(nm * 8));
     SP64_ = static_cast<double*>(mem_.alloc(nm * 8));
+    for (double* p : {Y64_, Y64n_, SP64_})
+      TRM_CUDA(cudaMemsetAsync(p, 0, nm * 8, s_));
     sdiag64_ = static_cast<double*>(mem_.alloc((size_t)N_ * 8));
     sdiag32_ = static_cast<float*>(mem_.alloc((size_t)N_ * 4));
   }
@@ -546,7 +564,7 @@ bool Solver::line_grams_fusable(const T* C, const T* P, const T* G) const {
     b.p[2] = G;
     a.cols = b.cols = m_;
     a.count = b.count = 3;
-    return gram_tc_pairs_eligible(N_, m_, a, b);
+    return gram_tc_pairs_eligible(ld_, m_, a, b);
   }
 }
 
@@ -576,7 +594,7 @@ void Solver::line_grams_fused(const T* C, const T* P, const T* G) {
     also.f32 = Bm32_;
     // algorithmic: 2 m^2 N per product, m^2 N for the symmetric one
     TRM_PROF(KC_GRAM32, 5 * m2N, 12 * nm,
-             gram_tc_pairs(N_, m_, a, b, Bm_, part_, part_cap_, &sc_->status,
+             gram_tc_pairs(ld_, m_, a, b, Bm_, part_, part_cap_, &sc_->status,
                            s_, also, /*sym_seg=*/1));
   }
 }
@@ -626,10 +644,10 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
   } else {
     TRM_PROF(ksp, sfl, sby, apply_h(op_, C, X, m_, s_));             // (1)
     TRM_PROF(KC_ROWOPS, 2 * nm, 2 * es * nm,
-             energy_diag<T>(N_, m_, C, X, HD_, sc_, part_, s_));      // (2), (3)
+             energy_diag<T>(ld_, m_, C, X, HD_, sc_, part_, s_));      // (2), (3)
   }
   TRM_PROF(KC_ROWOPS, 2 * nm, 3 * es * nm,
-           xprime<T>(N_, m_, Yc, X, HD_, nullptr, nullptr, s_));      // (5)
+           xprime<T>(ld_, m_, Yc, X, HD_, nullptr, nullptr, s_));      // (5)
   Blocks<T> bx;
   bx.p[0] = X;
   bx.cols = m_;
@@ -643,13 +661,13 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
   }
   bool hsplit = false;  // H' is in tw_.msplit as the gradient reads it
   TRM_PROF(kgr, 2 * m2N, 2 * es * nm,
-           hsplit = gram<T>(N_, m_, C, bx, Hp_, part_, part_cap_, s_,
+           hsplit = gram<T>(ld_, m_, C, bx, Hp_, part_, part_cap_, s_,
                             &sc_->status, hp_also));                  // (6)
   TRM_PROF(kgd, 2 * m2N, 5 * es * nm,
-           gradient<T>(N_, m_, Yc, X, Hp_, G, Gp, P, minv, sc_, part_,
+           gradient<T>(ld_, m_, Yc, X, Hp_, G, Gp, P, minv, sc_, part_,
                        part_cap_, s_, &tw_, hsplit));                 // (7)
   TRM_PROF(KC_ROWOPS, 2 * nm, 3 * es * nm,
-           update_p<T>(N_, m_, G, P, minv, sc_, s_));                 // P
+           update_p<T>(ld_, m_, G, P, minv, sc_, s_));                 // P
   const bool fused = !gen && line_grams_fusable<T>(C, P, G);
   int hp_chunks = 0;  // > 0: tr(P^T H P) from the stencil's column dots
   if constexpr (sizeof(T) == 4) {
@@ -680,7 +698,7 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
     bp.cols = m_;
     bp.count = 1;
     TRM_PROF(kgr, 2 * m2N, 2 * es * nm,
-             gram<T>(N_, m_, Yc, bp, Bm_, part_, part_cap_, s_, &sc_->status,
+             gram<T>(ld_, m_, Yc, bp, Bm_, part_, part_cap_, s_, &sc_->status,
                      bm_also));                                  // C^T (S) P
     Blocks<T> b3;
     b3.p[0] = SPt;
@@ -689,7 +707,7 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
     b3.cols = m_;
     b3.count = 3;
     TRM_PROF(kgr, 6 * m2N, 4 * es * nm,
-             gram<T>(N_, m_, P, b3, PG_, part_, part_cap_, s_, &sc_->status,
+             gram<T>(ld_, m_, P, b3, PG_, part_, part_cap_, s_, &sc_->status,
                      pg_also));                                       // P^T[P HP G]
   }
   const double m3 = md * md * md;
@@ -698,8 +716,8 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
   if constexpr (sizeof(T) == 4 && sizeof(Tm) == 4) {
     // alpha, Fig. ONFIG; for the tensor-core rotations the factor goes
     // straight into their operand format
-    const bool tc = rotate_on_tc(N_, m_, C, P, &tw_) &&
-                    (!gen || rotate_on_tc(N_, m_, Yc, SPt, &tw_));
+    const bool tc = rotate_on_tc(ld_, m_, C, P, &tw_) &&
+                    (!gen || rotate_on_tc(ld_, m_, Yc, SPt, &tw_));
     if (line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
                       PG32_ + woff, R_, sc_, mmw_, T1_, s_,
                       tc ? rw_.msplit : nullptr, mul_tc_ldm(m_)))
@@ -710,17 +728,17 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
                     sizeof(Tm) == 4, s_);
   prof.end(KC_SMALL, 4 * m3 + 2 * m3 / 3, 0.0, s_);
   TRM_PROF(krt, m2N, 3 * es * nm,
-           (rotate<T, T>(N_, m_, C, P, R, Cn, sc_, s_,
+           (rotate<T, T>(ld_, m_, C, P, R, Cn, sc_, s_,
                          R ? &tw_ : &rw_)));  // (C+aP)L^-T
   if (gen) {  // S (C + aP) L^-T = (Y + a S P) L^-T
     if constexpr (sizeof(T) == 8) {
       TRM_PROF(krt, m2N, 3 * es * nm,
-               (rotate<double, double>(N_, m_, Y64_, SP64_, R_, Y64n_, sc_,
+               (rotate<double, double>(ld_, m_, Y64_, SP64_, R_, Y64n_, sc_,
                                        s_, &tw_)));
       std::swap(Y64_, Y64n_);
     } else {
       TRM_PROF(krt, m2N, 3 * es * nm,
-               (rotate<float, float>(N_, m_, Y32_, SP32_, R, Y32n_, sc_, s_,
+               (rotate<float, float>(ld_, m_, Y32_, SP32_, R, Y32n_, sc_, s_,
                                      R ? &tw_ : &rw_)));
       std::swap(Y32_, Y32n_);
     }
@@ -744,7 +762,7 @@ void Solver::iter_mp2() {
   float* HP = static_cast<float*>(HPb_);
   const float* minv = opt_.precond ? minv32_ : nullptr;
   const size_t mm = (size_t)m_ * m_;
-  const size_t nm = (size_t)N_ * m_;
+  const size_t nm = (size_t)ld_ * m_;
   const double Nd = (double)N_, md = m_;
   const double dnm = Nd * md, m2N = dnm * md, m3 = md * md * md;
   float* Ch = Cdf_;
@@ -764,23 +782,23 @@ void Solver::iter_mp2() {
   } else {
     TRM_PROF(KC_SPMMDF, f64, b64, apply_h_df(op_, Ch, Cl, Xh, Xl, m_, s_));
     TRM_PROF(KC_ROWOPS, 2 * dnm, 16 * dnm,
-             energy_diag_df(N_, m_, Ch, Cl, Xh, Xl, HD_, sc_, part_, s_));
+             energy_diag_df(ld_, m_, Ch, Cl, Xh, Xl, HD_, sc_, part_, s_));
   }
   TRM_PROF(KC_ROWOPS, 2 * dnm, 20 * dnm,
-           xprime_df(N_, m_, Ch, Cl, Xh, Xl, HD_, X32_, s_));  // (5) FP32 X'
+           xprime_df(ld_, m_, Ch, Cl, Xh, Xl, HD_, X32_, s_));  // (5) FP32 X'
   Blocks<float> bx;
   bx.p[0] = X32_;
   bx.cols = m_;
   bx.count = 1;
   bool hsplit = false;
   TRM_PROF(KC_GRAM32, 2 * m2N, 8 * dnm,
-           hsplit = gram<float>(N_, m_, Ch, bx, Hp_, part_, part_cap_, s_,
+           hsplit = gram<float>(ld_, m_, Ch, bx, Hp_, part_, part_cap_, s_,
                                 &sc_->status, hprime_out()));         // (6)
   TRM_PROF(KC_GRAD32, 2 * m2N, 20 * dnm,
-           gradient<float>(N_, m_, Ch, X32_, Hp_, G, Gp, P, minv, sc_,
+           gradient<float>(ld_, m_, Ch, X32_, Hp_, G, Gp, P, minv, sc_,
                            part_, part_cap_, s_, &tw_, hsplit));      // (7)
   TRM_PROF(KC_ROWOPS, 2 * dnm, 12 * dnm,
-           update_p<float>(N_, m_, G, P, minv, sc_, s_));
+           update_p<float>(ld_, m_, G, P, minv, sc_, s_));
   const bool fused = line_grams_fusable<float>(Ch, P, G);
   const double* hpd = nullptr;
   const double* trp = nullptr;
@@ -805,7 +823,7 @@ void Solver::iter_mp2() {
     bp.cols = m_;
     bp.count = 1;
     TRM_PROF(KC_GRAM32, 2 * m2N, 8 * dnm,
-             gram<float>(N_, m_, Ch, bp, Bm_, part_, part_cap_, s_,
+             gram<float>(ld_, m_, Ch, bp, Bm_, part_, part_cap_, s_,
                          &sc_->status, bm_also));
     Blocks<float> b3;
     b3.p[0] = P;
@@ -814,11 +832,11 @@ void Solver::iter_mp2() {
     b3.cols = m_;
     b3.count = 3;
     TRM_PROF(KC_GRAM32, 6 * m2N, 16 * dnm,
-             gram<float>(N_, m_, P, b3, PG_, part_, part_cap_, s_,
+             gram<float>(ld_, m_, P, b3, PG_, part_, part_cap_, s_,
                          &sc_->status, pg_also));
   }
   prof.begin(KC_SMALL, s_);
-  const bool tc = rotate_on_tc(N_, m_, Ch, P, &tw_);
+  const bool tc = rotate_on_tc(ld_, m_, Ch, P, &tw_);
   const double* R = R_;
   if (line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
                     PG32_ + woff, R_, sc_, mmw_, T1_, s_,
@@ -827,7 +845,7 @@ void Solver::iter_mp2() {
     R = nullptr;
   prof.end(KC_SMALL, 4 * m3 + 2 * m3 / 3, 0.0, s_);
   TRM_PROF(KC_ROTDF, m2N, 24 * dnm,
-           rotate_split_df(N_, m_, Ch, Cl, P, R, Cdfn_, Cdfn_ + nm, sc_, s_,
+           rotate_split_df(ld_, m_, Ch, Cl, P, R, Cdfn_, Cdfn_ + nm, sc_, s_,
                            R ? &tw_ : &rw_));
   std::swap(Cdf_, Cdfn_);
   std::swap(Gb_[0], Gb_[1]);
@@ -836,11 +854,11 @@ void Solver::iter_mp2() {
 // The MP2 blocks between FP64 and FP32 pairs (at re-orthonormalizations,
 // Rayleigh-Ritz rotations and phase changes).
 void Solver::c64_to_df() {
-  const size_t nm = (size_t)N_ * m_;
+  const size_t nm = (size_t)ld_ * m_;
   split_df(C64_, Cdf_, Cdf_ + nm, (int64_t)nm, s_);
 }
 void Solver::df_to_c64() {
-  const size_t nm = (size_t)N_ * m_;
+  const size_t nm = (size_t)ld_ * m_;
   join_df(Cdf_, Cdf_ + nm, C64_, (int64_t)nm, s_);
 }
 
@@ -848,17 +866,17 @@ void Solver::df_to_c64() {
 // (FP64-class, on the FP32 pipe) in the mixed ladder.
 void Solver::gram64(const double* A, const Blocks<double>& b, double* out) {
   if (opt_.precision == TRM_FP64)
-    gram<double>(N_, m_, A, b, out, part_, part_cap_, s_, &sc_->status);
+    gram<double>(ld_, m_, A, b, out, part_, part_cap_, s_, &sc_->status);
   else
-    gram_df(N_, m_, A, b, out, part_, part_cap_, s_);
+    gram_df(ld_, m_, A, b, out, part_, part_cap_, s_);
 }
 
 // N x m times m x m products of FP64 blocks, FP64 or double-float as gram64.
 void Solver::mult64(const double* A, const double* M, double* Y) {
   if (opt_.precision == TRM_FP64)
-    mult(N_, m_, m_, A, M, Y, s_);
+    mult(ld_, m_, m_, A, M, Y, s_);
   else
-    mult_df(N_, m_, m_, A, M, Y, false, s_);
+    mult_df(ld_, m_, m_, A, M, Y, false, s_);
 }
 
 // Fig. ONFIG in FP64: S = C^T C, S = L L^T, C <- C L^{-T} (generalized
@@ -880,12 +898,12 @@ void Solver::orth_fp64(double*& C, double*& Cn) {
            chol_inv<double>(m_, S_, Linv_, R_, sc_, mmw_, s_));
   if (opt_.precision == TRM_FP64)
     TRM_PROF(KC_ROT64, m2N, 16 * nm,
-             (rotate<double, double>(N_, m_, C, nullptr, R_, Cn, nullptr, s_)));
+             (rotate<double, double>(ld_, m_, C, nullptr, R_, Cn, nullptr, s_)));
   else  // C L^{-T} in double-float
-    TRM_PROF(KC_ROT64, m2N, 16 * nm, mult_df(N_, m_, m_, C, R_, Cn, true, s_));
+    TRM_PROF(KC_ROT64, m2N, 16 * nm, mult_df(ld_, m_, m_, C, R_, Cn, true, s_));
   if (has_S_) {
     TRM_PROF(KC_ROT64, m2N, 16 * nm,
-             (rotate<double, double>(N_, m_, Y64_, nullptr, R_, Y64n_, nullptr,
+             (rotate<double, double>(ld_, m_, Y64_, nullptr, R_, Y64n_, nullptr,
                                      s_)));
     std::swap(Y64_, Y64n_);
   }
@@ -906,13 +924,13 @@ void Solver::orth_uniform(T*& C, T*& Cn) {
       gen = true;
     }
   }
-  gram<T>(N_, m_, C, b, S_, part_, part_cap_, s_, &sc_->status);
+  gram<T>(ld_, m_, C, b, S_, part_, part_cap_, s_, &sc_->status);
   chol_inv<T>(m_, S_, Linv_, R_, sc_, mmw_, s_);
-  rotate<T, T>(N_, m_, C, static_cast<const T*>(nullptr), R_, Cn, nullptr,
+  rotate<T, T>(ld_, m_, C, static_cast<const T*>(nullptr), R_, Cn, nullptr,
                s_, &tw_);
   if constexpr (sizeof(T) == 4) {
     if (gen) {  // Y follows C
-      rotate<float, float>(N_, m_, Y32_, static_cast<const float*>(nullptr),
+      rotate<float, float>(ld_, m_, Y32_, static_cast<const float*>(nullptr),
                            R_, Y32n_, nullptr, s_, &tw_);
       std::swap(Y32_, Y32n_);
     }
@@ -961,7 +979,7 @@ void Solver::final_rr(double* C, double* Cfin, double* Xfin) {
   // the overlap in FP64 in every mode: the returned block is orthonormalized
   // by its factor (the double-float Gram's sum over N rows is good to about
   // sqrt(N) 2^-48, which left C^T C - I near 1e-12 at N ~ 1e6)
-  gram<double>(N_, m_, C, bc, S_, part_, part_cap_, s_);
+  gram<double>(ld_, m_, C, bc, S_, part_, part_cap_, s_);
   chol_inv<double>(m_, S_, Linv_, R_, sc_, mmw_, s_);
   mm_gemm(m_, Linv_, false, Hp_, false, T1_, 1.0, 0.0, s_);
   mm_gemm(m_, T1_, false, Linv_, true, T2_, 1.0, 0.0, s_);
@@ -970,16 +988,16 @@ void Solver::final_rr(double* C, double* Cfin, double* Xfin) {
   mm_gemm(m_, R_, false, Z_, false, T1_, 1.0, 0.0, s_);
   // the returned block in FP64 in every mode; H C Y, used only for the
   // residual norms, keeps the FP64-class product
-  mult(N_, m_, m_, C, T1_, Cfin, s_);
+  mult(ld_, m_, m_, C, T1_, Cfin, s_);
   mult64(X64_, T1_, Xfin);
   if (has_S_) {  // ||H c_j - theta_j S c_j|| (sign independent)
     mult64(Y64_, T1_, SP64_);
-    column_residuals(N_, m_, Xfin, SP64_, lam_, res_, part_, s_);
-    fix_signs(N_, m_, Cfin, Xfin, part_, s_);
+    column_residuals(ld_, m_, Xfin, SP64_, lam_, res_, part_, s_);
+    fix_signs(ld_, m_, Cfin, Xfin, part_, s_);
     return;
   }
-  fix_signs(N_, m_, Cfin, Xfin, part_, s_);
-  column_residuals(N_, m_, Xfin, Cfin, lam_, res_, part_, s_);
+  fix_signs(ld_, m_, Cfin, Xfin, part_, s_);
+  column_residuals(ld_, m_, Xfin, Cfin, lam_, res_, part_, s_);
 }
 
 // ---------------------------------------------------------------------------
@@ -1061,13 +1079,14 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
                   const double* C0_host, trm_stats* stats) {
   const auto t_start = std::chrono::steady_clock::now();
   const long long launches0 = thread_launch_count();
-  const size_t nm = (size_t)N_ * m_;
+  const size_t nm = (size_t)ld_ * m_;
   history_.clear();
+  clear_padding(8);
+  clear_padding(4);
   if (C0_host)
-    TRM_CUDA(cudaMemcpyAsync(C64_, C0_host, nm * 8, cudaMemcpyHostToDevice,
-                             s_));
+    copy_in(C0_host, C64_, cudaMemcpyHostToDevice);
   else
-    random_block(N_, m_, opt_.seed, C64_, s_);
+    random_block(N_, m_, opt_.seed, C64_, s_, ld_);
 
   enum { PH_SP = 0, PH_MP2 = 1, PH_FP64 = 2 };
   const int prec = opt_.precision;
@@ -1298,6 +1317,7 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
     }
   }
   drain();
+  pad_es_ = 0;  // final_rr uses G as scratch
   if (prof.on) prof.resolve();
   if (phase == PH_SP) to_f64(C32_, C64_, (int64_t)nm, s_);
   if (phase == PH_MP2) df_to_c64();
@@ -1310,10 +1330,8 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
   TRM_CUDA(cudaMemcpyAsync(res.data(), res_, m_ * 8, cudaMemcpyDeviceToHost,
                            s_));
   if (C_out)
-    TRM_CUDA(cudaMemcpyAsync(C_out, Cfin, nm * 8,
-                             C_on_device ? cudaMemcpyDeviceToDevice
-                                         : cudaMemcpyDeviceToHost,
-                             s_));
+    copy_out(Cfin, C_out,
+             C_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost);
   TRM_CUDA(cudaStreamSynchronize(s_));
   if (lambda) std::memcpy(lambda, lam.data(), m_ * 8);
   if (E_G) *E_G = neumaier_sum(lam.data(), m_);
@@ -1341,48 +1359,106 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
 }
 
 // ---------------------------------------------------------------------------
+// Blocks from and to callers (columns N apart) and the padding rows.
+// ---------------------------------------------------------------------------
+static void copy_cols(const double* src, int64_t lds, double* dst, int64_t ldd,
+                      int64_t N, int m, cudaMemcpyKind kind, cudaStream_t s) {
+  if (lds == ldd)
+    TRM_CUDA(cudaMemcpyAsync(dst, src, (size_t)N * m * 8, kind, s));
+  else if (kind == cudaMemcpyDeviceToDevice)
+    copy_columns(N, m, src, lds, dst, ldd, s);
+  else
+    TRM_CUDA(cudaMemcpy2DAsync(dst, ldd * 8, src, lds * 8, N * 8, m, kind, s));
+}
+void Solver::copy_in(const double* src, double* dst, cudaMemcpyKind kind) {
+  copy_cols(src, N_, dst, ld_, N_, m_, kind, s_);
+}
+void Solver::copy_out(const double* src, double* dst, cudaMemcpyKind kind) {
+  copy_cols(src, ld_, dst, N_, N_, m_, kind, s_);
+}
+// The padding rows of G, P and HP lie elsewhere in FP64 (es = 8) than in FP32
+// (es = 4), a block used as scratch may hold anything there, and non-finite
+// values of an earlier call may have reached the others: they are cleared
+// where a solve or a CG sequence starts and before an iteration in a precision
+// that is not the one they were last clear for. (At the other precision's
+// places lie entries.)
+void Solver::clear_padding(int es) {
+  pad_es_ = es;
+  if (ld_ == N_) return;
+  PadList l;
+  for (double* p : {C64_, C64n_, X64_, Y64_, Y64n_, SP64_}) l.add(p, 8);
+  for (void* p : {Gb_[0], Gb_[1], Pb_, HPb_}) l.add(p, es);
+  for (float* p : {C32_, C32n_, X32_, Y32_, Y32n_, SP32_}) l.add(p, 4);
+  const size_t nm = (size_t)ld_ * m_;
+  for (float* p : {Cdf_, Cdfn_, Xdf_}) {
+    l.add(p, 4);
+    l.add(p + nm, 4);
+  }
+  clear_pad_rows(l, N_, ld_, m_, s_);
+}
+
+// ---------------------------------------------------------------------------
 // Step operations
 // ---------------------------------------------------------------------------
 void Solver::apply(int din, const void* in, int dout, void* out, int ncols) {
+  Operator op = op_;  // the caller's columns are N entries apart
+  op.ld = N_;
   if (din == TRM_F32 && dout == TRM_F32)
-    apply_h(op_, static_cast<const float*>(in), static_cast<float*>(out),
+    apply_h(op, static_cast<const float*>(in), static_cast<float*>(out),
             ncols, s_);
   else if (din == TRM_F64 && dout == TRM_F64)
-    apply_h(op_, static_cast<const double*>(in), static_cast<double*>(out),
+    apply_h(op, static_cast<const double*>(in), static_cast<double*>(out),
             ncols, s_);
   else
     throw Error(-1, "apply: unsupported dtype combination");
   TRM_CUDA(cudaStreamSynchronize(s_));
 }
 
-void Solver::energy_gradient(const double* C, double* E, double* HD,
-                             double* Hprime, void* G, int G_dtype,
+void Solver::energy_gradient(const double* C_dev, double* E, double* HD,
+                             double* Hprime, void* G_dev, int G_dtype,
                              int zdiag) {
+  // padded columns: C from a copy, G through a scratch block
+  const double* C = C_dev;
+  void* G = G_dev;
+  if (ld_ != N_) {
+    copy_in(C_dev, C64n_, cudaMemcpyDeviceToDevice);
+    C = C64n_;
+    G = HPb_;
+    pad_es_ = 0;
+  }
   apply_h(op_, C, X64_, m_, s_);
-  energy_diag<double>(N_, m_, C, X64_, HD_, sc_, part_, s_);
+  energy_diag<double>(ld_, m_, C, X64_, HD_, sc_, part_, s_);
   set_restart();
   GramOut also;
   also.zero_diag = zdiag != 0;
   if (G_dtype == TRM_F64) {
-    xprime<double>(N_, m_, C, X64_, HD_, nullptr, nullptr, s_);
+    xprime<double>(ld_, m_, C, X64_, HD_, nullptr, nullptr, s_);
     Blocks<double> b;
     b.p[0] = X64_;
     b.cols = m_;
     b.count = 1;
-    gram<double>(N_, m_, C, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
-    gradient<double>(N_, m_, C, X64_, Hp_, static_cast<double*>(G), nullptr,
+    gram<double>(ld_, m_, C, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
+    gradient<double>(ld_, m_, C, X64_, Hp_, static_cast<double*>(G), nullptr,
                      nullptr, nullptr, sc_, part_, part_cap_, s_);
   } else if (G_dtype == TRM_F32) {
-    xprime<double>(N_, m_, C, X64_, HD_, C32_, X32_, s_, false);
+    xprime<double>(ld_, m_, C, X64_, HD_, C32_, X32_, s_, false);
     Blocks<float> b;
     b.p[0] = X32_;
     b.cols = m_;
     b.count = 1;
-    gram<float>(N_, m_, C32_, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
-    gradient<float>(N_, m_, C32_, X32_, Hp_, static_cast<float*>(G), nullptr,
+    gram<float>(ld_, m_, C32_, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
+    gradient<float>(ld_, m_, C32_, X32_, Hp_, static_cast<float*>(G), nullptr,
                     nullptr, nullptr, sc_, part_, part_cap_, s_, &tw_);
   } else {
     throw Error(-1, "energy_gradient: G_dtype must be TRM_F32 or TRM_F64");
+  }
+  if (G != G_dev) {
+    if (G_dtype == TRM_F64)
+      copy_columns(N_, m_, static_cast<const double*>(G), ld_,
+                   static_cast<double*>(G_dev), N_, s_);
+    else
+      copy_columns(N_, m_, static_cast<const float*>(G), ld_,
+                   static_cast<float*>(G_dev), N_, s_);
   }
   if (HD)
     TRM_CUDA(cudaMemcpyAsync(HD, HD_, m_ * 8, cudaMemcpyDeviceToDevice, s_));
@@ -1396,26 +1472,27 @@ void Solver::energy_gradient(const double* C, double* E, double* HD,
 }
 
 void Solver::set_block(const double* C_dev) {
-  TRM_CUDA(cudaMemcpyAsync(C64_, C_dev, (size_t)N_ * m_ * 8,
-                           cudaMemcpyDeviceToDevice, s_));
+  copy_in(C_dev, C64_, cudaMemcpyDeviceToDevice);
   cg_fresh_ = true;
   set_restart();
   TRM_CUDA(cudaStreamSynchronize(s_));
 }
 
 void Solver::get_block(double* C_dev) {
-  TRM_CUDA(cudaMemcpyAsync(C_dev, C64_, (size_t)N_ * m_ * 8,
-                           cudaMemcpyDeviceToDevice, s_));
+  copy_out(C64_, C_dev, cudaMemcpyDeviceToDevice);
   TRM_CUDA(cudaStreamSynchronize(s_));
 }
 
 void Solver::iterate(int mode, int restart, double* E, double* rms,
                      double* alpha) {
-  const size_t nm = (size_t)N_ * m_;
+  const size_t nm = (size_t)ld_ * m_;
   // a new CG sequence reads no value of G_prev or P (gamma = 0), whatever
   // they hold: the flag is set here, last before the iteration
-  if (restart || cg_fresh_) set_restart();
+  const bool fresh = restart || cg_fresh_;
+  if (fresh) set_restart();
   cg_fresh_ = false;
+  const int es = mode == TRM_FP64 ? 8 : 4;
+  if (fresh || pad_es_ != es) clear_padding(es);
   if (mode == TRM_FP64) {
     double* G = static_cast<double*>(Gb_[0]);
     double* Gp = static_cast<double*>(Gb_[1]);
@@ -1453,9 +1530,14 @@ void Solver::iterate(int mode, int restart, double* E, double* rms,
 void Solver::rayleigh_ritz(double* C_dev, double* lambda_host,
                            double* res_host) {
   double* Xfin = static_cast<double*>(Gb_[0]);
-  final_rr(C_dev, C64n_, Xfin);
-  TRM_CUDA(cudaMemcpyAsync(C_dev, C64n_, (size_t)N_ * m_ * 8,
-                           cudaMemcpyDeviceToDevice, s_));
+  double* C = C_dev;
+  if (ld_ != N_) {
+    clear_padding(8);
+    C = static_cast<double*>(Pb_);  // (a new CG sequence follows)
+    copy_in(C_dev, C, cudaMemcpyDeviceToDevice);
+  }
+  final_rr(C, C64n_, Xfin);
+  copy_out(C64n_, C_dev, cudaMemcpyDeviceToDevice);
   if (lambda_host)
     TRM_CUDA(cudaMemcpyAsync(lambda_host, lam_, m_ * 8, cudaMemcpyDeviceToHost,
                              s_));
@@ -1464,6 +1546,7 @@ void Solver::rayleigh_ritz(double* C_dev, double* lambda_host,
                              s_));
   TRM_CUDA(cudaStreamSynchronize(s_));
   cg_fresh_ = true;  // final_rr used G as scratch
+  pad_es_ = 0;
   set_restart();
 }
 

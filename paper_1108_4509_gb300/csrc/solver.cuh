@@ -164,7 +164,17 @@ class Solver {
   void set_restart();
   void read_scalars(IterScalars* out);
 
-  int64_t N_;
+  // Columns of the solver's own blocks are ld_ entries apart: N rounded up to
+  // a multiple of four, so that every column starts on a 16-byte boundary (TMA
+  // and vector loads) whatever the grid. The padding rows are zero and stay so:
+  // every block kernel runs over ld_ rows and maps zeros to zeros, and the
+  // operator writes its N rows only.
+  int64_t N_, ld_;
+  static int64_t padded(int64_t N) { return (N + 3) & ~(int64_t)3; }
+  void copy_in(const double* src, double* dst, cudaMemcpyKind kind);
+  void copy_out(const double* src, double* dst, cudaMemcpyKind kind);
+  void clear_padding(int es);
+  int pad_es_ = 0;  // element size G, P and HP's padding is clear for
   int m_;
   double tol_;
   trm_options opt_;

@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1)
 // One point per thread, any nx.
 template <typename T, int R, bool DOTS>
 __global__ void __launch_bounds__(256)
-    k_stencil_1(StencilOp st, int64_t N, const double* __restrict__ d64,
+    k_stencil_1(StencilOp st, int64_t N, int64_t ld, const double* __restrict__ d64,
                 const float* __restrict__ d32, const T* __restrict__ X,
                 T* __restrict__ Y, int ncols, double* __restrict__ dots) {
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256)
   for (int q = 0; q < kCpb; ++q) {
     const int c = cb + q;
     if (c >= ncols || (DOTS && !valid)) continue;
-    const T* xp = X + (int64_t)c * N + i;
+    const T* xp = X + (int64_t)c * ld + i;
     T s1 = 0, s2 = 0;
     if (x >= 1) s1 += xp[-1];
     if (x + 1 < st.nx) s1 += xp[1];
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(256)
       if (z + 2 < st.nz) s2 += xp[2 * sz];
       acc += c2 * s2;
     }
-    if (!DOTS || Y) Y[(int64_t)c * N + i] = acc;
+    if (!DOTS || Y) Y[(int64_t)c * ld + i] = acc;
     if (DOTS) dsum[q] = xp[0] * acc;
   }
   if (DOTS) {
@@ -228,7 +228,7 @@ constexpr int kCsrCache = 16;
 
 template <typename T, typename TV, bool DOTS>
 __global__ void __launch_bounds__(256)
-    k_csr(int64_t N, const int32_t* __restrict__ rowptr,
+    k_csr(int64_t N, int64_t ld, const int32_t* __restrict__ rowptr,
           const int32_t* __restrict__ cols, const TV* __restrict__ vals,
           const T* __restrict__ X, T* __restrict__ Y, int ncols,
           double* __restrict__ dots) {
@@ -253,12 +253,12 @@ __global__ void __launch_bounds__(256)
       if (c >= ncols) break;
       T d = 0;
       if (valid) {
-        const T* x = X + (int64_t)c * N;
+        const T* x = X + (int64_t)c * ld;
         T acc = 0;
 #pragma unroll
         for (int k = 0; k < kCsrCache; ++k)
           if (k < nnz) acc += cv[k] * __ldg(x + ci[k]);
-        if (!DOTS || Y) Y[(int64_t)c * N + r] = acc;
+        if (!DOTS || Y) Y[(int64_t)c * ld + r] = acc;
         d = x[r] * acc;
       }
       if (DOTS) warp_dot(d, red, q);
@@ -269,10 +269,10 @@ __global__ void __launch_bounds__(256)
       if (c >= ncols) break;
       T d = 0;
       if (valid) {
-        const T* x = X + (int64_t)c * N;
+        const T* x = X + (int64_t)c * ld;
         T acc = 0;
         for (int k = b; k < e; ++k) acc += (T)vals[k] * __ldg(x + cols[k]);
-        if (!DOTS || Y) Y[(int64_t)c * N + r] = acc;
+        if (!DOTS || Y) Y[(int64_t)c * ld + r] = acc;
         d = x[r] * acc;
       }
       if (DOTS) warp_dot(d, red, q);
@@ -822,10 +822,10 @@ int launch_vec(const Operator& op, const T* X, T* Y, int ncols, double* dots,
       grid = dim3(ceil_div(op.N, threads), gy);
       if (st.radius == 1)
         k_stencil_1<T, 1, DOTS><<<grid, threads, 0, s>>>(
-            st, op.N, op.diag64, op.diag32, X, Y, ncols, dots);
+            st, op.N, op.ld, op.diag64, op.diag32, X, Y, ncols, dots);
       else
         k_stencil_1<T, 2, DOTS><<<grid, threads, 0, s>>>(
-            st, op.N, op.diag64, op.diag32, X, Y, ncols, dots);
+            st, op.N, op.ld, op.diag64, op.diag32, X, Y, ncols, dots);
     }
   } else {
     grid = dim3(ceil_div(op.N, threads), gy);
@@ -833,10 +833,10 @@ int launch_vec(const Operator& op, const T* X, T* Y, int ncols, double* dots,
     // holds them (the same products, no conversion per nonzero)
     if (op.csr.vals64 && (sizeof(T) == 8 || !op.csr.vals32))
       k_csr<T, double, DOTS><<<grid, threads, 0, s>>>(
-          op.N, op.csr.rowptr, op.csr.cols, op.csr.vals64, X, Y, ncols, dots);
+          op.N, op.ld, op.csr.rowptr, op.csr.cols, op.csr.vals64, X, Y, ncols, dots);
     else
       k_csr<T, float, DOTS><<<grid, threads, 0, s>>>(
-          op.N, op.csr.rowptr, op.csr.cols, op.csr.vals32, X, Y, ncols, dots);
+          op.N, op.ld, op.csr.rowptr, op.csr.cols, op.csr.vals32, X, Y, ncols, dots);
   }
   TRM_CHECK_LAUNCH();
   return (int)grid.x;

@@ -121,3 +121,91 @@ def test_step_factorisation_edges(trm, mode, m):
     bound = (a * np.linalg.norm(dG) + 2 * np.linalg.norm(dS)
              + np.linalg.norm(prod) + 1e-12)
     assert np.linalg.norm(C1 - Y @ R) <= bound
+
+
+# Grids whose size is not a multiple of four: the solver's blocks are padded.
+ODD = [((13, 11, 9), 40), ((7, 5, 3), 6), ((15, 14, 13), 33), ((9, 21, 1), 20)]
+
+
+@pytest.mark.parametrize("csr", [0, 1])
+@pytest.mark.parametrize("shape,m", ODD)
+def test_padded_columns_modes_in_turn(trm, shape, m, csr):
+    """On one handle with padded columns: every mode after every other, the
+    step operations in between and a start that overflows give the bytes a
+    fresh handle gives."""
+    V = ti.gaussian_wells(shape, 4, seed=2)
+    N = V.size
+    assert N % 4
+    H = op.grid_hamiltonian(shape, 4, 1.0, V)
+    cd = gu.to_dev(_near(H, m, 3))
+    opt = trm.trm_default_options(stream=gu.stream(), precond=1)
+
+    def make():
+        if csr:
+            return trm.trm_create_csr(N, *ti.grid_csr(shape, 4, 1.0, V), m, 1e-10,
+                                      opt)
+        nx, ny, nz = (tuple(shape) + (1, 1))[:3]
+        return trm.trm_create_stencil(nx, ny, nz, 4, 1.0, V, m, 1e-10, opt)
+
+    def two(h, mode):
+        trm.trm_set_block(h, cd.data_ptr())
+        r = [trm.trm_iterate(h, mode) for _ in range(2)]
+        out = gu.empty(N, m, np.float64)
+        trm.trm_get_block(h, out.data_ptr())
+        return r, gu.from_dev(out)
+
+    modes = [trm.TRM_FULL_SP, trm.TRM_FP64, trm.TRM_MP2]
+    ref = {}
+    for md in modes:
+        h = make()
+        ref[md] = two(h, md)
+        trm.trm_destroy(h)
+    h = make()
+    try:
+        g = gu.empty(N, m, np.float64)
+        big = gu.to_dev(np.full((N, m), 1e200) * (1 + ti.random_block(N, m, 1)))
+        for k, md in enumerate(modes + modes[::-1] + [trm.TRM_FP64]):
+            r, C = two(h, md)
+            assert r == ref[md][0] and np.array_equal(C, ref[md][1]), (k, md)
+            if k % 3 == 0:
+                trm.trm_energy_gradient(h, cd.data_ptr(), 0, 0, g.data_ptr(),
+                                        trm.TRM_F64, True)
+            elif k % 3 == 1:
+                other = gu.to_dev(_near(H, m, 5))
+                trm.trm_rayleigh_ritz(h, other.data_ptr(), m)
+            else:
+                trm.trm_set_block(h, big.data_ptr())
+                try:
+                    trm.trm_iterate(h, md)
+                except trm.TrmError:
+                    pass
+    finally:
+        trm.trm_destroy(h)
+
+
+@pytest.mark.parametrize("shape,m", ODD)
+def test_padded_columns_solve(trm, shape, m):
+    """A mixed solve on padded columns from a host block, the block returned to
+    the host and to the device: the oracle's eigenvalues, the same bytes."""
+    V = ti.gaussian_wells(shape, 4, seed=2)
+    N = V.size
+    H = op.grid_hamiltonian(shape, 4, 1.0, V)
+    w = np.linalg.eigvalsh(H.toarray())[:m]
+    C0 = np.asfortranarray(_near(H, m, 3))
+    nx, ny, nz = (tuple(shape) + (1, 1))[:3]
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_stencil(nx, ny, nz, 4, 1.0, V, m, 1e-10, opt)
+    try:
+        Ch = np.zeros((N, m), order="F")
+        lam, eg, _, status = trm.trm_solve(h, N, m, C_out=Ch, C0=C0)
+        assert status == 0
+        cd = gu.empty(N, m, np.float64)
+        lam2, _, _, status2 = trm.trm_solve(h, N, m, C_out=cd.data_ptr(),
+                                            C_on_device=True, C0=C0)
+        assert status2 == 0 and np.array_equal(lam, lam2)
+        assert np.array_equal(gu.from_dev(cd), Ch)
+        assert np.max(np.abs(lam - w)) < 1e-9
+        assert np.max(np.abs(Ch.T @ Ch - np.eye(m))) < 1e-12
+        assert np.max(np.abs(op.apply_h(H, Ch) - Ch * lam)) < 1e-8
+    finally:
+        trm.trm_destroy(h)
