@@ -6,6 +6,8 @@
 #include <mutex>
 #include <string>
 
+#include <optional>
+
 #include "solver.cuh"
 
 struct trm_ctx {
@@ -76,6 +78,64 @@ trm_options resolve(const trm_options* opt) {
   if (o.lag < 1) o.lag = 1;
   return o;
 }
+
+// Device memory of one call, stream-ordered, freed when the call returns.
+class Scratch {
+ public:
+  explicit Scratch(cudaStream_t s) : s_(s) {}
+  ~Scratch() {
+    if (p_) cudaFreeAsync(p_, s_);
+  }
+  Scratch(const Scratch&) = delete;
+  Scratch& operator=(const Scratch&) = delete;
+  bool get(size_t bytes, bool may_fail) {
+    const cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&p_), bytes, s_);
+    if (e == cudaSuccess) {
+      left_ = bytes;
+      at_ = p_;
+      return true;
+    }
+    p_ = nullptr;
+    if (!may_fail) TRM_CUDA(e);
+    cudaGetLastError();
+    return false;
+  }
+  // the next n elements, 16-byte aligned
+  template <typename T>
+  T* take(size_t n) {
+    const size_t b = (n * sizeof(T) + 15) & ~(size_t)15;
+    if (b > left_) throw trm::Error(TRM_ENOMEM, "scratch exhausted");
+    T* r = reinterpret_cast<T*>(at_);
+    at_ += b;
+    left_ -= b;
+    return r;
+  }
+
+ private:
+  cudaStream_t s_;
+  char* p_ = nullptr;
+  char* at_ = nullptr;
+  size_t left_ = 0;
+};
+
+// Digits of `blocks` N x m blocks and of an m x m factor, and their scales.
+struct OzScratch {
+  trm::OzBlock block[2];
+  trm::OzSmall small;
+  static size_t bytes(int64_t N, int m, int blocks) {
+    return blocks * (trm::oz_block_bytes(N, m) + 16) +
+           trm::oz_small_bytes(m, m) + 16 +
+           (blocks + 1) * ((size_t)m * sizeof(double) + 16);
+  }
+  OzScratch(Scratch& w, int64_t N, int m, int blocks) {
+    for (int k = 0; k < blocks; ++k) {
+      block[k].digits = w.take<char>(trm::oz_block_bytes(N, m));
+      block[k].scale = w.take<double>(m);
+    }
+    small.digits = w.take<char>(trm::oz_small_bytes(m, m));
+    small.scale = w.take<double>(m);
+  }
+};
 
 }  // namespace
 
@@ -337,20 +397,30 @@ trm_status trm_orthonormalize(int64_t N, int m, double* C, void* stream) {
     const size_t mm = (size_t)m * m;
     const size_t cap = trm::gram_partials_doubles(N, m, m);
     const size_t cw = trm::chol_work_elems(m);
-    const size_t bytes = (cap + 3 * mm + cw + (size_t)N * m) * sizeof(double) +
-                         sizeof(trm::IterScalars);
-    char* w = nullptr;
-    TRM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&w), bytes, s));
-    double* part = reinterpret_cast<double*>(w);
-    double* S = part + cap;
-    double* Linv = S + mm;
-    double* R = Linv + mm;
-    double* gw = R + mm;        // padded factorisation workspace
-    double* Cn = gw + cw;
-    auto* sc = reinterpret_cast<trm::IterScalars*>(Cn + (size_t)N * m);
+    const size_t fixed = (cap + 3 * mm + cw) * sizeof(double) +
+                         sizeof(trm::IterScalars) + 512;
+    // with the digits of C the result goes straight to C; else a second block
+    Scratch w(s);
+    const bool oz =
+        trm::oz_pays(N, m, m) &&
+        w.get(fixed + OzScratch::bytes(N, m, 1), /*may_fail=*/true);
+    if (!oz) w.get(fixed + (size_t)N * m * sizeof(double), false);
+    double* part = w.take<double>(cap);
+    double* S = w.take<double>(mm);
+    double* Linv = w.take<double>(mm);
+    double* R = w.take<double>(mm);
+    double* gw = w.take<double>(cw);  // padded factorisation workspace
+    auto* sc = w.take<trm::IterScalars>(1);
     int status = 0;
-    try {
-      TRM_CUDA(cudaMemsetAsync(sc, 0, sizeof(trm::IterScalars), s));
+    TRM_CUDA(cudaMemsetAsync(sc, 0, sizeof(trm::IterScalars), s));
+    if (oz) {
+      OzScratch z(w, N, m, 1);
+      trm::oz_slice(N, m, C, N, z.block[0], s);
+      trm::oz_gram(&z.block[0], 1, z.block[0], S, part, cap, &sc->status, s);
+      trm::chol_inv<double>(m, S, Linv, R, sc, gw, s);
+      trm::oz_mult(z.block[0], m, R, true, z.small, C, N, &sc->status, s);
+    } else {
+      double* Cn = w.take<double>((size_t)N * m);
       trm::Blocks<double> b;
       b.p[0] = C;
       b.cols = m;
@@ -360,15 +430,12 @@ trm_status trm_orthonormalize(int64_t N, int m, double* C, void* stream) {
       trm::rotate<double, double>(N, m, C, nullptr, R, Cn, nullptr, s);
       TRM_CUDA(cudaMemcpyAsync(C, Cn, (size_t)N * m * 8,
                                cudaMemcpyDeviceToDevice, s));
-      TRM_CUDA(cudaMemcpyAsync(&status, &sc->status, sizeof(int),
-                               cudaMemcpyDeviceToHost, s));
-      TRM_CUDA(cudaStreamSynchronize(s));
-    } catch (...) {
-      cudaFreeAsync(w, s);
-      throw;
     }
-    TRM_CUDA(cudaFreeAsync(w, s));
+    TRM_CUDA(cudaMemcpyAsync(&status, &sc->status, sizeof(int),
+                             cudaMemcpyDeviceToHost, s));
     TRM_CUDA(cudaStreamSynchronize(s));
+    if (status & 2)
+      return fail(nullptr, TRM_ETIMEOUT, "trm_orthonormalize: a device wait timed out");
     if (status & 1)
       return fail(nullptr, TRM_ENOTPD, "C^T C is not positive definite");
     return (int)TRM_OK;
@@ -388,68 +455,77 @@ trm_status trm_extrapolate(int64_t N, int m, const double* C_prev,
     const size_t cap = trm::gram_partials_doubles(N, m, m);
     const size_t pw = trm::polar_work_doubles(m);
     const size_t cw = trm::chol_work_elems(m);
-    const size_t bytes = (cap + 5 * mm + pw + cw + Nm) * sizeof(double) +
-                         sizeof(trm::IterScalars) + 2 * sizeof(int);
-    char* w = nullptr;
-    TRM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&w), bytes, s));
-    double* part = reinterpret_cast<double*>(w);
-    double* M = part + cap;
-    double* U = M + mm;
-    double* S = U + mm;
-    double* Linv = S + mm;
-    double* R = Linv + mm;
-    double* pwork = R + mm;
-    double* gw = pwork + pw;
-    double* Y = gw + cw;
-    auto* sc = reinterpret_cast<trm::IterScalars*>(Y + Nm);
-    int* info = reinterpret_cast<int*>(sc + 1);  // [eig sweeps, polar status]
+    const size_t fixed = (cap + 5 * mm + pw + cw + Nm) * sizeof(double) +
+                         sizeof(trm::IterScalars) + 2 * sizeof(int) + 512;
+    Scratch w(s);
+    const bool oz =
+        trm::oz_pays(N, m, m) &&
+        w.get(fixed + OzScratch::bytes(N, m, 2), /*may_fail=*/true);
+    if (!oz) w.get(fixed, false);
+    double* part = w.take<double>(cap);
+    double* M = w.take<double>(mm);
+    double* U = w.take<double>(mm);
+    double* S = w.take<double>(mm);
+    double* Linv = w.take<double>(mm);
+    double* R = w.take<double>(mm);
+    double* pwork = w.take<double>(pw);
+    double* gw = w.take<double>(cw);
+    double* Y = w.take<double>(Nm);
+    auto* sc = w.take<trm::IterScalars>(1);
+    int* info = w.take<int>(2);  // [eig sweeps, polar status]
     int flags[2] = {0, 0};
     int status = 0;
-    try {
-      TRM_CUDA(cudaMemsetAsync(sc, 0, sizeof(trm::IterScalars) + 2 * sizeof(int), s));
-      // align C_prev to C_cur: U = polar(C_prev^T C_cur)
+    TRM_CUDA(cudaMemsetAsync(sc, 0, sizeof(trm::IterScalars), s));
+    TRM_CUDA(cudaMemsetAsync(info, 0, 2 * sizeof(int), s));
+    // align C_prev to C_cur: U = polar(C_prev^T C_cur)
+    std::optional<OzScratch> z;
+    if (oz) {
+      z.emplace(w, N, m, 2);
+      trm::oz_slice(N, m, C_prev, N, z->block[0], s);
+      trm::oz_slice(N, m, C_cur, N, z->block[1], s);
+      trm::oz_gram(&z->block[0], 1, z->block[1], M, part, cap, &sc->status, s);
+    } else {
       trm::Blocks<double> b;
       b.p[0] = C_cur;
       b.cols = m;
       b.count = 1;
       trm::gram<double>(N, m, C_prev, b, M, part, cap, s);
-      trm::polar_factor(m, M, U, pwork, info + 1, info, s);
-      TRM_CUDA(cudaMemcpyAsync(flags, info, 2 * sizeof(int),
-                               cudaMemcpyDeviceToHost, s));
-      TRM_CUDA(cudaStreamSynchronize(s));
-    } catch (...) {
-      cudaFreeAsync(w, s);
-      throw;
     }
-    if (flags[1] & 1) {
-      TRM_CUDA(cudaFreeAsync(w, s));
-      TRM_CUDA(cudaStreamSynchronize(s));
+    trm::polar_factor(m, M, U, pwork, info + 1, info, s);
+    TRM_CUDA(cudaMemcpyAsync(flags, info, 2 * sizeof(int),
+                             cudaMemcpyDeviceToHost, s));
+    TRM_CUDA(cudaStreamSynchronize(s));
+    if (flags[1] & 1)
       return fail(nullptr, TRM_ENOTPD,
                   "C_prev^T C_cur is singular: the subspaces are too far "
                   "apart to align");
-    }
-    try {
-      trm::Blocks<double> b;
-      b.cols = m;
-      b.count = 1;
-      // C_next = (1 + alpha) C_cur - alpha C_prev U
+    // C_next = (1 + alpha) C_cur - alpha C_prev U, then Fig. ONFIG:
+    // C_next <- C_next L^{-T}
+    if (oz) {
+      // (C_next before its orthonormalization is needed as digits only)
+      trm::oz_mult(z->block[0], m, U, false, z->small, Y, N, &sc->status, s);
+      trm::oz_slice(N, m, C_cur, N, z->block[1], s, Y, nullptr, 1.0 + alpha,
+                    -alpha);
+      trm::oz_gram(&z->block[1], 1, z->block[1], S, part, cap, &sc->status, s);
+      trm::chol_inv<double>(m, S, Linv, R, sc, gw, s);
+      trm::oz_mult(z->block[1], m, R, true, z->small, C_next, N, &sc->status, s);
+    } else {
       trm::mult(N, m, m, C_prev, U, Y, s);
       trm::lin_comb((int64_t)Nm, 1.0 + alpha, C_cur, -alpha, Y, C_next, s);
-      // Fig. ONFIG: C_next <- C_next L^{-T}
+      trm::Blocks<double> b;
       b.p[0] = C_next;
+      b.cols = m;
+      b.count = 1;
       trm::gram<double>(N, m, C_next, b, S, part, cap, s);
       trm::chol_inv<double>(m, S, Linv, R, sc, gw, s);
       trm::rotate<double, double>(N, m, C_next, nullptr, R, Y, nullptr, s);
       TRM_CUDA(cudaMemcpyAsync(C_next, Y, Nm * 8, cudaMemcpyDeviceToDevice, s));
-      TRM_CUDA(cudaMemcpyAsync(&status, &sc->status, sizeof(int),
-                               cudaMemcpyDeviceToHost, s));
-      TRM_CUDA(cudaStreamSynchronize(s));
-    } catch (...) {
-      cudaFreeAsync(w, s);
-      throw;
     }
-    TRM_CUDA(cudaFreeAsync(w, s));
+    TRM_CUDA(cudaMemcpyAsync(&status, &sc->status, sizeof(int),
+                             cudaMemcpyDeviceToHost, s));
     TRM_CUDA(cudaStreamSynchronize(s));
+    if (status & 2)
+      return fail(nullptr, TRM_ETIMEOUT, "trm_extrapolate: a device wait timed out");
     if (status & 1)
       return fail(nullptr, TRM_ENOTPD, "C_next^T C_next is not positive definite");
     return (int)TRM_OK;

@@ -672,6 +672,14 @@ void energy_from_dots(const double* dots, int chunks, int m, double* HD,
   colsum(dots, chunks, m, HD, sc, 0, s);
 }
 
+int column_dots(int64_t N, int m, const double* A, const double* B,
+                double* dots, cudaStream_t s) {
+  const int chunks = ceil_div(N, RCHUNK);
+  k_coldot<double><<<dim3(chunks, m), 256, 0, s>>>(N, m, A, B, dots);
+  TRM_CHECK_LAUNCH();
+  return chunks;
+}
+
 template <typename T>
 void energy_diag(int64_t N, int m, const T* C, const T* X, double* HD,
                  IterScalars* sc, double* partials, cudaStream_t s) {
@@ -727,9 +735,14 @@ void gradient(int64_t N, int m, const T* C, const T* Xp, const double* Hp,
   k_gradient<T><<<grid, 256, 0, s>>>(N, m, C, Xp, Hp, G, Gprev, Pprev, minv,
                                      partials);
   TRM_CHECK_LAUNCH();
+  cg_from_parts(partials, (int)nparts, m, sc, s);
+}
+
+void cg_from_parts(const double* part, int n, int m, IterScalars* sc,
+                   cudaStream_t s) {
   // (one SM adds them two a cycle: more threads than records only wait)
-  const int ct = nparts <= 256 ? 128 : nparts <= 1024 ? 256 : 512;
-  k_cg_scalars<<<1, ct, 0, s>>>(partials, (int)nparts, m, sc);
+  const int ct = n <= 256 ? 128 : n <= 1024 ? 256 : 512;
+  k_cg_scalars<<<1, ct, 0, s>>>(part, n, m, sc);
   TRM_CHECK_LAUNCH();
 }
 

@@ -177,12 +177,57 @@ void gram_in_scratch(int64_t N, int m, const T* A, const Blocks<T>& B,
                      cudaStream_t s);
 
 // ---------------------------------------------------------------------------
+// FP64 Grams and products on the tensor cores (oz.cu): a block is cut into
+// eight BF16 digit arrays (oz_slice), which Grams (contraction over rows) and
+// products with a small matrix (over columns) both read.
+// ---------------------------------------------------------------------------
+struct OzBlock {
+  void* digits = nullptr;   // oz_block_bytes(N, m), 16-byte aligned
+  double* scale = nullptr;  // m column scales
+  int64_t N = 0;            // set by oz_slice
+  int m = 0;
+};
+struct OzSmall {            // the same for a product's small factor (k x n)
+  void* digits = nullptr;   // oz_small_bytes(k, n)
+  double* scale = nullptr;  // n
+};
+// Does the product of this size run faster this way than in FP64 arithmetic?
+bool oz_pays(int64_t N, int m, int n);
+size_t oz_block_bytes(int64_t N, int m);
+size_t oz_small_bytes(int k, int n);
+// digits of C (columns ldc apart), or, with P, of fc C + fp P (fp = sc->alpha
+// when sc is given)
+void oz_slice(int64_t N, int m, const double* C, int64_t ldc, OzBlock& out,
+              cudaStream_t s, const double* P = nullptr,
+              const IterScalars* sc = nullptr, double fc = 1.0,
+              double fp = 0.0);
+// out = [A_0 | A_1 ...]^T B per segment (segs <= 2): segs m x n matrices one
+// after the other; partials as gram's; err receives bit 2 on a timeout
+void oz_gram(const OzBlock* a, int segs, const OzBlock& b, double* out,
+             double* partials, size_t cap, int* err, cudaStream_t s);
+// Y = A M (M: a.m x n FP64, upper triangular if tri; columns of Y ldy apart)
+void oz_mult(const OzBlock& a, int n, const double* M, bool tri,
+             const OzSmall& w, double* Y, int64_t ldy, int* err, cudaStream_t s);
+// CTAs of a product: oz_grad writes four sums each
+int oz_product_parts(int64_t N, int n);
+// G = -2 (X' - A H') and the Polak-Ribiere sums, from which the CG scalars in
+// sc are updated (part: four doubles per CTA)
+void oz_grad(const OzBlock& a, const double* Hp, const OzSmall& w,
+             const double* Xp, double* G, const double* Gprev,
+             const double* Pprev, const double* minv, int64_t ld, double* part,
+             IterScalars* sc, cudaStream_t s);
+
+// ---------------------------------------------------------------------------
 // Tall-skinny products and fused row-local updates
 // ---------------------------------------------------------------------------
 // H_D[j] = sum_i C_ij X_ij (FP64), E = sum_j H_D[j] into sc->E
 template <typename T>
 void energy_diag(int64_t N, int m, const T* C, const T* X, double* HD,
                  IterScalars* sc, double* partials, cudaStream_t s);
+// dots[chunk * m + j] = column dots of A and B per chunk of rows (FP64);
+// returns the number of chunks
+int column_dots(int64_t N, int m, const double* A, const double* B,
+                double* dots, cudaStream_t s);
 // H_D[j] = sum over chunks of dots (from apply_h_dots), E into sc->E
 void energy_from_dots(const double* dots, int chunks, int m, double* HD,
                       IterScalars* sc, cudaStream_t s);
@@ -239,6 +284,9 @@ void gradient(int64_t N, int m, const T* C, const T* Xp, const double* Hp,
               T* G, const T* Gprev, const T* Pprev, const T* minv,
               IterScalars* sc, double* partials, size_t partials_cap,
               cudaStream_t s, const TcWork* tw = nullptr, bool split = false);
+// The CG scalars from n records of the four gradient sums.
+void cg_from_parts(const double* part, int n, int m, IterScalars* sc,
+                   cudaStream_t s);
 // P = M G + gamma P (gamma from sc)
 template <typename T>
 void update_p(int64_t N, int m, const T* G, T* P, const T* minv,

@@ -247,6 +247,7 @@ size_t Solver::footprint(int64_t n_rows, int m) {
   b += sym_eig_work_doubles(m) * 8 + 5 * mm * 4;
   b += part_capacity(N, m) * 8 + sizeof(IterScalars) + 16;
   b += 2 * mul_tc_work_floats(m, m) * 4;
+  b += 1024 + 3 * m * 8;                     // slack of the pool, scales
   b += (size_t)N * (8 + 4 + 4 + 8 + 4 + 8);  // diagonals, M, V
   return b + (64u << 10);                    // allocation granularity
 }
@@ -262,12 +263,21 @@ Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
   C64_ = d(nm);
   C64n_ = d(nm);
   X64_ = d(nm);
-  C32_ = f(nm);
-  C32n_ = f(nm);
-  X32_ = f(nm);
-  Cdf_ = f(2 * nm);  // MP2 blocks as FP32 pairs: hi at [0, nm), lo after
-  Cdfn_ = f(2 * nm);
-  Xdf_ = f(2 * nm);
+  // The FP32 blocks in one allocation: FP64 Grams and products on the tensor
+  // cores keep the digits of two blocks there (32 of the 36 bytes an entry),
+  // always while none of them holds anything
+  float* pool = f(9 * nm + 256);
+  ozA_.digits = pool;
+  ozB_.digits = reinterpret_cast<char*>(pool) + oz_block_bytes(ld_, m) / 256 * 256;
+  C32_ = pool;
+  C32n_ = C32_ + nm;
+  X32_ = C32n_ + nm;
+  Cdf_ = X32_ + nm;  // MP2 blocks as FP32 pairs: hi at [0, nm), lo after
+  Cdfn_ = Cdf_ + 2 * nm;
+  Xdf_ = Cdfn_ + 2 * nm;
+  ozA_.scale = d(3 * m);
+  ozB_.scale = ozA_.scale + m;
+  ozw_.scale = ozB_.scale + m;
   Gb_[0] = d(nm);
   Gb_[1] = d(nm);
   Pb_ = d(nm);
@@ -300,6 +310,10 @@ Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
   Z_ = d(mm);
   mmw_ = d(std::max(2 * mm, chol_work_elems(m)));
   eigws_ = d(sym_eig_work_doubles(m));
+  ozw_.digits = eigws_;
+  oz_ = oz_pays(N, m, m) &&
+        2 * oz_block_bytes(ld_, m) <= (9 * nm + 256) * sizeof(float) &&
+        oz_small_bytes(m, m) <= sym_eig_work_doubles(m) * sizeof(double);
   Hp32_ = f(mm);
   Bm32_ = f(4 * mm);
   PG32_ = Bm32_ + mm;
@@ -648,6 +662,14 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
   }
   TRM_PROF(KC_ROWOPS, 2 * nm, 3 * es * nm,
            xprime<T>(ld_, m_, Yc, X, HD_, nullptr, nullptr, s_));      // (5)
+  if constexpr (sizeof(T) == 8) {
+    if (oz_) {
+      iter_fp64_tail(C, Cn, X, G, Gp, P, HP, gen);
+      std::swap(C, Cn);
+      std::swap(G, Gp);
+      return;
+    }
+  }
   Blocks<T> bx;
   bx.p[0] = X;
   bx.cols = m_;
@@ -745,6 +767,74 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
   }
   std::swap(C, Cn);
   std::swap(G, Gp);
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 iteration from (6) on with its contractions on the tensor cores
+// (oz.cu): each block is cut into digits once for all the products it enters.
+// The digits of at most two blocks are held at a time, so the line search's
+// Grams run as [C P]^T P and P^T G; of P^T H P only the trace is needed, as the
+// column dots of P and H P. (Generalized problem: Y = S C in C's place after
+// H', S P in P's in the overlap's Gram, and Y is rotated along with C.)
+// ---------------------------------------------------------------------------
+void Solver::iter_fp64_tail(double* C, double* Cn, const double* X, double* G,
+                            const double* Gp, double* P, double* HP, bool gen) {
+  const double* minv = opt_.precond ? minv64_ : nullptr;
+  const size_t mm = (size_t)m_ * m_;
+  const double md = m_, nm = (double)N_ * md, m2N = nm * md;
+  int* err = &sc_->status;
+  double sfl, sby;
+  spmm_cost(op_, m_, 8, &sfl, &sby);
+  auto slice = [&](const double* B, OzBlock& o, const double* Q = nullptr) {
+    TRM_PROF(KC_ROWOPS, 0.0, (Q ? 32.0 : 24.0) * nm,
+             oz_slice(ld_, m_, B, ld_, o, s_, Q, Q ? sc_ : nullptr));
+  };
+  slice(C, ozA_);
+  slice(X, ozB_);
+  TRM_PROF(KC_GRAM64, 2 * m2N, 16 * nm,
+           oz_gram(&ozA_, 1, ozB_, Hp_, part_, part_cap_, err, s_));   // (6)
+  if (gen) slice(Y64_, ozA_);
+  TRM_PROF(KC_GRAD64, 2 * m2N, 40 * nm,
+           oz_grad(ozA_, Hp_, ozw_, X, G, Gp, P, minv, ld_, part_, sc_,
+                   s_));                                               // (7)
+  TRM_PROF(KC_ROWOPS, 2 * nm, 24 * nm,
+           update_p<double>(ld_, m_, G, P, minv, sc_, s_));            // P
+  TRM_PROF(KC_SPMM64, sfl, sby, apply_h(op_, P, HP, m_, s_));          // H P
+  int chunks = 0;
+  TRM_PROF(KC_ROWOPS, 2 * nm, 16 * nm,
+           chunks = column_dots(ld_, m_, P, HP, hpdots_, s_));
+  slice(P, ozB_);
+  if (gen) {
+    double ffl, fby;
+    spmm_cost(sop_, m_, 8, &ffl, &fby);
+    TRM_PROF(KC_GRAM64, 2 * m2N, 16 * nm,
+             oz_gram(&ozA_, 1, ozB_, Bm_, part_, part_cap_, err, s_));  // Y^T P
+    TRM_PROF(KC_SPMM64, ffl, fby, apply_h(sop_, P, SP64_, m_, s_));     // S P
+    slice(SP64_, ozA_);
+    TRM_PROF(KC_GRAM64, 2 * m2N, 16 * nm,
+             oz_gram(&ozB_, 1, ozA_, PG_, part_, part_cap_, err, s_));  // P^T S P
+  } else {
+    const OzBlock cp[2] = {ozA_, ozB_};
+    TRM_PROF(KC_GRAM64, 4 * m2N, 16 * nm,
+             oz_gram(cp, 2, ozB_, Bm_, part_, part_cap_, err, s_));  // [C P]^T P
+  }
+  slice(G, ozA_);
+  TRM_PROF(KC_GRAM64, 2 * m2N, 16 * nm,
+           oz_gram(&ozB_, 1, ozA_, PG_ + mm, part_, part_cap_, err, s_));  // P^T G
+  prof.begin(KC_SMALL, s_);
+  line_factor<double>(m_, Hp_, HD_, Bm_, PG_, nullptr, m_ + 1, hpdots_,
+                      chunks * m_, PG_ + mm, nullptr, R_, sc_, mmw_, T1_, false,
+                      s_);
+  prof.end(KC_SMALL, 4 * md * md * md + 2 * md * md * md / 3, 0.0, s_);
+  slice(C, ozA_, P);                                           // C + alpha P
+  TRM_PROF(KC_ROT64, m2N, 16 * nm,
+           oz_mult(ozA_, m_, R_, true, ozw_, Cn, ld_, err, s_));
+  if (gen) {
+    slice(Y64_, ozA_, SP64_);
+    TRM_PROF(KC_ROT64, m2N, 16 * nm,
+             oz_mult(ozA_, m_, R_, true, ozw_, Y64n_, ld_, err, s_));
+    std::swap(Y64_, Y64n_);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -856,27 +946,54 @@ void Solver::iter_mp2() {
 void Solver::c64_to_df() {
   const size_t nm = (size_t)ld_ * m_;
   split_df(C64_, Cdf_, Cdf_ + nm, (int64_t)nm, s_);
+  if (oz_ && ld_ != N_) {  // digits lay where X and X' keep zero rows
+    PadList l;
+    l.add(X32_, 4);
+    l.add(Xdf_, 4);
+    l.add(Xdf_ + nm, 4);
+    clear_pad_rows(l, N_, ld_, m_, s_);
+  }
 }
 void Solver::df_to_c64() {
   const size_t nm = (size_t)ld_ * m_;
   join_df(Cdf_, Cdf_ + nm, C64_, (int64_t)nm, s_);
 }
 
-// The N-deep Grams of FP64 blocks: FP64 in the all-FP64 mode, double-float
-// (FP64-class, on the FP32 pipe) in the mixed ladder.
+// The N-deep Grams of FP64 blocks: on the tensor cores where that pays, else
+// FP64 in the all-FP64 mode, double-float (FP64-class, on the FP32 pipe) in the
+// mixed ladder. Leaves the digits of A in ozA_ and, if it is another block,
+// those of b in ozB_.
 void Solver::gram64(const double* A, const Blocks<double>& b, double* out) {
-  if (opt_.precision == TRM_FP64)
+  if (oz_) {
+    oz_slice(ld_, m_, A, ld_, ozA_, s_);
+    if (b.p[0] != A) oz_slice(ld_, m_, b.p[0], ld_, ozB_, s_);
+    oz_gram(&ozA_, 1, b.p[0] != A ? ozB_ : ozA_, out, part_, part_cap_,
+            &sc_->status, s_);
+  } else if (opt_.precision == TRM_FP64) {
     gram<double>(ld_, m_, A, b, out, part_, part_cap_, s_, &sc_->status);
-  else
+  } else {
     gram_df(ld_, m_, A, b, out, part_, part_cap_, s_);
+  }
 }
 
-// N x m times m x m products of FP64 blocks, FP64 or double-float as gram64.
-void Solver::mult64(const double* A, const double* M, double* Y) {
-  if (opt_.precision == TRM_FP64)
-    mult(ld_, m_, m_, A, M, Y, s_);
-  else
-    mult_df(ld_, m_, m_, A, M, Y, false, s_);
+// N x m times m x m products of FP64 blocks, as gram64 (tri: M is upper
+// triangular). digits: those of A, when they are at hand.
+void Solver::mult64(const double* A, const double* M, double* Y, bool tri,
+                    OzBlock* digits) {
+  if (oz_) {
+    if (!digits) {
+      digits = &ozA_;
+      oz_slice(ld_, m_, A, ld_, ozA_, s_);
+    }
+    oz_mult(*digits, m_, M, tri, ozw_, Y, ld_, &sc_->status, s_);
+  } else if (opt_.precision == TRM_FP64) {
+    if (tri)
+      rotate<double, double>(ld_, m_, A, nullptr, M, Y, nullptr, s_);
+    else
+      mult(ld_, m_, m_, A, M, Y, s_);
+  } else {
+    mult_df(ld_, m_, m_, A, M, Y, tri, s_);
+  }
 }
 
 // Fig. ONFIG in FP64: S = C^T C, S = L L^T, C <- C L^{-T} (generalized
@@ -896,15 +1013,16 @@ void Solver::orth_fp64(double*& C, double*& Cn) {
   TRM_PROF(KC_GRAM64, 2 * m2N, 16 * nm, gram64(C, b, S_));
   TRM_PROF(KC_SMALL, 2.0 * m_ * m_ * m_ / 3, 0.0,
            chol_inv<double>(m_, S_, Linv_, R_, sc_, mmw_, s_));
-  if (opt_.precision == TRM_FP64)
-    TRM_PROF(KC_ROT64, m2N, 16 * nm,
-             (rotate<double, double>(ld_, m_, C, nullptr, R_, Cn, nullptr, s_)));
-  else  // C L^{-T} in double-float
-    TRM_PROF(KC_ROT64, m2N, 16 * nm, mult_df(ld_, m_, m_, C, R_, Cn, true, s_));
+  TRM_PROF(KC_ROT64, m2N, 16 * nm,
+           mult64(C, R_, Cn, true, &ozA_));  // C L^{-T}, from gram64's digits
   if (has_S_) {
-    TRM_PROF(KC_ROT64, m2N, 16 * nm,
-             (rotate<double, double>(ld_, m_, Y64_, nullptr, R_, Y64n_, nullptr,
-                                     s_)));
+    if (oz_)
+      TRM_PROF(KC_ROT64, m2N, 16 * nm,
+               mult64(Y64_, R_, Y64n_, true, &ozB_));
+    else
+      TRM_PROF(KC_ROT64, m2N, 16 * nm,
+               (rotate<double, double>(ld_, m_, Y64_, nullptr, R_, Y64n_,
+                                       nullptr, s_)));
     std::swap(Y64_, Y64n_);
   }
   std::swap(C, Cn);
@@ -949,10 +1067,10 @@ void Solver::rr_rotate_fp64() {
   make_A0(m_, Hp_, nullptr, A0_, s_);
   TRM_PROF(KC_EIG, 0.0, 0.0, sym_eig(m_, A0_, eigw_, Z_, eigws_, info_, s_));
   const double nm = (double)N_ * m_;
-  TRM_PROF(KC_ROT64, 2 * nm * m_, 16 * nm, mult64(C64_, Z_, C64n_));
+  TRM_PROF(KC_ROT64, 2 * nm * m_, 16 * nm, mult64(C64_, Z_, C64n_, false, &ozA_));
   std::swap(C64_, C64n_);
   if (has_S_) {  // Y = S C follows the rotation
-    TRM_PROF(KC_ROT64, 2 * nm * m_, 16 * nm, mult64(Y64_, Z_, Y64n_));
+    TRM_PROF(KC_ROT64, 2 * nm * m_, 16 * nm, mult64(Y64_, Z_, Y64n_, false, nullptr));
     std::swap(Y64_, Y64n_);
   }
 }
@@ -979,7 +1097,14 @@ void Solver::final_rr(double* C, double* Cfin, double* Xfin) {
   // the overlap in FP64 in every mode: the returned block is orthonormalized
   // by its factor (the double-float Gram's sum over N rows is good to about
   // sqrt(N) 2^-48, which left C^T C - I near 1e-12 at N ~ 1e6)
-  gram<double>(ld_, m_, C, bc, S_, part_, part_cap_, s_);
+  if (oz_) {
+    // (gram64 above left the digits of C in ozA_ and of X in ozB_)
+    if (has_S_) oz_slice(ld_, m_, Y64_, ld_, ozB_, s_);
+    oz_gram(&ozA_, 1, has_S_ ? ozB_ : ozA_, S_, part_, part_cap_, &sc_->status,
+            s_);
+  } else {
+    gram<double>(ld_, m_, C, bc, S_, part_, part_cap_, s_);
+  }
   chol_inv<double>(m_, S_, Linv_, R_, sc_, mmw_, s_);
   mm_gemm(m_, Linv_, false, Hp_, false, T1_, 1.0, 0.0, s_);
   mm_gemm(m_, T1_, false, Linv_, true, T2_, 1.0, 0.0, s_);
@@ -988,10 +1113,13 @@ void Solver::final_rr(double* C, double* Cfin, double* Xfin) {
   mm_gemm(m_, R_, false, Z_, false, T1_, 1.0, 0.0, s_);
   // the returned block in FP64 in every mode; H C Y, used only for the
   // residual norms, keeps the FP64-class product
-  mult(ld_, m_, m_, C, T1_, Cfin, s_);
-  mult64(X64_, T1_, Xfin);
+  if (oz_)
+    oz_mult(ozA_, m_, T1_, false, ozw_, Cfin, ld_, &sc_->status, s_);
+  else
+    mult(ld_, m_, m_, C, T1_, Cfin, s_);
+  mult64(X64_, T1_, Xfin, false, has_S_ ? nullptr : &ozB_);
   if (has_S_) {  // ||H c_j - theta_j S c_j|| (sign independent)
-    mult64(Y64_, T1_, SP64_);
+    mult64(Y64_, T1_, SP64_, false, &ozB_);
     column_residuals(ld_, m_, Xfin, SP64_, lam_, res_, part_, s_);
     fix_signs(ld_, m_, Cfin, Xfin, part_, s_);
     return;

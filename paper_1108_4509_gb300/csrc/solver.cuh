@@ -125,7 +125,10 @@ class Solver {
   void iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP);
   void iter_mp2();
   void gram64(const double* A, const Blocks<double>& b, double* out);
-  void mult64(const double* A, const double* M, double* Y);
+  void mult64(const double* A, const double* M, double* Y, bool tri,
+              OzBlock* digits);
+  void iter_fp64_tail(double* C, double* Cn, const double* X, double* G,
+                      const double* Gp, double* P, double* HP, bool gen);
   // The line-search Grams as one tensor-core launch [C P P]^T [P P G]
   // (C^T P, P^T P upper tiles mirrored, P^T G), with the diagonal of
   // P^T H P taken as column dots of the stencil applied to P (hpd_), when
@@ -200,6 +203,11 @@ class Solver {
   int* info_;
   // FP32 copies of H', B = C^T P and P^T [P HP G] (the Gram sums write them)
   float *Hp32_ = nullptr, *Bm32_ = nullptr, *PG32_ = nullptr;
+  // digits of two FP64 blocks and of a product's small factor (oz.cu), and
+  // whether products of this size take them
+  OzBlock ozA_, ozB_;
+  OzSmall ozw_;
+  bool oz_ = false;
   double* part_;
   size_t part_cap_;
   IterScalars* sc_;

@@ -209,3 +209,84 @@ def test_padded_columns_solve(trm, shape, m):
         assert np.max(np.abs(op.apply_h(H, Ch) - Ch * lam)) < 1e-8
     finally:
         trm.trm_destroy(h)
+
+
+@pytest.mark.parametrize("N,m", [(500009, 8), (20001, 63), (20002, 64),
+                                 (20003, 65), (6000, 127), (6000, 128),
+                                 (6001, 129), (3000, 200), (1031, 256),
+                                 (1024, 300)])
+def test_digit_products_orthonormalize(trm, N, m):
+    """Fig. ONFIG through the digit Gram and product at the edges of their
+    128 x 64 tiles and 32-row stages. Columns of very different size are
+    scaled one by one, so they cost no accuracy: the result is that of the
+    unscaled columns to rounding times the condition of the overlap (at most
+    a few for random columns of these shapes; 40 with m = N / 4)."""
+    C = ti.random_block(N, m, seed=4)
+    scale = 10.0 ** np.linspace(-15, 15, m)
+    ref = otrm.orthonormalize(C)
+    for block in (C, C * scale):
+        cd = gu.to_dev(block)
+        trm.trm_orthonormalize(N, m, cd.data_ptr(), gu.stream())
+        got = gu.from_dev(cd)
+        assert np.max(np.abs(got.T @ got - np.eye(m))) < 1e-13
+        assert np.max(np.abs(got - ref)) < 1e-13
+
+
+def test_digit_products_constant_and_non_finite(trm):
+    """The integer sums at their largest (equal entries, all digits at an
+    extreme), a zero column, and an infinity or NaN, which must not vanish."""
+    N, m = 8192, 64
+    x = np.nextafter(1.0, 0.0)
+    C = np.zeros((N, m), order="F")
+    step = N // m
+    for j in range(m):  # orthogonal: one constant stretch per column
+        C[j * step:(j + 1) * step, j] = x * 2.0 ** (j - 30)
+    cd = gu.to_dev(C)
+    trm.trm_orthonormalize(N, m, cd.data_ptr(), gu.stream())
+    got = gu.from_dev(cd)
+    ref = (C != 0) / np.sqrt(step)
+    assert np.max(np.abs(got - ref)) < 1e-15
+    one = np.full((N, 8), x)
+    one[:, 1:] *= (np.arange(N)[:, None] % np.arange(2, 9) == 0)
+    wide = np.concatenate([one] + [ti.random_block(N, 56, seed=2)], axis=1)
+    cd = gu.to_dev(wide)
+    trm.trm_orthonormalize(N, m, cd.data_ptr(), gu.stream())
+    assert np.max(np.abs(gu.from_dev(cd) - otrm.orthonormalize(wide))) < 1e-12
+    for bad in (np.inf, np.nan, 0.0):
+        D = np.array(wide, order="F")
+        if bad == 0.0:
+            D[:, 5] = 0.0
+        else:
+            D[77, 5] = bad
+        cd = gu.to_dev(D)
+        with pytest.raises(trm.TrmError) as e:
+            trm.trm_orthonormalize(N, m, cd.data_ptr(), gu.stream())
+        assert e.value.status == -3
+
+
+@pytest.mark.parametrize("shape,m", [((15, 14, 13), 200), ((16, 16, 12), 130),
+                                     ((31, 33, 35), 33)])
+def test_digit_products_fp64_step(trm, shape, m):
+    """One FP64 iteration whose contractions run on digits, against the same
+    step formed in FP64 on the host: rounding times the magnitudes involved."""
+    V = ti.gaussian_wells(shape, 4, seed=6)
+    H = op.grid_hamiltonian(shape, 4, 1.0, V)
+    N = V.size
+    C = otrm.orthonormalize(ti.random_block(N, m, seed=3))
+    E0, G0, _, _ = otrm.energy_gradient_alg1(H, C)
+    opt = trm.trm_default_options(stream=gu.stream(), precision=trm.TRM_FP64)
+    h = trm.trm_create_stencil(*shape, 4, 1.0, V, m, 1e-10, opt)
+    try:
+        cd = gu.to_dev(C)
+        trm.trm_set_block(h, cd.data_ptr())
+        E, r, a = trm.trm_iterate(h, trm.TRM_FP64)
+        out = gu.empty(N, m, np.float64)
+        trm.trm_get_block(h, out.data_ptr())
+        C1 = gu.from_dev(out)
+    finally:
+        trm.trm_destroy(h)
+    assert E == pytest.approx(E0, rel=1e-13)
+    assert r == pytest.approx(otrm.rms_residual(G0), rel=1e-12)
+    Y = C + a * G0
+    L = np.linalg.cholesky(Y.T @ Y)
+    assert np.max(np.abs(C1 - np.linalg.solve(L, Y.T).T)) < 1e-12
