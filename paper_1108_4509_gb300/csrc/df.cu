@@ -17,18 +17,6 @@ namespace trm {
 
 namespace {
 
-// Neighbour-sum accumulator: the hi parts are added exactly (TwoSum), the
-// lo parts and the rounding errors plainly; normalised once at the end.
-struct Acc {
-  float h = 0.f, l = 0.f;
-  __device__ __forceinline__ void add(float vh, float vl) {
-    const F2 t = two_sum(h, vh);
-    h = t.h;
-    l += t.l + vl;
-  }
-  __device__ __forceinline__ F2 get() const { return quick_two_sum(h, l); }
-};
-
 // hi + lo in FP64, widened on the integer pipe: one FP64 instruction (the
 // sum) instead of three.
 __device__ __forceinline__ double widen(float f) {
@@ -84,243 +72,262 @@ __global__ void __launch_bounds__(256)
 
 constexpr int kCols = 4;  // columns per CTA (grid.y walks column groups)
 
-// X = H C for the stencil operator, one grid point per thread.
-template <int R>
-__global__ void __launch_bounds__(256)
-    k_stencil_df(StencilOp st, int64_t N, int64_t ld, const float* __restrict__ dh,
+// ---------------------------------------------------------------------------
+// X = H C for the stencil operator as a register z-march (see k_stencil_zm): a
+// thread owns VW (2 or 1) consecutive x points of one column and walks a chunk
+// of planes with the 2R + 1 pairs of each along z in registers. The FP32 pipe is
+// what bounds it, so the pairs are summed without intermediate normalisations:
+// the hi parts by TwoSum, the lo parts and rounding errors plainly, the three
+// products as (fl, error) by fused multiply-adds, one renormalisation at the
+// end: about 112 operations a point, the errors a few units of 2^-48 of the
+// magnitudes as before. The column dots H_D = c_j . (H c)_j of
+// Fig. EGFIG step (2) are formed from the pairs in registers (double-float per
+// thread and warp, one FP64 add per warp): CTA (t, u) writes
+// dots[(u gridDim.x + t) ncols + column].
+// It replaces kernels that took the z neighbours through L2 with two CTAs per
+// SM (98 registers): 160 us at 48^3 x 128, 4.94 ms at 96^3 x 512.
+// ---------------------------------------------------------------------------
+// s + l += (h, l) of a neighbour
+__device__ __forceinline__ void acc_add(F2& a, float h, float l) {
+  const F2 t = two_sum(a.h, h);
+  a.h = t.h;
+  a.l += t.l + l;
+}
+// p + e = a b with |e| at 2^-48 of the product (not renormalised)
+__device__ __forceinline__ F2 prod_df(F2 a, F2 b) {
+  const float p = a.h * b.h;
+  float e = fmaf(a.h, b.h, -p);
+  e = fmaf(a.h, b.l, e);
+  return {p, fmaf(a.l, b.h, e)};
+}
+template <int VW>
+struct PairV {
+  float h[VW], l[VW];
+};
+template <int VW>
+__device__ __forceinline__ PairV<VW> ldp(const float* h, const float* l,
+                                         int64_t o, bool in) {
+  PairV<VW> v;
+  if constexpr (VW == 2) {
+    const float2 z = make_float2(0.f, 0.f);
+    const float2 a = in ? __ldg(reinterpret_cast<const float2*>(h + o)) : z;
+    const float2 b = in ? __ldg(reinterpret_cast<const float2*>(l + o)) : z;
+    v.h[0] = a.x; v.h[1] = a.y;
+    v.l[0] = b.x; v.l[1] = b.y;
+  } else {
+    v.h[0] = in ? __ldg(h + o) : 0.f;
+    v.l[0] = in ? __ldg(l + o) : 0.f;
+  }
+  return v;
+}
+
+template <int R, int VW>
+__global__ void __launch_bounds__(256, 3)
+    k_stencil_df(StencilOp st, int64_t ld, const float* __restrict__ dh,
                  const float* __restrict__ dl, const float* __restrict__ Ch,
                  const float* __restrict__ Cl, float* __restrict__ Xh,
-                 float* __restrict__ Xl, int ncols) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const int x = (int)(i % st.nx);
-  const int64_t yz = i / st.nx;
-  const int y = (int)(yz % st.ny);
-  const int z = (int)(yz / st.ny);
-  const int64_t sy = st.nx, sz = (int64_t)st.nx * st.ny;
-  const F2 d = {dh[i], dl[i]};
+                 float* __restrict__ Xl, int ncols, int zc,
+                 double* __restrict__ dots) {
+  __shared__ double red[8];
+  const int nx = st.nx, ny = st.ny, nz = st.nz, nxq = nx / VW;
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;  // group in the plane
+  const bool active = p < nxq * ny;
+  const int x0 = active ? VW * (p % nxq) : 0, y = active ? p / nxq : 0;
+  const int col = blockIdx.z;
+  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc);
+  const int64_t sz = (int64_t)nx * ny;
+  const int64_t rowoff = (int64_t)y * nx + x0;
+  const float* ch = Ch + (int64_t)col * ld + rowoff;
+  const float* cl = Cl + (int64_t)col * ld + rowoff;
+  const bool ym1 = y >= 1, yp1 = y + 1 < ny, ym2 = y >= 2, yp2 = y + 2 < ny;
   const F2 c1 = {st.c1h, st.c1l}, c2 = {st.c2h, st.c2l};
-  // neighbours present at this point (Dirichlet: absent ones are 0)
-  const bool xm1 = x >= 1, xp1 = x + 1 < st.nx, ym1 = y >= 1,
-             yp1 = y + 1 < st.ny, zm1 = z >= 1, zp1 = z + 1 < st.nz;
-  const bool xm2 = x >= 2, xp2 = x + 2 < st.nx, ym2 = y >= 2,
-             yp2 = y + 2 < st.ny, zm2 = z >= 2, zp2 = z + 2 < st.nz;
-  const int cb = blockIdx.y * kCols;
-  for (int q = 0; q < kCols; ++q) {
-    const int c = cb + q;
-    if (c >= ncols) break;
-    const int64_t base = (int64_t)c * ld + i;
-    const float* ph = Ch + base;
-    const float* pl = Cl + base;
-    Acc s1, s2;
-    if (xm1) s1.add(__ldg(ph - 1), __ldg(pl - 1));
-    if (xp1) s1.add(__ldg(ph + 1), __ldg(pl + 1));
-    if (ym1) s1.add(__ldg(ph - sy), __ldg(pl - sy));
-    if (yp1) s1.add(__ldg(ph + sy), __ldg(pl + sy));
-    if (zm1) s1.add(__ldg(ph - sz), __ldg(pl - sz));
-    if (zp1) s1.add(__ldg(ph + sz), __ldg(pl + sz));
-    if (R == 2) {
-      if (xm2) s2.add(__ldg(ph - 2), __ldg(pl - 2));
-      if (xp2) s2.add(__ldg(ph + 2), __ldg(pl + 2));
-      if (ym2) s2.add(__ldg(ph - 2 * sy), __ldg(pl - 2 * sy));
-      if (yp2) s2.add(__ldg(ph + 2 * sy), __ldg(pl + 2 * sy));
-      if (zm2) s2.add(__ldg(ph - 2 * sz), __ldg(pl - 2 * sz));
-      if (zp2) s2.add(__ldg(ph + 2 * sz), __ldg(pl + 2 * sz));
+  PairV<VW> q[2 * R + 2];  // planes z - R .. z + R, and z + R + 1 in flight
+#pragma unroll
+  for (int k = 0; k < 2 * R + 1; ++k) {
+    const int pz = z0 - R + k;
+    q[k] = ldp<VW>(ch, cl, pz * sz, active && pz >= 0 && pz < nz);
+  }
+  F2 dacc = {0.f, 0.f};
+  for (int z = z0; z < z1; ++z) {
+    const int64_t o = z * sz;
+    q[2 * R + 1] = ldp<VW>(ch, cl, o + (R + 1) * sz,
+                           active && z + R + 1 < nz && z + 1 < z1);
+    if (active) {
+      // the row's values x0 - 2 .. x0 + VW + 1
+      float eh[VW + 4], el[VW + 4];
+#pragma unroll
+      for (int k = 0; k < VW; ++k) {
+        eh[k + 2] = q[R].h[k];
+        el[k + 2] = q[R].l[k];
+      }
+      if constexpr (VW == 2) {
+        const PairV<2> a = ldp<2>(ch, cl, o - 2, x0 >= 2);
+        const PairV<2> b = ldp<2>(ch, cl, o + 2, x0 + 2 < nx);
+        eh[0] = a.h[0]; eh[1] = a.h[1]; eh[4] = b.h[0]; eh[5] = b.h[1];
+        el[0] = a.l[0]; el[1] = a.l[1]; el[4] = b.l[0]; el[5] = b.l[1];
+      } else {
+        const PairV<1> a = ldp<1>(ch, cl, o - 1, x0 >= 1);
+        const PairV<1> b = ldp<1>(ch, cl, o + 1, x0 + 1 < nx);
+        eh[1] = a.h[0]; eh[3] = b.h[0];
+        el[1] = a.l[0]; el[3] = b.l[0];
+        if (R == 2) {
+          const PairV<1> a2 = ldp<1>(ch, cl, o - 2, x0 >= 2);
+          const PairV<1> b2 = ldp<1>(ch, cl, o + 2, x0 + 2 < nx);
+          eh[0] = a2.h[0]; eh[4] = b2.h[0];
+          el[0] = a2.l[0]; el[4] = b2.l[0];
+        }
+      }
+      const PairV<VW> d = ldp<VW>(dh, dl, o + rowoff, true);
+      F2 s1[VW], s2[VW];
+      {
+        const PairV<VW> a = ldp<VW>(ch, cl, o - nx, ym1);
+        const PairV<VW> b = ldp<VW>(ch, cl, o + nx, yp1);
+#pragma unroll
+        for (int k = 0; k < VW; ++k) {
+          s1[k] = F2{a.h[k], a.l[k]};
+          acc_add(s1[k], b.h[k], b.l[k]);
+          acc_add(s1[k], q[R - 1].h[k], q[R - 1].l[k]);
+          acc_add(s1[k], q[R + 1].h[k], q[R + 1].l[k]);
+          acc_add(s1[k], eh[k + 1], el[k + 1]);
+          acc_add(s1[k], eh[k + 3], el[k + 3]);
+        }
+      }
+      if (R == 2) {
+        const PairV<VW> a = ldp<VW>(ch, cl, o - 2 * nx, ym2);
+        const PairV<VW> b = ldp<VW>(ch, cl, o + 2 * nx, yp2);
+#pragma unroll
+        for (int k = 0; k < VW; ++k) {
+          s2[k] = F2{a.h[k], a.l[k]};
+          acc_add(s2[k], b.h[k], b.l[k]);
+          acc_add(s2[k], q[0].h[k], q[0].l[k]);
+          acc_add(s2[k], q[2 * R].h[k], q[2 * R].l[k]);
+          acc_add(s2[k], eh[k], el[k]);
+          acc_add(s2[k], eh[k + 4], el[k + 4]);
+        }
+      }
+      float oh[VW], ol[VW];
+#pragma unroll
+      for (int k = 0; k < VW; ++k) {
+        const F2 c = {q[R].h[k], q[R].l[k]};
+        const F2 a = prod_df(F2{d.h[k], d.l[k]}, c);
+        const F2 b = prod_df(c1, s1[k]);
+        F2 t = two_sum(a.h, b.h);
+        t.l += a.l + b.l;
+        if (R == 2) {
+          const F2 e = prod_df(c2, s2[k]);
+          const F2 u = two_sum(t.h, e.h);
+          t.h = u.h;
+          t.l += u.l + e.l;
+        }
+        t = quick_two_sum(t.h, t.l);
+        oh[k] = t.h;
+        ol[k] = t.l;
+        const F2 w = prod_df(c, t);
+        const F2 u = two_sum(dacc.h, w.h);
+        dacc.h = u.h;
+        dacc.l += u.l + w.l;
+      }
+      const int64_t x = (int64_t)col * ld + rowoff + o;
+      if constexpr (VW == 2) {
+        *reinterpret_cast<float2*>(Xh + x) = make_float2(oh[0], oh[1]);
+        *reinterpret_cast<float2*>(Xl + x) = make_float2(ol[0], ol[1]);
+      } else {
+        Xh[x] = oh[0];
+        Xl[x] = ol[0];
+      }
+      dacc = quick_two_sum(dacc.h, dacc.l);
     }
-    F2 r = df_mul(d, F2{__ldg(ph), __ldg(pl)});
-    r = df_add(r, df_mul(c1, s1.get()));
-    if (R == 2) r = df_add(r, df_mul(c2, s2.get()));
-    Xh[base] = r.h;
-    Xl[base] = r.l;
+#pragma unroll
+    for (int k = 0; k < 2 * R + 1; ++k) q[k] = q[k + 1];
+  }
+  {
+    F2 w = dacc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      w = df_add(w, F2{__shfl_xor_sync(0xffffffffu, w.h, o),
+                       __shfl_xor_sync(0xffffffffu, w.l, o)});
+    if ((threadIdx.x & 31) == 0)
+      red[threadIdx.x >> 5] = to_f64(w.h) + to_f64(w.l);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int k = 0; k < (int)(blockDim.x + 31) / 32; ++k) t += red[k];
+      dots[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * ncols + col] = t;
+    }
   }
 }
 
-// The same four grid points at a time (nx % 4 == 0): one thread owns points
-// x0..x0+3 of a row, loads the centre, the neighbouring quads along x and the
-// y/z neighbours as 16-byte (hi, lo) vectors, and takes the x neighbours
-// from registers, which cuts loads and boundary logic per point fourfold.
-//
-// With DOTS the column dots H_D = c_j . (H c)_j of Fig. EGFIG step (2) are
-// formed from the pairs in registers (the arithmetic of k_coldot_df per
-// thread, double-float warp sums, one FP64 add per warp), so the MP2 step
-// does not read C and X again: CTA b writes dots[b * ncols + column].
-template <int R, bool DOTS>
+// X = H C for a CSR operator (values split into hi + lo at creation), one row
+// per thread and kCols columns together: an entry's index and value are read
+// once for them, the products are added as in k_stencil_df (hi parts by TwoSum,
+// the rest plainly), and the column dots c_j . (H c)_j: CTA b writes
+// dots[b ncols + column]. One column at a time with normalised sums it took 44
+// instructions an entry (420 us at N = 48^3, 13 entries a row, 128 columns) and
+// the dots 43 us in a kernel of their own.
 __global__ void __launch_bounds__(256)
-    k_stencil_df_v4(StencilOp st, int64_t N, const float* __restrict__ dh,
-                    const float* __restrict__ dl, const float* __restrict__ Ch,
-                    const float* __restrict__ Cl, float* __restrict__ Xh,
-                    float* __restrict__ Xl, int ncols,
-                    double* __restrict__ dots) {
-  const int64_t v0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = v0 < (N >> 2);
-  if (!DOTS && !valid) return;  // with DOTS every thread joins the sums
-  const int64_t v = valid ? v0 : 0;
+    k_csr_df(int64_t N, int64_t ld, const int32_t* __restrict__ rowptr,
+             const int32_t* __restrict__ cols, const float* __restrict__ vh,
+             const float* __restrict__ vl, const float* __restrict__ Ch,
+             const float* __restrict__ Cl, float* __restrict__ Xh,
+             float* __restrict__ Xl, int ncols, double* __restrict__ dots) {
   __shared__ double red[kCols][8];
-  F2 dacc[kCols];
-#pragma unroll
-  for (int q = 0; q < kCols; ++q) dacc[q] = F2{0.f, 0.f};
-  const int nxv = st.nx >> 2;
-  const int xv = (int)(v % nxv);
-  const int64_t yz = v / nxv;
-  const int y = (int)(yz % st.ny);
-  const int z = (int)(yz / st.ny);
-  const int64_t i0 = v << 2;
-  const int64_t sy = st.nx, sz = (int64_t)st.nx * st.ny;
-  const bool xl = xv > 0, xr = xv + 1 < nxv;
-  const bool ym1 = y >= 1, yp1 = y + 1 < st.ny, zm1 = z >= 1,
-             zp1 = z + 1 < st.nz;
-  const bool ym2 = y >= 2, yp2 = y + 2 < st.ny, zm2 = z >= 2,
-             zp2 = z + 2 < st.nz;
-  const float4 d4h = *reinterpret_cast<const float4*>(dh + i0);
-  const float4 d4l = *reinterpret_cast<const float4*>(dl + i0);
-  const float dH[4] = {d4h.x, d4h.y, d4h.z, d4h.w};
-  const float dL[4] = {d4l.x, d4l.y, d4l.z, d4l.w};
-  const F2 c1 = {st.c1h, st.c1l}, c2 = {st.c2h, st.c2l};
-  auto ld = [](const float* p) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
-    return t;
-  };
-  auto add4 = [](Acc (&a)[4], const float4& h, const float4& l) {
-    a[0].add(h.x, l.x);
-    a[1].add(h.y, l.y);
-    a[2].add(h.z, l.z);
-    a[3].add(h.w, l.w);
-  };
-  const int cb = blockIdx.y * kCols;
+  const int64_t r0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool valid = r0 < N;
+  const int64_t r = valid ? r0 : 0;
+  const int b = valid ? rowptr[r] : 0, e = valid ? rowptr[r + 1] : 0;
+  const int cb = blockIdx.y * kCols, nc = min(kCols, ncols - cb);
+  // (columns past the last read the last one's entries and are not written)
+  const float* ph[kCols];
+  const float* pl[kCols];
+  F2 acc[kCols];
 #pragma unroll
   for (int q = 0; q < kCols; ++q) {
-    const int c = cb + q;
-    if (c >= ncols || !valid) break;
-    const int64_t base = (int64_t)c * N + i0;
-    const float* ph = Ch + base;
-    const float* pl = Cl + base;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 ch = ld(ph), cl = ld(pl);
-    const float4 lh = xl ? ld(ph - 4) : zero, ll = xl ? ld(pl - 4) : zero;
-    const float4 rh = xr ? ld(ph + 4) : zero, rl = xr ? ld(pl + 4) : zero;
-    Acc s1[4], s2[4];
-    if (ym1) add4(s1, ld(ph - sy), ld(pl - sy));
-    if (yp1) add4(s1, ld(ph + sy), ld(pl + sy));
-    if (zm1) add4(s1, ld(ph - sz), ld(pl - sz));
-    if (zp1) add4(s1, ld(ph + sz), ld(pl + sz));
-    // x neighbours at distance 1: (l.w, c.x, c.y, c.z) and (c.y, c.z, c.w, r.x)
-    s1[0].add(lh.w, ll.w); s1[0].add(ch.y, cl.y);
-    s1[1].add(ch.x, cl.x); s1[1].add(ch.z, cl.z);
-    s1[2].add(ch.y, cl.y); s1[2].add(ch.w, cl.w);
-    s1[3].add(ch.z, cl.z); s1[3].add(rh.x, rl.x);
-    if (R == 2) {
-      if (ym2) add4(s2, ld(ph - 2 * sy), ld(pl - 2 * sy));
-      if (yp2) add4(s2, ld(ph + 2 * sy), ld(pl + 2 * sy));
-      if (zm2) add4(s2, ld(ph - 2 * sz), ld(pl - 2 * sz));
-      if (zp2) add4(s2, ld(ph + 2 * sz), ld(pl + 2 * sz));
-      // distance 2: (l.z, l.w, c.x, c.y) and (c.z, c.w, r.x, r.y)
-      s2[0].add(lh.z, ll.z); s2[0].add(ch.z, cl.z);
-      s2[1].add(lh.w, ll.w); s2[1].add(ch.w, cl.w);
-      s2[2].add(ch.x, cl.x); s2[2].add(rh.x, rl.x);
-      s2[3].add(ch.y, cl.y); s2[3].add(rh.y, rl.y);
-    }
-    const float cH[4] = {ch.x, ch.y, ch.z, ch.w};
-    const float cL[4] = {cl.x, cl.y, cl.z, cl.w};
-    float oh[4], ol[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      F2 r = df_mul(F2{dH[k], dL[k]}, F2{cH[k], cL[k]});
-      r = df_add(r, df_mul(c1, s1[k].get()));
-      if (R == 2) r = df_add(r, df_mul(c2, s2[k].get()));
-      oh[k] = r.h;
-      ol[k] = r.l;
-    }
-    *reinterpret_cast<float4*>(Xh + base) = make_float4(oh[0], oh[1], oh[2], oh[3]);
-    *reinterpret_cast<float4*>(Xl + base) = make_float4(ol[0], ol[1], ol[2], ol[3]);
-    if (DOTS) {
-      F2 a = dacc[q];
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        a = df_add(a, df_mul(F2{cH[k], cL[k]}, F2{oh[k], ol[k]}));
-      dacc[q] = a;
-    }
+    const int64_t o = (int64_t)(cb + min(q, nc - 1)) * ld;
+    ph[q] = Ch + o;
+    pl[q] = Cl + o;
+    acc[q] = F2{0.f, 0.f};
   }
-  if (DOTS) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 2
+  for (int k = b; k < e; ++k) {
+    const int j = cols[k];
+    const F2 v = {vh[k], vl[k]};
 #pragma unroll
     for (int q = 0; q < kCols; ++q) {
-      F2 w = dacc[q];
+      const F2 t = prod_df(v, F2{__ldg(ph[q] + j), __ldg(pl[q] + j)});
+      acc_add(acc[q], t.h, t.l);
+    }
+  }
+  F2 d[kCols];
+#pragma unroll
+  for (int q = 0; q < kCols; ++q) {
+    d[q] = F2{0.f, 0.f};
+    if (valid && q < nc) {
+      const F2 t = quick_two_sum(acc[q].h, acc[q].l);
+      const int64_t o = (int64_t)(cb + q) * ld + r;
+      Xh[o] = t.h;
+      Xl[o] = t.l;
+      d[q] = df_mul(F2{ph[q][r], pl[q][r]}, t);
+    }
+  }
+  {
+#pragma unroll
+    for (int q = 0; q < kCols; ++q) {
+      F2 w = d[q];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1)
         w = df_add(w, F2{__shfl_xor_sync(0xffffffffu, w.h, o),
                          __shfl_xor_sync(0xffffffffu, w.l, o)});
-      if (lane == 0) red[q][warp] = to_f64(w.h) + to_f64(w.l);
+      if ((threadIdx.x & 31) == 0)
+        red[q][threadIdx.x >> 5] = to_f64(w.h) + to_f64(w.l);
     }
     __syncthreads();
-    if (threadIdx.x < kCols && cb + (int)threadIdx.x < ncols) {
+    if ((int)threadIdx.x < nc) {
       double t = red[threadIdx.x][0];
 #pragma unroll
       for (int w = 1; w < 8; ++w) t += red[threadIdx.x][w];
       dots[(size_t)blockIdx.x * ncols + cb + threadIdx.x] = t;
     }
   }
-}
-
-// X = H C for a CSR operator (values split into hi + lo at creation).
-__global__ void __launch_bounds__(256)
-    k_csr_df(int64_t N, int64_t ld, const int32_t* __restrict__ rowptr,
-             const int32_t* __restrict__ cols, const float* __restrict__ vh,
-             const float* __restrict__ vl, const float* __restrict__ Ch,
-             const float* __restrict__ Cl, float* __restrict__ Xh,
-             float* __restrict__ Xl, int ncols) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= N) return;
-  const int b = rowptr[r], e = rowptr[r + 1];
-  const int cb = blockIdx.y * kCols;
-  for (int q = 0; q < kCols; ++q) {
-    const int c = cb + q;
-    if (c >= ncols) break;
-    const int64_t off = (int64_t)c * ld;
-    F2 acc = {0.f, 0.f};
-    for (int k = b; k < e; ++k) {
-      const int64_t j = off + cols[k];
-      acc = df_add(acc, df_mul(F2{vh[k], vl[k]}, F2{__ldg(Ch + j), __ldg(Cl + j)}));
-    }
-    Xh[off + r] = acc.h;
-    Xl[off + r] = acc.l;
-  }
-}
-
-constexpr int kRowChunk = 4096;  // rows per partial of the column dots
-
-// dots[chunk * m + j] = sum_{i in chunk} C_ij X_ij (16-byte vectors when
-// N % 4 == 0 and the blocks are 16-byte aligned)
-__global__ void __launch_bounds__(256)
-    k_coldot_df(int64_t N, int m, const float* __restrict__ Ch,
-                const float* __restrict__ Cl, const float* __restrict__ Xh,
-                const float* __restrict__ Xl, double* __restrict__ dots,
-                int vec) {
-  __shared__ double red[32];
-  const int j = blockIdx.y;
-  const int64_t rb = (int64_t)blockIdx.x * kRowChunk;
-  const int64_t re = min(N, rb + kRowChunk);
-  const int64_t off = (int64_t)j * N;
-  F2 acc = {0.f, 0.f};
-  if (vec) {
-    const float4* ch = reinterpret_cast<const float4*>(Ch + off);
-    const float4* cl = reinterpret_cast<const float4*>(Cl + off);
-    const float4* xh = reinterpret_cast<const float4*>(Xh + off);
-    const float4* xl = reinterpret_cast<const float4*>(Xl + off);
-    for (int64_t i = (rb >> 2) + threadIdx.x; i < (re >> 2); i += blockDim.x) {
-      const float4 a = ch[i], b = cl[i], c = xh[i], d = xl[i];
-      acc = df_add(acc, df_mul(F2{a.x, b.x}, F2{c.x, d.x}));
-      acc = df_add(acc, df_mul(F2{a.y, b.y}, F2{c.y, d.y}));
-      acc = df_add(acc, df_mul(F2{a.z, b.z}, F2{c.z, d.z}));
-      acc = df_add(acc, df_mul(F2{a.w, b.w}, F2{c.w, d.w}));
-    }
-  } else {
-    for (int64_t i = rb + threadIdx.x; i < re; i += blockDim.x)
-      acc = df_add(acc, df_mul(F2{Ch[off + i], Cl[off + i]},
-                               F2{Xh[off + i], Xl[off + i]}));
-  }
-  double v[1] = {to_double(acc)};
-  block_sum<1>(v, red);
-  if (threadIdx.x == 0) dots[(size_t)blockIdx.x * m + j] = v[0];
 }
 
 // X32 = fl32(X - C diag(H_D))
@@ -391,74 +398,59 @@ void join_df(const float* hi, const float* lo, double* x, int64_t n,
   TRM_CHECK_LAUNCH();
 }
 
-void apply_h_df(const Operator& op, const float* Ch, const float* Cl,
-                float* Xh, float* Xl, int ncols, cudaStream_t s) {
-  if (ncols <= 0) return;
+namespace {
+
+template <int R, int VW>
+int launch_df(const Operator& op, const float* Ch, const float* Cl, float* Xh,
+              float* Xl, int ncols, double* dots, cudaStream_t s) {
+  const StencilOp st = zm_axes(op.st);
+  const ZmShape z =
+      zm_shape(st, op.N, ncols, VW, (int)apply_h_dots_doubles(op, 1));
+  k_stencil_df<R, VW><<<dim3(z.tiles, z.chunks, ncols), z.threads, 0, s>>>(
+      st, op.ld, op.diag32, op.diaglo, Ch, Cl, Xh, Xl, ncols, z.zc, dots);
+  TRM_CHECK_LAUNCH();
+  return z.tiles * z.chunks;  // partial dots per column
+}
+
+int stencil_df(const Operator& op, const float* Ch, const float* Cl, float* Xh,
+               float* Xl, int ncols, double* dots, cudaStream_t s) {
+  if (ncols > 65535) throw Error(-1, "too many columns for one launch");
+  const uintptr_t a = reinterpret_cast<uintptr_t>(Ch) |
+                      reinterpret_cast<uintptr_t>(Cl) |
+                      reinterpret_cast<uintptr_t>(Xh) |
+                      reinterpret_cast<uintptr_t>(Xl) |
+                      reinterpret_cast<uintptr_t>(op.diag32) |
+                      reinterpret_cast<uintptr_t>(op.diaglo);
+  // (short rows of a one-plane grid: one point a thread fills the warps better)
+  const bool two = (op.st.nx | op.ld) % 2 == 0 && a % 8 == 0 &&
+                   !(op.st.nz == 1 && op.st.nx < 64);
+  if (op.st.radius == 1)
+    return two ? launch_df<1, 2>(op, Ch, Cl, Xh, Xl, ncols, dots, s)
+               : launch_df<1, 1>(op, Ch, Cl, Xh, Xl, ncols, dots, s);
+  return two ? launch_df<2, 2>(op, Ch, Cl, Xh, Xl, ncols, dots, s)
+             : launch_df<2, 1>(op, Ch, Cl, Xh, Xl, ncols, dots, s);
+}
+
+int csr_df(const Operator& op, const float* Ch, const float* Cl, float* Xh,
+           float* Xl, int ncols, double* dots, cudaStream_t s) {
   const int gy = ceil_div(ncols, kCols);
   if (gy > 65535) throw Error(-1, "too many columns for one launch");
-  dim3 grid(ceil_div(op.N, 256), gy);
-  const bool v4 = op.kind == 0 && op.st.nx % 4 == 0 && op.N % 4 == 0 &&
-                  ((reinterpret_cast<uintptr_t>(Ch) | reinterpret_cast<uintptr_t>(Cl) |
-                    reinterpret_cast<uintptr_t>(Xh) | reinterpret_cast<uintptr_t>(Xl) |
-                    reinterpret_cast<uintptr_t>(op.diag32) |
-                    reinterpret_cast<uintptr_t>(op.diaglo)) & 15) == 0;
-  if (v4) {
-    dim3 g4(ceil_div(op.N / 4, 256), gy);
-    if (op.st.radius == 1)
-      k_stencil_df_v4<1, false><<<g4, 256, 0, s>>>(
-          op.st, op.N, op.diag32, op.diaglo, Ch, Cl, Xh, Xl, ncols, nullptr);
-    else
-      k_stencil_df_v4<2, false><<<g4, 256, 0, s>>>(
-          op.st, op.N, op.diag32, op.diaglo, Ch, Cl, Xh, Xl, ncols, nullptr);
-  } else if (op.kind == 0) {
-    if (op.st.radius == 1)
-      k_stencil_df<1><<<grid, 256, 0, s>>>(op.st, op.N, op.ld, op.diag32, op.diaglo,
-                                           Ch, Cl, Xh, Xl, ncols);
-    else
-      k_stencil_df<2><<<grid, 256, 0, s>>>(op.st, op.N, op.ld, op.diag32, op.diaglo,
-                                           Ch, Cl, Xh, Xl, ncols);
-  } else {
-    k_csr_df<<<grid, 256, 0, s>>>(op.N, op.ld, op.csr.rowptr, op.csr.cols,
-                                  op.csr.valshi, op.csr.valslo, Ch, Cl, Xh,
-                                  Xl, ncols);
-  }
+  const dim3 grid(ceil_div(op.N, 256), gy);
+  k_csr_df<<<grid, 256, 0, s>>>(op.N, op.ld, op.csr.rowptr, op.csr.cols,
+                                      op.csr.valshi, op.csr.valslo, Ch, Cl, Xh,
+                                      Xl, ncols, dots);
   TRM_CHECK_LAUNCH();
+  return (int)grid.x;
 }
+
+}  // namespace
 
 int apply_h_df_dots(const Operator& op, const float* Ch, const float* Cl,
                     float* Xh, float* Xl, int ncols, double* dots,
                     cudaStream_t s) {
   if (ncols <= 0) return 0;
-  const bool v4 = op.kind == 0 && op.st.nx % 4 == 0 && op.N % 4 == 0 &&
-                  ((reinterpret_cast<uintptr_t>(Ch) | reinterpret_cast<uintptr_t>(Cl) |
-                    reinterpret_cast<uintptr_t>(Xh) | reinterpret_cast<uintptr_t>(Xl) |
-                    reinterpret_cast<uintptr_t>(op.diag32) |
-                    reinterpret_cast<uintptr_t>(op.diaglo)) & 15) == 0;
-  const int gy = ceil_div(ncols, kCols);
-  if (!v4 || gy > 65535) return 0;  // the caller forms the dots separately
-  dim3 g4(ceil_div(op.N / 4, 256), gy);
-  if (op.st.radius == 1)
-    k_stencil_df_v4<1, true><<<g4, 256, 0, s>>>(
-        op.st, op.N, op.diag32, op.diaglo, Ch, Cl, Xh, Xl, ncols, dots);
-  else
-    k_stencil_df_v4<2, true><<<g4, 256, 0, s>>>(
-        op.st, op.N, op.diag32, op.diaglo, Ch, Cl, Xh, Xl, ncols, dots);
-  TRM_CHECK_LAUNCH();
-  return (int)g4.x;  // partial dots per column
-}
-
-void energy_diag_df(int64_t N, int m, const float* Ch, const float* Cl,
-                    const float* Xh, const float* Xl, double* HD,
-                    IterScalars* sc, double* partials, cudaStream_t s) {
-  const int chunks = ceil_div(N, kRowChunk);
-  const int vec = N % 4 == 0 &&
-                  ((reinterpret_cast<uintptr_t>(Ch) | reinterpret_cast<uintptr_t>(Cl) |
-                    reinterpret_cast<uintptr_t>(Xh) | reinterpret_cast<uintptr_t>(Xl)) &
-                   15) == 0;
-  k_coldot_df<<<dim3(chunks, m), 256, 0, s>>>(N, m, Ch, Cl, Xh, Xl, partials,
-                                               vec);
-  TRM_CHECK_LAUNCH();
-  energy_from_dots(partials, chunks, m, HD, sc, s);
+  return op.kind == 0 ? stencil_df(op, Ch, Cl, Xh, Xl, ncols, dots, s)
+                      : csr_df(op, Ch, Cl, Xh, Xl, ncols, dots, s);
 }
 
 void xprime_df(int64_t N, int m, const float* Ch, const float* Cl,

@@ -52,6 +52,16 @@ void apply_h(const Operator& op, const double* X, double* Y, int ncols,
 int apply_h_dots(const Operator& op, const float* X, float* Y, int ncols,
                  double* dots, cudaStream_t s);
 size_t apply_h_dots_doubles(const Operator& op, int ncols);
+// Geometry of the register z-march stencils: CTAs of `threads` threads over
+// `tiles` parts of a plane (vw points per thread), `chunks` runs of zc planes
+// and the columns; tiles * chunks partial dots per column, at most max_dots
+// where one run of all planes allows.
+struct ZmShape {
+  int tiles, threads, chunks, zc;
+};
+ZmShape zm_shape(const StencilOp& st, int64_t N, int ncols, int vw, int max_dots);
+// the axes as the march takes them (a 2-D grid's y in z's place)
+StencilOp zm_axes(const StencilOp& st);
 
 // ---------------------------------------------------------------------------
 // Double-float (FP32 pair, ~48-bit) arithmetic for the FP64-accuracy steps
@@ -62,19 +72,12 @@ void split_df(const double* x, float* hi, float* lo, int64_t n,
 void join_df(const float* hi, const float* lo, double* x, int64_t n,
              cudaStream_t s);
 // X = H C in double-float (needs Operator::diaglo, and valshi/valslo for CSR)
-void apply_h_df(const Operator& op, const float* Ch, const float* Cl,
-                float* Xh, float* Xl, int ncols, cudaStream_t s);
-// The same with the column dots sum_i C_ij X_ij of each CTA in
-// dots[chunk * ncols + j] (apply_h_dots_doubles entries; energy_from_dots
-// adds them up); returns the number of chunks, or 0 when this operator or
-// these buffers take the unfused kernels (then nothing is launched).
+// with the column dots sum_i C_ij X_ij of each CTA in dots[chunk * ncols + j]
+// (apply_h_dots_doubles entries; energy_from_dots adds them up); returns the
+// number of chunks.
 int apply_h_df_dots(const Operator& op, const float* Ch, const float* Cl,
                     float* Xh, float* Xl, int ncols, double* dots,
                     cudaStream_t s);
-// H_D[j] = sum_i C_ij X_ij, E = sum_j H_D[j] into sc->E
-void energy_diag_df(int64_t N, int m, const float* Ch, const float* Cl,
-                    const float* Xh, const float* Xl, double* HD,
-                    IterScalars* sc, double* partials, cudaStream_t s);
 // X32 = fl32(X - C diag(H_D))
 void xprime_df(int64_t N, int m, const float* Ch, const float* Cl,
                const float* Xh, const float* Xl, const double* HD, float* X32,

@@ -5,8 +5,8 @@
 // x points of one (y, z) row and walks a few columns, so the grid-index work
 // and the diagonal are shared across columns and every access is a 16-byte
 // vector load (x neighbours come from the vectors left and right of it).
-// CSR operators: one thread per row keeps the row's entries in registers and
-// walks the columns of its column group.
+// CSR operators: one thread per row takes the columns of its column group
+// together.
 #include <algorithm>
 #include <atomic>
 #include <cstdlib>
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1)
   }
 }
 
-// One point per thread, any nx.
+// One point per thread, any nx (FP64).
 template <typename T, int R, bool DOTS>
 __global__ void __launch_bounds__(256)
     k_stencil_1(StencilOp st, int64_t N, int64_t ld, const double* __restrict__ d64,
@@ -224,7 +224,13 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-constexpr int kCsrCache = 16;
+// CSR: one row per thread, KC columns at a time, so an entry's column index and
+// value are read once for KC products and KC gathers are in flight together
+// (one column at a time, the row cached in registers: 236 us in FP32 at
+// N = 48^3, 13 entries a row, 128 columns). A row's products are added in the
+// order of its entries.
+template <typename T>
+__host__ __device__ constexpr int csr_cols() { return sizeof(T) == 4 ? 8 : 4; }
 
 template <typename T, typename TV, bool DOTS>
 __global__ void __launch_bounds__(256)
@@ -232,53 +238,51 @@ __global__ void __launch_bounds__(256)
           const int32_t* __restrict__ cols, const TV* __restrict__ vals,
           const T* __restrict__ X, T* __restrict__ Y, int ncols,
           double* __restrict__ dots) {
+  constexpr int KC = csr_cols<T>();
   const int64_t r0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = r0 < N;
   if (!DOTS && !valid) return;
   const int64_t r = valid ? r0 : 0;
-  __shared__ double red[kCpb][8];
+  __shared__ double red[KC][8];
   const int b = valid ? rowptr[r] : 0, e = valid ? rowptr[r + 1] : 0;
-  const int nnz = e - b;
-  const int cb = blockIdx.y * kCpb;
-  if (nnz <= kCsrCache) {
-    int ci[kCsrCache];
-    T cv[kCsrCache];
+  const int cb = blockIdx.y * KC, nc = min(KC, ncols - cb);
+  // (columns past the last read the last one's entries and are not written)
+  const T* x[KC];
 #pragma unroll
-    for (int k = 0; k < kCsrCache; ++k) {
-      ci[k] = k < nnz ? cols[b + k] : 0;
-      cv[k] = k < nnz ? (T)vals[b + k] : (T)0;
-    }
-    for (int q = 0; q < kCpb; ++q) {
-      const int c = cb + q;
-      if (c >= ncols) break;
-      T d = 0;
-      if (valid) {
-        const T* x = X + (int64_t)c * ld;
-        T acc = 0;
+  for (int q = 0; q < KC; ++q) x[q] = X + (int64_t)(cb + min(q, nc - 1)) * ld;
+  T acc[KC];
 #pragma unroll
-        for (int k = 0; k < kCsrCache; ++k)
-          if (k < nnz) acc += cv[k] * __ldg(x + ci[k]);
-        if (!DOTS || Y) Y[(int64_t)c * ld + r] = acc;
-        d = x[r] * acc;
-      }
-      if (DOTS) warp_dot(d, red, q);
-    }
-  } else {
-    for (int q = 0; q < kCpb; ++q) {
-      const int c = cb + q;
-      if (c >= ncols) break;
-      T d = 0;
-      if (valid) {
-        const T* x = X + (int64_t)c * ld;
-        T acc = 0;
-        for (int k = b; k < e; ++k) acc += (T)vals[k] * __ldg(x + cols[k]);
-        if (!DOTS || Y) Y[(int64_t)c * ld + r] = acc;
-        d = x[r] * acc;
-      }
-      if (DOTS) warp_dot(d, red, q);
+  for (int q = 0; q < KC; ++q) acc[q] = (T)0;
+#pragma unroll 2
+  for (int k = b; k < e; ++k) {
+    const int j = cols[k];
+    const T v = (T)vals[k];
+#pragma unroll
+    for (int q = 0; q < KC; ++q) acc[q] += v * __ldg(x[q] + j);
+  }
+  T d[KC];
+#pragma unroll
+  for (int q = 0; q < KC; ++q) {
+    d[q] = (T)0;
+    if (valid && q < nc) {
+      if (!DOTS || Y) Y[(int64_t)(cb + q) * ld + r] = acc[q];
+      if (DOTS) d[q] = x[q][r] * acc[q];
     }
   }
-  if (DOTS) write_dots(red, dots, cb, ncols);
+  if (DOTS) {
+#pragma unroll
+    for (int q = 0; q < KC; ++q) {
+      const T t = warp_sum(d[q]);
+      if ((threadIdx.x & 31) == 0) red[q][threadIdx.x >> 5] = to_f64(t);
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < nc) {
+      double t = red[threadIdx.x][0];
+#pragma unroll
+      for (int w = 1; w < 8; ++w) t += red[threadIdx.x][w];
+      dots[(size_t)blockIdx.x * ncols + cb + threadIdx.x] = t;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -510,114 +514,137 @@ int launch_vec(const Operator& op, const T* X, T* Y, int ncols, double* dots,
                cudaStream_t s);
 
 // ---------------------------------------------------------------------------
-// Register z-march (FP32, nx % 4 == 0): a CTA owns a tile of quads (four
-// consecutive x points of one row) of an x-y plane, one column and a chunk
-// of z planes; each thread walks z over its quad keeping the 2R + 1 values
-// of the quad along z in registers, so per plane it reads one new plane
-// value from DRAM and its x and y neighbours, which the neighbouring
-// threads of the same tile have just read as their own quads (L1 hits),
-// instead of four more planes through L2. There is no barrier inside the
-// march, so every warp keeps its loads in flight on its own. Every point
-// gets the same operations in the same order as k_stencil_v4; with DOTS the
-// column dot is accumulated in double-float per thread and the CTA's sum
-// goes to dots[(blockIdx.y * gridDim.x + blockIdx.x) * ncols + column].
+// Register z-march (FP32): a CTA owns a tile of an x-y plane, one column and a
+// chunk of z planes; a thread owns VW consecutive x points of one row (4, 2 or
+// 1, as nx is a multiple of them) and walks z keeping their 2R + 1 values along
+// z in registers, so per plane it reads one new value of each from DRAM and its
+// x and y neighbours, which the neighbouring threads of the same tile have just
+// read as their own (L1 hits), instead of four more planes through L2. There is
+// no barrier inside the march, so every warp keeps its loads in flight on its
+// own. Every point gets the same operations in the same order as in
+// k_stencil_v4; with DOTS the column dot is accumulated in double-float per
+// thread and the CTA's sum goes to
+// dots[(blockIdx.y * gridDim.x + blockIdx.x) * ncols + column].
+// Odd grids (VW = 1) took a kernel that read all twelve neighbours through L1
+// and L2 for each point: 34 us at 39 x 41 x 37, 90 columns.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float4 ldg4f(const float* p) {
-  return __ldg(reinterpret_cast<const float4*>(p));
+template <int VW>
+__device__ __forceinline__ void ldv(const float* p, bool in, float (&v)[VW]) {
+  if constexpr (VW == 4) {
+    const float4 t = in ? __ldg(reinterpret_cast<const float4*>(p))
+                        : make_float4(0.f, 0.f, 0.f, 0.f);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  } else if constexpr (VW == 2) {
+    const float2 t = in ? __ldg(reinterpret_cast<const float2*>(p))
+                        : make_float2(0.f, 0.f);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+    v[0] = in ? __ldg(p) : 0.f;
+  }
+}
+template <int VW>
+__device__ __forceinline__ void stv(float* p, const float (&v)[VW]) {
+  if constexpr (VW == 4)
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  else if constexpr (VW == 2)
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  else
+    *p = v[0];
+}
+// Values x0 - 2 .. x0 + VW + 1 of a row, c holding x0 .. x0 + VW - 1 and x0 a
+// multiple of VW; zeros outside [0, nx).
+template <int R, int VW>
+__device__ __forceinline__ void row_ext(const float* p, const float (&c)[VW],
+                                        int x0, int nx, float (&e)[VW + 4]) {
+#pragma unroll
+  for (int k = 0; k < VW; ++k) e[k + 2] = c[k];
+  if constexpr (VW == 1) {
+    e[1] = x0 >= 1 ? __ldg(p - 1) : 0.f;
+    e[3] = x0 + 1 < nx ? __ldg(p + 1) : 0.f;
+    e[0] = R == 2 && x0 >= 2 ? __ldg(p - 2) : 0.f;
+    e[4] = R == 2 && x0 + 2 < nx ? __ldg(p + 2) : 0.f;
+  } else {
+    float a[VW], b[VW];
+    ldv<VW>(p - VW, x0 >= VW, a);
+    ldv<VW>(p + VW, x0 + VW < nx, b);
+    e[0] = a[VW - 2];
+    e[1] = a[VW - 1];
+    e[VW + 2] = b[0];
+    e[VW + 3] = b[1];
+  }
 }
 
-template <int R, bool DOTS>
-__global__ void __launch_bounds__(256, 4)
-    k_stencil_zm(StencilOp st, int64_t N, const float* __restrict__ d32,
+template <int R, bool DOTS, int VW>
+__global__ void __launch_bounds__(256, VW == 1 ? 6 : 4)
+    k_stencil_zm(StencilOp st, int64_t ld, const float* __restrict__ d32,
                  const float* __restrict__ X, float* __restrict__ Y,
                  int ncols, int zc, double* __restrict__ dots) {
   __shared__ double red[8];
-  const int nx = st.nx, ny = st.ny, nz = st.nz, nxq = nx >> 2;
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;  // quad in the plane
+  const int nx = st.nx, ny = st.ny, nz = st.nz, nxq = nx / VW;
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;  // group in the plane
   const bool active = p < nxq * ny;
-  const int qx = active ? p % nxq : 0, y = active ? p / nxq : 0;
+  const int x0 = active ? VW * (p % nxq) : 0, y = active ? p / nxq : 0;
   const int col = blockIdx.z;
   const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc);
   const int64_t sz = (int64_t)nx * ny;
-  const int64_t rowoff = (int64_t)y * nx + 4 * qx;
-  const float* xb = X + (int64_t)col * N + rowoff;
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  const bool xl_in = qx > 0, xr_in = qx + 1 < nxq;
+  const int64_t rowoff = (int64_t)y * nx + x0;
+  const float* xb = X + (int64_t)col * ld + rowoff;
   const bool ym1 = y >= 1, yp1 = y + 1 < ny, ym2 = y >= 2, yp2 = y + 2 < ny;
   const float c1 = st.c1h, c2 = st.c2h;  // rounded on the host
-  // q[k]: the quad in plane z - R + k (zeros outside the grid: Dirichlet);
+  // q[k]: the points in plane z - R + k (zeros outside the grid: Dirichlet);
   // q[2R + 1], plane z + R + 1, is loaded one step before it is needed so
   // that a plane's DRAM latency overlaps the arithmetic of the step before
-  float4 q[2 * R + 2];
+  float q[2 * R + 2][VW];
 #pragma unroll
   for (int k = 0; k < 2 * R + 1; ++k) {
     const int pz = z0 - R + k;
-    q[k] = (active && pz >= 0 && pz < nz) ? ldg4f(xb + pz * sz) : zero;
+    ldv<VW>(xb + pz * sz, active && pz >= 0 && pz < nz, q[k]);
   }
   F2 dacc = {0.f, 0.f};
   for (int z = z0; z < z1; ++z) {
-    q[2 * R + 1] =
-        (active && z + R + 1 < nz && z + 1 < z1) ? ldg4f(xb + (z + R + 1) * sz)
-                                                 : zero;
+    ldv<VW>(xb + (z + R + 1) * sz, active && z + R + 1 < nz && z + 1 < z1,
+            q[2 * R + 1]);
     if (active) {
       const float* pc = xb + z * sz;
-      const float4 xc = q[R];
-      const float4 xl = xl_in ? ldg4f(pc - 4) : zero;
-      const float4 xr = xr_in ? ldg4f(pc + 4) : zero;
-      const float4 a1v = ym1 ? ldg4f(pc - nx) : zero;
-      const float4 b1v = yp1 ? ldg4f(pc + nx) : zero;
-      const float4 e1v = q[R - 1], f1v = q[R + 1];
-      const float4 d4 = ldg4f(d32 + z * sz + rowoff);
-      const float c[4] = {xc.x, xc.y, xc.z, xc.w};
-      const float a1[4] = {a1v.x, a1v.y, a1v.z, a1v.w};
-      const float b1[4] = {b1v.x, b1v.y, b1v.z, b1v.w};
-      const float e1[4] = {e1v.x, e1v.y, e1v.z, e1v.w};
-      const float f1[4] = {f1v.x, f1v.y, f1v.z, f1v.w};
-      const float l1[4] = {xl.w, xc.x, xc.y, xc.z};
-      const float r1[4] = {xc.y, xc.z, xc.w, xr.x};
-      const float d[4] = {d4.x, d4.y, d4.z, d4.w};
-      float a2[4] = {0, 0, 0, 0}, b2[4] = {0, 0, 0, 0}, e2[4] = {0, 0, 0, 0},
-            f2[4] = {0, 0, 0, 0};
-      float l2[4] = {0, 0, 0, 0}, r2[4] = {0, 0, 0, 0};
+      float e[VW + 4], a1[VW], b1[VW], a2[VW], b2[VW], d[VW];
+      row_ext<R, VW>(pc, q[R], x0, nx, e);
+      ldv<VW>(pc - nx, ym1, a1);
+      ldv<VW>(pc + nx, yp1, b1);
+      ldv<VW>(d32 + z * sz + rowoff, true, d);
       if (R == 2) {
-        const float4 a2v = ym2 ? ldg4f(pc - 2 * nx) : zero;
-        const float4 b2v = yp2 ? ldg4f(pc + 2 * nx) : zero;
-        const float4 e2v = q[0], f2v = q[2 * R];
-        a2[0] = a2v.x; a2[1] = a2v.y; a2[2] = a2v.z; a2[3] = a2v.w;
-        b2[0] = b2v.x; b2[1] = b2v.y; b2[2] = b2v.z; b2[3] = b2v.w;
-        e2[0] = e2v.x; e2[1] = e2v.y; e2[2] = e2v.z; e2[3] = e2v.w;
-        f2[0] = f2v.x; f2[1] = f2v.y; f2[2] = f2v.z; f2[3] = f2v.w;
-        l2[0] = xl.z; l2[1] = xl.w; l2[2] = xc.x; l2[3] = xc.y;
-        r2[0] = xc.z; r2[1] = xc.w; r2[2] = xr.x; r2[3] = xr.y;
+        ldv<VW>(pc - 2 * nx, ym2, a2);
+        ldv<VW>(pc + 2 * nx, yp2, b2);
       }
-      float out[4];
+      float out[VW];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < VW; ++k) {
         float s1 = 0.f, s2 = 0.f;
         s1 += a1[k];
         s1 += b1[k];
-        s1 += e1[k];
-        s1 += f1[k];
-        float acc = d[k] * c[k] + c1 * (s1 + l1[k] + r1[k]);
+        s1 += q[R - 1][k];
+        s1 += q[R + 1][k];
+        float acc = d[k] * q[R][k] + c1 * (s1 + e[k + 1] + e[k + 3]);
         if (R == 2) {
           s2 += a2[k];
           s2 += b2[k];
-          s2 += e2[k];
-          s2 += f2[k];
-          acc += c2 * (s2 + l2[k] + r2[k]);
+          s2 += q[0][k];
+          s2 += q[2 * R][k];
+          acc += c2 * (s2 + e[k] + e[k + 4]);
         }
         out[k] = acc;
       }
-      if (!DOTS || Y)
-        *reinterpret_cast<float4*>(Y + (int64_t)col * N + z * sz + rowoff) =
-            make_float4(out[0], out[1], out[2], out[3]);
-      if (DOTS)
-        dacc = df_add(dacc, F2{c[0] * out[0] + c[1] * out[1] +
-                                   c[2] * out[2] + c[3] * out[3],
-                               0.f});
+      if (!DOTS || Y) stv<VW>(Y + (int64_t)col * ld + z * sz + rowoff, out);
+      if (DOTS) {
+        float t = q[R][0] * out[0];
+#pragma unroll
+        for (int k = 1; k < VW; ++k) t += q[R][k] * out[k];
+        dacc = df_add(dacc, F2{t, 0.f});
+      }
     }
 #pragma unroll
-    for (int k = 0; k < 2 * R + 1; ++k) q[k] = q[k + 1];
+    for (int k = 0; k < 2 * R + 1; ++k)
+#pragma unroll
+      for (int u = 0; u < VW; ++u) q[k][u] = q[k + 1][u];
   }
   if (DOTS) {
     F2 w = dacc;
@@ -636,58 +663,93 @@ __global__ void __launch_bounds__(256, 4)
   }
 }
 
-// Launch geometry of the z-march: plane tiles of at most 256 quads (a
-// multiple of 32 threads, evened out over the tiles), z chunks so that
-// about eight CTAs per SM are launched (at least four planes each), and no
-// more partial dots per column than apply_h_dots_doubles allows.
-struct ZmShape {
-  int tiles, threads, chunks, zc;
-};
-ZmShape zm_shape(const Operator& op, int ncols) {
-  const StencilOp& st = op.st;
-  const int nq = (st.nx / 4) * st.ny;
+}  // namespace
+
+// A grid of one plane is marched along y (its rows in the planes' place).
+// Launch geometry of the z-march: plane tiles of at most 256 threads (a
+// multiple of 32, evened out over the tiles), z chunks so that about 3072 threads
+// per SM are launched (at least four planes each; half as many leave a last
+// wave, twice as many read more halo planes: 115, 112, 112 us for the
+// double-float kernel at 48^3 x 128 with 2048, 3072 and 4096), and no more
+// partial dots per column than apply_h_dots_doubles allows.
+StencilOp zm_axes(const StencilOp& st) {
+  StencilOp t = st;
+  if (t.nz == 1) std::swap(t.ny, t.nz);
+  return t;
+}
+ZmShape zm_shape(const StencilOp& st, int64_t N, int ncols, int vw, int max_dots) {
+  const int nq = (st.nx / vw) * st.ny;
   ZmShape z{};
   z.tiles = ceil_div(nq, 256);
   z.threads = 32 * ceil_div(nq, 32 * z.tiles);
-  const int want = ceil_div(8 * sm_count(), z.tiles * ncols);
-  const int cap = (int)std::max<int64_t>(1, ceil_div(op.N / 4, (int64_t)256) /
-                                                 z.tiles);
+  const int want = ceil_div((int64_t)12 * 256 * sm_count(),
+                            (int64_t)z.threads * z.tiles * ncols);
+  const int cap = std::max(1, max_dots / z.tiles);
   const int chunks = std::max(1, std::min({want, ceil_div(st.nz, 4), cap}));
   z.zc = ceil_div(st.nz, chunks);
   z.chunks = ceil_div(st.nz, z.zc);
   return z;
 }
 
-template <int R, bool DOTS>
-int launch_zm(const Operator& op, const float* X, float* Y, int ncols,
-              double* dots, cudaStream_t s) {
-  const ZmShape z = zm_shape(op, ncols);
-  k_stencil_zm<R, DOTS><<<dim3(z.tiles, z.chunks, ncols), z.threads, 0, s>>>(
-      op.st, op.N, op.diag32, X, Y, ncols, z.zc, dots);
-  TRM_CHECK_LAUNCH();
+namespace {
+
+// x points per thread of the z-march for this grid and these buffers (16- and
+// 8-byte vectors need the row length and the columns' spacing to match).
+int zm_width(const Operator& op, const float* X, const float* Y) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(X) |
+                      reinterpret_cast<uintptr_t>(Y) |
+                      reinterpret_cast<uintptr_t>(op.diag32);
+  const int64_t n = op.st.nx | op.ld;
+  if (n % 4 == 0 && a % 16 == 0) return 4;
+  return n % 2 == 0 && a % 8 == 0 ? 2 : 1;
+}
+
+int max_dots_per_column(const Operator& op) {
+  return (int)(apply_h_dots_doubles(op, 1));
+}
+
+template <int R, bool DOTS, int VW>
+int launch_zm_v(const Operator& op, const float* X, float* Y, int ncols,
+                double* dots, cudaStream_t s) {
+  const StencilOp st = zm_axes(op.st);
+  const ZmShape z = zm_shape(st, op.N, std::min(ncols, 65535), VW,
+                             max_dots_per_column(op));
+  // (the columns are the grid's last dimension: batches of what it takes)
+  for (int c0 = 0; c0 < ncols; c0 += 65535) {
+    const int nc = std::min(65535, ncols - c0);
+    k_stencil_zm<R, DOTS, VW><<<dim3(z.tiles, z.chunks, nc), z.threads, 0, s>>>(
+        st, op.ld, op.diag32, X + c0 * op.ld, Y ? Y + c0 * op.ld : nullptr,
+        ncols, z.zc, DOTS ? dots + c0 : nullptr);
+    TRM_CHECK_LAUNCH();
+  }
   return z.tiles * z.chunks;  // partial dots per column
 }
 
 template <bool DOTS>
 int launch_zm_r(const Operator& op, const float* X, float* Y, int ncols,
                 double* dots, cudaStream_t s) {
-  return op.st.radius == 1 ? launch_zm<1, DOTS>(op, X, Y, ncols, dots, s)
-                           : launch_zm<2, DOTS>(op, X, Y, ncols, dots, s);
+  const int vw = zm_width(op, X, Y);
+  if (op.st.radius == 1)
+    return vw == 4   ? launch_zm_v<1, DOTS, 4>(op, X, Y, ncols, dots, s)
+           : vw == 2 ? launch_zm_v<1, DOTS, 2>(op, X, Y, ncols, dots, s)
+                     : launch_zm_v<1, DOTS, 1>(op, X, Y, ncols, dots, s);
+  return vw == 4   ? launch_zm_v<2, DOTS, 4>(op, X, Y, ncols, dots, s)
+         : vw == 2 ? launch_zm_v<2, DOTS, 2>(op, X, Y, ncols, dots, s)
+                   : launch_zm_v<2, DOTS, 1>(op, X, Y, ncols, dots, s);
 }
 
-// The z-march takes FP32 stencils with nx % 4 == 0 on 16-byte-aligned
-// blocks, at most 65535 columns, and partial dots within the buffer.
+// With nx % 4 == 0 the z-march is one of the autotuned kernels where its
+// partial dots fit; on other grids it is the FP32 stencil.
 template <typename T>
 bool zm_eligible(const Operator& op, const T* X, const T* Y, int ncols) {
   if constexpr (sizeof(T) != 4) {
     return false;
   } else {
     if (op.kind != 0 || op.st.nx % 4 != 0 || ncols > 65535) return false;
-    if (((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y) |
-          reinterpret_cast<uintptr_t>(op.diag32)) & 15) != 0)
-      return false;
-    const ZmShape z = zm_shape(op, ncols);
-    return (int64_t)z.tiles * z.chunks <= ceil_div(op.N / 4, (int64_t)256);
+    if (zm_width(op, X, Y) != 4) return false;
+    const ZmShape z =
+        zm_shape(zm_axes(op.st), op.N, ncols, 4, max_dots_per_column(op));
+    return z.tiles * z.chunks <= max_dots_per_column(op);
   }
 }
 
@@ -782,6 +844,8 @@ template <typename T, bool DOTS>
 int launch_apply(const Operator& op, const T* X, T* Y, int ncols, double* dots,
                  cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
+    if (op.kind == 0 && op.st.nx % 4 != 0)
+      return launch_zm_r<DOTS>(op, X, Y, ncols, dots, s);
     if (op.kind == 0 && op.st.nx % 4 == 0) {
       // TRM_STENCIL_KERNEL=vec|planes|zm overrides the tuned choice (for
       // tests and measurements; an ineligible kernel falls back to vec)
@@ -818,7 +882,7 @@ int launch_vec(const Operator& op, const T* X, T* Y, int ncols, double* dots,
       else
         k_stencil_v4<T, 2, DOTS><<<grid, threads, 0, s>>>(
             st, op.N, op.diag64, op.diag32, X, Y, ncols, dots);
-    } else {
+    } else if constexpr (sizeof(T) == 8) {
       grid = dim3(ceil_div(op.N, threads), gy);
       if (st.radius == 1)
         k_stencil_1<T, 1, DOTS><<<grid, threads, 0, s>>>(
@@ -828,7 +892,9 @@ int launch_vec(const Operator& op, const T* X, T* Y, int ncols, double* dots,
             st, op.N, op.ld, op.diag64, op.diag32, X, Y, ncols, dots);
     }
   } else {
-    grid = dim3(ceil_div(op.N, threads), gy);
+    const int gc = ceil_div(ncols, csr_cols<T>());
+    if (gc > 65535) throw Error(-1, "too many columns for one launch");
+    grid = dim3(ceil_div(op.N, threads), gc);
     // FP32 blocks take the FP32 roundings of the values when the operator
     // holds them (the same products, no conversion per nonzero)
     if (op.csr.vals64 && (sizeof(T) == 8 || !op.csr.vals32))
