@@ -128,10 +128,18 @@ constexpr uint32_t kIdesc = idesc_tf32(BM, BN, false, false);
 // them, or for a symmetric segment only those on or above its diagonal.
 constexpr int kMaxTiles = 256;  // 8 x 32: m = 1024, four m-column segments
 
+// Narrow blocks (at most 64 columns) would leave three quarters of a 128 x 128
+// tile empty. Their CTAs stack two operands in the tile's two halves instead and
+// use two or three of its four quadrants:
+//   kLine: A = [C P], B = [P G] gives C^T P, P^T P and P^T G in one tile;
+//   kRows: A and B at two row offsets, two row slices' partials in one tile.
+enum Stack { kWhole = 0, kLine = 1, kRows = 2 };
+
 struct TcArgs {
   int64_t N;
   int m, n;               // output is m x n
-  int64_t rows_per_split;
+  int stack;
+  int64_t rows_per_split;  // kRows: of each of the two slices
   int kc;                 // stages per accumulation chunk of long slices
   int seg_cols;           // columns per segment
   int tps;                // column tiles per segment (the last one ragged:
@@ -156,7 +164,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int split = blockIdx.x;
   const int i0 = args.ti[blockIdx.y] * BM;
-  const int64_t rb = (int64_t)split * args.rows_per_split;
+  const int stack = args.stack;
+  const int64_t rb =
+      (int64_t)split * args.rows_per_split * (stack == kRows ? 2 : 1);
   const int64_t re = min(args.N, rb + args.rows_per_split);
   const int nk = (int)((re - rb + BK - 1) / BK);
   const int seg = args.tj[blockIdx.y] / args.tps;
@@ -202,8 +212,16 @@ __global__ void __launch_bounds__(THREADS, 1)
           break;
         mbar_expect_tx(&sm->full[s], 2 * BM * BK * sizeof(float));
         const int x = (int)(rb + (int64_t)k * BK);
-        tma_load_2d(sm->raw[s][0], mapA, x, i0, &sm->full[s]);
-        tma_load_2d(sm->raw[s][1], mapB, x, jb, &sm->full[s]);
+        if (stack == kWhole) {
+          tma_load_2d(sm->raw[s][0], mapA, x, i0, &sm->full[s]);
+          tma_load_2d(sm->raw[s][1], mapB, x, jb, &sm->full[s]);
+        } else {  // halves of 64 lines (rows past N read as zeros)
+          const int x2 = stack == kRows ? x + (int)args.rows_per_split : x;
+          tma_load_2d(sm->raw[s][0], &maps.a[0], x, 0, &sm->full[s]);
+          tma_load_2d(sm->raw[s][0] + 64 * BK, &maps.a[1], x2, 0, &sm->full[s]);
+          tma_load_2d(sm->raw[s][1], &maps.b[0], x, 0, &sm->full[s]);
+          tma_load_2d(sm->raw[s][1] + 64 * BK, &maps.b[1], x2, 0, &sm->full[s]);
+        }
         ++issued;
       }
       // Before the CTA may exit, the copies it issued must have landed (they
@@ -279,11 +297,23 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint32_t lrow = (uint32_t)(32 * q) << 16;
     const int kcl = nk <= kSingleChunk ? nk : args.kc;
     const int nch = nk > 0 ? (nk + kcl - 1) / kcl : 0;
-    const int row = i0 + 32 * q + lane;
+    // where this thread's row and columns 64 g .. +63 of the tile go: row `row`
+    // and columns col0 .. col0 + ncol - 1 (tile columns from cb0) of partial
+    // `part`; nothing when ncol is 0
+    int row = i0 + 32 * q + lane, part = split;
+    int col0 = j0 + 64 * g, ncol = args.seg_cols - jb - 64 * g;
+    if (stack != kWhole) {
+      const int hr = q >> 1;  // half of the tile's rows
+      row -= 64 * hr;
+      col0 = stack == kLine ? (hr + g) * args.m : 0;
+      ncol = stack == kLine ? (hr || !g ? args.m : 0)
+                            : (hr == g ? args.n : 0);
+      if (stack == kRows) part = 2 * split + g;
+    }
     // partials as FP32 pairs: split s holds hi at [2 s count, (2 s + 1)
     // count) and lo after it (no FP64 instruction in this kernel)
     const size_t count = (size_t)args.m * args.n;
-    float* out_hi = reinterpret_cast<float*>(args.part) + 2 * (size_t)split * count;
+    float* out_hi = reinterpret_cast<float*>(args.part) + 2 * (size_t)part * count;
     float* out_lo = out_hi + count;
     bool ok = nch > 0;
     for (int c = 0; c < nch && ok; ++c) {
@@ -317,9 +347,9 @@ __global__ void __launch_bounds__(THREADS, 1)
           if (row < args.m) {
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
-              const int col = j0 + cb + e;
-              if (jb + cb + e < args.seg_cols) {
-                const size_t idx = row + (size_t)col * args.m;
+              const int c = cb - 64 * g + e;
+              if (c < ncol) {
+                const size_t idx = row + (size_t)(col0 + c) * args.m;
                 out_hi[idx] = __uint_as_float(hi[e]);
                 out_lo[idx] = __uint_as_float(lo[e]);
               }
@@ -338,10 +368,10 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     __syncwarp();
     if (!ok && row < args.m) {  // a wait gave up: zero partial, error set
-      for (int cb = 64 * g; cb < 64 * g + 64; ++cb)
-        if (jb + cb < args.seg_cols) {
-          out_hi[row + (size_t)(j0 + cb) * args.m] = 0.f;
-          out_lo[row + (size_t)(j0 + cb) * args.m] = 0.f;
+      for (int c = 0; c < 64; ++c)
+        if (c < ncol) {
+          out_hi[row + (size_t)(col0 + c) * args.m] = 0.f;
+          out_lo[row + (size_t)(col0 + c) * args.m] = 0.f;
         }
     }
   }
@@ -355,8 +385,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-CUtensorMap block_map(const float* p, int64_t N, int cols) {
-  return f32_map(p, N, cols, N, BK, BM);
+CUtensorMap block_map(const float* p, int64_t N, int cols, int lines = BM) {
+  return f32_map(p, N, cols, N, BK, lines);
 }
 
 }  // namespace
@@ -519,8 +549,17 @@ void gram_tc_pairs(int64_t N, int m, const Blocks<float>& A,
   if (sym_seg >= 0 && (sym_seg >= B.count || B.cols != m))
     throw Error(-1, "gram_tc: a symmetric segment must be m x m");
   TcArgs a{};
+  int stack = kWhole;
+  if (m <= 64 && B.cols <= 64) {
+    if (A.count == 3 && A.p[1] == A.p[2] && B.p[0] == B.p[1] && B.cols == m)
+      stack = kLine;
+    else if (nseg == 1 && N >= 2 * BK)
+      stack = kRows;
+  }
+  if (stack == kLine) sym_seg = -1;  // (P^T P comes whole)
   int tiles = 0;
-  for (int tj = 0; tj < nseg * tps; ++tj) {
+  if (stack != kWhole) tiles = 1;
+  for (int tj = 0; stack == kWhole && tj < nseg * tps; ++tj) {
     const int seg = tj / tps;
     const int tjs = tj - seg * tps;  // column tile in its segment
     for (int ti = 0; ti < tiles_m; ++ti) {
@@ -541,6 +580,16 @@ void gram_tc_pairs(int64_t N, int m, const Blocks<float>& A,
     const int kb = k < B.count ? k : 0;
     maps.a[k] = block_map(A.p[A.count > 1 ? kb : 0], N, m);
     maps.b[k] = block_map(B.p[kb], N, B.cols);
+  }
+  TcMaps half;  // the stacked operands
+  if (stack != kWhole) {
+    const bool line = stack == kLine;
+    half.a[0] = block_map(A.p[0], N, m, 64);
+    half.a[1] = line ? block_map(A.p[1], N, m, 64) : half.a[0];
+    half.b[0] = block_map(B.p[0], N, B.cols, 64);
+    half.b[1] = line ? block_map(B.p[2], N, m, 64) : half.b[0];
+    half.a[2] = half.a[3] = half.a[0];
+    half.b[2] = half.b[3] = half.b[0];
   }
   a.N = N;
   a.m = m;
@@ -567,16 +616,26 @@ void gram_tc_pairs(int64_t N, int m, const Blocks<float>& A,
   auto run = [&](int want) {
     int64_t rows = (N + want - 1) / want;
     rows = ((rows + BK - 1) / BK) * BK;
-    const int splits = (int)((N + rows - 1) / rows);
+    int splits = (int)((N + rows - 1) / rows);  // partials
+    a.stack = stack == kRows && splits < 2 ? kWhole : stack;
+    int ctas = splits;
+    if (a.stack == kRows) {  // two slices a CTA
+      ctas = (splits + 1) / 2;
+      splits = 2 * ctas;
+    }
     if ((size_t)splits * count > cap)
       throw Error(-2, "gram_tc: partials buffer too small");
     a.rows_per_split = rows;
-    k_gram_tc<<<dim3(splits, tiles), THREADS, smem, s>>>(maps, a);
+    k_gram_tc<<<dim3(ctas, tiles), THREADS, smem, s>>>(
+        a.stack == kWhole ? maps : half, a);
     TRM_CHECK_LAUNCH();
     sum_splits_pairs(reinterpret_cast<const float*>(partials), splits, count,
                      out, s, m, also, SymSeg{sym_seg, m, segcols, BM});
   };
-  run(tuned_splits(N, m, n, tiles, sym_seg, smax, s, run));
+  // (an odd count of kRows slices takes one more partial: even caps)
+  if (stack == kRows && smax > 1) smax &= ~1;
+  run(tuned_splits(N, m, n, tiles, stack == kWhole ? sym_seg : -1 - stack, smax,
+                   s, run));
 }
 
 }  // namespace trm

@@ -235,39 +235,39 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else if (warp == 3) {
     // ------- TMA: the gradient's epilogue operands into the slots -------
-    // Slot sequence: tile tl, column half g, 8-column group q (0..7) is
-    // number j = 8 tl + q of half g and lands in slot 2 g + (j & 1).
+    // Slot sequence: half g's 8-column groups, those with a column below n,
+    // tile after tile; its number j lands in slot 2 g + (j & 1).
     if (MODE == kGrad && lane == 0) {
       const bool hg = args.gprev != nullptr, hp = args.pprev != nullptr;
       const uint32_t bytes = (uint32_t)(EC * BM * 4) * (1 + hg + hp);
       float* slots = &sm->rawp[0][0];
-      int last[NSLOT] = {-1, -1, -1, -1};  // the number last loaded per slot
-      int j = 0;
+      int jn[2] = {0, 0};  // groups loaded per half
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         int r0, c0;
         tile_rc(args, t, r0, c0);
-        for (int q = 0; q < 8 && ok; ++q, ++j)
+        for (int q = 0; q < 8 && ok; ++q)
           for (int g = 0; g < 2 && ok; ++g) {
-            const int e = 2 * g + (j & 1);
+            const int c = c0 + g * (NC / 2) + q * EC;
+            if (c >= args.n) continue;
+            const int j = jn[g], e = 2 * g + (j & 1);
             if (j >= 2 && !mbar_wait(&sm->eempty[e], ((j >> 1) - 1) & 1,
                                      args.err, &sm->failed)) {
               ok = false;
               break;
             }
             float* d = slots + e * ESLOT;
-            const int c = c0 + g * (NC / 2) + q * EC;
             mbar_expect_tx(&sm->efull[e], bytes);
             tma_load_2d(d, &mapX, r0, c, &sm->efull[e]);
             if (hg) tma_load_2d(d + EC * BM, &mapGp, r0, c, &sm->efull[e]);
             if (hp) tma_load_2d(d + 2 * EC * BM, &mapPp, r0, c, &sm->efull[e]);
-            last[e] = j;
+            jn[g] = j + 1;
           }
       }
       // the copies in flight must land before the CTA may exit
-      for (int e = 0; e < NSLOT; ++e)
-        if (last[e] >= 0)
-          mbar_wait_own(&sm->efull[e], (last[e] >> 1) & 1, args.err);
+      for (int g = 0; g < 2; ++g)
+        for (int j = jn[g] > 2 ? jn[g] - 2 : 0; j < jn[g]; ++j)
+          mbar_wait_own(&sm->efull[2 * g + (j & 1)], (j >> 1) & 1, args.err);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int half = cbeg ? 1 : 0;
     const bool hg = args.gprev != nullptr, hp = args.pprev != nullptr;
     bool dead = false;
-    int tl = 0;
+    int tl = 0, jslot = 0;
     for (int t = blockIdx.x; t < ntiles && !dead; t += gridDim.x, ++tl) {
       const int b = tl & 1;
       // warp-uniform outcome: the TMEM loads below are .sync.aligned
@@ -397,8 +397,10 @@ __global__ void __launch_bounds__(THREADS, 1)
       const bool rin = row < N;
       float mi = 1.f;
       if (MODE == kGrad && rin && args.minv) mi = args.minv[row];
+      // (columns past n: nothing is staged, read or written for them)
+      const int cend = min(cbeg + NC / 2, args.n - c0);
 #pragma unroll 1
-      for (int cb = cbeg; cb < cbeg + NC / 2; cb += 16) {
+      for (int cb = cbeg; cb < cend; cb += 16) {
         uint32_t r[16];
         tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * NC + cb), r);
         if (MODE == kGrad) {
@@ -406,7 +408,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           // thread of the half arrives, rows past N included)
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            const int j = 8 * tl + (cb - cbeg) / EC + h;
+            if (cb + h * EC >= cend) break;  // (no slot was filled for it)
+            const int j = jslot++;
             const int e = 2 * half + (j & 1);
             const bool in_slot =
                 mbar_wait(&sm->efull[e], (j >> 1) & 1, args.err, &sm->failed);
@@ -511,17 +514,15 @@ __global__ void __launch_bounds__(THREADS, 1)
       mbar_arrive(&sm->accempty[b]);
     }
     if (MODE == kGrad) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-          s_sum[j] = df_add(s_sum[j],
-                            F2{__shfl_xor_sync(0xffffffffu, s_sum[j].h, o),
-                               __shfl_xor_sync(0xffffffffu, s_sum[j].l, o)});
-      if (lane == 0)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          sm->red[warp - EPI0][j] = (double)s_sum[j].h + (double)s_sum[j].l;
+      const F2 w4 = warp_sum4(
+          s_sum,
+          [](F2 x, int o) {
+            return F2{__shfl_xor_sync(0xffffffffu, x.h, o),
+                      __shfl_xor_sync(0xffffffffu, x.l, o)};
+          },
+          [](F2 x, F2 y) { return df_add(x, y); });
+      if ((lane & 7) == 0)
+        sm->red[warp - EPI0][lane >> 3] = (double)w4.h + (double)w4.l;
       asm volatile("bar.sync 1, %0;" ::"n"(NEPI * 32) : "memory");
       if (threadIdx.x == EPI0 * 32) {
 #pragma unroll
@@ -547,15 +548,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int c = t; c < (int)gridDim.x; c += NEPI * 32)
 #pragma unroll
           for (int j = 0; j < 4; ++j) v[j] += __ldcg(&args.part[(size_t)c * 4 + j]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1)
-            v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+        const double w8 = warp_sum4(v);
         asm volatile("bar.sync 1, %0;" ::"n"(NEPI * 32) : "memory");
-        if (lane == 0)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) sm->red[warp - EPI0][j] = v[j];
+        if ((lane & 7) == 0) sm->red[warp - EPI0][lane >> 3] = w8;
         asm volatile("bar.sync 1, %0;" ::"n"(NEPI * 32) : "memory");
         if (t == 0) {
           double tot[4];
