@@ -363,10 +363,14 @@ void random_block(int64_t N, int m, uint64_t seed, double* C, cudaStream_t s,
 // m x m FP64 matrices on the device
 // ---------------------------------------------------------------------------
 // Cm = alpha op(A) op(B) + beta Cm (all m x m FP64, column-major)
-// (fp32: products and sums in FP32, inputs and outputs FP64)
 void mm_gemm(int m, const double* A, bool trA, const double* B, bool trB,
-             double* Cm, double alpha, double beta, cudaStream_t s,
-             bool fp32 = false);
+             double* Cm, double alpha, double beta, cudaStream_t s);
+// Newton-Schulz steps X <- X (3 I - X^T X) / 2 towards the nearest matrix with
+// orthonormal columns, at most `steps`: none is run after one that started
+// within 1e-10 of it. X and Xn swap per step (X the result); G: m x m work; dev:
+// `steps` words, zeroed.
+void newton_schulz(int m, double*& X, double*& Xn, double* G,
+                   unsigned long long* dev, int steps, cudaStream_t s);
 // A0 = sym(H') + diag(H_D)
 void make_A0(int m, const double* Hp, const double* HD, double* A0,
              cudaStream_t s);
@@ -422,6 +426,8 @@ void sym_eig(int m, const double* A, double* w, double* Z, double* work,
 // 1e-12 of the largest sets *status bit 1. work: polar_work_doubles(m);
 // info as sym_eig's.
 size_t polar_work_doubles(int m);
+// Near-orthogonal M takes Newton-Schulz steps instead (info 0); the stream is
+// waited for once, to see which.
 void polar_factor(int m, const double* M, double* U, double* work, int* status,
                   int* info, cudaStream_t s);
 

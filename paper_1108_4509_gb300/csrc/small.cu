@@ -16,36 +16,101 @@ namespace trm {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Cm = alpha op(A) op(B) + beta Cm, 16 x 16 tiles, one output per thread.
+// Cm = alpha op(A) op(B) + beta Cin, 8 x 8 tiles on 256 threads: four threads
+// share an output, each a quarter of every 64-deep stage, in two chains. An
+// SM does two FP64 multiply-adds a cycle, so these matrices are spread over as
+// many SMs as they fill: 4.9 us at m = 48, 5.6 at 64, 8.3 at 128, 35 at 256
+// with launches back to back; 16 x 16 tiles, one thread per output, take 8.2,
+// 8.3, 14 and 41 (m = 512: 231 and 238, m = 1024: 1780 and 1762).
+//
+// skip (may be null): when *skip is below kNsDone the product is not formed
+// and Cm becomes a copy of Cin (is left alone without one). dev (may be null):
+// receives max |Cm - I|, as the bits of a non-negative double.
 // ---------------------------------------------------------------------------
-template <typename Tc>
+// A Newton-Schulz step takes X^T X - I = E to 3/4 E^2 + 1/4 E^3: from entries
+// below 1e-10 to below m 1e-20, less than rounding leaves, so the steps after
+// that one change nothing.
+constexpr double kNsDone = 1e-10;
+
+struct GemmOpt {
+  const double* cin = nullptr;
+  const unsigned long long* skip = nullptr;
+  unsigned long long* dev = nullptr;
+};
+
 __global__ void __launch_bounds__(256)
     k_mm_gemm(int m, const double* __restrict__ A, int trA,
-              const double* __restrict__ B, int trB, double* Cm,
-              double alpha, double beta) {
-  __shared__ Tc As[16][17], Bs[16][17];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int i = blockIdx.x * 16 + tx;
-  const int j = blockIdx.y * 16 + ty;
-  Tc acc = 0;
-  for (int k0 = 0; k0 < m; k0 += 16) {
-    const int ka = k0 + ty;
-    As[ty][tx] = (i < m && ka < m) ? (Tc)(trA ? A[ka + (int64_t)i * m]
-                                              : A[i + (int64_t)ka * m])
-                                   : (Tc)0;
-    const int kb = k0 + tx;
-    Bs[ty][tx] = (kb < m && j < m) ? (Tc)(trB ? B[j + (int64_t)kb * m]
-                                              : B[kb + (int64_t)j * m])
-                                   : (Tc)0;
+              const double* __restrict__ B, int trB, double* __restrict__ Cm,
+              double alpha, double beta, GemmOpt opt) {
+  constexpr int TT = 8;   // tile
+  constexpr int KS = 4;   // threads per output
+  constexpr int KD = 64;  // stage depth
+  __shared__ double As[KD][TT + 1], Bs[KD][TT + 1];
+  __shared__ double part[KS][TT * TT];
+  const int tid = threadIdx.x;
+  const int o = tid % (TT * TT), ks = tid / (TT * TT);
+  const int tx = o % TT, ty = o / TT;
+  const int i0 = blockIdx.x * TT, j0 = blockIdx.y * TT;
+  const int i = i0 + tx, j = j0 + ty;
+  const bool in = i < m && j < m;
+  const int64_t e = i + (int64_t)j * m;
+  if (opt.skip && __longlong_as_double((long long)*opt.skip) < kNsDone) {
+    if (in && ks == 0 && opt.cin) Cm[e] = opt.cin[e];
+    return;
+  }
+  double a0 = 0.0, a1 = 0.0;
+  for (int k0 = 0; k0 < m; k0 += KD) {
+    for (int q = tid; q < KD * TT; q += 256) {
+      // each operand along its contiguous index
+      const int kr = trA ? q % KD : q / TT, r = trA ? q / KD : q % TT;
+      As[kr][r] = (i0 + r < m && k0 + kr < m)
+                      ? (trA ? A[(k0 + kr) + (int64_t)(i0 + r) * m]
+                             : A[(i0 + r) + (int64_t)(k0 + kr) * m])
+                      : 0.0;
+      const int kc = trB ? q / TT : q % KD, c = trB ? q % TT : q / KD;
+      Bs[kc][c] = (k0 + kc < m && j0 + c < m)
+                      ? (trB ? B[(j0 + c) + (int64_t)(k0 + kc) * m]
+                             : B[(k0 + kc) + (int64_t)(j0 + c) * m])
+                      : 0.0;
+    }
     __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) acc += As[kk][tx] * Bs[ty][kk];
+    for (int k = 0; k < 16; k += 2) {
+      a0 = fma(As[16 * ks + k][tx], Bs[16 * ks + k][ty], a0);
+      a1 = fma(As[16 * ks + k + 1][tx], Bs[16 * ks + k + 1][ty], a1);
+    }
     __syncthreads();
   }
-  if (i < m && j < m) {
-    const int64_t o = i + (int64_t)j * m;
-    Cm[o] = alpha * (double)acc + (beta != 0.0 ? beta * Cm[o] : 0.0);
+  double acc = a0 + a1;
+  part[ks][o] = acc;
+  __syncthreads();
+  if (ks == 0)
+#pragma unroll
+    for (int q = 1; q < KS; ++q) acc += part[q][o];
+  double d = 0.0;
+  if (in && ks == 0) {
+    const double v = alpha * acc + (beta != 0.0 ? beta * opt.cin[e] : 0.0);
+    Cm[e] = v;
+    d = fabs(v - (i == j ? 1.0 : 0.0));
   }
+  if (opt.dev) {
+    // (a NaN's bits are above every number's: it never reads as converged)
+    unsigned long long b = (unsigned long long)__double_as_longlong(fabs(d));
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+      const unsigned long long x = __shfl_xor_sync(0xffffffffu, b, s);
+      b = x > b ? x : b;
+    }
+    if ((tid & 31) == 0 && b) atomicMax(opt.dev, b);
+  }
+}
+
+static void mm_launch(int m, const double* A, bool trA, const double* B, bool trB,
+                      double* Cm, double alpha, double beta, const GemmOpt& opt,
+                      cudaStream_t s) {
+  const int t = ceil_div(m, 8);
+  k_mm_gemm<<<dim3(t, t), 256, 0, s>>>(m, A, trA, B, trB, Cm, alpha, beta, opt);
+  TRM_CHECK_LAUNCH();
 }
 
 // A0 = sym(H') + diag(H_D): the projected matrix C^T H C when C^T C = I
@@ -1464,6 +1529,9 @@ __global__ void __launch_bounds__(1024)
 // stop when one applied no rotation or the off-diagonal part is below
 // conv_tol of the whole (squared Frobenius norms).
 // ---------------------------------------------------------------------------
+//
+// Before a sweep all pairs are looked at together: when none would be rotated,
+// its rounds are not run (m = 64 in FP64: 110 us of rounds).
 template <typename T>
 __global__ void __launch_bounds__(1024)
     k_jacobi(int m, const double* __restrict__ Ain, T* __restrict__ Ag,
@@ -1488,6 +1556,7 @@ __global__ void __launch_bounds__(1024)
   const int M = m + (m & 1);
   const int np = M / 2;
   int sweeps = 0;
+  bool settled = false;
   if (tid == 0) rotated = 1;
   __syncthreads();
   for (int sweep = 0; sweep <= max_sweeps; ++sweep) {
@@ -1509,7 +1578,17 @@ __global__ void __launch_bounds__(1024)
     }
     __syncthreads();
     if (done) break;
+    int any = 0;
+    for (int c = warp; c < m; c += nw)
+      for (int r = lane; r < c; r += 32) {
+        const T x = A[r + c * ld];
+        any |= x != (T)0 &&
+               fabs(x) > rot_tol * (fabs(A[r + r * ld]) + fabs(A[c + c * ld])) +
+                             abs_tol;
+      }
+    settled = !__syncthreads_or(any);
     sweeps = sweep + 1;
+    if (settled) break;
     for (int r = 0; r < M - 1; ++r) {
       for (int k = tid; k < np; k += nt) {
         const int a0 = (k == 0) ? 0 : 1 + ((k - 1 + r) % (M - 1));
@@ -1597,18 +1676,20 @@ __global__ void __launch_bounds__(1024)
       __syncthreads();
     }
   }
-  // ascending order (stable on ties)
-  for (int i = tid; i < m; i += nt) {
+  // ascending order (stable on ties), a column per warp
+  __syncthreads();
+  for (int i = warp; i < m; i += nw) {
     const T wi = A[i + i * ld];
     int rank = 0;
-    for (int j = 0; j < m; ++j) {
+    for (int j = lane; j < m; j += 32) {
       const T wj = A[j + j * ld];
       rank += (wj < wi) || (wj == wi && j < i);
     }
-    w[rank] = (double)wi;
-    for (int r = 0; r < m; ++r) Z[r + rank * m] = (double)Zw[r + i * m];
+    rank = __reduce_add_sync(0xffffffffu, rank);
+    if (lane == 0) w[rank] = (double)wi;
+    for (int r = lane; r < m; r += 32) Z[r + rank * m] = (double)Zw[r + i * m];
   }
-  if (tid == 0 && info) *info = done ? sweeps : -1;
+  if (tid == 0 && info) *info = (done || settled) ? sweeps : -1;
 }
 
 // ---------------------------------------------------------------------------
@@ -1622,57 +1703,92 @@ __global__ void __launch_bounds__(1024)
 //   e_ij = r_ij / 2 otherwise, and also where the first-order step would
 //          exceed 0.01 (inside a cluster only orthonormality is restored;
 //          the closing FP64 Jacobi separates the cluster),
-// and X <- X + X E. Frobenius norms stand for the 2-norms (a larger delta)
-// and max |lambda_i| for ||A||. One CTA; G = X^T X, S = X^T A X in, E out.
+// and X <- X + X E. The 2-norms in delta are taken as 2 / sqrt(m) of the
+// Frobenius norms, as for a matrix of random entries (m >= 128; the factor of
+// m = 128 below that: a delta as large as the Frobenius norms leaves pairs of
+// close eigenvalues to the FP64 sweeps, 170 us of them at m = 64, and with
+// couplings up to their threshold), max |lambda_i| as ||A||. G = X^T X,
+// S = X^T A X in, E out.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024)
-    k_refine_eig(int m, const double* __restrict__ G,
-                 const double* __restrict__ S, double* __restrict__ E) {
-  __shared__ double lam[1024];
+// Partial sums of ||S - D||^2 and ||R||^2 (R = I - G, D = diag(s_ii / g_ii)) and
+// max |lambda|, three doubles per CTA.
+__global__ void __launch_bounds__(256)
+    k_refine_norms(int m, const double* __restrict__ G,
+                   const double* __restrict__ S, double* __restrict__ part) {
   __shared__ double red[2 * 32];
-  __shared__ unsigned long long amax;  // max |lambda| (bits of a double >= 0)
-  const int tid = threadIdx.x, nt = blockDim.x;
-  if (tid == 0) amax = 0ull;
+  __shared__ unsigned long long amax;
+  if (threadIdx.x == 0) amax = 0ull;
   __syncthreads();
-  for (int i = tid; i < m; i += nt) {
-    lam[i] = S[i + (size_t)i * m] / G[i + (size_t)i * m];
-    // non-negative doubles order like their bit patterns
-    atomicMax(&amax, (unsigned long long)__double_as_longlong(fabs(lam[i])));
-  }
-  __syncthreads();
-  double v[2] = {0.0, 0.0};  // ||S - D||^2, ||R||^2
-  for (size_t e = tid; e < (size_t)m * m; e += nt) {
+  double v[2] = {0.0, 0.0};
+  unsigned long long mx = 0ull;
+  for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < (size_t)m * m;
+       e += (size_t)gridDim.x * 256) {
     const int i = (int)(e % m), j = (int)(e / m);
-    const double r = (i == j ? 1.0 : 0.0) - G[e];
-    const double d = S[e] - (i == j ? lam[i] : 0.0);
-    v[0] += d * d;
-    v[1] += r * r;
+    double r = -G[e], d = S[e];
+    if (i == j) {
+      r += 1.0;
+      const double lam = S[e] / G[e];
+      d -= lam;
+      // non-negative doubles order like their bit patterns
+      mx = max(mx, (unsigned long long)__double_as_longlong(fabs(lam)));
+    }
+    v[0] = fma(d, d, v[0]);
+    v[1] = fma(r, r, v[1]);
   }
+  if (mx) atomicMax(&amax, mx);
   block_sum<2>(v, red);
-  const double anorm = __longlong_as_double((long long)amax);
-  const double delta = 2.0 * (sqrt(v[0]) + anorm * sqrt(v[1]));
-  for (size_t e = tid; e < (size_t)m * m; e += nt) {
-    const int i = (int)(e % m), j = (int)(e / m);
-    const double r = (i == j ? 1.0 : 0.0) - G[e];
-    const double dl = lam[j] - lam[i];
-    const double num = S[e] + lam[j] * r;
-    E[e] = (i != j && fabs(dl) > delta && fabs(num) <= 0.01 * fabs(dl))
-               ? num / dl
-               : 0.5 * r;
+  if (threadIdx.x == 0) {
+    part[3 * blockIdx.x] = v[0];
+    part[3 * blockIdx.x + 1] = v[1];
+    part[3 * blockIdx.x + 2] = __longlong_as_double((long long)amax);
   }
+}
+
+// E of the refinement (see sym_eig), an entry per thread; the nparts partial
+// norms are added by every CTA alike. (On one CTA its m^2 FP64 divisions took
+// 33 us at m = 64.)
+__global__ void __launch_bounds__(256)
+    k_refine_eig(int m, const double* __restrict__ G,
+                 const double* __restrict__ S, const double* __restrict__ part,
+                 int nparts, double* __restrict__ E) {
+  __shared__ double sdelta;
+  if (threadIdx.x < 32) {
+    double a = 0.0, b = 0.0, c = 0.0;
+    for (int k = threadIdx.x; k < nparts; k += 32) {
+      a += part[3 * k];
+      b += part[3 * k + 1];
+      c = fmax(c, part[3 * k + 2]);
+    }
+    a = warp_sum(a);
+    b = warp_sum(b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      c = fmax(c, __shfl_xor_sync(0xffffffffu, c, o));
+    if (threadIdx.x == 0)
+      sdelta = 4.0 * rsqrt((double)max(m, 128)) * (sqrt(a) + c * sqrt(b));
+  }
+  __syncthreads();
+  const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (e >= (size_t)m * m) return;
+  const double delta = sdelta;
+  const int i = (int)(e % m), j = (int)(e / m);
+  const double lj = S[j + (size_t)j * m] / G[j + (size_t)j * m];
+  const double li = S[i + (size_t)i * m] / G[i + (size_t)i * m];
+  const double r = (i == j ? 1.0 : 0.0) - G[e];
+  const double dl = lj - li;
+  const double num = S[e] + lj * r;
+  E[e] = (i != j && fabs(dl) > delta && fabs(num) <= 0.01 * fabs(dl))
+             ? num / dl
+             : 0.5 * r;
 }
 
 }  // namespace
 
 void mm_gemm(int m, const double* A, bool trA, const double* B, bool trB,
-             double* Cm, double alpha, double beta, cudaStream_t s,
-             bool fp32) {
-  dim3 grid(ceil_div(m, 16), ceil_div(m, 16));
-  if (fp32)
-    k_mm_gemm<float><<<grid, 256, 0, s>>>(m, A, trA, B, trB, Cm, alpha, beta);
-  else
-    k_mm_gemm<double><<<grid, 256, 0, s>>>(m, A, trA, B, trB, Cm, alpha, beta);
-  TRM_CHECK_LAUNCH();
+             double* Cm, double alpha, double beta, cudaStream_t s) {
+  GemmOpt o;
+  o.cin = Cm;
+  mm_launch(m, A, trA, B, trB, Cm, alpha, beta, o, s);
 }
 
 void make_A0(int m, const double* Hp, const double* HD, double* A0,
@@ -1936,7 +2052,26 @@ static void jacobi_launch(int m, const double* A, const double* Z0, double* w,
   TRM_CHECK_LAUNCH();
 }
 
-size_t sym_eig_work_doubles(int m) { return (size_t)8 * m * m; }
+// 8 m x m matrices, 2 x 4 deviations, the partial norms
+constexpr int kNormParts = 64;
+size_t sym_eig_work_doubles(int m) {
+  return (size_t)8 * m * m + 8 + 3 * kNormParts;
+}
+
+void newton_schulz(int m, double*& X, double*& Xn, double* G,
+                   unsigned long long* dev, int steps, cudaStream_t s) {
+  for (int k = 0; k < steps; ++k) {
+    GemmOpt g;
+    g.skip = k ? dev + k - 1 : nullptr;
+    g.dev = dev + k;  // stays 0 when skipped: so are all later ones
+    mm_launch(m, X, true, X, false, G, 1.0, 0.0, g, s);
+    GemmOpt h;
+    h.cin = X;
+    h.skip = g.skip;
+    mm_launch(m, X, false, G, false, Xn, -0.5, 1.5, h, s);
+    std::swap(X, Xn);
+  }
+}
 
 // FP32 Jacobi sweeps (the FP64 pipe is 1/64 of the FP32 one); then twice:
 // one FP64 refinement of the eigenvectors by matrix products on many CTAs,
@@ -1963,24 +2098,28 @@ void sym_eig(int m, const double* A, double* w, double* Z, double* work,
   jacobi_launch<float>(m, A, nullptr, w, X, reinterpret_cast<float*>(jw),
                        reinterpret_cast<float*>(jw) + mm, info, 20, 4e-7f,
                        1e-6f, 0.0f, s);
+  constexpr int kNs = 4;
+  auto* dev = reinterpret_cast<unsigned long long*>(work + 8 * mm);
+  double* norms = work + 8 * mm + 2 * kNs;
+  const int nparts = std::min(ceil_div((int64_t)mm, 1024), kNormParts);
+  TRM_CUDA(cudaMemsetAsync(dev, 0, 2 * kNs * sizeof(*dev), s));
   for (int it = 0; it < 2; ++it) {
-    mm_gemm(m, A, false, X, false, T, 1.0, 0.0, s, false);   // A X
-    mm_gemm(m, X, true, T, false, Sx, 1.0, 0.0, s, false);   // X^T A X
-    mm_gemm(m, X, true, X, false, G, 1.0, 0.0, s, false);    // X^T X
-    k_refine_eig<<<1, 1024, 0, s>>>(m, G, Sx, E);
+    mm_gemm(m, A, false, X, false, T, 1.0, 0.0, s);   // A X
+    mm_gemm(m, X, true, T, false, Sx, 1.0, 0.0, s);   // X^T A X
+    mm_gemm(m, X, true, X, false, G, 1.0, 0.0, s);    // X^T X
+    k_refine_norms<<<nparts, 256, 0, s>>>(m, G, Sx, norms);
     TRM_CHECK_LAUNCH();
-    TRM_CUDA(cudaMemcpyAsync(Xn, X, mm * 8, cudaMemcpyDeviceToDevice, s));
-    mm_gemm(m, X, false, E, false, Xn, 1.0, 1.0, s, false);  // X + X E
+    k_refine_eig<<<ceil_div((int64_t)mm, 256), 256, 0, s>>>(m, G, Sx, norms,
+                                                            nparts, E);
+    TRM_CHECK_LAUNCH();
+    GemmOpt o;
+    o.cin = X;
+    mm_launch(m, X, false, E, false, Xn, 1.0, 1.0, o, s);  // X + X E
     std::swap(X, Xn);
-    for (int ns = 0; ns < 4; ++ns) {
-      mm_gemm(m, X, true, X, false, G, 1.0, 0.0, s, false);  // X^T X
-      TRM_CUDA(cudaMemcpyAsync(Xn, X, mm * 8, cudaMemcpyDeviceToDevice, s));
-      mm_gemm(m, X, false, G, false, Xn, -0.5, 1.5, s, false);  // 1.5 X - X G / 2
-      std::swap(X, Xn);
-    }
+    newton_schulz(m, X, Xn, G, dev + it * kNs, kNs, s);
   }
-  mm_gemm(m, A, false, X, false, T, 1.0, 0.0, s, false);
-  mm_gemm(m, X, true, T, false, Sx, 1.0, 0.0, s, false);
+  mm_gemm(m, A, false, X, false, T, 1.0, 0.0, s);
+  mm_gemm(m, X, true, T, false, Sx, 1.0, 0.0, s);
   jacobi_launch<double>(m, Sx, X, w, Z, jw, jw + mm, info, 8, 1e-13, 1e-15,
                         0.0, s);
 }

@@ -290,3 +290,27 @@ def test_digit_products_fp64_step(trm, shape, m):
     Y = C + a * G0
     L = np.linalg.cholesky(Y.T @ Y)
     assert np.max(np.abs(C1 - np.linalg.solve(L, Y.T).T)) < 1e-12
+
+
+@pytest.mark.parametrize("side", [-1, 1])
+@pytest.mark.parametrize("m", [1, 7, 8, 9, 160, 161])
+def test_polar_factor_on_both_sides_of_its_rule(trm, m, side):
+    """||M^T M - I||_F a little below 1/2 takes Newton-Schulz steps, above it
+    the eigensolver: both give the oracle's extrapolation. The sizes lie at the
+    edges of the products' tiles. Rounding: m eps in each of some ten products
+    of matrices of norm up to 2."""
+    N = 2 * m + 50
+    rng = np.random.default_rng(m)
+    full = np.linalg.qr(rng.standard_normal((N, 2 * m)))[0]
+    q1 = np.linalg.qr(rng.standard_normal((m, m)))[0]
+    q2 = np.linalg.qr(rng.standard_normal((m, m)))[0]
+    d = rng.uniform(0.2, 1.0, m)  # 1 - cos^2 of the principal angles
+    d *= (0.5 + side * 1e-3) / np.linalg.norm(d)
+    C0 = full[:, :m]
+    C1 = (C0 @ q1 * np.sqrt(1 - d) + full[:, m:] * np.sqrt(d)) @ q2
+    want = otrm.extrapolate(C0, C1, 1.0)
+    d0, d1 = gu.to_dev(C0), gu.to_dev(C1)
+    dn = gu.empty(N, m, np.float64)
+    trm.trm_extrapolate(N, m, d0.data_ptr(), d1.data_ptr(), 1.0, dn.data_ptr(),
+                        gu.stream())
+    assert np.max(np.abs(gu.from_dev(dn) - want)) < 20 * m * 2.3e-16 + 1e-14
