@@ -32,10 +32,23 @@ namespace {
 // that one change nothing.
 constexpr double kNsDone = 1e-10;
 
+// Acceptance of chol_refined's result: max |X S X^T - I| after one correction
+// (another then leaves m 1e-20), max |X - I| after both
+__device__ __forceinline__ bool refined_ok(const unsigned long long* dev) {
+  return __longlong_as_double((long long)dev[1]) < 1e-10 &&
+         __longlong_as_double((long long)dev[2]) < 0.5;
+}
+
+// tri: which operands are lower triangular (the products then leave out what
+// lies beyond their tiles), and Phi: 1 where only the lower triangle of
+// Cm - I is wanted, with half its diagonal (dev as before).
+enum { kTriA = 1, kTriB = 2, kTriBt = 4, kTriOut = 8, kPhi = 16 };
+
 struct GemmOpt {
   const double* cin = nullptr;
   const unsigned long long* skip = nullptr;
   unsigned long long* dev = nullptr;
+  int tri = 0;
 };
 
 __global__ void __launch_bounds__(256)
@@ -58,17 +71,22 @@ __global__ void __launch_bounds__(256)
     if (in && ks == 0 && opt.cin) Cm[e] = opt.cin[e];
     return;
   }
+  if ((opt.tri & kTriOut) && j0 > i0) return;
+  int kb = 0, ke = m;  // the sum's range
+  if (opt.tri & kTriA) ke = min(ke, i0 + TT);
+  if (opt.tri & kTriBt) ke = min(ke, j0 + TT);
+  if (opt.tri & kTriB) kb = j0;
   double a0 = 0.0, a1 = 0.0;
-  for (int k0 = 0; k0 < m; k0 += KD) {
+  for (int k0 = kb; k0 < ke; k0 += KD) {
     for (int q = tid; q < KD * TT; q += 256) {
       // each operand along its contiguous index
       const int kr = trA ? q % KD : q / TT, r = trA ? q / KD : q % TT;
-      As[kr][r] = (i0 + r < m && k0 + kr < m)
+      As[kr][r] = (i0 + r < m && k0 + kr < ke)
                       ? (trA ? A[(k0 + kr) + (int64_t)(i0 + r) * m]
                              : A[(i0 + r) + (int64_t)(k0 + kr) * m])
                       : 0.0;
       const int kc = trB ? q / TT : q % KD, c = trB ? q % TT : q / KD;
-      Bs[kc][c] = (k0 + kc < m && j0 + c < m)
+      Bs[kc][c] = (k0 + kc < ke && j0 + c < m)
                       ? (trB ? B[(j0 + c) + (int64_t)(k0 + kc) * m]
                              : B[(k0 + kc) + (int64_t)(j0 + c) * m])
                       : 0.0;
@@ -90,8 +108,8 @@ __global__ void __launch_bounds__(256)
   double d = 0.0;
   if (in && ks == 0) {
     const double v = alpha * acc + (beta != 0.0 ? beta * opt.cin[e] : 0.0);
-    Cm[e] = v;
-    d = fabs(v - (i == j ? 1.0 : 0.0));
+    d = v - (i == j ? 1.0 : 0.0);
+    Cm[e] = !(opt.tri & kPhi) ? v : i > j ? d : i == j ? 0.5 * d : 0.0;
   }
   if (opt.dev) {
     // (a NaN's bits are above every number's: it never reads as converged)
@@ -318,7 +336,9 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
                const double* __restrict__ Q, const float* __restrict__ Bf,
                const float* __restrict__ Qf, double* __restrict__ Linv,
                double* __restrict__ R, IterScalars* sc, Tm* gwork,
-               const double* __restrict__ lpart, int nlpart) {
+               const double* __restrict__ lpart, int nlpart,
+               const unsigned long long* refined) {
+  if (refined && refined_ok(refined)) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int bad;
   __shared__ Tm rdiag[1024];  // 1 / L_cc, all columns (mp <= 1024)
@@ -1145,7 +1165,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
       hi[i + (size_t)i * out.ldm] = h;
       lo[i + (size_t)i * out.ldm] = l;
     }
-  } else {
+  } else if (out.R) {
     for (int i = warp; i < m; i += nw)
       for (int k = lane; k < m; k += 32)
         out.R[k + i * m] = k < i ? to_f64(entry(k, i))
@@ -1181,6 +1201,50 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
 constexpr int CB = 32;
 
 // The line step alpha from the line-term partials (one CTA).
+// A power of two whose square brings a positive number into [1/2, 2) (finite
+// for any bits); 1 for a number on either side of 1
+__device__ __forceinline__ double half_exp_scale(double x) {
+  const int e = (int)((__double_as_longlong(x) >> 52) & 0x7ff) - 1023;
+  return __longlong_as_double((long long)(1023 - ((e + 1) >> 1)) << 52);
+}
+
+// S' = D S D (D from S's diagonal; the lower triangle of S, mirrored), or S(a)
+// = I + a (B + B^T) + a^2 (Q + Q^T) / 2. Clears the three deviations.
+__global__ void __launch_bounds__(256)
+    k_ref_form(int m, const double* __restrict__ S,
+               const double* __restrict__ Bm, const double* __restrict__ Q,
+               const IterScalars* __restrict__ sc, double* __restrict__ Sp,
+               unsigned long long* dev) {
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e < 3) dev[e] = 0ull;
+  if (e >= m * m) return;
+  const int i = max(e % m, e / m), k = min(e % m, e / m);
+  if (Bm) {
+    const double al = sc->alpha;
+    Sp[e] = al * (Bm[i + k * m] + Bm[k + i * m]) +
+            0.5 * al * al * (Q[i + k * m] + Q[k + i * m]) + (i == k ? 1.0 : 0.0);
+  } else {
+    Sp[e] = S[i + k * m] * half_exp_scale(S[i + i * m]) *
+            half_exp_scale(S[k + k * m]);
+  }
+}
+
+// L^{-1} = X D and its transpose, where the corrections converged
+__global__ void __launch_bounds__(256)
+    k_ref_out(int m, const double* __restrict__ S, const double* __restrict__ X,
+              const unsigned long long* __restrict__ dev,
+              double* __restrict__ Linv, double* __restrict__ R) {
+  if (!refined_ok(dev)) return;
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e >= m * m) return;
+  const int i = e % m, k = e / m;
+  const double lo = i >= k ? X[e] * (S ? half_exp_scale(S[k + k * m]) : 1.0) : 0.0;
+  const double up = i <= k ? X[k + i * m] * (S ? half_exp_scale(S[i + i * m]) : 1.0)
+                           : 0.0;
+  if (Linv) Linv[e] = lo;
+  R[e] = up;
+}
+
 __global__ void k_cb_alpha(int m, const double* __restrict__ lpart, int nlpart,
                            IterScalars* sc) {
   __shared__ double lred[4 * 32];
@@ -1812,12 +1876,17 @@ static int chol_blocked_from() {
   return v;
 }
 
+// FP64 factor and inverse by correcting FP32 ones: S' (S scaled by powers of
+// two to a diagonal near 1), X, two temporaries, Phi, three deviations
+static size_t refine_elems(int m) { return (size_t)5 * m * m + 3; }
+
 // elements of the padded working copy plus the inverse's temporary (one
-// CTA), or of W, L, X, T and the failure flag (blocked)
+// CTA; FP64: or of refine_elems), or of W, L, X, T and the failure flag
+// (blocked)
 size_t chol_work_elems(int m) {
   const size_t mp = (size_t)((m + 31) & ~31);
   if (m >= chol_blocked_from() || m >= kPanelMax) return 4 * mp * mp + 8;
-  return mp * (mp + 1) + 33 * mp;
+  return std::max(mp * (mp + 1) + 33 * mp, refine_elems(m));
 }
 
 template <typename Tm, bool dev>
@@ -1888,6 +1957,58 @@ static bool panel_fits(int m) {
   return m <= kPanelMax && (m < chol_blocked_from() || m == kPanelMax);
 }
 
+// The FP64 factorisation on one CTA is bound by its SM's two FP64 multiply-adds
+// a cycle and the pivots' chain. Here the panel kernel's FP32 inverse factor X
+// is corrected to FP64 by products, which every SM shares: with F = X S X^T - I
+// and Phi the lower triangle of F with half its diagonal,
+// (I - Phi) X S X^T (I - Phi)^T = I + O(F^2), so X <- X - Phi X squares the
+// error. Two corrections suffice (dev[1], see refined_ok). The rounding errors of
+// the products grow with the condition, a little faster than the
+// elimination's: max |X - I| < 1/2 (dev[2]) holds it at about 20, within which
+// they are smaller (max |X S X^T - I| at m = 64: 3.3e-16 against 5.7e-16 at
+// condition 1.5; m = 48, condition 10: 2.8e-16 against 6.0e-16). Otherwise
+// nothing is written and k_chol_inv, launched behind it, does its work; it
+// returns at once where the result stands. 67 us instead of 166 at m = 64, 101
+// instead of 485 at 128; a matrix that is handed on loses 60 and 100 us.
+// m <= 32 has one panel and gains little (45 us instead of 60): left out.
+constexpr int kRefineFrom = 33;
+
+static const unsigned long long* chol_refined(int m, const double* S,
+                                              const double* Bm, const double* Q,
+                                              double* Linv, double* R,
+                                              IterScalars* sc, double* gwork,
+                                              cudaStream_t s) {
+  const size_t mm = (size_t)m * m;
+  double* Sp = gwork;
+  double* X = Sp + mm;
+  double* Xn = X + mm;
+  double* T = Xn + mm;
+  double* Phi = T + mm;
+  auto* dev = reinterpret_cast<unsigned long long*>(Phi + mm);
+  const int blocks = ceil_div((int64_t)mm, 256);
+  k_ref_form<<<blocks, 256, 0, s>>>(m, S, Bm, Q, sc, Sp, dev);
+  TRM_CHECK_LAUNCH();
+  PanelOut out;
+  out.Linv = X;
+  panel_launch<false>(m, Sp, nullptr, nullptr, out, nullptr, s, nullptr, 0);
+  for (int k = 0; k < 2; ++k) {
+    GemmOpt a, f, x;
+    a.tri = kTriA;
+    mm_launch(m, X, false, Sp, false, T, 1.0, 0.0, a, s);  // X S'
+    f.tri = kTriBt | kTriOut | kPhi;
+    f.dev = dev + k;
+    mm_launch(m, T, false, X, true, Phi, 1.0, 0.0, f, s);  // X S' X^T
+    x.tri = kTriA | kTriB | kTriOut;
+    x.cin = X;
+    if (k == 1) x.dev = dev + 2;
+    mm_launch(m, Phi, false, X, false, Xn, -1.0, 1.0, x, s);  // X - Phi X
+    std::swap(X, Xn);
+  }
+  k_ref_out<<<blocks, 256, 0, s>>>(m, S, X, dev, Linv, R);
+  TRM_CHECK_LAUNCH();
+  return dev;
+}
+
 template <typename Tm, bool dev>
 static void chol_launch(int m, const double* S, const double* Bm,
                         const double* Q, const float* Bf, const float* Qf,
@@ -1911,7 +2032,17 @@ static void chol_launch(int m, const double* S, const double* Bm,
                             nlpart);
       return;
     }
-    const size_t bytes = chol_work_elems(m) * sizeof(Tm);
+    const unsigned long long* refined = nullptr;
+    if (!dev && m >= kRefineFrom && panel_fits(m)) {
+      if (lpart) {
+        k_cb_alpha<<<1, 256, 0, s>>>(m, lpart, nlpart, sc);
+        TRM_CHECK_LAUNCH();
+        lpart = nullptr;
+      }
+      refined = chol_refined(m, S, Bm, Q, Linv, R, sc, gwork, s);
+    }
+    const size_t mp = (size_t)((m + 31) & ~31);
+    const size_t bytes = (mp * (mp + 1) + 33 * mp) * sizeof(Tm);
     const bool smem = bytes <= 200 * 1024;
     if (smem) {
       static std::atomic<int> done[64] = {};  // per device; any thread may launch
@@ -1926,11 +2057,11 @@ static void chol_launch(int m, const double* S, const double* Bm,
     }
     if (smem)
       k_chol_inv<Tm, dev, true><<<1, chol_threads<Tm>(), bytes, s>>>(
-          m, S, Bm, Q, Bf, Qf, Linv, R, sc, nullptr, lpart, nlpart);
+          m, S, Bm, Q, Bf, Qf, Linv, R, sc, nullptr, lpart, nlpart, refined);
     else
       k_chol_inv<Tm, dev, false><<<1, chol_threads<Tm>(), 0, s>>>(
           m, S, Bm, Q, Bf, Qf, Linv, R, sc, reinterpret_cast<Tm*>(gwork), lpart,
-          nlpart);
+          nlpart, refined);
     TRM_CHECK_LAUNCH();
   }
 }

@@ -314,3 +314,25 @@ def test_polar_factor_on_both_sides_of_its_rule(trm, m, side):
     trm.trm_extrapolate(N, m, d0.data_ptr(), d1.data_ptr(), 1.0, dn.data_ptr(),
                         gu.stream())
     assert np.max(np.abs(gu.from_dev(dn) - want)) < 20 * m * 2.3e-16 + 1e-14
+
+
+@pytest.mark.parametrize("cond", [4.0, 1e4])
+@pytest.mark.parametrize("m", [32, 33, 64, 129, 255, 256])
+def test_fp64_factor_corrected_and_eliminated(trm, m, cond):
+    """C^T C of condition 4 takes the corrected FP32 factor (33 <= m < 256), of
+    condition 1e4 the FP64 elimination behind it; the columns' scales span
+    2^+-40, which the factor's scaling takes out. Rounding of the Gram matrix
+    and the factor: m eps times the condition, a factor of 20 above."""
+    N = 2 * m + 100
+    rng = np.random.default_rng(m)
+    U = np.linalg.qr(rng.standard_normal((N, m)))[0]
+    V = np.linalg.qr(rng.standard_normal((m, m)))[0]
+    s = np.geomspace(1.0, cond ** 0.5, m)
+    C = (U * s) @ V * 2.0 ** np.floor(rng.uniform(-40, 40, m))
+    ref = otrm.orthonormalize(C)
+    t = gu.to_dev(C)
+    trm.trm_orthonormalize(N, m, t.data_ptr(), gu.stream())
+    got = gu.from_dev(t)
+    tol = 20 * m * 2.3e-16 * cond
+    assert np.max(np.abs(got.T @ got - np.eye(m))) < tol
+    assert np.max(np.abs(got - ref)) < tol
