@@ -85,7 +85,8 @@ constexpr int kCols = 4;  // columns per CTA (grid.y walks column groups)
 // thread and warp, one FP64 add per warp): CTA (t, u) writes
 // dots[(u gridDim.x + t) ncols + column].
 // It replaces kernels that took the z neighbours through L2 with two CTAs per
-// SM (98 registers): 160 us at 48^3 x 128, 4.94 ms at 96^3 x 512.
+// SM (98 registers): 160 us at 48^3 x 128 and 4.94 ms at 96^3 x 512, now 113 us
+// and 2.94 ms. The pairs' arithmetic is the bound (0.30 of the copy bandwidth).
 // ---------------------------------------------------------------------------
 // s + l += (h, l) of a neighbour
 __device__ __forceinline__ void acc_add(F2& a, float h, float l) {
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(256, 3)
 // the rest plainly), and the column dots c_j . (H c)_j: CTA b writes
 // dots[b ncols + column]. One column at a time with normalised sums it took 44
 // instructions an entry (420 us at N = 48^3, 13 entries a row, 128 columns) and
-// the dots 43 us in a kernel of their own.
+// the dots 43 us in a kernel of their own; now 252 us with the dots.
 __global__ void __launch_bounds__(256)
     k_csr_df(int64_t N, int64_t ld, const int32_t* __restrict__ rowptr,
              const int32_t* __restrict__ cols, const float* __restrict__ vh,

@@ -404,15 +404,10 @@ bool line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
 size_t chol_work_elems(int m);
 // S = L L^T (lower); writes Linv = L^{-1} (unless null) and R = L^{-T}. Non-PD sets
 // sc->status bit 1 and returns identities. gwork: chol_work_elems(m)
-// doubles (used when the working copy does not fit in shared memory).
+// doubles. FP64: see chol_refined.
 template <typename Tm>
 void chol_inv(int m, const double* S, double* Linv, double* R,
               IterScalars* sc, double* gwork, cudaStream_t s);
-// The same for S close to I, in deviation form (L = I + F, L^{-1} = I + Y):
-// FP32 arithmetic on the small parts gives FP64 accuracy relative to I.
-template <typename Tm>
-void chol_inv_dev(int m, const double* S, double* Linv, double* R,
-                  IterScalars* sc, double* gwork, cudaStream_t s);
 // symmetric eigenproblem A = Z diag(w) Z^T to FP64 accuracy (FP32 cyclic
 // Jacobi, FP64 refinement of the eigenvectors, FP64 Jacobi on the refined
 // projection), w ascending; work: sym_eig_work_doubles(m); info (device

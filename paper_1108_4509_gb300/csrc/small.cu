@@ -333,8 +333,7 @@ constexpr int chol_threads() { return 256; }
 template <typename Tm, bool dev, bool SM>
 __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
     k_chol_inv(int m, const double* __restrict__ S, const double* __restrict__ Bm,
-               const double* __restrict__ Q, const float* __restrict__ Bf,
-               const float* __restrict__ Qf, double* __restrict__ Linv,
+               const double* __restrict__ Q, double* __restrict__ Linv,
                double* __restrict__ R, IterScalars* sc, Tm* gwork,
                const double* __restrict__ lpart, int nlpart,
                const unsigned long long* refined) {
@@ -354,14 +353,12 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
     line_alpha_block(m, lpart, nlpart, sc, lred);
     __syncthreads();
   }
-  if (Bm || Bf) {
+  if (Bm) {
     // half of a (B + B^T) + a^2/2 (Q + Q^T) from each triangle, read in
     // column order (four loads of each matrix in flight per thread), then
-    // the lower triangle adds its mirror. With FP32 copies of B and Q (Bf,
-    // Qf) the FP32 factorisation does no FP64 work here.
+    // the lower triangle adds its mirror.
     const double al = sc->alpha;
     const double hq = 0.5 * al * al;
-    const float alf = (float)al, hqf = (float)hq;
     for (int k = warp; k < mp; k += nw)
       for (int i0 = lane; i0 < mp; i0 += 128) {
         Tm t[4];
@@ -369,10 +366,7 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
         for (int u = 0; u < 4; ++u) {
           const int i = i0 + 32 * u;
           const bool in = i < m && k < m;
-          if (Bf)
-            t[u] = in ? (Tm)(alf * Bf[i + k * m] + hqf * Qf[i + k * m]) : (Tm)0;
-          else
-            t[u] = in ? (Tm)(al * Bm[i + k * m] + hq * Q[i + k * m]) : (Tm)0;
+          t[u] = in ? (Tm)(al * Bm[i + k * m] + hq * Q[i + k * m]) : (Tm)0;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -431,7 +425,7 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
             // diagonal entry marks a (numerically) singular S
             const int cc = c0 + c;
             const double sjj =
-                (Bm || Bf || cc >= m) ? 1.0 : fabs(S[cc + cc * m]);
+                (Bm || cc >= m) ? 1.0 : fabs(S[cc + cc * m]);
             if (!(d > (Tm)(4 * m) * eps * (Tm)sjj)) {
               b = true;
               d = (Tm)1;
@@ -653,7 +647,9 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
 //       update the next diagonal block first and two go on with (1) for it,
 //       so the pivot chain runs beside the updates.
 // What bounds it is that chain (one dependent rsqrt, multiply, shuffle per
-// column, about 110 cycles) and one SM's FP32 rate. In deviation form (dev,
+// column, about 110 cycles) and one SM's FP32 rate: 38 us at m = 128 and 86 at
+// 220 from cold caches, where a kernel with separate factor, solve and inverse
+// phases took 78 and 376. In deviation form (dev,
 // S = I + E, see above) only the diagonal needs care: it holds the deviation
 // d of the pivot from 1, and y_cc = -f_cc / L_cc is kept apart (ydiag).
 // With `split` the inverse goes out as the two TF32 terms the product kernels
@@ -2057,10 +2053,10 @@ static void chol_launch(int m, const double* S, const double* Bm,
     }
     if (smem)
       k_chol_inv<Tm, dev, true><<<1, chol_threads<Tm>(), bytes, s>>>(
-          m, S, Bm, Q, Bf, Qf, Linv, R, sc, nullptr, lpart, nlpart, refined);
+          m, S, Bm, Q, Linv, R, sc, nullptr, lpart, nlpart, refined);
     else
       k_chol_inv<Tm, dev, false><<<1, chol_threads<Tm>(), 0, s>>>(
-          m, S, Bm, Q, Bf, Qf, Linv, R, sc, reinterpret_cast<Tm*>(gwork), lpart,
+          m, S, Bm, Q, Linv, R, sc, reinterpret_cast<Tm*>(gwork), lpart,
           nlpart, refined);
     TRM_CHECK_LAUNCH();
   }
@@ -2071,13 +2067,6 @@ void chol_inv(int m, const double* S, double* Linv, double* R, IterScalars* sc,
               double* gwork, cudaStream_t s) {
   chol_launch<Tm, false>(m, S, nullptr, nullptr, nullptr, nullptr, Linv, R,
                          sc, gwork, s);
-}
-
-template <typename Tm>
-void chol_inv_dev(int m, const double* S, double* Linv, double* R,
-                  IterScalars* sc, double* gwork, cudaStream_t s) {
-  chol_launch<Tm, true>(m, S, nullptr, nullptr, nullptr, nullptr, Linv, R,
-                        sc, gwork, s);
 }
 
 // k-splits of the line terms: about 64 CTAs when the m x m tiles are few
@@ -2145,10 +2134,6 @@ bool line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
   return false;
 }
 
-template void chol_inv_dev<float>(int, const double*, double*, double*,
-                                  IterScalars*, double*, cudaStream_t);
-template void chol_inv_dev<double>(int, const double*, double*, double*,
-                                   IterScalars*, double*, cudaStream_t);
 template void line_factor<float>(int, const double*, const double*,
                                  const double*, const double*, const double*,
                                  int, const double*, int, const double*,

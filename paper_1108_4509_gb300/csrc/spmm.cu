@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(256)
 // CSR: one row per thread, KC columns at a time, so an entry's column index and
 // value are read once for KC products and KC gathers are in flight together
 // (one column at a time, the row cached in registers: 236 us in FP32 at
-// N = 48^3, 13 entries a row, 128 columns). A row's products are added in the
+// N = 48^3, 13 entries a row, 128 columns; now 127). A row's products are added in the
 // order of its entries.
 template <typename T>
 __host__ __device__ constexpr int csr_cols() { return sizeof(T) == 4 ? 8 : 4; }
