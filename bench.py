@@ -331,7 +331,7 @@ class ClockSampler:
 PROFILE_OF_CLASS = {
     "grad_f32": "k_mul_tc_grad_grid48_m128.md",
     "gram_f32": "k_gram_tc_line_grams_grid48_m128.md",
-    "spmm_df": "k_stencil_df_v4_mp2_grid48_m128.md",
+    "spmm_df": "k_stencil_df_mp2_grid48_m128.md",
     "rotate_df": "k_mul_tc_splitdf_mp2_grid48_m128.md",
     "spmm_f32": "k_stencil_zm_f32_grid48_m128.md",
 }
