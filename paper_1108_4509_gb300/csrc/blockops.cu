@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(512)
     a += b;
     if (do_sqrt) a = sqrt(a);
     if (j < m) out[j] = a;
+    __syncwarp();  // thread 0's fence then orders every lane's sum
   }
   if (!sc) return;
   if (threadIdx.x == 0) {

@@ -1,0 +1,43 @@
+"""Calls at the edges of what they accept, through the C ABI: widths, padded
+columns, long rows, blocks with a wide range of magnitudes."""
+import numpy as np
+import pytest
+
+import trm_inputs as ti
+from oracle import operator as op
+from oracle import trm as otrm
+
+from . import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def trm():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1108_4509_gb300 as mod
+    return mod
+
+
+@pytest.mark.parametrize("m", [1, 31, 32, 33, 65, 257])
+def test_energy_is_the_sum_of_its_columns(trm, m):
+    """E is added up by the CTA of the column sums that finishes last, from
+    what the others stored: the H_D of the same call, to the rounding of m
+    additions, in each of several calls with other blocks."""
+    shape = (9, 8, 7)
+    V = ti.gaussian_wells(shape, 4, seed=2)
+    N = V.size
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_stencil(*shape, 4, 1.0, V, m, 1e-10, opt)
+    try:
+        for seed in range(4):
+            C = otrm.orthonormalize(ti.random_block(N, m, seed)) * (seed + 1)
+            cd, g = gu.to_dev(C), gu.empty(N, m, np.float64)
+            hd = gu.to_dev(np.zeros(m))
+            E = trm.trm_energy_gradient(h, cd.data_ptr(), hd.data_ptr(), 0,
+                                        g.data_ptr(), trm.TRM_F64, True)
+            HD = gu.from_dev(hd)
+            assert abs(E - HD.sum()) <= m * 2.3e-16 * np.abs(HD).sum()
+    finally:
+        trm.trm_destroy(h)
