@@ -1876,13 +1876,25 @@ static int chol_blocked_from() {
 // two to a diagonal near 1), X, two temporaries, Phi, three deviations
 static size_t refine_elems(int m) { return (size_t)5 * m * m + 3; }
 
-// elements of the padded working copy plus the inverse's temporary (one
-// CTA; FP64: or of refine_elems), or of W, L, X, T and the failure flag
-// (blocked)
+// Does the FP64 factorisation of this size correct an FP32 one (chol_refined)?
+// m <= 32 has one panel and gains little (45 us instead of 60): left out.
+constexpr int kRefineFrom = 33;
+static bool panel_fits(int m);
+static bool refines(int m) {
+  return m >= kRefineFrom && m < chol_blocked_from() && panel_fits(m);
+}
+
+// The largest of what the kernels that may factor this size keep: the padded
+// working copy plus the inverse's temporary (one CTA); W, L, X, T and the
+// failure flag (blocked: FP64 from chol_blocked_from() on, FP32 above kPanelMax
+// too); refine_elems.
 size_t chol_work_elems(int m) {
   const size_t mp = (size_t)((m + 31) & ~31);
-  if (m >= chol_blocked_from() || m >= kPanelMax) return 4 * mp * mp + 8;
-  return std::max(mp * (mp + 1) + 33 * mp, refine_elems(m));
+  size_t n = mp * (mp + 1) + 33 * mp;
+  if (m >= chol_blocked_from() || m > kPanelMax)
+    n = std::max(n, 4 * mp * mp + 8);
+  if (refines(m)) n = std::max(n, refine_elems(m));
+  return n;
 }
 
 template <typename Tm, bool dev>
@@ -1966,9 +1978,6 @@ static bool panel_fits(int m) {
 // nothing is written and k_chol_inv, launched behind it, does its work; it
 // returns at once where the result stands. 67 us instead of 166 at m = 64, 101
 // instead of 485 at 128; a matrix that is handed on loses 60 and 100 us.
-// m <= 32 has one panel and gains little (45 us instead of 60): left out.
-constexpr int kRefineFrom = 33;
-
 static const unsigned long long* chol_refined(int m, const double* S,
                                               const double* Bm, const double* Q,
                                               double* Linv, double* R,
@@ -2029,7 +2038,7 @@ static void chol_launch(int m, const double* S, const double* Bm,
       return;
     }
     const unsigned long long* refined = nullptr;
-    if (!dev && m >= kRefineFrom && panel_fits(m)) {
+    if (!dev && refines(m)) {
       if (lpart) {
         k_cb_alpha<<<1, 256, 0, s>>>(m, lpart, nlpart, sc);
         TRM_CHECK_LAUNCH();

@@ -1,5 +1,9 @@
 """Calls at the edges of what they accept, through the C ABI: widths, padded
 columns, long rows, blocks with a wide range of magnitudes."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -41,3 +45,32 @@ def test_energy_is_the_sum_of_its_columns(trm, m):
             assert abs(E - HD.sum()) <= m * 2.3e-16 * np.abs(HD).sum()
     finally:
         trm.trm_destroy(h)
+
+
+_FACTOR_256 = """
+import numpy as np
+import trm_inputs as ti
+from oracle import trm as otrm
+from tests import gpu_util as gu
+import paper_1108_4509_gb300 as trm
+N, m = 900, 256
+C = ti.random_block(N, m, 7)
+t = gu.to_dev(C)
+trm.trm_orthonormalize(N, m, t.data_ptr(), gu.stream())
+got = gu.from_dev(t)
+tol = 20 * m * 2.3e-16 * np.linalg.cond(C) ** 2
+assert np.max(np.abs(got.T @ got - np.eye(m))) < tol
+assert np.max(np.abs(got - otrm.orthonormalize(C))) < tol
+"""
+
+
+def test_factor_of_256_columns_on_one_cta(trm):
+    """m = 256 with the line to the blocked launches moved above it: the
+    corrected factor at its largest, in a process of its own (the line is read
+    once). Rounding: m eps times the overlap's condition (about 11 for this
+    shape), a factor of 20 above."""
+    env = dict(os.environ, TRM_CHOL_BLOCKED_FROM="300")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FACTOR_256], cwd=root, env=env,
+                       capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
