@@ -626,11 +626,11 @@ __global__ void k_random(int64_t N, int64_t total, int64_t ld, uint64_t seed,
   }
 }
 
-template <typename T>
-__global__ void k_copy_columns(int64_t N, const T* __restrict__ src,
-                               int64_t lds, T* __restrict__ dst, int64_t ldd) {
-  const T* a = src + (int64_t)blockIdx.y * lds;
-  T* b = dst + (int64_t)blockIdx.y * ldd;
+__global__ void k_copy_columns(int64_t N, const double* __restrict__ src,
+                               int64_t lds, double* __restrict__ dst,
+                               int64_t ldd) {
+  const double* a = src + (int64_t)blockIdx.y * lds;
+  double* b = dst + (int64_t)blockIdx.y * ldd;
 #pragma unroll 4
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -846,17 +846,11 @@ void fix_signs(int64_t N, int m, double* C, double* X, double* work,
   TRM_CHECK_LAUNCH();
 }
 
-template <typename T>
-void copy_columns(int64_t N, int m, const T* src, int64_t lds, T* dst,
+void copy_columns(int64_t N, int m, const double* src, int64_t lds, double* dst,
                   int64_t ldd, cudaStream_t s) {
-  k_copy_columns<T><<<dim3(elem_grid_x(N), m), 256, 0, s>>>(N, src, lds, dst,
-                                                            ldd);
+  k_copy_columns<<<dim3(elem_grid_x(N), m), 256, 0, s>>>(N, src, lds, dst, ldd);
   TRM_CHECK_LAUNCH();
 }
-template void copy_columns<float>(int64_t, int, const float*, int64_t, float*,
-                                  int64_t, cudaStream_t);
-template void copy_columns<double>(int64_t, int, const double*, int64_t,
-                                   double*, int64_t, cudaStream_t);
 
 void clear_pad_rows(const PadList& l, int64_t N, int64_t ld, int m,
                     cudaStream_t s) {

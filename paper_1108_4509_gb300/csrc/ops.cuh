@@ -338,8 +338,7 @@ void fix_signs(int64_t N, int m, double* C, double* X, double* work,
 void to_f32(const double* x, float* y, int64_t n, cudaStream_t s);
 void to_f64(const float* x, double* y, int64_t n, cudaStream_t s);
 // N x m entries between blocks whose columns are lds and ldd entries apart
-template <typename T>
-void copy_columns(int64_t N, int m, const T* src, int64_t lds, T* dst,
+void copy_columns(int64_t N, int m, const double* src, int64_t lds, double* dst,
                   int64_t ldd, cudaStream_t s);
 // Blocks whose rows N .. ld - 1 clear_pad_rows sets to zero (element sizes 4
 // and 8; null pointers are skipped).

@@ -1536,51 +1536,40 @@ void Solver::apply(int din, const void* in, int dout, void* out, int ncols) {
   TRM_CUDA(cudaStreamSynchronize(s_));
 }
 
-void Solver::energy_gradient(const double* C_dev, double* E, double* HD,
-                             double* Hprime, void* G_dev, int G_dtype,
+// On the caller's columns, N apart: no padding row is read, so nothing that an
+// earlier call left in one (a block that overflowed leaves NaN) reaches the
+// result. The scratch blocks then hold entries where their padding lies.
+void Solver::energy_gradient(const double* C, double* E, double* HD,
+                             double* Hprime, void* G, int G_dtype,
                              int zdiag) {
-  // padded columns: C from a copy, G through a scratch block
-  const double* C = C_dev;
-  void* G = G_dev;
-  if (ld_ != N_) {
-    copy_in(C_dev, C64n_, cudaMemcpyDeviceToDevice);
-    C = C64n_;
-    G = HPb_;
-    pad_es_ = 0;
-  }
-  apply_h(op_, C, X64_, m_, s_);
-  energy_diag<double>(ld_, m_, C, X64_, HD_, sc_, part_, s_);
+  if (G_dtype != TRM_F32 && G_dtype != TRM_F64)
+    throw Error(-1, "energy_gradient: G_dtype must be TRM_F32 or TRM_F64");
+  Operator op = op_;
+  op.ld = N_;
+  pad_es_ = 0;
+  apply_h(op, C, X64_, m_, s_);
+  energy_diag<double>(N_, m_, C, X64_, HD_, sc_, part_, s_);
   set_restart();
   GramOut also;
   also.zero_diag = zdiag != 0;
   if (G_dtype == TRM_F64) {
-    xprime<double>(ld_, m_, C, X64_, HD_, nullptr, nullptr, s_);
+    xprime<double>(N_, m_, C, X64_, HD_, nullptr, nullptr, s_);
     Blocks<double> b;
     b.p[0] = X64_;
     b.cols = m_;
     b.count = 1;
-    gram<double>(ld_, m_, C, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
-    gradient<double>(ld_, m_, C, X64_, Hp_, static_cast<double*>(G), nullptr,
+    gram<double>(N_, m_, C, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
+    gradient<double>(N_, m_, C, X64_, Hp_, static_cast<double*>(G), nullptr,
                      nullptr, nullptr, sc_, part_, part_cap_, s_);
-  } else if (G_dtype == TRM_F32) {
-    xprime<double>(ld_, m_, C, X64_, HD_, C32_, X32_, s_, false);
+  } else {
+    xprime<double>(N_, m_, C, X64_, HD_, C32_, X32_, s_, false);
     Blocks<float> b;
     b.p[0] = X32_;
     b.cols = m_;
     b.count = 1;
-    gram<float>(ld_, m_, C32_, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
-    gradient<float>(ld_, m_, C32_, X32_, Hp_, static_cast<float*>(G), nullptr,
+    gram<float>(N_, m_, C32_, b, Hp_, part_, part_cap_, s_, &sc_->status, also);
+    gradient<float>(N_, m_, C32_, X32_, Hp_, static_cast<float*>(G), nullptr,
                     nullptr, nullptr, sc_, part_, part_cap_, s_, &tw_);
-  } else {
-    throw Error(-1, "energy_gradient: G_dtype must be TRM_F32 or TRM_F64");
-  }
-  if (G != G_dev) {
-    if (G_dtype == TRM_F64)
-      copy_columns(N_, m_, static_cast<const double*>(G), ld_,
-                   static_cast<double*>(G_dev), N_, s_);
-    else
-      copy_columns(N_, m_, static_cast<const float*>(G), ld_,
-                   static_cast<float*>(G_dev), N_, s_);
   }
   if (HD)
     TRM_CUDA(cudaMemcpyAsync(HD, HD_, m_ * 8, cudaMemcpyDeviceToDevice, s_));

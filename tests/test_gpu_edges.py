@@ -74,3 +74,55 @@ def test_factor_of_256_columns_on_one_cta(trm):
     r = subprocess.run([sys.executable, "-c", _FACTOR_256], cwd=root, env=env,
                        capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("how", ["gradient", "gradient32", "iterate"])
+@pytest.mark.parametrize("csr", [0, 1])
+@pytest.mark.parametrize("shape,m", [((13, 11, 9), 40), ((7, 5, 3), 6),
+                                     ((9, 21, 1), 20)])
+def test_energy_gradient_after_an_overflow(trm, shape, m, csr, how):
+    """A block that overflows leaves no trace on a handle with padded columns
+    (N % 4 != 0): the next trm_energy_gradient gives E, H_D, H' and G of a
+    fresh handle, byte for byte, in either type of G."""
+    V = ti.gaussian_wells(shape, 4, seed=2)
+    N = V.size
+    assert N % 4
+    opt = trm.trm_default_options(stream=gu.stream(), precond=1)
+
+    def make():
+        if csr:
+            return trm.trm_create_csr(N, *ti.grid_csr(shape, 4, 1.0, V), m, 1e-10,
+                                      opt)
+        return trm.trm_create_stencil(*shape, 4, 1.0, V, m, 1e-10, opt)
+
+    def energy_gradient(h, block, dt):
+        g = gu.empty(N, m, [np.float32, np.float64][dt == trm.TRM_F64])
+        hd, hp = gu.to_dev(np.zeros(m)), gu.empty(m, m, np.float64)
+        E = trm.trm_energy_gradient(h, block.data_ptr(), hd.data_ptr(),
+                                    hp.data_ptr(), g.data_ptr(), dt, True)
+        return E, gu.from_dev(hd), gu.from_dev(hp), gu.from_dev(g)
+
+    good = gu.to_dev(otrm.orthonormalize(ti.random_block(N, m, 3)))
+    big = gu.to_dev(np.full((N, m), 1e200) * (1 + ti.random_block(N, m, 1)))
+    types = (trm.TRM_F64, trm.TRM_F32)
+    h = make()
+    ref = [energy_gradient(h, good, dt) for dt in types]
+    trm.trm_destroy(h)
+    assert all(np.all(np.isfinite(x)) for r in ref for x in r)
+    h = make()
+    try:
+        for k, dt in enumerate(types):
+            if how == "iterate":
+                trm.trm_set_block(h, big.data_ptr())
+                try:
+                    trm.trm_iterate(h, trm.TRM_FP64)
+                except trm.TrmError:
+                    pass
+            else:
+                energy_gradient(h, big, trm.TRM_F64 if how == "gradient"
+                                else trm.TRM_F32)
+            got = energy_gradient(h, good, dt)
+            for a, b in zip(got, ref[k]):
+                assert np.array_equal(a, b)
+    finally:
+        trm.trm_destroy(h)
