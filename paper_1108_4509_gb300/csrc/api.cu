@@ -494,7 +494,11 @@ trm_status trm_extrapolate(int64_t N, int m, const double* C_prev,
     trm::polar_factor(m, M, U, pwork, info + 1, info, s);
     TRM_CUDA(cudaMemcpyAsync(flags, info, 2 * sizeof(int),
                              cudaMemcpyDeviceToHost, s));
+    TRM_CUDA(cudaMemcpyAsync(&status, &sc->status, sizeof(int),
+                             cudaMemcpyDeviceToHost, s));
     TRM_CUDA(cudaStreamSynchronize(s));
+    if (status & 2)
+      return fail(nullptr, TRM_ETIMEOUT, "trm_extrapolate: a device wait timed out");
     if (flags[1] & 1)
       return fail(nullptr, TRM_ENOTPD,
                   "C_prev^T C_cur is singular: the subspaces are too far "

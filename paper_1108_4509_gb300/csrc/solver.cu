@@ -19,10 +19,11 @@ namespace trm {
 namespace {
 
 constexpr int kRing = Solver::kRingSize;
+constexpr int kTimedOut = 2;  // IterScalars::status: a bounded wait gave up
 
-__global__ void k_set_restart(IterScalars* sc) {
+__global__ void k_set_restart(IterScalars* sc, int keep) {
   sc->restart = 1;
-  sc->status = 0;
+  sc->status &= keep;
 }
 
 double neumaier_sum(const double* x, int n) {
@@ -543,7 +544,12 @@ static void spmm_cost(const Operator& op, int ncols, int es, double* fl,
   } while (0)
 
 void Solver::set_restart() {
-  k_set_restart<<<1, 1, 0, s_>>>(sc_);
+  k_set_restart<<<1, 1, 0, s_>>>(sc_, kTimedOut);
+  TRM_CHECK_LAUNCH();
+}
+
+void Solver::begin_call() {
+  k_set_restart<<<1, 1, 0, s_>>>(sc_, 0);
   TRM_CHECK_LAUNCH();
 }
 
@@ -1203,6 +1209,7 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
   const long long launches0 = thread_launch_count();
   const size_t nm = (size_t)ld_ * m_;
   history_.clear();
+  begin_call();
   clear_padding(8);
   clear_padding(4);
   if (C0_host)
@@ -1326,7 +1333,7 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
                    std::to_string(i);
       break;
     }
-    if (v.status & 2) {  // a bounded device wait gave up
+    if (v.status & kTimedOut) {
       status = TRM_ETIMEOUT;
       last_error = "a tensor-core pipeline wait timed out";
       break;
@@ -1454,7 +1461,13 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
   if (C_out)
     copy_out(Cfin, C_out,
              C_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost);
-  TRM_CUDA(cudaStreamSynchronize(s_));
+  IterScalars v;
+  read_scalars(&v);
+  if (v.status & kTimedOut) {  // in the closing step, or in an iteration
+    converged = false;         // after the last one the host read
+    status = TRM_ETIMEOUT;
+    last_error = "a tensor-core pipeline wait timed out";
+  }
   if (lambda) std::memcpy(lambda, lam.data(), m_ * 8);
   if (E_G) *E_G = neumaier_sum(lam.data(), m_);
   if (stats) {
@@ -1549,7 +1562,7 @@ void Solver::energy_gradient(const double* C, double* E, double* HD,
   pad_es_ = 0;
   apply_h(op, C, X64_, m_, s_);
   energy_diag<double>(N_, m_, C, X64_, HD_, sc_, part_, s_);
-  set_restart();
+  begin_call();
   GramOut also;
   also.zero_diag = zdiag != 0;
   if (G_dtype == TRM_F64) {
@@ -1578,14 +1591,14 @@ void Solver::energy_gradient(const double* C, double* E, double* HD,
                              cudaMemcpyDeviceToDevice, s_));
   IterScalars v;
   read_scalars(&v);
-  if (v.status & 2) throw Error(-6, "a bounded device wait gave up");
+  if (v.status & kTimedOut) throw Error(-6, "a bounded device wait gave up");
   if (E) *E = v.E;
 }
 
 void Solver::set_block(const double* C_dev) {
   copy_in(C_dev, C64_, cudaMemcpyDeviceToDevice);
   cg_fresh_ = true;
-  set_restart();
+  begin_call();
   TRM_CUDA(cudaStreamSynchronize(s_));
 }
 
@@ -1600,7 +1613,7 @@ void Solver::iterate(int mode, int restart, double* E, double* rms,
   // a new CG sequence reads no value of G_prev or P (gamma = 0), whatever
   // they hold: the flag is set here, last before the iteration
   const bool fresh = restart || cg_fresh_;
-  if (fresh) set_restart();
+  if (fresh) begin_call();
   cg_fresh_ = false;
   const int es = mode == TRM_FP64 ? 8 : 4;
   if (fresh || pad_es_ != es) clear_padding(es);
@@ -1634,7 +1647,7 @@ void Solver::iterate(int mode, int restart, double* E, double* rms,
   if (E) *E = v.E;
   if (rms) *rms = v.rms;
   if (alpha) *alpha = v.alpha;
-  if (v.status & 2) throw Error(-6, "a bounded device wait gave up");
+  if (v.status & kTimedOut) throw Error(-6, "a bounded device wait gave up");
   if (v.status & 1) throw Error(-3, "overlap matrix not positive definite");
 }
 
@@ -1642,6 +1655,7 @@ void Solver::rayleigh_ritz(double* C_dev, double* lambda_host,
                            double* res_host) {
   double* Xfin = static_cast<double*>(Gb_[0]);
   double* C = C_dev;
+  begin_call();
   if (ld_ != N_) {
     clear_padding(8);
     C = static_cast<double*>(Pb_);  // (a new CG sequence follows)
@@ -1655,10 +1669,11 @@ void Solver::rayleigh_ritz(double* C_dev, double* lambda_host,
   if (res_host)
     TRM_CUDA(cudaMemcpyAsync(res_host, res_, m_ * 8, cudaMemcpyDeviceToHost,
                              s_));
-  TRM_CUDA(cudaStreamSynchronize(s_));
   cg_fresh_ = true;  // final_rr used G as scratch
   pad_es_ = 0;
-  set_restart();
+  IterScalars v;
+  read_scalars(&v);
+  if (v.status & kTimedOut) throw Error(-6, "a bounded device wait gave up");
 }
 
 template void Solver::orth_uniform<float>(float*&, float*&);

@@ -164,6 +164,10 @@ class Solver {
   void rr_rotate_fp64();  // C64 <- C64 Z diagonalising C^T H C
   // Final FP64 Rayleigh-Ritz on C64: writes lam_dev, res_dev, Cfin (=C64b)
   void final_rr(double* C, double* Cfin, double* Xfin);
+  // begin_call: at the start of a call, clears sc_->status. set_restart: a new
+  // CG sequence within one; a timeout stays in the word until the host, which
+  // reads it once more before the call returns, has seen it.
+  void begin_call();
   void set_restart();
   void read_scalars(IterScalars* out);
 
