@@ -1498,12 +1498,16 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
 // ---------------------------------------------------------------------------
 static void copy_cols(const double* src, int64_t lds, double* dst, int64_t ldd,
                       int64_t N, int m, cudaMemcpyKind kind, cudaStream_t s) {
+  constexpr int64_t kMaxPitch = INT32_MAX;  // bytes, of a 2-D copy
   if (lds == ldd)
     TRM_CUDA(cudaMemcpyAsync(dst, src, (size_t)N * m * 8, kind, s));
   else if (kind == cudaMemcpyDeviceToDevice)
     copy_columns(N, m, src, lds, dst, ldd, s);
-  else
+  else if (std::max(lds, ldd) * 8 <= kMaxPitch)
     TRM_CUDA(cudaMemcpy2DAsync(dst, ldd * 8, src, lds * 8, N * 8, m, kind, s));
+  else
+    for (int j = 0; j < m; ++j)
+      TRM_CUDA(cudaMemcpyAsync(dst + j * ldd, src + j * lds, N * 8, kind, s));
 }
 void Solver::copy_in(const double* src, double* dst, cudaMemcpyKind kind) {
   copy_cols(src, N_, dst, ld_, N_, m_, kind, s_);

@@ -145,7 +145,28 @@ static int timeouts() {
   return bad;
 }
 
+// A block from and to the host whose columns are 2^31 bytes and more apart
+// (N % 4 != 0: the solver's own are padded).
+static int large_columns() {
+  const int64_t N = ((int64_t)1 << 28) + 1;
+  trm::Solver s(N, 2, 1e-10, options(TRM_FP64));
+  s.init_stencil((int)N, 1, 1, 2, 1.0, nullptr);
+  g_copies1d = 0;
+  double lam[2], eg, C[2];  // (the fake moves nothing of this size)
+  const int st = s.solve(lam, &eg, C, 0, C, nullptr);
+  std::printf("large columns: %d, %d copies, %d refused\n", st, g_copies1d,
+              g_bad_pitch);
+  return st != TRM_OK || g_copies1d != 4 || g_bad_pitch != 0;
+}
+
 int main(int argc, char** argv) {
-  if (argc < 2 || std::strcmp(argv[1], "timeouts") == 0) return timeouts() != 0;
+  const char* what = argc > 1 ? argv[1] : "";
+  try {
+    if (!std::strcmp(what, "timeouts")) return timeouts() != 0;
+    if (!std::strcmp(what, "large_columns")) return large_columns();
+  } catch (const std::exception& e) {
+    std::printf("%s: %s\n", what, e.what());
+    return 1;
+  }
   return 2;
 }

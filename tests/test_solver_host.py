@@ -62,3 +62,9 @@ def test_every_timeout_reaches_the_caller(harness):
     a phase change, an iteration, the closing step) the solve returns
     TRM_ETIMEOUT, trm_rayleigh_ritz likewise, and the next call starts clean."""
     _run(harness, "timeouts")
+
+
+def test_host_blocks_with_columns_over_2_gb(harness):
+    """trm_solve's C0 and C on the host, N % 4 != 0, N >= 2^28: the columns go
+    one by one where a 2-D copy's pitch would not be accepted."""
+    _run(harness, "large_columns")
