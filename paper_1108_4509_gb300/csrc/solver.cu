@@ -1393,7 +1393,10 @@ int Solver::solve(double* lambda, double* E_G, double* C_out, int C_on_device,
         rr_rotate_fp64();
         // the generalized problem goes on in FP64 (its double-float MP2
         // would need Y and S C as FP32 pairs)
-        if (!has_S_) c64_to_df();
+        if (has_S_)
+          clear_padding(8);  // (G, P and HP held FP32 blocks until here)
+        else
+          c64_to_df();
         set_restart();
         phase = has_S_ ? PH_FP64 : PH_MP2;
         best = INFINITY;

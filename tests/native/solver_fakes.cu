@@ -6,13 +6,14 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <map>
+#include <vector>
 
 #include "solver.cuh"
 
 namespace {
 int g_grams = 0, g_fail_at = 0;     // digit Grams run, and which one times out
 int g_copies1d = 0, g_bad_pitch = 0;
+int g_clear_es = 0, g_dirty = 0;    // what G, P and HP were last cleared for
 constexpr size_t kLarge = (size_t)64 << 20;  // larger requests move nothing
 }  // namespace
 
@@ -21,6 +22,18 @@ bool oz_pays(int64_t, int, int) { return true; }
 void oz_gram(const OzBlock*, int, const OzBlock&, double*, double*, size_t,
              int* err, cudaStream_t) {
   if (++g_grams == g_fail_at) *err |= 2;
+}
+// (the list of a clear has the FP64 blocks, then G, G_prev, P and HP)
+void clear_pad_rows(const PadList& l, int64_t, int64_t, int, cudaStream_t) {
+  int fp64 = 0;
+  while (fp64 < l.n && l.es[fp64] == 8) ++fp64;
+  g_clear_es = fp64 >= 7 ? 8 : 4;
+}
+// the FP64 iteration's first use of H P over the padded rows
+int column_dots(int64_t, int, const double*, const double*, double*,
+                cudaStream_t) {
+  g_dirty += g_clear_es != 8;
+  return 0;
 }
 }  // namespace trm
 
@@ -159,11 +172,31 @@ static int large_columns() {
   return st != TRM_OK || g_copies1d != 4 || g_bad_pitch != 0;
 }
 
+// The generalized mixed ladder on padded columns: full SP with FP32 blocks in
+// G, P and HP, then FP64 ones in the same places.
+static int generalized_padding() {
+  const int n = 5, N = n * n * n;
+  std::vector<int> rp(N + 1), ci(N);
+  std::vector<double> v(N, 1.0);
+  for (int i = 0; i < N; ++i) {
+    ci[i] = i;
+    rp[i + 1] = i + 1;
+  }
+  trm::Solver s(N, 8, 1e-10, options(TRM_MIXED));
+  s.init_stencil(n, n, n, 2, 1.0, nullptr);
+  s.init_overlap(rp.data(), ci.data(), v.data());
+  const int st = solve_status(s, 0);
+  std::printf("generalized: %d, %d digit Grams, %d on uncleared padding\n", st,
+              g_grams, g_dirty);
+  return st != TRM_OK || g_grams < 6 || g_dirty != 0;
+}
+
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
   try {
     if (!std::strcmp(what, "timeouts")) return timeouts() != 0;
     if (!std::strcmp(what, "large_columns")) return large_columns();
+    if (!std::strcmp(what, "generalized")) return generalized_padding();
   } catch (const std::exception& e) {
     std::printf("%s: %s\n", what, e.what());
     return 1;

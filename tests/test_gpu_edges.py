@@ -126,3 +126,33 @@ def test_energy_gradient_after_an_overflow(trm, shape, m, csr, how):
                 assert np.array_equal(a, b)
     finally:
         trm.trm_destroy(h)
+
+
+def test_generalized_mixed_solve_on_padded_columns(trm):
+    """The mixed ladder of the generalized problem on a grid with N % 4 != 0:
+    the dense eigenvalues, an S-orthonormal block, and the same bytes from a
+    second solve on the handle."""
+    import scipy.linalg as sla
+    import scipy.sparse as sp
+    shape, m = (9, 11, 7), 10
+    V = ti.gaussian_wells(shape, 4, seed=2)
+    N = V.size
+    assert N % 4
+    H = op.grid_hamiltonian(shape, 4, 1.0, V)
+    rp, ci, v = ti.hat_overlap_csr(shape)
+    S = sp.csr_matrix((v, ci, rp), shape=(N, N))
+    w = sla.eigh(H.toarray(), S.toarray(), eigvals_only=True)[:m]
+    opt = trm.trm_default_options(stream=gu.stream(), precision=trm.TRM_MIXED,
+                                  seed=3)
+    h = trm.trm_create_stencil(*shape, 4, 1.0, V, m, 1e-10, opt)
+    try:
+        trm.trm_set_overlap_csr(h, rp, ci, v)
+        C, D = np.zeros((N, m), order="F"), np.zeros((N, m), order="F")
+        lam, _, st, status = trm.trm_solve(h, N, m, C_out=C)
+        lam2, _, _, status2 = trm.trm_solve(h, N, m, C_out=D)
+        assert status == 0 and status2 == 0 and st.iterations_phase[0] > 0
+        assert np.array_equal(lam, lam2) and np.array_equal(C, D)
+        assert np.max(np.abs(lam - w)) < 1e-9
+        assert np.max(np.abs(C.T @ (S @ C) - np.eye(m))) < 1e-10
+    finally:
+        trm.trm_destroy(h)

@@ -68,3 +68,9 @@ def test_host_blocks_with_columns_over_2_gb(harness):
     """trm_solve's C0 and C on the host, N % 4 != 0, N >= 2^28: the columns go
     one by one where a 2-D copy's pitch would not be accepted."""
     _run(harness, "large_columns")
+
+
+def test_padding_cleared_where_the_generalized_ladder_turns_to_fp64(harness):
+    """Full SP leaves FP32 entries where FP64 blocks have their padding rows:
+    they are cleared before the first FP64 iteration."""
+    _run(harness, "generalized")
