@@ -418,7 +418,10 @@ trm_status trm_orthonormalize(int64_t N, int m, double* C, void* stream) {
       trm::oz_slice(N, m, C, N, z.block[0], s);
       trm::oz_gram(&z.block[0], 1, z.block[0], S, part, cap, &sc->status, s);
       trm::chol_inv<double>(m, S, Linv, R, sc, gw, s);
-      trm::oz_mult(z.block[0], m, R, true, z.small, C, N, &sc->status, s);
+      // (digits hold less of an entry far below its column's largest than FP64
+      // does: a C that cannot be factored stays as it is)
+      trm::oz_mult(z.block[0], m, R, true, z.small, C, N, &sc->status, s,
+                   &sc->status);
     } else {
       double* Cn = w.take<double>((size_t)N * m);
       trm::Blocks<double> b;

@@ -208,9 +208,12 @@ void oz_slice(int64_t N, int m, const double* C, int64_t ldc, OzBlock& out,
 // after the other; partials as gram's; err receives bit 2 on a timeout
 void oz_gram(const OzBlock* a, int segs, const OzBlock& b, double* out,
              double* partials, size_t cap, int* err, cudaStream_t s);
-// Y = A M (M: a.m x n FP64, upper triangular if tri; columns of Y ldy apart)
+// Y = A M (M: a.m x n FP64, upper triangular if tri; columns of Y ldy apart).
+// halt (device, may be null): Y is left alone when the factorisation before it
+// set bit 1 there.
 void oz_mult(const OzBlock& a, int n, const double* M, bool tri,
-             const OzSmall& w, double* Y, int64_t ldy, int* err, cudaStream_t s);
+             const OzSmall& w, double* Y, int64_t ldy, int* err, cudaStream_t s,
+             const int* halt = nullptr);
 // CTAs of a product: oz_grad writes four sums each
 int oz_product_parts(int64_t N, int n);
 // G = -2 (X' - A H') and the Polak-Ribiere sums, from which the CG scalars in

@@ -245,6 +245,8 @@ struct OzArgs {
   const double* pprev;
   const double* minv;
   int* err;
+  const int* halt;         // product (may be null): nothing is written when
+                           // bit 1 of *halt is set
 };
 
 // BF16 instruction descriptor, FP32 accumulation; a_mn: A is MN-major.
@@ -293,6 +295,7 @@ __global__ void __launch_bounds__(OTHREADS, 1)
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr bool gram = MODE == kOzGram;
+  if (MODE == kOzStore && args.halt && (*args.halt & 1)) return;
   // Jobs: Gram, one (split, tile); products, tiles blockIdx.x, + gridDim.x, ...
   // with the column tile fastest (the tiles of a row tile share A in L2).
   const int njobs = gram ? 1 : args.tiles_m * args.tiles_n;
@@ -690,8 +693,9 @@ int oz_product_parts(int64_t N, int n) {
 
 void oz_mult(const OzBlock& a, int n, const double* M, bool tri,
              const OzSmall& w, double* Y, int64_t ldy, int* err,
-             cudaStream_t s) {
+             cudaStream_t s, const int* halt) {
   OzArgs g{};
+  g.halt = halt;
   g.out = Y;
   g.ldo = ldy;
   g.tri = tri ? 1 : 0;

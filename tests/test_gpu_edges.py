@@ -156,3 +156,17 @@ def test_generalized_mixed_solve_on_padded_columns(trm):
         assert np.max(np.abs(C.T @ (S @ C) - np.eye(m))) < 1e-10
     finally:
         trm.trm_destroy(h)
+
+
+@pytest.mark.parametrize("N,m", [(400, 12), (8192, 64)])
+def test_block_that_cannot_be_factored_stays(trm, N, m):
+    """trm_orthonormalize of a singular block returns TRM_ENOTPD and leaves the
+    block as it was, the entries far below their column's largest too, on the
+    FP64 products (the smaller size) and on the digits."""
+    C = ti.random_block(N, m, seed=3) * 10.0 ** -np.linspace(0, 40, N)[:, None]
+    C[:, m // 2] = 2.0 * C[:, 1]
+    cd = gu.to_dev(C)
+    with pytest.raises(trm.TrmError) as e:
+        trm.trm_orthonormalize(N, m, cd.data_ptr(), gu.stream())
+    assert e.value.status == -3
+    assert np.array_equal(gu.from_dev(cd), C)
