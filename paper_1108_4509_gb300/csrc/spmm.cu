@@ -843,6 +843,9 @@ int choose_kernel(const Operator& op, const float* X, float* Y, int ncols,
 template <typename T, bool DOTS>
 int launch_apply(const Operator& op, const T* X, T* Y, int ncols, double* dots,
                  cudaStream_t s) {
+  // one limit for every operator and type, whatever a kernel's own would be
+  if (ceil_div(ncols, kCpb) > 65535)
+    throw Error(-1, "too many columns for one launch");
   if constexpr (sizeof(T) == 4) {
     if (op.kind == 0 && op.st.nx % 4 != 0)
       return launch_zm_r<DOTS>(op, X, Y, ncols, dots, s);
@@ -870,7 +873,6 @@ int launch_vec(const Operator& op, const T* X, T* Y, int ncols, double* dots,
                cudaStream_t s) {
   const int threads = 256;
   const int gy = ceil_div(ncols, kCpb);
-  if (gy > 65535) throw Error(-1, "too many columns for one launch");
   dim3 grid;
   if (op.kind == 0) {
     const StencilOp& st = op.st;
@@ -892,9 +894,7 @@ int launch_vec(const Operator& op, const T* X, T* Y, int ncols, double* dots,
             st, op.N, op.ld, op.diag64, op.diag32, X, Y, ncols, dots);
     }
   } else {
-    const int gc = ceil_div(ncols, csr_cols<T>());
-    if (gc > 65535) throw Error(-1, "too many columns for one launch");
-    grid = dim3(ceil_div(op.N, threads), gc);
+    grid = dim3(ceil_div(op.N, threads), ceil_div(ncols, csr_cols<T>()));
     // FP32 blocks take the FP32 roundings of the values when the operator
     // holds them (the same products, no conversion per nonzero)
     if (op.csr.vals64 && (sizeof(T) == 8 || !op.csr.vals32))

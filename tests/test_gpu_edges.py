@@ -170,3 +170,32 @@ def test_block_that_cannot_be_factored_stays(trm, N, m):
         trm.trm_orthonormalize(N, m, cd.data_ptr(), gu.stream())
     assert e.value.status == -3
     assert np.array_equal(gu.from_dev(cd), C)
+
+
+@pytest.mark.parametrize("csr", [0, 1])
+@pytest.mark.parametrize("nx", [4, 5])
+def test_most_columns_of_an_application(trm, nx, csr):
+    """trm_apply_h takes 4 * 65535 columns and refuses one more, for every
+    operator and type."""
+    import torch
+    V = np.arange(1.0, nx + 1)
+    opt = trm.trm_default_options(stream=gu.stream())
+    if csr:
+        h = trm.trm_create_csr(nx, *ti.grid_csr((nx, 1, 1), 2, 1.0, V), 1, 1e-10,
+                               opt)
+    else:
+        h = trm.trm_create_stencil(nx, 1, 1, 2, 1.0, V, 1, 1e-10, opt)
+    H = torch.tensor(op.grid_hamiltonian((nx, 1, 1), 2, 1.0, V).toarray()).cuda()
+    most = 4 * 65535
+    try:
+        for dt, td in ((trm.TRM_F32, torch.float32), (trm.TRM_F64, torch.float64)):
+            X = torch.ones(most + 1, nx, dtype=td, device="cuda")
+            Y = torch.zeros_like(X)
+            trm.trm_apply_h(h, dt, X.data_ptr(), dt, Y.data_ptr(), most)
+            want = (X.double() @ H)[:most]
+            assert float((Y[:most].double() - want).abs().max()) < 1e-5
+            with pytest.raises(trm.TrmError) as e:
+                trm.trm_apply_h(h, dt, X.data_ptr(), dt, Y.data_ptr(), most + 1)
+            assert e.value.status == -1
+    finally:
+        trm.trm_destroy(h)
