@@ -296,6 +296,7 @@ __global__ void __launch_bounds__(256)
     for (int q = 0; q < kCols; ++q) {
       const F2 t = prod_df(v, F2{__ldg(ph[q] + j), __ldg(pl[q] + j)});
       acc_add(acc[q], t.h, t.l);
+      acc[q] = quick_two_sum(acc[q].h, acc[q].l);
     }
   }
   F2 d[kCols];

@@ -199,3 +199,31 @@ def test_most_columns_of_an_application(trm, nx, csr):
             assert e.value.status == -1
     finally:
         trm.trm_destroy(h)
+
+
+def test_mp2_energy_of_a_matrix_with_long_rows(trm):
+    """1500 equal entries a row: the double-float sum of a row is renormalised
+    at every entry, so that its low part rounds against what one addition
+    leaves and not against what all before it have. Per entry at most 2^-46.6
+    of the partial sum (two low parts added, then added to the sum's), half
+    the final one on average, and 2^-47 of the product: n 2^-46.6 of the sum.
+    With one renormalisation at the end the errors add up in step here, and
+    the energy was 7.6e-11 off."""
+    n, m, v = 1500, 2, 0.7
+    N = n * m
+    rp = (np.arange(N + 1) * n).astype(np.int32)
+    first = (np.arange(N) // n * n)[:, None]
+    cols = (first + np.arange(n)[None, :]).astype(np.int32).reshape(-1)
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_csr(N, rp, cols, np.full(N * n, v), m, 1e-10, opt)
+    try:
+        C = np.zeros((N, m), order="F")
+        for j in range(m):
+            C[j * n:(j + 1) * n, j] = 1.0 / np.sqrt(n)
+        cd = gu.to_dev(C)
+        trm.trm_set_block(h, cd.data_ptr())
+        E, _, _ = trm.trm_iterate(h, trm.TRM_MP2)
+    finally:
+        trm.trm_destroy(h)
+    want = m * n * n * v / n
+    assert abs(E - want) <= n * 2.0 ** -46.6 * want
