@@ -317,7 +317,9 @@ bool gram(int64_t N, int m, const T* A, const Blocks<T>& B, double* out,
   const int n = B.total();
   if (m <= 0 || n <= 0) return false;
   if constexpr (sizeof(T) == 4) {
-    if (gram_tc_eligible(N, m, A, B)) {  // tensor cores, FP32-class accuracy
+    // tensor cores, FP32-class accuracy
+    if (gram_tc_eligible(N, m, A, B) &&
+        (!also.fine || gram_tc_fine_pays(N, m))) {
       gram_tc(N, m, A, B, out, partials, partials_cap, err, s, also);
       return true;
     }

@@ -8,7 +8,7 @@
 // the product to 2e-8 of sum |a||b|, with lo from rna_tf32(x) instead to
 // 1e-5), so hi = trunc_tf32(x) is the TMA-loaded tile itself and only lo is
 // formed (lo = rna_tf32(x - hi), |lo| < 2^-10 |x|, rounding error < 2^-21
-// |x|). The three products hi.hi + hi.lo + lo.hi are accumulated in FP32 in
+// |x|). The three products lo.hi + hi.lo + hi.hi are accumulated in FP32 in
 // tensor memory; the dropped lo.lo and the rounding of lo are below 2^-19 of
 // |a b|: FP32-class accuracy. A TMA box of 32 rows x 128 columns of a
 // column-major FP32 block, loaded with the 128-byte swizzle, is already the
@@ -28,8 +28,22 @@
 // is bounded by KC * 12 steps of 2^-23 of the chunk sums. Row slices of at
 // most kSingleChunk stages (512 rows) are one chunk and fold nothing: at 96
 // stages (all of the 48^3 case) that bias was the largest error of a step
-// (2e-5 of the step length; the MP2 block after two steps 4.6e-11 off, with
-// chunks 1.4e-11) for 1 % less time.
+// (2e-5 of the step length). Within a stage the small products come first, so
+// that at its end only hi.hi has been added to a sum of full size.
+//
+// Fine sums (GramOut::fine) are for blocks that FP32 multiply-adds served
+// until their columns were padded (grids with N % 4 != 0), and are no further
+// off than those: every stage is folded, so a sum is truncated four times in
+// 32 rows, and lo.lo, which has the sign of the product on both truncated
+// operands, is formed too. MP2 blocks after two steps against 64 bits:
+//                                  39x41x37,90  13x11x9,40  31x33x35,50
+//   FP32 multiply-adds              1.7e-12      4.4e-13     1.1e-12
+//   chunks as above, large first    1.7e-11      2.5e-11     2.5e-11
+//   fine                            1.4e-12      4.4e-13     1.1e-12
+// Folding a stage takes longer than its MMAs, so short slices serve these
+// best: from two stages on (16 stages: 40 us more an iteration of a small
+// problem). An FP32 iteration at 37^3, 90 columns: 341 us, 282 with chunks, 816
+// with multiply-adds; at 25^3, 48: 148, 152, 237.
 //
 // Warp roles (576 threads): warp 0 issues the TMA loads (one box of A and one
 // of B per 32-row stage into a ring of raw stages, each freed when the MMAs
@@ -75,6 +89,11 @@ constexpr int OSTAGES = TRM_GRAM_OSTAGES;  // lo stages
 constexpr int THREADS = 576;  // 18 warps
 constexpr int KC = 8;         // stages per accumulation chunk (default)
 constexpr int kSingleChunk = 16;  // row slices this short are one chunk
+constexpr int kFineStages = 2;    // the shortest row slices of fine sums
+// From this N m^2 on fine sums run faster here than with FP32 multiply-adds
+// (an FP32 iteration, here and there: 13^3, 33 columns 112 and 111 us; 13^3, 48:
+// 116 and 117; 17^3, 33: 118 and 128; 13^3, 90: 160 and 176).
+constexpr double kFineFrom = 4e6;
 // Row slices of at least this many stages: a small problem takes fewer CTAs
 // (each holds a whole SM) and leaves the rest of the GPU to concurrent solves.
 constexpr int kMinStages = 16;
@@ -142,6 +161,8 @@ struct TcArgs {
   int stack;
   int64_t rows_per_split;  // kRows: of each of the two slices
   int kc;                 // stages per accumulation chunk of long slices
+  int single;             // slices of at most this many stages are one chunk
+  int lolo;               // form lo lo too
   int seg_cols;           // columns per segment
   int tps;                // column tiles per segment (the last one ragged:
                           // its columns past seg_cols load as zeros)
@@ -234,7 +255,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       bool ok = true;
-      const int kcl = nk <= kSingleChunk ? nk : args.kc;  // stages per chunk
+      const int kcl = nk <= args.single ? nk : args.kc;  // stages per chunk
+      const int p0 = args.lolo ? 0 : 1;  // the first product
       for (int k = 0; k < nk && ok; ++k) {
         const int s = k % OSTAGES, r = k % RSTAGES;
         const int kc = k % kcl, c = k / kcl, b = c & 1;
@@ -255,14 +277,16 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint32_t bH = smem_u32(sm->raw[r][1]);
         const uint32_t aL = smem_u32(sm->op[s][0]);
         const uint32_t bL = smem_u32(sm->op[s][1]);
-        const uint32_t pa[3] = {aH, aH, aL};
-        const uint32_t pb[3] = {bH, bL, bH};
+        // (small products first: a large sum is truncated only by hi hi)
+        const uint32_t pa[4] = {aL, aL, aH, aH};
+        const uint32_t pb[4] = {bL, bH, bL, bH};
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
+        for (int p = 0; p < 4; ++p) {
+          if (p < p0) continue;
 #pragma unroll
           for (int kk = 0; kk < BK / 8; ++kk)  // K = 8 per TF32 MMA (32 bytes)
             mma_tf32(d, kdesc(pa[p] + kk * 32), kdesc(pb[p] + kk * 32),
-                     kIdesc, (kc > 0 || p > 0 || kk > 0) ? 1u : 0u);
+                     kIdesc, (kc > 0 || p > p0 || kk > 0) ? 1u : 0u);
         }
         mma_commit(&sm->opfree[s]);   // lo and the raw stage reusable
         mma_commit(&sm->rawfree[r]);  // once these MMAs are done
@@ -296,7 +320,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int q = warp & 3;            // TMEM lane quarter of this warp
     const int g = (warp - 10) >> 2;    // column half of the tile
     const uint32_t lrow = (uint32_t)(32 * q) << 16;
-    const int kcl = nk <= kSingleChunk ? nk : args.kc;
+    const int kcl = nk <= args.single ? nk : args.kc;
     const int nch = nk > 0 ? (nk + kcl - 1) / kcl : 0;
     // where this thread's row and columns 64 g .. +63 of the tile go: row `row`
     // and columns col0 .. col0 + ncol - 1 (tile columns from cb0) of partial
@@ -415,14 +439,19 @@ bool gram_tc_pairs_eligible(int64_t N, int m, const Blocks<float>& A,
   return tc::encode_fn() != nullptr;
 }
 
+bool gram_tc_fine_pays(int64_t N, int m) {
+  return (double)N * m * m >= kFineFrom;
+}
+
 // Row slices for a launch of `tiles` output tiles: among the counts that
-// keep at least kMinStages stages per slice, launch at most 8 waves of CTAs
+// keep at least min_stages stages per slice, launch at most 8 waves of CTAs
 // and stay within max_splits, the one whose CTAs fill the SMs most evenly,
 // less 1 % per extra wave (each wave refills the pipelines). Every CTA of a
 // launch does the same work, so with one slice per tile a launch of 164
 // tiles would run a second wave of 12 CTAs as long as the first.
-static int tc_splits(int64_t N, int tiles, int max_splits, int sms) {
-  const int64_t by_rows = ceil_div(N, (int64_t)BK * kMinStages);
+static int tc_splits(int64_t N, int tiles, int max_splits, int sms,
+                     int min_stages = kMinStages) {
+  const int64_t by_rows = ceil_div(N, (int64_t)BK * min_stages);
   const int smax = (int)std::max<int64_t>(
       1, std::min<int64_t>({by_rows, (int64_t)8 * sms / tiles,
                             (int64_t)max_splits}));
@@ -455,34 +484,35 @@ static int tc_splits(int64_t N, int tiles, int max_splits, int sms) {
 // fixed per process and repeated solves agree bit for bit.
 struct SliceKey {
   int64_t N;
-  int m, n, tiles, sym;
+  int m, n, tiles, sym, fine;
   bool operator<(const SliceKey& o) const {
-    return std::tie(N, m, n, tiles, sym) <
-           std::tie(o.N, o.m, o.n, o.tiles, o.sym);
+    return std::tie(N, m, n, tiles, sym, fine) <
+           std::tie(o.N, o.m, o.n, o.tiles, o.sym, o.fine);
   }
 };
 std::mutex g_slice_mu;
 std::map<SliceKey, int> g_slices;
 
 template <typename Run>
-int tuned_splits(int64_t N, int m, int n, int tiles, int sym, int smax,
-                 cudaStream_t s, Run& run) {
+int tuned_splits(int64_t N, int m, int n, int tiles, int sym, int fine,
+                 int smax, cudaStream_t s, Run& run) {
   const int sms = sm_count();
-  const int base = tc_splits(N, tiles, smax, sms);
+  const int min_stages = fine ? kFineStages : kMinStages;
+  const int base = tc_splits(N, tiles, smax, sms, min_stages);
   // TRM_GRAM_SLICES=formula (or a count) fixes the slices instead (for
   // profilers, whose serialised replay would distort the timing)
   if (const char* f = std::getenv("TRM_GRAM_SLICES")) {
     const int v = std::atoi(f);
     return v > 0 ? std::min(v, smax) : base;
   }
-  const SliceKey key{N, m, n, tiles, sym};
+  const SliceKey key{N, m, n, tiles, sym, fine};
   {
     std::lock_guard<std::mutex> lock(g_slice_mu);
     auto it = g_slices.find(key);
     if (it != g_slices.end()) return std::min(it->second, smax);
   }
   const int most = (int)std::max<int64_t>(
-      1, std::min<int64_t>(smax, ceil_div(N, (int64_t)BK * kMinStages)));
+      1, std::min<int64_t>(smax, ceil_div(N, (int64_t)BK * min_stages)));
   int cand[2], nc = 0;
   for (int c : {base, base / 2}) {
     c = std::max(1, std::min(c, most));
@@ -599,7 +629,9 @@ void gram_tc_pairs(int64_t N, int m, const Blocks<float>& A,
   a.tps = tps;
   // TRM_GRAM_KC overrides the chunk length (measurements of the
   // accumulation error against the fold's cost)
-  a.kc = KC;
+  a.kc = also.fine ? 1 : KC;
+  a.single = also.fine ? 1 : kSingleChunk;
+  a.lolo = also.fine;
   if (const char* f = std::getenv("TRM_GRAM_KC")) {
     const int v = std::atoi(f);
     if (v >= 1 && v <= kSingleChunk) a.kc = v;
@@ -635,8 +667,8 @@ void gram_tc_pairs(int64_t N, int m, const Blocks<float>& A,
   };
   // (an odd count of kRows slices takes one more partial: even caps)
   if (stack == kRows && smax > 1) smax &= ~1;
-  run(tuned_splits(N, m, n, tiles, stack == kWhole ? sym_seg : -1 - stack, smax,
-                   s, run));
+  run(tuned_splits(N, m, n, tiles, stack == kWhole ? sym_seg : -1 - stack,
+                   also.fine, smax, s, run));
 }
 
 }  // namespace trm

@@ -5,9 +5,15 @@
 //
 // Precision: as in the Gram kernel, each FP32 value of Y is split in shared
 // memory into two TF32 terms (hi = rna_tf32(y), lo = rna_tf32(y - hi)), M is
-// split the same way from FP64 by k_split_small, and hi.hi + hi.lo + lo.hi is
-// accumulated in FP32 in tensor memory (FP32-class accuracy, ~2^-22 relative
-// per term).
+// split the same way from FP64 by k_split_small, and lo.hi + hi.lo + hi.hi is
+// accumulated in FP32 in tensor memory (~2^-22 relative per term). Each MMA
+// truncates its sum, so a product on top of a large sum costs a fraction of
+// its last place. The two small products therefore have an accumulator of
+// their own, which the epilogue adds, rounded once, and only the hi.hi of
+// every eight k are truncated against the result (the split update, where the
+// product is a small correction, keeps one accumulator, small products first).
+// With one accumulator, large products first: an FP32 step at 13 x 11 x 9,
+// m = 40 was 4.2e-7 off, an FMA chain's is 2.2e-7.
 //
 // Layout: Y is column-major (rows contiguous), so a TMA box of 32 rows x 32
 // columns with the 128-byte swizzle holds 32 lines of 32 rows each (the
@@ -19,7 +25,7 @@
 //
 // Rings: staging (TMA -> converters; raw Y and P tiles), operand (converters
 // and TMA -> MMA; hi, lo and the M tiles), accumulator (MMA -> epilogue; two
-// 128-column TMEM buffers, so the epilogue of one tile overlaps the next).
+// buffers in TMEM, so the epilogue of one tile overlaps the next).
 // Persistent CTAs (one per SM) walk (128-row, 128-column) tiles. Warp roles
 // (512 threads): warp 0 TMA for Y/P, warp 1 TMEM allocation and MMA issue
 // (one thread), warp 2 TMA for M, warp 3 TMA for the gradient's epilogue
@@ -144,6 +150,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   MulSmem* sm = reinterpret_cast<MulSmem*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr bool kTwoAcc = MODE == kStore || MODE == kGrad;
+  constexpr int kTmem = kTwoAcc ? 4 * NC : 2 * NC;
   const int ntiles = args.ntr * args.nch;
   const int nk = (args.k + BK - 1) / BK;
 
@@ -169,7 +177,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     sm->failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(&sm->tmem_base, 2 * NC);
+  if (warp == 1) tmem_alloc(&sm->tmem_base, kTmem);
   fence_before();
   __syncthreads();
   fence_after();
@@ -298,15 +306,18 @@ __global__ void __launch_bounds__(THREADS, 1)
           fence_after();
           const uint32_t aH = smem_u32(sm->ah[s]), aL = smem_u32(sm->al[s]);
           const uint32_t bH = smem_u32(sm->bh[s]), bL = smem_u32(sm->bl[s]);
-          const uint32_t pa[3] = {aH, aH, aL};
+          const uint32_t pa[3] = {aL, aH, aH};
           const uint32_t pb[3] = {bH, bL, bH};
 #pragma unroll
-          for (int p = 0; p < 3; ++p)
+          for (int p = 0; p < 3; ++p) {
+            const uint32_t dp = kTwoAcc && p < 2 ? d + 2 * NC : d;
 #pragma unroll
             for (int kk = 0; kk < BK / 8; ++kk)  // K = 8 per MMA (32 bytes)
-              mma_tf32(d, smem_desc(pa[p] + kk * 32, 16, 1024),
+              mma_tf32(dp, smem_desc(pa[p] + kk * 32, 16, 1024),
                        smem_desc(pb[p] + kk * 32, 16, 1024), idesc,
-                       (kb > 0 || p > 0 || kk > 0) ? 1u : 0u);
+                       (kb > 0 || kk > 0 || (kTwoAcc ? p == 1 : p > 0)) ? 1u
+                                                                       : 0u);
+          }
           mma_commit(&sm->op_empty[s]);
         }
         if (ok) mma_commit(&sm->accfull[b]);
@@ -402,7 +413,20 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll 1
       for (int cb = cbeg; cb < cend; cb += 16) {
         uint32_t r[16];
-        tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * NC + cb), r);
+        const uint32_t acc =
+            tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * NC + cb);
+        if (kTwoAcc) {
+          uint32_t x[16];
+          tmem_ld16_async(acc, r);
+          tmem_ld16_async(acc + 2 * NC, x);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 16; ++e)
+            r[e] = __float_as_uint(__uint_as_float(r[e]) +
+                                   __uint_as_float(x[e]));
+        } else {
+          tmem_ld16(acc, r);
+        }
         if (MODE == kGrad) {
           // the two slots of these 16 columns: wait, read, release (every
           // thread of the half arrives, rows past N included)
@@ -572,7 +596,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 1) {
     __syncwarp();
     fence_after();
-    tmem_dealloc(tmem, 2 * NC);
+    tmem_dealloc(tmem, kTmem);
   }
 }
 

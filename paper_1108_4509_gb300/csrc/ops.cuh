@@ -113,14 +113,17 @@ size_t gram_partials_doubles(int64_t N, int m, int n);
 // What the split sum of a Gram writes besides its FP64 result: the result
 // rounded to FP32, its two TF32 terms for the product kernels (hi, then lo
 // split_ldm * n floats on; tensor-core Grams only), and whether entries (i, i)
-// are zero instead of the sum.
+// are zero instead of the sum. fine: FP32 sums no further off than those of
+// FP32 multiply-adds (see gram_tc.cu).
 struct GramOut {
   float* f32 = nullptr;
   float* split = nullptr;
   int split_ldm = 0;
   int zero_diag = 0;
+  int fine = 0;
 };
-// FP32 inputs go to the tensor-core kernel when gram_tc_eligible; err (device
+// FP32 inputs go to the tensor-core kernel when gram_tc_eligible (and, for
+// fine sums, gram_tc_fine_pays); err (device
 // int, may be null) receives bit 2 if one of its bounded waits gave up.
 // Returns whether that kernel ran (and GramOut::split was written).
 template <typename T>
@@ -156,6 +159,8 @@ bool gram_tc_eligible(int64_t N, int m, const float* A, const Blocks<float>& B);
 // segments); up to four segments.
 bool gram_tc_pairs_eligible(int64_t N, int m, const Blocks<float>& A,
                             const Blocks<float>& B);
+// Do fine sums of these sizes run faster there than with FP32 multiply-adds?
+bool gram_tc_fine_pays(int64_t N, int m);
 // Doubles of split partials gram_tc / gram_tc_pairs need for an m x n result
 // (skipped_tiles: tiles of a symmetric segment that are mirrored, not run).
 size_t gram_tc_partials_doubles(int64_t N, int m, int n, int skipped_tiles = 0);

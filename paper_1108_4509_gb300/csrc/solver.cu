@@ -254,7 +254,7 @@ size_t Solver::footprint(int64_t n_rows, int m) {
 }
 
 Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
-    : N_(N), ld_(padded(N)), m_(m), tol_(tol), opt_(opt) {
+    : N_(N), ld_(padded(N)), fine_(ld_ != N), m_(m), tol_(tol), opt_(opt) {
   s_ = reinterpret_cast<cudaStream_t>(opt.stream);
   mem_.set_stream(s_);
   const size_t nm = (size_t)ld_ * m;
@@ -327,12 +327,14 @@ Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
   sc_ = static_cast<IterScalars*>(mem_.alloc(sizeof(IterScalars)));
   TRM_CUDA(cudaMemsetAsync(sc_, 0, sizeof(IterScalars), s_));
   op_.err = &sc_->status;
-  tw_.msplit_floats = mul_tc_work_floats(m, m);
-  tw_.msplit = f(tw_.msplit_floats);
   tw_.err = &sc_->status;
-  rw_ = tw_;
-  rw_.msplit = f(rw_.msplit_floats);
-  TRM_CUDA(cudaMemsetAsync(rw_.msplit, 0, rw_.msplit_floats * 4, s_));
+  if (!fine_ || gram_tc_fine_pays(ld_, m)) {  // else no product takes them
+    tw_.msplit_floats = mul_tc_work_floats(m, m);
+    tw_.msplit = f(tw_.msplit_floats);
+    rw_ = tw_;
+    rw_.msplit = f(rw_.msplit_floats);
+    TRM_CUDA(cudaMemsetAsync(rw_.msplit, 0, rw_.msplit_floats * 4, s_));
+  }
   diag64_ = d(N);
   diag32_ = f(N);
   diaglo_ = f(N);
@@ -584,7 +586,8 @@ bool Solver::line_grams_fusable(const T* C, const T* P, const T* G) const {
     b.p[2] = G;
     a.cols = b.cols = m_;
     a.count = b.count = 3;
-    return gram_tc_pairs_eligible(ld_, m_, a, b);
+    return gram_tc_pairs_eligible(ld_, m_, a, b) &&
+           (!fine_ || gram_tc_fine_pays(ld_, m_));
   }
 }
 
@@ -592,6 +595,7 @@ bool Solver::line_grams_fusable(const T* C, const T* P, const T* G) const {
 // line model and, as far as the tensor cores run, the gradient's operand.
 GramOut Solver::hprime_out() const {
   GramOut o;
+  o.fine = fine_;
   o.f32 = Hp32_;
   o.split = tw_.msplit;
   o.split_ldm = mul_tc_ldm(m_);
@@ -611,6 +615,7 @@ void Solver::line_grams_fused(const T* C, const T* P, const T* G) {
     a.count = b.count = 3;
     const double nm = (double)N_ * m_, m2N = nm * m_;
     GramOut also;
+    also.fine = fine_;
     also.f32 = Bm32_;
     // algorithmic: 2 m^2 N per product, m^2 N for the symmetric one
     TRM_PROF(KC_GRAM32, 5 * m2N, 12 * nm,
@@ -684,6 +689,7 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
   GramOut hp_also, bm_also, pg_also;
   if (sizeof(T) == 4) {
     hp_also = hprime_out();
+    bm_also.fine = pg_also.fine = fine_;
     bm_also.f32 = Bm32_;
     pg_also.f32 = PG32_;
   }
@@ -903,6 +909,7 @@ void Solver::iter_mp2() {
     line_grams_fused<float>(Ch, P, G);
   } else {
     GramOut bm_also, pg_also;
+    bm_also.fine = pg_also.fine = fine_;
     bm_also.f32 = Bm32_;
     pg_also.f32 = PG32_;
     TRM_PROF(KC_SPMM32, f32, b32, apply_h(op_, P, HP, m_, s_));
@@ -1042,7 +1049,9 @@ void Solver::orth_uniform(T*& C, T*& Cn) {
       gen = true;
     }
   }
-  gram<T>(ld_, m_, C, b, S_, part_, part_cap_, s_, &sc_->status);
+  GramOut also;
+  also.fine = fine_;
+  gram<T>(ld_, m_, C, b, S_, part_, part_cap_, s_, &sc_->status, also);
   chol_inv<T>(m_, S_, Linv_, R_, sc_, mmw_, s_);
   rotate<T, T>(ld_, m_, C, static_cast<const T*>(nullptr), R_, Cn, nullptr,
                s_, &tw_);

@@ -181,6 +181,9 @@ class Solver {
   void copy_in(const double* src, double* dst, cudaMemcpyKind kind);
   void copy_out(const double* src, double* dst, cudaMemcpyKind kind);
   void clear_padding(int es);
+  // FP32 Grams of padded blocks with sums as exact as FP32 multiply-adds: on
+  // such grids they ran on those before the columns were padded.
+  bool fine_;
   int pad_es_ = 0;  // element size G, P and HP's padding is clear for
   int m_;
   double tol_;

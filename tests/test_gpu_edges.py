@@ -1,5 +1,6 @@
 """Calls at the edges of what they accept, through the C ABI: widths, padded
 columns, long rows, blocks with a wide range of magnitudes."""
+import ctypes as ct
 import os
 import subprocess
 import sys
@@ -227,3 +228,97 @@ def test_mp2_energy_of_a_matrix_with_long_rows(trm):
         trm.trm_destroy(h)
     want = m * n * n * v / n
     assert abs(E - want) <= n * 2.0 ** -46.6 * want
+
+
+class _Blocks(ct.Structure):
+    _fields_ = [("p", ct.c_void_p * 4), ("cols", ct.c_int), ("count", ct.c_int)]
+
+
+class _GramOut(ct.Structure):
+    _fields_ = [("f32", ct.c_void_p), ("split", ct.c_void_p),
+                ("split_ldm", ct.c_int), ("zero_diag", ct.c_int),
+                ("fine", ct.c_int)]
+
+
+@pytest.mark.parametrize("N,m", [(1284, 60), (4096, 32), (36000, 64), (36000, 65),
+                                 (9000, 130), (60000, 200)])
+def test_fine_gram_of_positive_blocks(trm, N, m):
+    """The tensor-core Gram with fine sums, all terms of one sign, where every
+    truncation counts the same way: within a stage of 32 rows the sum is
+    truncated by 2^-23 at a quarter, half, three quarters and the whole of its
+    size (2.5 2^-23), and by the other products at 2^-10 of that. The operands'
+    second terms round at 2^-22 of the value, up and down alike over the rows:
+    half of that bound is more than what is left. (Chunks of eight stages are
+    about 1e-6 off.)"""
+    import torch
+    rng = np.random.default_rng(N + m)
+    A = rng.uniform(0.5, 1.0, (N, m)).astype(np.float32)
+    B = rng.uniform(0.5, 1.0, (N, m)).astype(np.float32)
+    a, b = gu.to_dev(A), gu.to_dev(B)
+    lib = ct.CDLL(trm.LIB_PATH)
+    size = lib._ZN3trm21gram_partials_doublesElii
+    size.restype = ct.c_size_t
+    assert lib._ZN3trm17gram_tc_fine_paysEli(ct.c_int64(N), m) & 1
+    cap = size(ct.c_int64(N), m, m)
+    part = torch.zeros(cap, dtype=torch.float64, device="cuda")
+    out, err = gu.empty(m, m, np.float64), gu.to_dev(np.zeros(4, np.int32))
+    blocks = _Blocks((ct.c_void_p * 4)(b.data_ptr(), None, None, None), m, 1)
+    also = _GramOut(None, None, 0, 0, 1)
+    f = lib._ZN3trm4gramIfEEbliPKT_RKNS_6BlocksIS1_EEPdS8_mP11CUstream_stPiRKNS_7GramOutE
+    f(ct.c_int64(N), m, ct.c_void_p(a.data_ptr()), ct.byref(blocks),
+      ct.c_void_p(out.data_ptr()), ct.c_void_p(part.data_ptr()),
+      ct.c_size_t(cap), ct.c_void_p(gu.stream()), ct.c_void_p(err.data_ptr()),
+      ct.byref(also))
+    G = gu.from_dev(out)
+    assert int(err[0]) == 0
+    want = A.astype(np.float64).T @ B.astype(np.float64)
+    assert np.max(np.abs(G / want - 1.0)) <= 2.5 * 2.0 ** -23 + 2.0 ** -22
+
+
+@pytest.mark.parametrize("shape,m", [((13, 11, 9), 33), ((13, 11, 9), 60),
+                                     ((17, 19, 21), 32), ((21, 23, 25), 40),
+                                     ((31, 33, 35), 70), ((9, 21, 1), 20)])
+def test_mp2_step_on_odd_grids_is_as_exact_as_multiply_adds(trm, shape, m):
+    """N % 4 != 0, close to the solution: the step's own error, relative to
+    the step. Grams and products of FP32 multiply-adds, or as exact: 6e-7 of
+    a Gram at most (the test above) in alpha, one 6e-8 each for G, P and the
+    update, a product's 2^-22: below 1e-6 in all. With the sums that other
+    grids take it was 3e-6 to 8e-6."""
+    order = 4
+    V = ti.gaussian_wells(shape, 4, seed=6)
+    N = V.size
+    assert N % 4
+    H = op.grid_hamiltonian(shape, order, 1.0, V)
+    import scipy.sparse.linalg as spla
+    w, v = (np.linalg.eigh(H.toarray()) if N < 2000 else
+            spla.eigsh(H, k=m, which="SA", tol=1e-12,
+                       v0=np.ones(N), ncv=4 * m))
+    C = np.linalg.qr(v[:, :m] + 5e-6 * np.sqrt(3.0 / N) * 2
+                     * ti.random_block(N, m, 3))[0]
+    X = op.apply_h(H, C)
+    HD = np.sum(C * X, axis=0)
+    Xp = X - C * HD
+    Hp = C.T @ Xp
+    np.fill_diagonal(Hp, 0.0)
+    G = -2.0 * (Xp - C @ Hp)
+    B, Q, W = C.T @ G, G.T @ G, G.T @ G
+    A0 = 0.5 * (Hp + Hp.T) + np.diag(HD)
+    D1 = A0 @ B - B @ A0 - 0.5 * (W + W.T)
+    curve = (np.sum(G * op.apply_h(H, G)) - np.sum(Q * A0)
+             - np.sum((B + B.T) * D1))
+    a = np.trace(W) / (2 * curve)
+    Y = C + a * G
+    want = np.linalg.solve(np.linalg.cholesky(Y.T @ Y), Y.T).T
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_stencil(*shape, order, 1.0, V, m, 1e-10, opt)
+    try:
+        cd = gu.to_dev(C)
+        trm.trm_set_block(h, cd.data_ptr())
+        trm.trm_iterate(h, trm.TRM_MP2, restart=True)
+        out = gu.empty(N, m, np.float64)
+        trm.trm_get_block(h, out.data_ptr())
+        got = gu.from_dev(out)
+    finally:
+        trm.trm_destroy(h)
+    step = np.linalg.norm(a * G)
+    assert np.linalg.norm(got - want) <= 1e-6 * step + 2.0 ** -46 * np.sqrt(m)
