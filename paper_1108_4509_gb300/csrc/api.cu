@@ -474,12 +474,16 @@ trm_status trm_extrapolate(int64_t N, int m, const double* C_prev,
     double* pwork = w.take<double>(pw);
     double* gw = w.take<double>(cw);
     double* Y = w.take<double>(Nm);
-    auto* sc = w.take<trm::IterScalars>(1);
-    int* info = w.take<int>(2);  // [eig sweeps, polar status]
-    int flags[2] = {0, 0};
+    struct Words {  // what the host reads, in one copy
+      trm::IterScalars sc;
+      int info[2];  // [eig sweeps, polar status]
+    };
+    auto* words = w.take<Words>(1);
+    trm::IterScalars* sc = &words->sc;
+    int* info = words->info;
+    Words seen{};
     int status = 0;
-    TRM_CUDA(cudaMemsetAsync(sc, 0, sizeof(trm::IterScalars), s));
-    TRM_CUDA(cudaMemsetAsync(info, 0, 2 * sizeof(int), s));
+    TRM_CUDA(cudaMemsetAsync(words, 0, sizeof(Words), s));
     // align C_prev to C_cur: U = polar(C_prev^T C_cur)
     std::optional<OzScratch> z;
     if (oz) {
@@ -495,14 +499,12 @@ trm_status trm_extrapolate(int64_t N, int m, const double* C_prev,
       trm::gram<double>(N, m, C_prev, b, M, part, cap, s);
     }
     trm::polar_factor(m, M, U, pwork, info + 1, info, s);
-    TRM_CUDA(cudaMemcpyAsync(flags, info, 2 * sizeof(int),
-                             cudaMemcpyDeviceToHost, s));
-    TRM_CUDA(cudaMemcpyAsync(&status, &sc->status, sizeof(int),
+    TRM_CUDA(cudaMemcpyAsync(&seen, words, sizeof(Words),
                              cudaMemcpyDeviceToHost, s));
     TRM_CUDA(cudaStreamSynchronize(s));
-    if (status & 2)
+    if (seen.sc.status & 2)
       return fail(nullptr, TRM_ETIMEOUT, "trm_extrapolate: a device wait timed out");
-    if (flags[1] & 1)
+    if (seen.info[1] & 1)
       return fail(nullptr, TRM_ENOTPD,
                   "C_prev^T C_cur is singular: the subspaces are too far "
                   "apart to align");
