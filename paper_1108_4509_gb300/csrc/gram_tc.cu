@@ -40,10 +40,12 @@
 //   FP32 multiply-adds              1.7e-12      4.4e-13     1.1e-12
 //   chunks as above, large first    1.7e-11      2.5e-11     2.5e-11
 //   fine                            1.4e-12      4.4e-13     1.1e-12
-// Folding a stage takes longer than its MMAs, so short slices serve these
-// best: from two stages on (16 stages: 40 us more an iteration of a small
-// problem). An FP32 iteration at 37^3, 90 columns: 341 us, 282 with chunks, 816
-// with multiply-adds; at 25^3, 48: 148, 152, 237.
+// Folding a stage takes longer than its MMAs, so short slices serve one problem
+// best, long ones many at once (2, 4, 8 and 16 stages at least: an FP32
+// iteration at 13^3, 48 columns 116, 127, 146 and 173 us, a server's 16 mixed
+// requests 357, 353, 337 and 338 ms): four. An FP32 iteration at 37^3, 90
+// columns: 342 us, 282 with chunks, 816 with multiply-adds; at 25^3, 48: 148,
+// 152, 237.
 //
 // Warp roles (576 threads): warp 0 issues the TMA loads (one box of A and one
 // of B per 32-row stage into a ring of raw stages, each freed when the MMAs
@@ -89,11 +91,12 @@ constexpr int OSTAGES = TRM_GRAM_OSTAGES;  // lo stages
 constexpr int THREADS = 576;  // 18 warps
 constexpr int KC = 8;         // stages per accumulation chunk (default)
 constexpr int kSingleChunk = 16;  // row slices this short are one chunk
-constexpr int kFineStages = 2;    // the shortest row slices of fine sums
+constexpr int kFineStages = 4;    // the shortest row slices of fine sums
 // From this N m^2 on fine sums run faster here than with FP32 multiply-adds
-// (an FP32 iteration, here and there: 13^3, 33 columns 112 and 111 us; 13^3, 48:
-// 116 and 117; 17^3, 33: 118 and 128; 13^3, 90: 160 and 176).
-constexpr double kFineFrom = 4e6;
+// (an FP32 iteration, here and there: 13^3, 33 columns 122 and 111 us; 13^3, 48:
+// 127 and 117; 17^3, 33: 125 and 128; 13^3, 90: 169 and 176; 16 mixed requests
+// 354 ms, 381 with the line at 3e7).
+constexpr double kFineFrom = 5e6;
 // Row slices of at least this many stages: a small problem takes fewer CTAs
 // (each holds a whole SM) and leaves the rest of the GPU to concurrent solves.
 constexpr int kMinStages = 16;
