@@ -127,15 +127,15 @@ __global__ void __launch_bounds__(256, 3)
     k_stencil_df(StencilOp st, int64_t ld, const float* __restrict__ dh,
                  const float* __restrict__ dl, const float* __restrict__ Ch,
                  const float* __restrict__ Cl, float* __restrict__ Xh,
-                 float* __restrict__ Xl, int ncols, int zc,
+                 float* __restrict__ Xl, int ncols, int zc, int pack,
                  double* __restrict__ dots) {
   __shared__ double red[8];
   const int nx = st.nx, ny = st.ny, nz = st.nz, nxq = nx / VW;
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;  // group in the plane
-  const bool active = p < nxq * ny;
+  int p, z0;  // group in the plane, first plane
+  const bool active = zm_place(nxq * ny, nz, zc, pack, p, z0);
   const int x0 = active ? VW * (p % nxq) : 0, y = active ? p / nxq : 0;
   const int col = blockIdx.z;
-  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc);
+  const int z1 = min(nz, z0 + zc);
   const int64_t sz = (int64_t)nx * ny;
   const int64_t rowoff = (int64_t)y * nx + x0;
   const float* ch = Ch + (int64_t)col * ld + rowoff;
@@ -409,7 +409,8 @@ int launch_df(const Operator& op, const float* Ch, const float* Cl, float* Xh,
   const ZmShape z =
       zm_shape(st, op.N, ncols, VW, (int)apply_h_dots_doubles(op, 1));
   k_stencil_df<R, VW><<<dim3(z.tiles, z.chunks, ncols), z.threads, 0, s>>>(
-      st, op.ld, op.diag32, op.diaglo, Ch, Cl, Xh, Xl, ncols, z.zc, dots);
+      st, op.ld, op.diag32, op.diaglo, Ch, Cl, Xh, Xl, ncols, z.zc,
+      z.pack, dots);
   TRM_CHECK_LAUNCH();
   return z.tiles * z.chunks;  // partial dots per column
 }

@@ -54,12 +54,27 @@ int apply_h_dots(const Operator& op, const float* X, float* Y, int ncols,
 size_t apply_h_dots_doubles(const Operator& op, int ncols);
 // Geometry of the register z-march stencils: CTAs of `threads` threads over
 // `tiles` parts of a plane (vw points per thread), `chunks` runs of zc planes
-// and the columns; tiles * chunks partial dots per column, at most max_dots
-// where one run of all planes allows.
+// (`pack` of them in a CTA where a plane is small) and the columns; tiles *
+// chunks partial dots per column, at most max_dots where one run of all planes
+// allows.
 struct ZmShape {
-  int tiles, threads, chunks, zc;
+  int tiles, threads, chunks, zc, pack;
 };
 ZmShape zm_shape(const StencilOp& st, int64_t N, int ncols, int vw, int max_dots);
+// The place of this thread in a march: group p of a plane of nq and the first
+// plane of its chunk; whether it has one.
+__device__ __forceinline__ bool zm_place(int nq, int nz, int zc, int pack,
+                                         int& p, int& z0) {
+  if (pack == 1) {
+    p = blockIdx.x * blockDim.x + threadIdx.x;
+    z0 = blockIdx.y * zc;
+    return p < nq;
+  }
+  const int sub = threadIdx.x / nq;
+  p = threadIdx.x - sub * nq;
+  z0 = (blockIdx.y * pack + sub) * zc;
+  return sub < pack && z0 < nz;
+}
 // the axes as the march takes them (a 2-D grid's y in z's place)
 StencilOp zm_axes(const StencilOp& st);
 

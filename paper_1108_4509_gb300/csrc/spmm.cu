@@ -578,14 +578,14 @@ template <int R, bool DOTS, int VW>
 __global__ void __launch_bounds__(256, VW == 1 ? 6 : 4)
     k_stencil_zm(StencilOp st, int64_t ld, const float* __restrict__ d32,
                  const float* __restrict__ X, float* __restrict__ Y,
-                 int ncols, int zc, double* __restrict__ dots) {
+                 int ncols, int zc, int pack, double* __restrict__ dots) {
   __shared__ double red[8];
   const int nx = st.nx, ny = st.ny, nz = st.nz, nxq = nx / VW;
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;  // group in the plane
-  const bool active = p < nxq * ny;
+  int p, z0;  // group in the plane, first plane
+  const bool active = zm_place(nxq * ny, nz, zc, pack, p, z0);
   const int x0 = active ? VW * (p % nxq) : 0, y = active ? p / nxq : 0;
   const int col = blockIdx.z;
-  const int z0 = blockIdx.y * zc, z1 = min(nz, z0 + zc);
+  const int z1 = min(nz, z0 + zc);
   const int64_t sz = (int64_t)nx * ny;
   const int64_t rowoff = (int64_t)y * nx + x0;
   const float* xb = X + (int64_t)col * ld + rowoff;
@@ -671,7 +671,9 @@ __global__ void __launch_bounds__(256, VW == 1 ? 6 : 4)
 // per SM are launched (at least four planes each; half as many leave a last
 // wave, twice as many read more halo planes: 115, 112, 112 us for the
 // double-float kernel at 48^3 x 128 with 2048, 3072 and 4096), and no more
-// partial dots per column than apply_h_dots_doubles allows.
+// partial dots per column than apply_h_dots_doubles allows. A small plane (thin
+// rods, 2-D grids with short rows) that would leave more than an eighth of its
+// warps' lanes idle shares a CTA of 128 threads with other chunks.
 StencilOp zm_axes(const StencilOp& st) {
   StencilOp t = st;
   if (t.nz == 1) std::swap(t.ny, t.nz);
@@ -681,13 +683,16 @@ ZmShape zm_shape(const StencilOp& st, int64_t N, int ncols, int vw, int max_dots
   const int nq = (st.nx / vw) * st.ny;
   ZmShape z{};
   z.tiles = ceil_div(nq, 256);
-  z.threads = 32 * ceil_div(nq, 32 * z.tiles);
-  const int want = ceil_div((int64_t)12 * 256 * sm_count(),
-                            (int64_t)z.threads * z.tiles * ncols);
-  const int cap = std::max(1, max_dots / z.tiles);
+  const int lanes = 32 * ceil_div(nq, 32);
+  z.pack = 8 * (lanes - nq) > lanes ? std::max(1, 128 / nq) : 1;
+  z.threads = 32 * ceil_div(nq * z.pack, 32 * z.tiles);
+  const int per = z.pack > 1 ? nq : z.threads * z.tiles;  // threads of a chunk
+  const int want =
+      ceil_div((int64_t)12 * 256 * sm_count(), (int64_t)per * ncols);
+  const int cap = std::max(1, max_dots / z.tiles) * z.pack;
   const int chunks = std::max(1, std::min({want, ceil_div(st.nz, 4), cap}));
   z.zc = ceil_div(st.nz, chunks);
-  z.chunks = ceil_div(st.nz, z.zc);
+  z.chunks = ceil_div(ceil_div(st.nz, z.zc), z.pack);
   return z;
 }
 
@@ -719,7 +724,7 @@ int launch_zm_v(const Operator& op, const float* X, float* Y, int ncols,
     const int nc = std::min(65535, ncols - c0);
     k_stencil_zm<R, DOTS, VW><<<dim3(z.tiles, z.chunks, nc), z.threads, 0, s>>>(
         st, op.ld, op.diag32, X + c0 * op.ld, Y ? Y + c0 * op.ld : nullptr,
-        ncols, z.zc, DOTS ? dots + c0 : nullptr);
+        ncols, z.zc, z.pack, DOTS ? dots + c0 : nullptr);
     TRM_CHECK_LAUNCH();
   }
   return z.tiles * z.chunks;  // partial dots per column

@@ -240,7 +240,7 @@ class _GramOut(ct.Structure):
                 ("fine", ct.c_int)]
 
 
-@pytest.mark.parametrize("N,m", [(1284, 60), (4096, 32), (36000, 64), (36000, 65),
+@pytest.mark.parametrize("N,m", [(1388, 64), (5000, 32), (36000, 64), (36000, 65),
                                  (9000, 130), (60000, 200)])
 def test_fine_gram_of_positive_blocks(trm, N, m):
     """The tensor-core Gram with fine sums, all terms of one sign, where every
@@ -322,3 +322,33 @@ def test_mp2_step_on_odd_grids_is_as_exact_as_multiply_adds(trm, shape, m):
         trm.trm_destroy(h)
     step = np.linalg.norm(a * G)
     assert np.linalg.norm(got - want) <= 1e-6 * step + 2.0 ** -46 * np.sqrt(m)
+
+
+@pytest.mark.parametrize("order", [2, 4])
+@pytest.mark.parametrize("shape", [(1, 200, 1), (2, 101, 1), (3, 3, 50),
+                                   (5, 5, 33), (4, 4, 40), (7, 300, 1),
+                                   (9, 9, 9), (6, 11, 13), (129, 1, 1),
+                                   (1, 1, 77), (1, 7, 30)])
+def test_marching_stencils_of_thin_grids(trm, shape, order):
+    """Planes of a few points, whose CTAs take several chunks: H C in FP32
+    against the dense operator (13 terms of FP32 rounding) and the MP2 energy,
+    whose H C and column dots are double-float pairs, against FP64."""
+    V = ti.gaussian_wells(shape, 2, seed=2)
+    N, m = V.size, 5
+    H = op.grid_hamiltonian(shape, order, 1.0, V).toarray()
+    C = otrm.orthonormalize(ti.random_block(N, m, seed=3))
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_stencil(*shape, order, 1.0, V, m, 1e-10, opt)
+    try:
+        x32 = gu.to_dev(C, np.float32)
+        y = gu.empty(N, m, np.float32)
+        trm.trm_apply_h(h, trm.TRM_F32, x32.data_ptr(), trm.TRM_F32,
+                        y.data_ptr(), m)
+        mag = np.abs(H) @ np.abs(C)
+        assert np.all(np.abs(gu.from_dev(y) - H @ C) <= 16 * 2.0 ** -24 * mag)
+        cd = gu.to_dev(C)
+        trm.trm_set_block(h, cd.data_ptr())
+        E, _, _ = trm.trm_iterate(h, trm.TRM_MP2)
+        assert abs(E - np.sum(C * (H @ C))) <= 2.0 ** -44 * np.sum(np.abs(C) * mag)
+    finally:
+        trm.trm_destroy(h)

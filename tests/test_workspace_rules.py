@@ -1,5 +1,6 @@
 """CPU checks that the sizes of workspaces follow the rules that choose the
 kernels which use them."""
+import ctypes as ct
 import os
 import subprocess
 import sys
@@ -50,3 +51,52 @@ def test_factorisation_workspace(blocked_from):
         if m > 256:
             need = max(need, (4 * mp * mp + 1) // 2 + 1)
         assert have[m - 1] >= need, m
+
+
+class _Stencil(ct.Structure):
+    _fields_ = [("nx", ct.c_int), ("ny", ct.c_int), ("nz", ct.c_int),
+                ("radius", ct.c_int), ("c1", ct.c_double), ("c2", ct.c_double),
+                ("c1h", ct.c_float), ("c1l", ct.c_float), ("c2h", ct.c_float),
+                ("c2l", ct.c_float)]
+
+
+class _March(ct.Structure):
+    _fields_ = [("tiles", ct.c_int), ("threads", ct.c_int), ("chunks", ct.c_int),
+                ("zc", ct.c_int), ("pack", ct.c_int)]
+
+
+def test_march_takes_every_point_once():
+    """The geometry of the marching stencils (trm::zm_shape) and the place of a
+    thread in it (zm_place, written out here): every group of every plane once,
+    no more partial dots than the buffer holds, CTAs of at most 256 threads."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1108_4509_gb300 as trm
+    shape = ct.CDLL(trm.LIB_PATH)._ZN3trm8zm_shapeERKNS_9StencilOpEliii
+    shape.restype = _March
+    edges = [1, 2, 3, 5, 8, 9, 16, 33, 129]
+    for nx in edges:
+        for ny in edges:
+            for nz in [1, 2, 5, 31, 70]:
+                vw = 4 if nx % 4 == 0 else 2 if nx % 2 == 0 else 1
+                N = nx * ny * nz
+                dots = -(-(N // 4 if nx % 4 == 0 else N) // 256)
+                for ncols in (1, 48):
+                    z = shape(ct.byref(_Stencil(nx, ny, nz, 2)), ct.c_int64(N),
+                              ncols, vw, dots)
+                    nq = nx // vw * ny
+                    assert z.threads % 32 == 0 and z.threads <= 256
+                    assert z.tiles * z.chunks <= max(dots, z.tiles)
+                    seen = []
+                    for by in range(z.chunks):
+                        for t in range(z.tiles * z.threads):
+                            if z.pack == 1:
+                                p, z0, on = t, by * z.zc, t < nq
+                            else:
+                                sub = t // nq
+                                p, z0 = t - sub * nq, (by * z.pack + sub) * z.zc
+                                on = sub < z.pack and z0 < nz
+                            if on:
+                                seen += [p * nz + k for k in
+                                         range(z0, min(nz, z0 + z.zc))]
+                    assert sorted(seen) == list(range(nq * nz)), (nx, ny, nz)
