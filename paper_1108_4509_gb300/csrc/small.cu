@@ -33,10 +33,13 @@ namespace {
 constexpr double kNsDone = 1e-10;
 
 // Acceptance of chol_refined's result: max |X S X^T - I| after one correction
-// (another then leaves m 1e-20), max |X - I| after both
+// (another then leaves m 1e-20), max |X - I| after both, and no kernel before
+// them that saw the attempt to be in vain (dev[kRefStop]).
+enum { kRefDev1 = 1, kRefDev2 = 2, kRefStop = 3, kRefWords = 4 };
 __device__ __forceinline__ bool refined_ok(const unsigned long long* dev) {
-  return __longlong_as_double((long long)dev[1]) < 1e-10 &&
-         __longlong_as_double((long long)dev[2]) < 0.5;
+  return dev[kRefStop] == 0ull &&
+         __longlong_as_double((long long)dev[kRefDev1]) < 1e-10 &&
+         __longlong_as_double((long long)dev[kRefDev2]) < 0.5;
 }
 
 // tri: which operands are lower triangular (the products then leave out what
@@ -47,6 +50,7 @@ enum { kTriA = 1, kTriB = 2, kTriBt = 4, kTriOut = 8, kPhi = 16 };
 struct GemmOpt {
   const double* cin = nullptr;
   const unsigned long long* skip = nullptr;
+  const unsigned long long* stop = nullptr;  // not null: nothing when not 0
   unsigned long long* dev = nullptr;
   int tri = 0;
 };
@@ -71,6 +75,7 @@ __global__ void __launch_bounds__(256)
     if (in && ks == 0 && opt.cin) Cm[e] = opt.cin[e];
     return;
   }
+  if (opt.stop && *opt.stop) return;
   if ((opt.tri & kTriOut) && j0 > i0) return;
   int kb = 0, ke = m;  // the sum's range
   if (opt.tri & kTriA) ke = min(ke, i0 + TT);
@@ -871,6 +876,11 @@ struct PanelOut {
   float* split = nullptr;  // TF32 hi and lo of L^{-T}
   int ldm = 0;
   int split_diag = 0;      // leave the diagonal out, written as pairs
+  // chol_refined: where any of nhopeless words is set, or max |Linv - I| is
+  // 1/2 or more, *stop becomes 1 and Linv is of no use; else *stop is 0
+  const int* hopeless = nullptr;
+  int nhopeless = 0;
+  unsigned long long* stop = nullptr;
 };
 
 template <bool dev>
@@ -890,6 +900,13 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
   float* lcol = Z + 32 * ldz;   // 32 x 32, and a line read past its end
   float* rd = lcol + 33 * 32;
   auto blk = [&](int i, int j) { return M + (panel_blocks(i) + j) * PSZ; };
+  if (!dev && out.stop) {
+    const bool any = tid < out.nhopeless && out.hopeless[tid];
+    if (__syncthreads_or(any)) {
+      if (tid == 0) *out.stop = 1ull;
+      return;
+    }
+  }
   if (tid == 0) bad = 0;
   // S (or S(a) from B and Q) into the blocks, minus I in deviation form; the
   // padding is the identity. A unit is eight columns of a block, read along
@@ -1168,12 +1185,19 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
                          : k > i ? 0.0
                                  : (dev ? 1.0 : 0.0) + (double)dfull(i);
   }
+  float far = 0.f;  // max |Linv - I|
   if (out.Linv)
     for (int k = warp; k < m; k += nw)
-      for (int i = lane; i < m; i += 32)
-        out.Linv[i + k * m] = i > k ? to_f64(entry(k, i))
-                            : i < k ? 0.0
-                                    : (dev ? 1.0 : 0.0) + (double)dfull(i);
+      for (int i = lane; i < m; i += 32) {
+        const float x = i > k ? entry(k, i) : i == k ? dfull(i) : 0.f;
+        far = fmaxf(far, fabsf(!dev && i == k ? x - 1.f : x));
+        out.Linv[i + k * m] =
+            i == k ? (dev ? 1.0 : 0.0) + (double)x : to_f64(x);
+      }
+  if (!dev && out.stop) {
+    const bool in_vain = __syncthreads_or(isbad || !(far < 0.5f));
+    if (tid == 0) *out.stop = in_vain ? 1ull : 0ull;
+  }
   if (tid == 0 && isbad && sc) sc->status |= 1;
 }
 
@@ -1205,24 +1229,35 @@ __device__ __forceinline__ double half_exp_scale(double x) {
 }
 
 // S' = D S D (D from S's diagonal; the lower triangle of S, mirrored), or S(a)
-// = I + a (B + B^T) + a^2 (Q + Q^T) / 2. Clears the three deviations.
+// = I + a (B + B^T) + a^2 (Q + Q^T) / 2. Clears the deviations. hopeless[CTA]:
+// does it hold two columns with a cosine above 1/2? Their own entry of L^{-1}
+// (c / sqrt(1 - c^2) for unit columns) is then about what refined_ok refuses,
+// and the attempt ends here.
 __global__ void __launch_bounds__(256)
     k_ref_form(int m, const double* __restrict__ S,
                const double* __restrict__ Bm, const double* __restrict__ Q,
                const IterScalars* __restrict__ sc, double* __restrict__ Sp,
-               unsigned long long* dev) {
+               unsigned long long* dev, int* hopeless) {
   const int e = blockIdx.x * 256 + threadIdx.x;
-  if (e < 3) dev[e] = 0ull;
-  if (e >= m * m) return;
-  const int i = max(e % m, e / m), k = min(e % m, e / m);
-  if (Bm) {
-    const double al = sc->alpha;
-    Sp[e] = al * (Bm[i + k * m] + Bm[k + i * m]) +
-            0.5 * al * al * (Q[i + k * m] + Q[k + i * m]) + (i == k ? 1.0 : 0.0);
-  } else {
-    Sp[e] = S[i + k * m] * half_exp_scale(S[i + i * m]) *
-            half_exp_scale(S[k + k * m]);
+  if (e < kRefStop) dev[e] = 0ull;
+  bool far = false;
+  if (e < m * m) {
+    const int i = max(e % m, e / m), k = min(e % m, e / m);
+    double v;
+    if (Bm) {
+      const double al = sc->alpha;
+      v = al * (Bm[i + k * m] + Bm[k + i * m]) +
+          0.5 * al * al * (Q[i + k * m] + Q[k + i * m]) + (i == k ? 1.0 : 0.0);
+    } else {
+      const double sii = S[i + i * m], skk = S[k + k * m];
+      const double di = half_exp_scale(sii), dk = half_exp_scale(skk);
+      v = S[i + k * m] * di * dk;
+      far = i != k && 4.0 * v * v > (sii * di * di) * (skk * dk * dk);
+    }
+    Sp[e] = v;
   }
+  const int any = __syncthreads_or(far);
+  if (threadIdx.x == 0) hopeless[blockIdx.x] = any;
 }
 
 // L^{-1} = X D and its transpose, where the corrections converged
@@ -1873,8 +1908,12 @@ static int chol_blocked_from() {
 }
 
 // FP64 factor and inverse by correcting FP32 ones: S' (S scaled by powers of
-// two to a diagonal near 1), X, two temporaries, Phi, three deviations
-static size_t refine_elems(int m) { return (size_t)5 * m * m + 3; }
+// two to a diagonal near 1), X, two temporaries, Phi, the words of refined_ok,
+// k_ref_form's flags (two to a double)
+static int ref_ctas(int m) { return ceil_div((int64_t)m * m, 256); }
+static size_t refine_elems(int m) {
+  return (size_t)5 * m * m + kRefWords + (ref_ctas(m) + 1) / 2;
+}
 
 // Does the FP64 factorisation of this size correct an FP32 one (chol_refined)?
 // m <= 32 has one panel and gains little (45 us instead of 60): left out.
@@ -1977,7 +2016,11 @@ static bool panel_fits(int m) {
 // condition 1.5; m = 48, condition 10: 2.8e-16 against 6.0e-16). Otherwise
 // nothing is written and k_chol_inv, launched behind it, does its work; it
 // returns at once where the result stands. 67 us instead of 166 at m = 64, 101
-// instead of 485 at 128; a matrix that is handed on loses 60 and 100 us.
+// instead of 485 at 128. A matrix that is handed on loses what the attempt took:
+// 60 and 100 us when it ran to its end, so two tests end it earlier, for
+// columns at small angles before it begins (their entry alone is too large) and
+// for a large FP32 X before the products; the launches behind them then return
+// at once.
 static const unsigned long long* chol_refined(int m, const double* S,
                                               const double* Bm, const double* Q,
                                               double* Linv, double* R,
@@ -1990,14 +2033,19 @@ static const unsigned long long* chol_refined(int m, const double* S,
   double* T = Xn + mm;
   double* Phi = T + mm;
   auto* dev = reinterpret_cast<unsigned long long*>(Phi + mm);
-  const int blocks = ceil_div((int64_t)mm, 256);
-  k_ref_form<<<blocks, 256, 0, s>>>(m, S, Bm, Q, sc, Sp, dev);
+  auto* hopeless = reinterpret_cast<int*>(dev + kRefWords);
+  const int blocks = ref_ctas(m);
+  k_ref_form<<<blocks, 256, 0, s>>>(m, S, Bm, Q, sc, Sp, dev, hopeless);
   TRM_CHECK_LAUNCH();
   PanelOut out;
   out.Linv = X;
+  out.hopeless = hopeless;
+  out.nhopeless = blocks;
+  out.stop = dev + kRefStop;
   panel_launch<false>(m, Sp, nullptr, nullptr, out, nullptr, s, nullptr, 0);
   for (int k = 0; k < 2; ++k) {
     GemmOpt a, f, x;
+    a.stop = f.stop = x.stop = dev + kRefStop;
     a.tri = kTriA;
     mm_launch(m, X, false, Sp, false, T, 1.0, 0.0, a, s);  // X S'
     f.tri = kTriBt | kTriOut | kPhi;
@@ -2005,7 +2053,7 @@ static const unsigned long long* chol_refined(int m, const double* S,
     mm_launch(m, T, false, X, true, Phi, 1.0, 0.0, f, s);  // X S' X^T
     x.tri = kTriA | kTriB | kTriOut;
     x.cin = X;
-    if (k == 1) x.dev = dev + 2;
+    if (k == 1) x.dev = dev + kRefDev2;
     mm_launch(m, Phi, false, X, false, Xn, -1.0, 1.0, x, s);  // X - Phi X
     std::swap(X, Xn);
   }

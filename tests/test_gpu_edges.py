@@ -352,3 +352,28 @@ def test_marching_stencils_of_thin_grids(trm, shape, order):
         assert abs(E - np.sum(C * (H @ C))) <= 2.0 ** -44 * np.sum(np.abs(C) * mag)
     finally:
         trm.trm_destroy(h)
+
+
+@pytest.mark.parametrize("cond", [15.0, 25.0, 300.0])
+@pytest.mark.parametrize("m", [33, 64, 100, 255])
+def test_fp64_factor_where_the_correction_is_left_early(trm, m, cond):
+    """Overlaps that the corrected FP32 factor refuses, before its products
+    (a large entry of the FP32 inverse) and before it begins (two columns at a
+    small angle), and one near the line: the elimination's result. Rounding: m
+    eps times the condition, a factor of 20 above."""
+    N = 2 * m + 100
+    rng = np.random.default_rng(m)
+    U = np.linalg.qr(rng.standard_normal((N, m)))[0]
+    Q = np.linalg.qr(rng.standard_normal((m, m)))[0]
+    C = (U * np.geomspace(1.0, cond ** 0.5, m)) @ Q
+    near = C.copy()
+    near[:, m - 1] = 0.9 * near[:, 3] + 0.3 * near[:, m - 1]
+    for block in (C, near, C * 2.0 ** np.floor(rng.uniform(-30, 30, m))):
+        ref = otrm.orthonormalize(block)
+        t = gu.to_dev(block)
+        trm.trm_orthonormalize(N, m, t.data_ptr(), gu.stream())
+        got = gu.from_dev(t)
+        unit = block / np.linalg.norm(block, axis=0)
+        tol = 20 * m * 2.3e-16 * np.linalg.cond(unit) ** 2
+        assert np.max(np.abs(got.T @ got - np.eye(m))) < tol
+        assert np.max(np.abs(got - ref)) < tol

@@ -29,7 +29,7 @@ def test_factorisation_workspace(blocked_from):
     workspace, wherever TRM_CHOL_BLOCKED_FROM puts the line to the blocked
     launches: FP64 on one CTA (padded copy and a 33-row temporary) or blocked
     (four padded copies), the corrected FP32 factor for 33 <= m <= 256 (five
-    m x m matrices, three deviations), FP32 above m = 256 blocked (four padded
+    m x m matrices, four words, a flag per 256 entries), FP32 above m = 256 blocked (four padded
     copies, in half as many doubles)."""
     env = dict(os.environ)
     env.pop("TRM_CHOL_BLOCKED_FROM", None)
@@ -47,7 +47,7 @@ def test_factorisation_workspace(blocked_from):
         else:
             need = mp * (mp + 1) + 33 * mp
             if 33 <= m <= 256:
-                need = max(need, 5 * m * m + 3)
+                need = max(need, 5 * m * m + 4 + (-(-m * m // 256) + 1) // 2)
         if m > 256:
             need = max(need, (4 * mp * mp + 1) // 2 + 1)
         assert have[m - 1] >= need, m
