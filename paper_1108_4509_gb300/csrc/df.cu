@@ -10,6 +10,8 @@
 // — far below what E_G at 1e-10 and residuals at 1e-10 need — while every
 // operation runs on the FP32 pipe. No FP64 instruction is executed per
 // element, except once per thread when an FP64 scalar is split.
+#include <type_traits>
+
 #include "dfmath.cuh"
 #include "ops.cuh"
 
@@ -277,7 +279,6 @@ __global__ void __launch_bounds__(256)
   const int64_t r = valid ? r0 : 0;
   const int b = valid ? rowptr[r] : 0, e = valid ? rowptr[r + 1] : 0;
   const int cb = blockIdx.y * kCols, nc = min(kCols, ncols - cb);
-  // (columns past the last read the last one's entries and are not written)
   const float* ph[kCols];
   const float* pl[kCols];
   F2 acc[kCols];
@@ -288,17 +289,24 @@ __global__ void __launch_bounds__(256)
     pl[q] = Cl + o;
     acc[q] = F2{0.f, 0.f};
   }
+  auto row = [&](auto full) {
 #pragma unroll 2
-  for (int k = b; k < e; ++k) {
-    const int j = cols[k];
-    const F2 v = {vh[k], vl[k]};
+    for (int k = b; k < e; ++k) {
+      const int j = cols[k];
+      const F2 v = {vh[k], vl[k]};
 #pragma unroll
-    for (int q = 0; q < kCols; ++q) {
-      const F2 t = prod_df(v, F2{__ldg(ph[q] + j), __ldg(pl[q] + j)});
-      acc_add(acc[q], t.h, t.l);
-      acc[q] = quick_two_sum(acc[q].h, acc[q].l);
+      for (int q = 0; q < kCols; ++q)
+        if (decltype(full)::value || q < nc) {
+          const F2 t = prod_df(v, F2{__ldg(ph[q] + j), __ldg(pl[q] + j)});
+          acc_add(acc[q], t.h, t.l);
+          acc[q] = quick_two_sum(acc[q].h, acc[q].l);
+        }
     }
-  }
+  };
+  if (nc == kCols)
+    row(std::true_type{});
+  else
+    row(std::false_type{});
   F2 d[kCols];
 #pragma unroll
   for (int q = 0; q < kCols; ++q) {

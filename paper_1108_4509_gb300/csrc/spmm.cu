@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdlib>
+#include <type_traits>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -227,8 +228,9 @@ __global__ void __launch_bounds__(256)
 // CSR: one row per thread, KC columns at a time, so an entry's column index and
 // value are read once for KC products and KC gathers are in flight together
 // (one column at a time, the row cached in registers: 236 us in FP32 at
-// N = 48^3, 13 entries a row, 128 columns; now 127). A row's products are added in the
-// order of its entries.
+// N = 48^3, 13 entries a row, 128 columns; now 127). The last columns of a block
+// that is no multiple of KC go without the others' gathers. A row's products are
+// added in the order of its entries.
 template <typename T>
 __host__ __device__ constexpr int csr_cols() { return sizeof(T) == 4 ? 8 : 4; }
 
@@ -246,20 +248,26 @@ __global__ void __launch_bounds__(256)
   __shared__ double red[KC][8];
   const int b = valid ? rowptr[r] : 0, e = valid ? rowptr[r + 1] : 0;
   const int cb = blockIdx.y * KC, nc = min(KC, ncols - cb);
-  // (columns past the last read the last one's entries and are not written)
   const T* x[KC];
 #pragma unroll
   for (int q = 0; q < KC; ++q) x[q] = X + (int64_t)(cb + min(q, nc - 1)) * ld;
   T acc[KC];
 #pragma unroll
   for (int q = 0; q < KC; ++q) acc[q] = (T)0;
+  auto row = [&](auto full) {
 #pragma unroll 2
-  for (int k = b; k < e; ++k) {
-    const int j = cols[k];
-    const T v = (T)vals[k];
+    for (int k = b; k < e; ++k) {
+      const int j = cols[k];
+      const T v = (T)vals[k];
 #pragma unroll
-    for (int q = 0; q < KC; ++q) acc[q] += v * __ldg(x[q] + j);
-  }
+      for (int q = 0; q < KC; ++q)
+        if (decltype(full)::value || q < nc) acc[q] += v * __ldg(x[q] + j);
+    }
+  };
+  if (nc == KC)
+    row(std::true_type{});
+  else
+    row(std::false_type{});
   T d[KC];
 #pragma unroll
   for (int q = 0; q < KC; ++q) {
