@@ -154,7 +154,10 @@ constexpr int kMaxTiles = 256;  // 8 x 32: m = 1024, four m-column segments
 // tile empty. Their CTAs stack two operands in the tile's two halves instead and
 // use two or three of its four quadrants:
 //   kLine: A = [C P], B = [P G] gives C^T P, P^T P and P^T G in one tile;
-//   kRows: A and B at two row offsets, two row slices' partials in one tile.
+//   kRows: A and B at two row offsets, two row slices' partials in one tile
+//          (half as long each: with slices as for whole tiles half the SMs
+//          idled, and a Gram of 100000 x 33 took 68 us a call instead of 59,
+//          now 57).
 // (The serving mix, m = 8..96, went from 357 to 314 ms for 16 requests.)
 enum Stack { kWhole = 0, kLine = 1, kRows = 2 };
 
@@ -448,20 +451,21 @@ bool gram_tc_fine_pays(int64_t N, int m) {
 
 // Row slices for a launch of `tiles` output tiles: among the counts that
 // keep at least min_stages stages per slice, launch at most 8 waves of CTAs
+// (of `per` slices each)
 // and stay within max_splits, the one whose CTAs fill the SMs most evenly,
 // less 1 % per extra wave (each wave refills the pipelines). Every CTA of a
 // launch does the same work, so with one slice per tile a launch of 164
 // tiles would run a second wave of 12 CTAs as long as the first.
 static int tc_splits(int64_t N, int tiles, int max_splits, int sms,
-                     int min_stages = kMinStages) {
+                     int min_stages = kMinStages, int per = 1) {
   const int64_t by_rows = ceil_div(N, (int64_t)BK * min_stages);
   const int smax = (int)std::max<int64_t>(
-      1, std::min<int64_t>({by_rows, (int64_t)8 * sms / tiles,
+      1, std::min<int64_t>({by_rows, (int64_t)8 * per * sms / tiles,
                             (int64_t)max_splits}));
   int best = 1;
   double beff = 0.0;
   for (int sp = 1; sp <= smax; ++sp) {
-    const int64_t ctas = (int64_t)tiles * sp;
+    const int64_t ctas = (int64_t)tiles * ceil_div(sp, per);
     const int64_t waves = ceil_div(ctas, (int64_t)sms);
     const double eff =
         (double)ctas / ((double)sms * (double)waves) - 0.01 * (double)(waves - 1);
@@ -500,8 +504,9 @@ template <typename Run>
 int tuned_splits(int64_t N, int m, int n, int tiles, int sym, int fine,
                  int smax, cudaStream_t s, Run& run) {
   const int sms = sm_count();
-  const int min_stages = fine ? kFineStages : kMinStages;
-  const int base = tc_splits(N, tiles, smax, sms, min_stages);
+  const int per = sym == -1 - kRows ? 2 : 1;
+  const int min_stages = (fine ? kFineStages : kMinStages) / per;
+  const int base = tc_splits(N, tiles, smax, sms, min_stages, per);
   // TRM_GRAM_SLICES=formula (or a count) fixes the slices instead (for
   // profilers, whose serialised replay would distort the timing)
   if (const char* f = std::getenv("TRM_GRAM_SLICES")) {
