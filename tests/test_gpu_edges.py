@@ -377,3 +377,41 @@ def test_fp64_factor_where_the_correction_is_left_early(trm, m, cond):
         tol = 20 * m * 2.3e-16 * np.linalg.cond(unit) ** 2
         assert np.max(np.abs(got.T @ got - np.eye(m))) < tol
         assert np.max(np.abs(got - ref)) < tol
+
+
+@pytest.mark.parametrize("gap", [1e-12, 1e-9, 1e-7, 1e-6, 1e-4])
+@pytest.mark.parametrize("m", [48, 128, 200])
+def test_eigenvalues_with_a_coupling_of_low_rank(trm, m, gap):
+    """Diagonal blocks whose neighbours lie `gap` apart, all coupled by a matrix
+    of rank one with entries just below what the FP32 sweeps rotate: its 2-norm
+    is its Frobenius norm, many times what the refinement's separation takes
+    for a random coupling of that size. The closing sweeps leave couplings of
+    1e-13 of two diagonal entries and 1e-15 of the whole; products round at m
+    eps."""
+    rng = np.random.default_rng(m)
+    d = np.repeat(np.linspace(1.0, 2.0, m // 8), 8)[:m]
+    d = d + gap * np.arange(len(d))
+    m = len(d)
+    v = rng.choice([-1.0, 1.0], m)
+    A = np.diag(d) + 0.9e-6 * np.linalg.norm(d) * np.outer(v, v)
+    N = m + 3
+    H = np.zeros((N, N))
+    H[:m, :m] = A
+    H[range(m, N), range(m, N)] = 9.0
+    rows, cols = np.nonzero(H)
+    rp = np.searchsorted(rows, np.arange(N + 1)).astype(np.int32)
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_csr(N, rp, cols.astype(np.int32), H[rows, cols], m, 1e-10,
+                           opt)
+    try:
+        t = gu.to_dev(np.eye(N)[:, :m])
+        lam, _ = trm.trm_rayleigh_ritz(h, t.data_ptr(), m)
+        C = gu.from_dev(t)
+    finally:
+        trm.trm_destroy(h)
+    w = np.linalg.eigvalsh(A)
+    scale = np.abs(w).max()
+    tol = (2e-13 * np.sqrt(m) + 1e-15 * m + 20 * m * 2.3e-16) * scale
+    assert np.max(np.abs(lam - w)) <= tol
+    assert np.max(np.linalg.norm(H @ C - C * lam, axis=0)) <= tol
+    assert np.max(np.abs(C.T @ C - np.eye(m))) <= 20 * m * 2.3e-16
