@@ -395,47 +395,8 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// MP1 (ii): Cn = Y L_D + fl32(Y) L', Y = C + alpha P; L_D = diag(R) in FP64,
-// L' = R - L_D in FP32.
-__global__ void __launch_bounds__(256)
-    k_rotate_split(int64_t N, int m, const double* __restrict__ C,
-                   const float* __restrict__ P, const double* __restrict__ R,
-                   double* __restrict__ Cn, const IterScalars* __restrict__ sc) {
-  __shared__ __align__(16) float As[GK][GLD];
-  __shared__ __align__(16) float Ms[GK][GLD];
-  const int64_t r0 = (int64_t)blockIdx.x * GT;
-  const int c0 = blockIdx.y * GT;
-  const double alpha = sc->alpha;
-  float acc[4][4] = {};
-  auto loadA = [&](int r, int k) -> float {
-    const int64_t row = r0 + r;
-    if (row >= N) return 0.f;
-    const int64_t idx = row + (int64_t)k * N;
-    return (float)(C[idx] + alpha * (double)P[idx]);
-  };
-  auto loadM = [&](int k, int c) -> float {
-    const int col = c0 + c;
-    return (col < m && k != col) ? (float)R[k + (int64_t)col * m] : 0.f;
-  };
-  const int kend = min(m, c0 + GT);
-  tile_product<float>(0, kend, loadA, loadM, acc, As, Ms);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-#pragma unroll
-  for (int x = 0; x < 4; ++x) {
-    const int64_t row = r0 + tx * 4 + x;
-    if (row >= N) continue;
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      const int col = c0 + ty * 4 + y;
-      if (col >= m) continue;
-      const int64_t idx = row + (int64_t)col * N;
-      const double yv = C[idx] + alpha * (double)P[idx];
-      Cn[idx] = yv * R[col + (int64_t)col * m] + (double)acc[x][y];
-    }
-  }
-}
-
-// The same split update with C and Cn as FP32 pairs: the FP32 operand is
+// MP1 (ii): Cn = Y L_D + fl32(Y) L', Y = C + alpha P; L_D = diag(R), L' = R - L_D in
+// FP32, with C and Cn as FP32 pairs: the FP32 operand is
 // Ch + alpha P, and Y diag(R) is formed in double-float.
 __global__ void __launch_bounds__(256)
     k_rotate_split_df(int64_t N, int m, const float* __restrict__ Ch,
@@ -781,18 +742,6 @@ void rotate(int64_t N, int m, const T* C, const TP* P, const double* R, T* Cn,
   }
   dim3 grid(ceil_div(N, GT), ceil_div(m, GT));
   k_rotate<T, TP><<<grid, 256, 0, s>>>(N, m, C, P, R, Cn, sc);
-  TRM_CHECK_LAUNCH();
-}
-
-void rotate_split(int64_t N, int m, const double* C, const float* P,
-                  const double* R, double* Cn, const IterScalars* sc,
-                  cudaStream_t s, const float* C32, const TcWork* tw) {
-  if (C32 && mul_tc_eligible(N, m, m, tw) && aligned16(C32) && aligned16(P)) {
-    mul_tc_split64(N, m, C32, P, C, sc, R, Cn, *tw, s);
-    return;
-  }
-  dim3 grid(ceil_div(N, GT), ceil_div(m, GT));
-  k_rotate_split<<<grid, 256, 0, s>>>(N, m, C, P, R, Cn, sc);
   TRM_CHECK_LAUNCH();
 }
 

@@ -62,7 +62,7 @@ constexpr int CS = 2;    // operand stages
 constexpr int THREADS = 512;
 constexpr int CONV0 = 4, NCONV = 4, EPI0 = 8, NEPI = 8;
 
-enum Mode { kStore = 0, kGrad = 1, kSplit64 = 2, kSplitDf = 3 };
+enum Mode { kStore = 0, kGrad = 1, kSplitDf = 3 };
 
 constexpr int EC = 8;                // columns per epilogue slot
 constexpr int ESLOT = 3 * EC * BM;   // X', G_prev, P_prev: EC columns each
@@ -99,11 +99,8 @@ struct MulArgs {
   const float* minv;
   double* part;    // kGrad: 4 sums per CTA
   IterScalars* scw;  // kGrad: the CG scalars (formed by the last CTA)
-  const double* c64;  // kSplit64: Cn = (C64 + alpha P) diag(R) + Y M
-  const float* p32;
-  const double* R;
-  double* out64;
-  const float* ch;     // kSplitDf: C as FP32 pairs, Cn written as pairs
+  const float* p32;    // kSplitDf: Cn = (C + alpha P) diag(R) + Y M, with C
+  const float* ch;     // as FP32 pairs and Cn written as pairs
   const float* cl;
   float* outh;
   float* outl;
@@ -386,8 +383,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     // Polak-Ribiere sums as double-float pairs (no FP64 instruction per
     // batch: GB300's FP64 pipe is 1/64 of its FP32 rate)
     F2 s_sum[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-    double alpha64 = 0.0;
-    if (MODE == kSplit64 && args.sc) alpha64 = args.sc->alpha;
     F2 alpha2 = {0.f, 0.f};
     if (MODE == kSplitDf && args.sc) alpha2 = df_of(args.sc->alpha);
     const float* slots = &sm->rawp[0][0];
@@ -505,30 +500,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const int64_t idx = row + (int64_t)col * N;
                 args.outh[idx] = t.h;
                 args.outl[idx] = t.l;
-              }
-            }
-          }
-        } else {
-#pragma unroll
-          for (int h = 0; h < 16; h += 8) {
-            double cv[8];
-            float pv[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int col = c0 + cb + h + e;
-              const int64_t idx = row + (int64_t)col * N;
-              const bool in = col < args.n;
-              cv[e] = in ? args.c64[idx] : 0.0;
-              pv[e] = in ? args.p32[idx] : 0.f;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int col = c0 + cb + h + e;
-              if (col < args.n) {
-                const double y = fma(alpha64, (double)pv[e], cv[e]);
-                args.out64[row + (int64_t)col * N] =
-                    fma(y, args.R[col + (int64_t)col * args.k],
-                        (double)__uint_as_float(r[h + e]));
               }
             }
           }
@@ -732,19 +703,9 @@ void mul_tc_splitdf(int64_t N, int m, const float* Ch, const float* Cl,
                     float* Cnh, float* Cnl, const TcWork& tw, cudaStream_t s) {
   MulArgs a{};
   a.N = N; a.k = m; a.n = m; a.sc = sc; a.ch = Ch; a.cl = Cl; a.p32 = P;
-  a.R = R; a.outh = Cnh; a.outl = Cnl; a.err = tw.err;
+  a.outh = Cnh; a.outl = Cnl; a.err = tw.err;
   a.tri = 1;
   launch<kSplitDf>(a, Ch, P, R, 1, tw.msplit, s, nullptr);
-}
-
-void mul_tc_split64(int64_t N, int m, const float* C32, const float* P,
-                    const double* C64, const IterScalars* sc, const double* R,
-                    double* Cn, const TcWork& tw, cudaStream_t s) {
-  MulArgs a{};
-  a.N = N; a.k = m; a.n = m; a.sc = sc; a.c64 = C64; a.p32 = P; a.R = R;
-  a.out64 = Cn; a.err = tw.err;
-  a.tri = 1;
-  launch<kSplit64>(a, C32, P, R, 1, tw.msplit, s, nullptr);
 }
 
 }  // namespace trm

@@ -291,12 +291,9 @@ int mul_tc_grad(int64_t N, int m, const float* C, const double* Hp,
                 const float* Xp, float* G, const float* Gprev,
                 const float* Pprev, const float* minv, double* part,
                 IterScalars* sc, const TcWork& tw, cudaStream_t s);
-// Cn = (C64 + alpha P) diag(R) + (C32 + alpha P) (R - diag(R))
-void mul_tc_split64(int64_t N, int m, const float* C32, const float* P,
-                    const double* C64, const IterScalars* sc, const double* R,
-                    double* Cn, const TcWork& tw, cudaStream_t s);
-// The same with C and Cn as FP32 pairs (C32 = Ch): Y = C + alpha P and
-// Y diag(R) in double-float, plus the tensor-core product
+// Cn = (C + alpha P) diag(R) + (Ch + alpha P) (R - diag(R)) with C and Cn as FP32
+// pairs: Y = C + alpha P and Y diag(R) in double-float, plus the tensor-core
+// product
 void mul_tc_splitdf(int64_t N, int m, const float* Ch, const float* Cl,
                     const float* P, const IterScalars* sc, const double* R,
                     float* Cnh, float* Cnl, const TcWork& tw, cudaStream_t s);
@@ -327,15 +324,9 @@ template <typename T, typename TP>
 void rotate(int64_t N, int m, const T* C, const TP* P, const double* R,
             T* Cn, const IterScalars* sc, cudaStream_t s,
             const TcWork* tw = nullptr);
-// MP1 (ii): Cn = Y L_D + fl32(Y) L', Y = C + alpha P; R = L^{-T} FP64.
-// With C32 = fl32(C) and tw, fl32(Y) is formed as C32 + alpha P in FP32 and
-// the product runs on the tensor cores.
-void rotate_split(int64_t N, int m, const double* C, const float* P,
-                  const double* R, double* Cn, const IterScalars* sc,
-                  cudaStream_t s, const float* C32 = nullptr,
-                  const TcWork* tw = nullptr);
-// The split update with C and Cn as FP32 pairs (hi, lo): the FP32 operand
-// is Ch + alpha P, Y diag(R) is formed in double-float
+// MP1 (ii): Cn = Y L_D + fl32(Y) L', Y = C + alpha P, R = L^{-T} FP64, with C and
+// Cn as FP32 pairs (hi, lo): the FP32 operand is Ch + alpha P, Y diag(R) is formed
+// in double-float
 void rotate_split_df(int64_t N, int m, const float* Ch, const float* Cl,
                      const float* P, const double* R, float* Cnh, float* Cnl,
                      const IterScalars* sc, cudaStream_t s,
@@ -399,23 +390,21 @@ void make_A0(int m, const double* Hp, const double* HD, double* A0,
 // The line step along P and the factor of the new overlap: the line-model
 // terms from H' (diag zeroed), H_D, B = C^T P, Q = P^T P, the trace of
 // P^T H P and W = P^T G give alpha (into sc); then S = I + a (B + B^T) +
-// a^2 Q is factorised (in deviation form when dev) into Linv (may be null)
-// and R = L^{-T}. The trace comes from the diagonal hpd[j * hpd_stride] (the
+// a^2 Q is factorised into R = L^{-T}. The trace comes from the diagonal hpd[j * hpd_stride] (the
 // matrix P^T H P with stride m + 1), or, when hpd is null, as the sum of the
 // n_tr_parts partial column dots in tr_parts (the stencil applied to P).
-// part: >= 16 * ceil(m/32)^2 doubles; gwork: max(2 m^2, chol_work_elems(m))
-// doubles (FP32 factorisations keep FP32 copies of B and Q there).
-template <typename Tm>
+// part: >= 16 * ceil(m/32)^2 doubles; gwork: chol_work_elems(m) doubles.
 void line_factor(int m, const double* Hp, const double* HD, const double* Bm,
                  const double* Q, const double* hpd, int hpd_stride,
                  const double* tr_parts, int n_tr_parts, const double* W,
-                 double* Linv, double* R, IterScalars* sc, double* gwork,
-                 double* part, bool dev, cudaStream_t s);
-// line_factor<float> with the m x m inputs given in FP32 (Gram copies). With
-// split (mul_tc_work_floats(m, m) floats, zero when first used) and m small enough for one CTA the
-// factor goes out as the TF32 terms the tensor-core rotations read (leading
-// dimension split_ldm; split_diag: the diagonal left out, as pairs) instead of
-// R, and the call returns true: the rotation then takes a null R.
+                 double* R, IterScalars* sc, double* gwork, double* part,
+                 cudaStream_t s);
+// The same in FP32 arithmetic, the m x m inputs given in FP32 (Gram copies) and
+// the factor formed in deviation form. With split (mul_tc_work_floats(m, m)
+// floats, zero when first used) and m small enough for one CTA the factor goes
+// out as the TF32 terms the tensor-core rotations read (leading dimension
+// split_ldm; split_diag: the diagonal left out, as pairs) instead of R, and the
+// call returns true: the rotation then takes a null R.
 bool line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
                    const float* Q, const double* hpd, int hpd_stride,
                    const double* tr_parts, int n_tr_parts, const float* W,

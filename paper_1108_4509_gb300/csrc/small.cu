@@ -229,7 +229,7 @@ __device__ void line_alpha_block(int m, const double* __restrict__ part,
 }
 
 // ---------------------------------------------------------------------------
-// Cholesky S = L L^T and L^{-1}, blocked in 32-column panels, one CTA of 256
+// FP64 Cholesky S = L L^T and L^{-1}, blocked in 32-column panels, one CTA of 256
 // threads. Writes Linv (lower) and R = L^{-T} (upper).
 //
 // m is padded to mp, a multiple of 32, with the identity, which changes
@@ -250,9 +250,9 @@ __device__ void line_alpha_block(int m, const double* __restrict__ part,
 // S is read from memory, or (Bm != null) formed on the fly as
 // S = I + a (B + B^T) + a^2 Q with a = sc->alpha (the line step's overlap).
 //
-// With dev = true the factorisation runs in deviation form for S = I + E:
+// With dev = true the other kernels here run in deviation form for S = I + E:
 // L = I + F and L^{-1} = I + Y with the identity kept exact and only the
-// small E, F, Y held in Tm. Pivot: d = E_cc - sum_k F_ck^2 and
+// small E, F, Y held. Pivot: d = E_cc - sum_k F_ck^2 and
 // f_cc = d / (1 + sqrt(1 + d)); off the diagonal L and F coincide; inverse
 // diagonal y_cc = -f_cc / (1 + f_cc). When S - I is small, FP32 arithmetic
 // here yields L to FP64 accuracy relative to I.
@@ -330,19 +330,19 @@ __device__ __forceinline__ void diag_inverse_warp(const Tm* B, int ldb,
 // 256 threads: the register-resident rows of the diagonal-block steps need
 // more than the 128 registers a 512-thread CTA allows (they spilled, and
 // the sequential pivot chain paid for it); the parallel phases lose less.
-template <typename Tm>
-constexpr int chol_threads() { return 256; }
+constexpr int kCholThreads = 256;
 
 // SM: the working copy lives in shared memory (a compile-time choice, so its
 // accesses compile to shared-memory instructions), else in gwork.
-template <typename Tm, bool dev, bool SM>
-__global__ void __launch_bounds__(chol_threads<Tm>(), 1)
+template <bool SM>
+__global__ void __launch_bounds__(kCholThreads, 1)
     k_chol_inv(int m, const double* __restrict__ S, const double* __restrict__ Bm,
                const double* __restrict__ Q, double* __restrict__ Linv,
-               double* __restrict__ R, IterScalars* sc, Tm* gwork,
+               double* __restrict__ R, IterScalars* sc, double* gwork,
                const double* __restrict__ lpart, int nlpart,
                const unsigned long long* refined) {
   if (refined && refined_ok(refined)) return;
+  using Tm = double;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int bad;
   __shared__ Tm rdiag[1024];  // 1 / L_cc, all columns (mp <= 1024)
@@ -351,8 +351,7 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
   const int mp = (m + 31) & ~31, ld = mp + 1, P = mp >> 5;
   Tm* a = SM ? reinterpret_cast<Tm*>(smraw) : gwork;
   Tm* tb = a + (size_t)mp * ld;  // 32 x mp, leading dimension 33
-  const Tm one = dev ? (Tm)1 : (Tm)0;
-  const Tm eps = sizeof(Tm) == 4 ? (Tm)1.2e-7 : (Tm)2.3e-16;
+  const Tm eps = 2.3e-16;
   if (lpart) {  // the line step first (it sets sc->alpha)
     __shared__ double lred[4 * 32];
     line_alpha_block(m, lpart, nlpart, sc, lred);
@@ -380,17 +379,11 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
     __syncthreads();
     for (int k = warp; k < mp; k += nw)
       for (int i = k + lane; i < mp; i += 32)
-        a[i + k * ld] = a[i + k * ld] + a[k + i * ld] +
-                        ((!dev && i == k) ? (Tm)1 : (Tm)0);
+        a[i + k * ld] = a[i + k * ld] + a[k + i * ld] + (i == k ? 1.0 : 0.0);
   } else {
     for (int k = warp; k < mp; k += nw)
       for (int i = k + lane; i < mp; i += 32) {
-        double v;
-        if (i < m && k < m)
-          v = S[i + k * m] - (dev && i == k ? 1.0 : 0.0);
-        else
-          v = (!dev && i == k) ? 1.0 : 0.0;
-        a[i + k * ld] = (Tm)v;
+        a[i + k * ld] = i < m && k < m ? S[i + k * m] : i == k ? 1.0 : 0.0;
       }
   }
   if (tid == 0) bad = 0;
@@ -416,34 +409,21 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
         const int q = c >> 3;
         if (warp == (c & 7)) {
           Tm d = __shfl_sync(0xffffffffu, v[q], c);
-          // 1 / L_cc is all the column needs: rsqrt(1 + d) (rsqrt(d)) on the
-          // pivot chain; L_cc itself is formed after the column is out
-          Tm rl;
-          if (dev) {
-            if (!(d > (Tm)-0.999)) {  // pivot 1 + d not positive: singular S
-              b = true;
-              d = (Tm)0;
-            }
-            rl = piv_rsqrt((Tm)1 + d);
-          } else {
-            // a pivot that has lost all but 4m roundings of its original
-            // diagonal entry marks a (numerically) singular S
-            const int cc = c0 + c;
-            const double sjj =
-                (Bm || cc >= m) ? 1.0 : fabs(S[cc + cc * m]);
-            if (!(d > (Tm)(4 * m) * eps * (Tm)sjj)) {
-              b = true;
-              d = (Tm)1;
-            }
-            rl = piv_rsqrt(d);
+          // 1 / L_cc is all the column needs: rsqrt(d) on the pivot chain; L_cc
+          // itself is formed after the column is out
+          // a pivot that has lost all but 4m roundings of its original
+          // diagonal entry marks a (numerically) singular S
+          const int cc = c0 + c;
+          const double sjj = (Bm || cc >= m) ? 1.0 : fabs(S[cc + cc * m]);
+          if (!(d > (Tm)(4 * m) * eps * sjj)) {
+            b = true;
+            d = 1.0;
           }
+          const Tm rl = piv_rsqrt(d);
           if (lane > c) v[q] *= rl;
           colbuf[c & 1][lane] = v[q];  // the diagonal entry is not read
           if (lane == 0) rdiag[c0 + c] = rl;
-          // L_cc (deviation form: L_cc - 1 = d / (1 + sqrt(1 + d)), with
-          // sqrt(1 + d) = (1 + d) rl, which keeps small d accurate)
-          if (lane == c)
-            v[q] = dev ? d * piv_rcp((Tm)1 + ((Tm)1 + d) * rl) : d * rl;
+          if (lane == c) v[q] = d * rl;
         }
         __syncthreads();
         const Tm lrc = colbuf[c & 1][lane];
@@ -511,16 +491,13 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
   // (d) inverse X = L_pp^{-1} of each diagonal block, one warp per block,
   // in place, row by row: lane j forms X_ij = (delta_ij - sum_{k=j}^{i-1}
   // L_ik X_kj) / L_ii from row i of L and its own column of X (rolled loops:
-  // code run once per launch would stall on instruction fetch). In
-  // deviation form (L = I + F, X = I + Y) the same recurrence reads
-  // y_jj = -f_jj / (1 + f_jj) and, for i > j,
-  // y_ij = -(f_ij + sum_{k=j}^{i-1} f_ik y_kj) / (1 + f_ii).
+  // code run once per launch would stall on instruction fetch).
   for (int pb = warp; pb < P; pb += nw) {
     Tm* B = a + 32 * pb + (size_t)(32 * pb) * ld;  // block (i, k) at B[i + k ld]
     const Tm* rd = rdiag + 32 * pb;
     const int j = lane;
     for (int i = 0; i < 32; ++i) {
-      Tm s0 = (dev && i > j) ? B[i + j * ld] : (Tm)0, s1 = 0;
+      Tm s0 = 0, s1 = 0;
       int k = j;
 #pragma unroll 2
       for (; k + 1 < i; k += 2) {
@@ -529,7 +506,7 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
       }
       if (k < i) s0 += B[i + k * ld] * B[k + j * ld];
       Tm x = 0;
-      if (i == j) x = dev ? -B[i + i * ld] * rd[i] : rd[i];
+      if (i == j) x = rd[i];
       else if (i > j) x = -(s0 + s1) * rd[i];
       __syncwarp();  // row i of L is read by every lane before it is replaced
       if (i >= j) B[i + j * ld] = x;
@@ -545,12 +522,7 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
     const int nblk = 2 * ri;  // 8 row groups x ri/4 column groups
     for (int bq = tid; bq < nblk; bq += nt) {
       const int r0 = 4 * (bq & 7), cb = 4 * (bq >> 3);
-      Tm acc[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v)  // identity part of X (deviation form)
-          acc[u][v] = dev ? a[(ri + r0 + u) + (cb + v) * ld] : (Tm)0;
+      Tm acc[4][4] = {};
 #pragma unroll 4
       for (int col = cb; col < ri; ++col) {
         Tm lr[4], xc[4];
@@ -572,12 +544,7 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
     __syncthreads();
     for (int bq = tid; bq < nblk; bq += nt) {
       const int r0 = 4 * (bq & 7), cb = 4 * (bq >> 3);
-      Tm acc[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-          acc[u][v] = dev ? tb[(r0 + u) + (cb + v) * 33] : (Tm)0;
+      Tm acc[4][4] = {};
 #pragma unroll 4
       for (int q = 0; q <= r0 + 3; ++q) {
         Tm xr[4], tv[4];
@@ -599,20 +566,11 @@ __global__ void __launch_bounds__(chol_threads<Tm>(), 1)
     __syncthreads();
   }
   const int isbad = bad;
-  // Linv(i, k) column by column, then R(k, i) = Linv(i, k) column by column
-  // (FP64 work only where it is needed: a conversion per lower-triangle
-  // entry, the identity added on the diagonal alone)
-  // (four entries per thread in flight; an FP64 conversion per
-  // lower-triangle entry, the identity added on the diagonal alone)
+  // Linv(i, k) column by column, then R(k, i) = Linv(i, k) column by column,
+  // four entries per thread in flight
   auto entry = [&](int i, int k) -> double {
-    double v = 0.0;
-    if (isbad) {
-      if (i == k) v = 1.0;
-    } else if (i >= k) {
-      v = (double)a[i + k * ld];
-      if (dev && i == k) v += 1.0;
-    }
-    return v;
+    if (isbad) return i == k ? 1.0 : 0.0;
+    return i >= k ? a[i + k * ld] : 0.0;
   };
   for (int o = 0; o < (Linv ? 2 : 1); ++o) {
     double* out = o ? Linv : R;
@@ -1214,13 +1172,12 @@ __global__ void __launch_bounds__(kPanelThreads, 1)
 // [A 0; B C], its inverse is [A^{-1} 0; -C^{-1} B A^{-1}  C^{-1}], so with the
 // 32 x 32 inverses from k_cb_diag, levels of block size 32, 64, ... each form
 // T = B A^{-1}, then X_CA = -C^{-1} T, for all blocks of the level at once
-// (k_cb_inv). Deviation form (dev) as in k_chol_inv: W holds S - I, L = I + F
+// (k_cb_inv). Deviation form (dev): W holds S - I, L = I + F
 // and X = I + Y with the identities implicit, so FP32 arithmetic keeps L to
 // FP64 accuracy relative to I when S is close to I.
 // ---------------------------------------------------------------------------
 constexpr int CB = 32;
 
-// The line step alpha from the line-term partials (one CTA).
 // A power of two whose square brings a positive number into [1/2, 2) (finite
 // for any bits); 1 for a number on either side of 1
 __device__ __forceinline__ double half_exp_scale(double x) {
@@ -1276,6 +1233,7 @@ __global__ void __launch_bounds__(256)
   R[e] = up;
 }
 
+// The line step alpha from the line-term partials (one CTA).
 __global__ void k_cb_alpha(int m, const double* __restrict__ lpart, int nlpart,
                            IterScalars* sc) {
   __shared__ double lred[4 * 32];
@@ -1515,15 +1473,14 @@ __global__ void k_cb_out(int m, int mp, const Tm* __restrict__ X,
 // to tr(A0 (B B^T - B^T B)) by cyclic invariance, so no m x m product is
 // stored.
 // ---------------------------------------------------------------------------
-template <typename Tm, typename Tin>
+template <typename Tm>
 __global__ void __launch_bounds__(1024)
-    k_line_terms(int m, const Tin* __restrict__ Hp,
-                 const double* __restrict__ HD, const Tin* __restrict__ Bm,
-                 const Tin* __restrict__ Q, const double* __restrict__ hpd,
+    k_line_terms(int m, const Tm* __restrict__ Hp,
+                 const double* __restrict__ HD, const Tm* __restrict__ Bm,
+                 const Tm* __restrict__ Q, const double* __restrict__ hpd,
                  int hpd_stride, const double* __restrict__ tr_parts,
-                 int n_tr_parts, const Tin* __restrict__ W,
-                 double* __restrict__ part,
-                 float* __restrict__ Bf, float* __restrict__ Qf) {
+                 int n_tr_parts, const Tm* __restrict__ W,
+                 double* __restrict__ part) {
   __shared__ Tm t0[32][33], t1[32][33], t2[32][33], t3[32][33];
   __shared__ double red[4 * 32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -1556,10 +1513,6 @@ __global__ void __launch_bounds__(1024)
     v2 = a0 * M;
     if (ks == 0) {
       const Tm bij = (Tm)Bm[e], qij = (Tm)Q[e];
-      if (Bf) {  // FP32 copies for the factorisation that follows
-        Bf[e] = (float)bij;
-        Qf[e] = (float)qij;
-      }
       const Tm s1 = bij + t1[ty][tx];
       const Tm wij = (Tm)W[e], wji = t2[ty][tx];
       v2 -= (Tm)0.5 * s1 * (wij + wji);
@@ -2102,19 +2055,18 @@ static void chol_launch(int m, const double* S, const double* Bm,
       int dv = 0;
       cudaGetDevice(&dv);
       if (dv < 0 || dv >= 64 || !done[dv].load(std::memory_order_relaxed)) {
-        TRM_CUDA(cudaFuncSetAttribute(k_chol_inv<Tm, dev, true>,
+        TRM_CUDA(cudaFuncSetAttribute(k_chol_inv<true>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       200 * 1024));
         if (dv >= 0 && dv < 64) done[dv].store(1, std::memory_order_relaxed);
       }
     }
     if (smem)
-      k_chol_inv<Tm, dev, true><<<1, chol_threads<Tm>(), bytes, s>>>(
+      k_chol_inv<true><<<1, kCholThreads, bytes, s>>>(
           m, S, Bm, Q, Linv, R, sc, nullptr, lpart, nlpart, refined);
     else
-      k_chol_inv<Tm, dev, false><<<1, chol_threads<Tm>(), 0, s>>>(
-          m, S, Bm, Q, Linv, R, sc, reinterpret_cast<Tm*>(gwork), lpart,
-          nlpart, refined);
+      k_chol_inv<false><<<1, kCholThreads, 0, s>>>(
+          m, S, Bm, Q, Linv, R, sc, gwork, lpart, nlpart, refined);
     TRM_CHECK_LAUNCH();
   }
 }
@@ -2134,34 +2086,19 @@ static int line_ksplit(int m) {
   return std::max(1, ks);
 }
 
-template <typename Tm>
 void line_factor(int m, const double* Hp, const double* HD, const double* Bm,
                  const double* Q, const double* hpd, int hpd_stride,
                  const double* tr_parts, int n_tr_parts, const double* W,
-                 double* Linv, double* R, IterScalars* sc, double* gwork,
-                 double* part, bool dev, cudaStream_t s) {
+                 double* R, IterScalars* sc, double* gwork, double* part,
+                 cudaStream_t s) {
   const int t = ceil_div(m, 32);
   const int ksplit = line_ksplit(m);
-  // FP32 factorisations take B and Q as FP32 copies written by the line
-  // terms, placed after the factorisation's own FP32 working copy in gwork
-  // (gwork holds max(2 m^2, chol_work_elems(m)) doubles)
-  float* Bf = nullptr;
-  float* Qf = nullptr;
-  if (sizeof(Tm) == 4) {
-    Bf = reinterpret_cast<float*>(gwork) + chol_work_elems(m);
-    Qf = Bf + (size_t)m * m;
-  }
-  k_line_terms<Tm, double><<<dim3(t, t, ksplit), 1024, 0, s>>>(
-      m, Hp, HD, Bm, Q, hpd, hpd_stride, tr_parts, n_tr_parts, W, part, Bf,
-      Qf);
+  k_line_terms<double><<<dim3(t, t, ksplit), 1024, 0, s>>>(
+      m, Hp, HD, Bm, Q, hpd, hpd_stride, tr_parts, n_tr_parts, W, part);
   TRM_CHECK_LAUNCH();
   // the factorisation kernel takes the line step from the partials first
-  if (dev)
-    chol_launch<Tm, true>(m, nullptr, Bm, Q, Bf, Qf, Linv, R, sc, gwork, s,
-                          part, t * t * ksplit);
-  else
-    chol_launch<Tm, false>(m, nullptr, Bm, Q, Bf, Qf, Linv, R, sc, gwork, s,
-                           part, t * t * ksplit);
+  chol_launch<double, false>(m, nullptr, Bm, Q, nullptr, nullptr, nullptr, R, sc,
+                             gwork, s, part, t * t * ksplit);
 }
 
 // The FP32 path with the m x m inputs already in FP32 (copies the Gram sums
@@ -2174,9 +2111,8 @@ bool line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
                    bool split_diag) {
   const int t = ceil_div(m, 32);
   const int ksplit = line_ksplit(m);
-  k_line_terms<float, float><<<dim3(t, t, ksplit), 1024, 0, s>>>(
-      m, Hp, HD, Bm, Q, hpd, hpd_stride, tr_parts, n_tr_parts, W, part,
-      nullptr, nullptr);
+  k_line_terms<float><<<dim3(t, t, ksplit), 1024, 0, s>>>(
+      m, Hp, HD, Bm, Q, hpd, hpd_stride, tr_parts, n_tr_parts, W, part);
   TRM_CHECK_LAUNCH();
   if (split && panel_fits(m)) {
     PanelOut out;
@@ -2190,17 +2126,6 @@ bool line_factor32(int m, const float* Hp, const double* HD, const float* Bm,
                            gwork, s, part, t * t * ksplit);
   return false;
 }
-
-template void line_factor<float>(int, const double*, const double*,
-                                 const double*, const double*, const double*,
-                                 int, const double*, int, const double*,
-                                 double*, double*, IterScalars*, double*,
-                                 double*, bool, cudaStream_t);
-template void line_factor<double>(int, const double*, const double*,
-                                  const double*, const double*, const double*,
-                                  int, const double*, int, const double*,
-                                  double*, double*, IterScalars*, double*,
-                                  double*, bool, cudaStream_t);
 
 template <typename T>
 static void jacobi_launch(int m, const double* A, const double* Z0, double* w,

@@ -757,9 +757,8 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
                       tc ? rw_.msplit : nullptr, mul_tc_ldm(m_)))
       R = nullptr;
   } else
-    line_factor<Tm>(m_, Hp_, HD_, Bm_, PG_, hpd, m_ + 1, trp, ntrp,
-                    PG_ + woff, nullptr, R_, sc_, mmw_, T1_,
-                    sizeof(Tm) == 4, s_);
+    line_factor(m_, Hp_, HD_, Bm_, PG_, hpd, m_ + 1, trp, ntrp, PG_ + woff, R_,
+                sc_, mmw_, T1_, s_);
   prof.end(KC_SMALL, 4 * m3 + 2 * m3 / 3, 0.0, s_);
   TRM_PROF(krt, m2N, 3 * es * nm,
            (rotate<T, T>(ld_, m_, C, P, R, Cn, sc_, s_,
@@ -834,9 +833,8 @@ void Solver::iter_fp64_tail(double* C, double* Cn, const double* X, double* G,
   TRM_PROF(KC_GRAM64, 2 * m2N, 16 * nm,
            oz_gram(&ozB_, 1, ozA_, PG_ + mm, part_, part_cap_, err, s_));  // P^T G
   prof.begin(KC_SMALL, s_);
-  line_factor<double>(m_, Hp_, HD_, Bm_, PG_, nullptr, m_ + 1, hpdots_,
-                      chunks * m_, PG_ + mm, nullptr, R_, sc_, mmw_, T1_, false,
-                      s_);
+  line_factor(m_, Hp_, HD_, Bm_, PG_, nullptr, m_ + 1, hpdots_, chunks * m_,
+              PG_ + mm, R_, sc_, mmw_, T1_, s_);
   prof.end(KC_SMALL, 4 * md * md * md + 2 * md * md * md / 3, 0.0, s_);
   slice(C, ozA_, P);                                           // C + alpha P
   TRM_PROF(KC_ROT64, m2N, 16 * nm,
