@@ -13,11 +13,16 @@
 // every sum of up to kChunk * 32 rows of all products of equal weight exactly
 // (8 * 128 * 2^14 = 2^24): nothing is rounded until the integer sums, held in
 // 64 bits, are turned into one FP64 value. Dropped are r and the products of
-// weight below 2^-56 of the leading one (36 of 64 are kept): about 2^-61 of
-// max|a| max|b| per row, so that a column whose largest entry is 2^8 times its
-// usual one still loses less than an FP64 sum rounds. (Seven-bit digits, 2^-55,
-// left a step with max/rms = 8 columns 2.3 times further off than FP64
-// arithmetic did.)
+// weight below 2^-56 of the leading one (36 of 64 are kept): per term of a sum
+// less than 2^-57 max|a| max|b| of the two columns, usually about 2^-61. That is
+// FP64 norm-wise, for any block: a sum of random terms, or of columns whose
+// largest entry is up to 2^8 times their usual one, is no further off than an
+// FP64 chain leaves it (measured: at most as far for every FP64 call of the
+// repository's sizes; seven-bit digits, 2^-55, were 2.3 times further off at max
+// / rms = 8). It is not FP64 entry by entry: entries below 2^-9 of their column's
+// largest lose low bits and those below 2^-63 of it vanish, so in a column that
+// falls off exponentially the small entries of a product carry an error
+// relative to the large ones.
 //
 // One CTA owns a 128 x 64 output tile: eight accumulators (one per weight) of
 // 64 columns fill the 512 TMEM columns. Per 32-deep stage TMA brings all eight
@@ -578,8 +583,8 @@ int oz_ldk(int k) { return (k + 7) & ~7; }
 
 // The slicing passes and whole 128 x 64 tiles cost about 50 us however small
 // the product, the time of 3e7 multiply-adds on the FP64 pipe (110592 x 128:
-// Gram 153 us with 100 for the digits of a block, against 3020; 32768 x 64: 40
-// with 20, against 267).
+// Gram 165 us and 98 for the digits of a block, against 3020; 32768 x 64: 51
+// and 27, against 267).
 bool oz_pays(int64_t N, int m, int n) {
   return (double)N * m * n >= 3e7 && N >= 1024 && m >= 8 && n >= 8 &&
          N < ((int64_t)1 << 31) - 128 && encode_fn() != nullptr;
