@@ -22,6 +22,17 @@
  *    negative trm_status, with a message from trm_last_error() where a
  *    handle exists, or trm_last_global_error() otherwise.
  *  - A handle may be used by one host thread at a time.
+ *  - "FP64 products": Grams of FP64 blocks and their products with m x m
+ *    matrices run on the tensor cores from N m^2 = 3e7 on (N >= 1024, m >= 8),
+ *    in exact integer sums of the columns' leading 62 bits: each entry is held
+ *    in fixed point against the largest magnitude of its column. A result that
+ *    sums K products is rounded to FP64 and off by less than
+ *    K 2^-56 max|a| max|b| (usually sqrt(K) 2^-61) of the two columns a, b: as
+ *    FP64 arithmetic norm-wise, in orthonormality, eigenvalues and residuals.
+ *    It is not so entry by entry: an entry far below the largest of its column
+ *    does not keep FP64's own relative accuracy, and one below 2^-63 of it
+ *    counts as zero. Smaller products are FP64 multiply-adds (in the mixed
+ *    ladder FP32 pairs). trm_gram's FP64 products are always multiply-adds.
  */
 #ifndef TRM_H
 #define TRM_H
@@ -42,13 +53,14 @@ typedef enum {
   TRM_ENOTPD = -3,   /* an overlap matrix C^T C was not positive definite */
   TRM_ENOCONV = -4,  /* max_iter reached; outputs hold the best iterate */
   TRM_ECUDA = -5,    /* a CUDA runtime call failed */
-  TRM_ETIMEOUT = -6, /* a bounded device wait gave up */
+  TRM_ETIMEOUT = -6, /* a bounded device wait gave up; outputs hold no result */
   TRM_EGAP = -7      /* reserved: gap test failed */
 } trm_status;
 
 /* Precision modes (Sec. 2.2). */
 typedef enum {
-  TRM_FP64 = 0,    /* "full DP": every operation in FP64 */
+  TRM_FP64 = 0,    /* "full DP": every operation in FP64 (large products as
+                      "FP64 products" above) */
   TRM_MP1 = 1,     /* reserved: Sec. 2.2's MP1 (G, P stored FP32, split
                       rotation) is not offered -- its O(m^2 N) Grams stay
                       FP64, the slowest part on this GPU; create returns
@@ -247,9 +259,10 @@ trm_status trm_gram(int64_t N, int m, int n, int dtype, const void* A,
                     const void* B, double* out, void* stream);
 
 /*
- * Fig. ONFIG in FP64 on the device: S = C^T C, S = L L^T, C <- C L^{-T}.
+ * Fig. ONFIG in FP64 on the device: S = C^T C, S = L L^T, C <- C L^{-T}
+ * (large blocks: "FP64 products" above).
  * C: device, N x m FP64, overwritten. Returns TRM_ENOTPD if S is not
- * positive definite.
+ * positive definite; a finite C is then as it was.
  */
 trm_status trm_orthonormalize(int64_t N, int m, double* C, void* stream);
 
@@ -259,11 +272,12 @@ trm_status trm_orthonormalize(int64_t N, int m, double* C, void* stream);
  * the converged blocks of the two previous problems, a block for the next.
  * C_cur's columns are any basis of its subspace, so C_prev is first aligned
  * to it by the orthogonal U that minimises ||C_prev U - C_cur||_F (the polar
- * factor of M = C_prev^T C_cur, formed on the device as
- * M (M^T M)^{-1/2} from the eigendecomposition of M^T M); then
+ * factor of M = C_prev^T C_cur, M (M^T M)^{-1/2}, formed on the device by
+ * Newton-Schulz steps where M is near-orthogonal, else from the
+ * eigendecomposition of M^T M); then
  *   C_next = C_cur + alpha (C_cur - C_prev U),
  * orthonormalized as trm_orthonormalize does (C_next^T C_next = I, Cholesky
- * factor, so the result is unique). alpha = 1 is linear extrapolation in
+ * factor, so the result is unique; large blocks: "FP64 products" above). alpha = 1 is linear extrapolation in
  * equal steps; alpha = dt_next / dt_prev for unequal ones.
  * C_prev, C_cur: device, N x m column-major FP64, orthonormal, read only.
  * C_next: device, N x m, written (may not alias the inputs).
@@ -288,7 +302,8 @@ trm_status trm_iterate(trm_handle h, int mode, int restart, double* E_out,
                        double* rms_out, double* alpha_out);
 
 /*
- * Rayleigh-Ritz on span(C) in FP64 (Sec. 2.1): solves (C^T H C) y = theta
+ * Rayleigh-Ritz on span(C) in FP64 (Sec. 2.1; large blocks: "FP64 products"
+ * above): solves (C^T H C) y = theta
  * (C^T C) y, overwrites C (device, N x m FP64) with C Y (unit columns, each
  * column's largest-magnitude entry positive), and writes lambda (host, m,
  * ascending) and the residual norms ||H c_j - lambda_j c_j|| (host, m).
