@@ -14,6 +14,12 @@
 // product is a small correction, keeps one accumulator, small products first).
 // With one accumulator, large products first: an FP32 step at 13 x 11 x 9,
 // m = 40 was 4.2e-7 off, an FMA chain's is 2.2e-7.
+// Truncation goes one way: a rotation (M near I) shrinks the block, by half a place
+// an entry, with one accumulator by 2 (norms 6e-8 and 2.4e-7 short). Blocks that
+// FP32 multiply-adds rotated until their columns were padded (TcWork::fine)
+// therefore leave the diagonal out of the MMAs (kStoreDiag): the epilogue adds
+// Y diag(M) in two multiply-adds, with Y from memory again (two FP32 steps at
+// 39 x 41 x 37, m = 90: 905 -> 946 us; their energy 8e-8 -> 2e-9 off).
 //
 // Layout: Y is column-major (rows contiguous), so a TMA box of 32 rows x 32
 // columns with the 128-byte swizzle holds 32 lines of 32 rows each (the
@@ -62,7 +68,7 @@ constexpr int CS = 2;    // operand stages
 constexpr int THREADS = 512;
 constexpr int CONV0 = 4, NCONV = 4, EPI0 = 8, NEPI = 8;
 
-enum Mode { kStore = 0, kGrad = 1, kSplitDf = 3 };
+enum Mode { kStore = 0, kGrad = 1, kStoreDiag = 2, kSplitDf = 3 };
 
 constexpr int EC = 8;                // columns per epilogue slot
 constexpr int ESLOT = 3 * EC * BM;   // X', G_prev, P_prev: EC columns each
@@ -100,11 +106,12 @@ struct MulArgs {
   double* part;    // kGrad: 4 sums per CTA
   IterScalars* scw;  // kGrad: the CG scalars (formed by the last CTA)
   const float* p32;    // kSplitDf: Cn = (C + alpha P) diag(R) + Y M, with C
-  const float* ch;     // as FP32 pairs and Cn written as pairs
-  const float* cl;
+  const float* ch;     // as FP32 pairs and Cn written as pairs; kStoreDiag: the
+  const float* cl;     // same in FP32 (ch and out, p32 may be null)
   float* outh;
   float* outl;
-  const float* rdiag;  // kSplitDf: diag(R) as pairs (hi[0..n), lo[n..2n))
+  const float* rdiag;  // kSplitDf, kStoreDiag: diag(R) as pairs (hi[0..n),
+                       // lo[n..2n))
   int* err;
 };
 static_assert(NSLOT * ESLOT <= RS * BM * BK,
@@ -147,7 +154,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   MulSmem* sm = reinterpret_cast<MulSmem*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr bool kTwoAcc = MODE == kStore || MODE == kGrad;
+  constexpr bool kTwoAcc = MODE != kSplitDf;
   constexpr int kTmem = kTwoAcc ? 4 * NC : 2 * NC;
   const int ntiles = args.ntr * args.nch;
   const int nk = (args.k + BK - 1) / BK;
@@ -384,7 +391,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     // batch: GB300's FP64 pipe is 1/64 of its FP32 rate)
     F2 s_sum[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
     F2 alpha2 = {0.f, 0.f};
-    if (MODE == kSplitDf && args.sc) alpha2 = df_of(args.sc->alpha);
+    if ((MODE == kSplitDf || MODE == kStoreDiag) && args.sc)
+      alpha2 = df_of(args.sc->alpha);
     const float* slots = &sm->rawp[0][0];
     const int half = cbeg ? 1 : 0;
     const bool hg = args.gprev != nullptr, hp = args.pprev != nullptr;
@@ -474,6 +482,29 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int col = c0 + cb + e;
             if (col < args.n)
               args.out[row + (int64_t)col * N] = __uint_as_float(r[e]);
+          }
+        } else if (MODE == kStoreDiag) {
+#pragma unroll
+          for (int h = 0; h < 16; h += 8) {
+            float cv[8], pv[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const int col = c0 + cb + h + e;
+              const int64_t idx = row + (int64_t)col * N;
+              const bool in = col < args.n;
+              cv[e] = in ? args.ch[idx] : 0.f;
+              pv[e] = in && args.p32 ? args.p32[idx] : 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const int col = c0 + cb + h + e;
+              if (col < args.n) {
+                const float y = args.p32 ? fmaf(alpha2.h, pv[e], cv[e]) : cv[e];
+                const float t = fmaf(y, args.rdiag[args.n + col],
+                                     __uint_as_float(r[h + e]));
+                args.out[row + (int64_t)col * N] = fmaf(y, args.rdiag[col], t);
+              }
+            }
           }
         } else if (MODE == kSplitDf) {
 #pragma unroll
@@ -615,7 +646,8 @@ void launch(const MulArgs& a0, const float* A, const float* P,
   const int ldm = ldm_of(a.k);
   float* hi = ws;
   float* lo = ws + (size_t)ldm * a.n;
-  float* diag2 = MODE == kSplitDf ? lo + (size_t)ldm * a.n : nullptr;
+  float* diag2 = MODE == kSplitDf || MODE == kStoreDiag
+                     ? lo + (size_t)ldm * a.n : nullptr;
   if (diag2) a.rdiag = diag2;
   if (M) {  // (null: the terms are there already, from the factorisation)
     k_split_small<<<ceil_div((int64_t)ldm * a.n, 256), 256, 0, s>>>(
@@ -683,7 +715,13 @@ void mul_tc_store(int64_t N, int k, int n, const float* A, const float* P,
   MulArgs a{};
   a.N = N; a.k = k; a.n = n; a.sc = sc; a.out = out; a.err = tw.err;
   a.tri = 1;  // the rotation's L^{-T}
-  launch<kStore>(a, A, P, M, 0, tw.msplit, s, nullptr);
+  if (tw.fine) {
+    a.ch = A;
+    a.p32 = P;
+    launch<kStoreDiag>(a, A, P, M, 1, tw.msplit, s, nullptr);
+  } else {
+    launch<kStore>(a, A, P, M, 0, tw.msplit, s, nullptr);
+  }
 }
 
 int mul_tc_grad(int64_t N, int m, const float* C, const double* Hp,

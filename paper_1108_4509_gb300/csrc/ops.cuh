@@ -269,6 +269,7 @@ struct TcWork {
   float* msplit = nullptr;
   size_t msplit_floats = 0;
   int* err = nullptr;
+  int fine = 0;  // rotations as exact as FP32 multiply-adds (split_diag terms)
 };
 size_t mul_tc_work_floats(int k, int n);
 int mul_tc_ldm(int k);  // leading dimension of the split small matrix

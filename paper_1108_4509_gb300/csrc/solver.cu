@@ -328,6 +328,7 @@ Solver::Solver(int64_t N, int m, double tol, const trm_options& opt)
   TRM_CUDA(cudaMemsetAsync(sc_, 0, sizeof(IterScalars), s_));
   op_.err = &sc_->status;
   tw_.err = &sc_->status;
+  tw_.fine = fine_;
   if (!fine_ || gram_tc_fine_pays(ld_, m)) {  // else no product takes them
     tw_.msplit_floats = mul_tc_work_floats(m, m);
     tw_.msplit = f(tw_.msplit_floats);
@@ -754,7 +755,8 @@ void Solver::iter_uniform(T*& C, T*& Cn, T* X, T*& G, T*& Gp, T* P, T* HP) {
                     (!gen || rotate_on_tc(ld_, m_, Yc, SPt, &tw_));
     if (line_factor32(m_, Hp32_, HD_, Bm32_, PG32_, hpd, m_ + 1, trp, ntrp,
                       PG32_ + woff, R_, sc_, mmw_, T1_, s_,
-                      tc ? rw_.msplit : nullptr, mul_tc_ldm(m_)))
+                      tc ? rw_.msplit : nullptr, mul_tc_ldm(m_),
+                      /*split_diag=*/fine_))
       R = nullptr;
   } else
     line_factor(m_, Hp_, HD_, Bm_, PG_, hpd, m_ + 1, trp, ntrp, PG_ + woff, R_,

@@ -415,3 +415,39 @@ def test_eigenvalues_with_a_coupling_of_low_rank(trm, m, gap):
     assert np.max(np.abs(lam - w)) <= tol
     assert np.max(np.linalg.norm(H @ C - C * lam, axis=0)) <= tol
     assert np.max(np.abs(C.T @ C - np.eye(m))) <= 20 * m * 2.3e-16
+
+
+@pytest.mark.parametrize("shape,m", [((13, 11, 9), 64), ((21, 23, 25), 40),
+                                     ((17, 19, 21), 96), ((9, 11, 13), 260)])
+def test_full_sp_rotation_on_odd_grids_does_not_shrink(trm, shape, m):
+    """N % 4 != 0, tensor-core rotation, a step of some percent (so that no
+    entry's change is below half a place and lost): the mean square norm of the
+    columns. The entries of C before and after and the rotation's multiply-adds
+    round by 2^-24 in either direction, a few 2^-24 / sqrt(N m) together; the
+    overlap's small part is good to 2^-22 of its largest entry and the factor's
+    diagonal is held as a pair. A truncated sum takes half a place off every
+    entry, 6e-8 off the mean."""
+    V = ti.gaussian_wells(shape, 4, seed=6)
+    N = V.size
+    assert N % 4 and N * m * m >= 5e6
+    H = op.grid_hamiltonian(shape, 4, 1.0, V)
+    import scipy.sparse.linalg as spla
+    v = (np.linalg.eigh(H.toarray())[1] if N < 2000 else
+         spla.eigsh(H, k=m, which="SA", v0=np.ones(N))[1])
+    C = np.linalg.qr(v[:, :m] + 0.17 / np.sqrt(N) * ti.random_block(N, m, 3))[0]
+    _, G, _, _ = otrm.energy_gradient_alg1(H, C)
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_stencil(*shape, 4, 1.0, V, m, 1e-10, opt)
+    try:
+        cd = gu.to_dev(C)
+        trm.trm_set_block(h, cd.data_ptr())
+        _, _, a = trm.trm_iterate(h, trm.TRM_FULL_SP, restart=True)
+        out = gu.empty(N, m, np.float64)
+        trm.trm_get_block(h, out.data_ptr())
+        got = gu.from_dev(out)
+    finally:
+        trm.trm_destroy(h)
+    q = a * a * np.max(np.sum(G ** 2, axis=0))
+    assert q > 1e-5
+    bound = 16 * 2.0 ** -24 / np.sqrt(N * m) + 2.0 ** -20 * q
+    assert abs(np.sum(got ** 2) / m - 1.0) <= bound
