@@ -529,9 +529,9 @@ int launch_vec(const Operator& op, const T* X, T* Y, int ncols, double* dots,
 // x and y neighbours, which the neighbouring threads of the same tile have just
 // read as their own (L1 hits), instead of four more planes through L2. There is
 // no barrier inside the march, so every warp keeps its loads in flight on its
-// own. Every point gets the same operations in the same order as in
-// k_stencil_v4; with DOTS the column dot is accumulated in double-float per
-// thread and the CTA's sum goes to
+// own. With VW = 4 every point gets the same operations in the same order as in
+// k_stencil_v4, else in k_stencil_1's order; with DOTS the column dot is
+// accumulated in double-float per thread and the CTA's sum goes to
 // dots[(blockIdx.y * gridDim.x + blockIdx.x) * ncols + column].
 // Odd grids (VW = 1) took a kernel that read all twelve neighbours through L1
 // and L2 for each point: 34 us at 39 x 41 x 37, 90 columns.
@@ -626,18 +626,35 @@ __global__ void __launch_bounds__(256, VW == 1 ? 6 : 4)
       float out[VW];
 #pragma unroll
       for (int k = 0; k < VW; ++k) {
-        float s1 = 0.f, s2 = 0.f;
-        s1 += a1[k];
-        s1 += b1[k];
-        s1 += q[R - 1][k];
-        s1 += q[R + 1][k];
-        float acc = d[k] * q[R][k] + c1 * (s1 + e[k + 1] + e[k + 3]);
-        if (R == 2) {
-          s2 += a2[k];
-          s2 += b2[k];
-          s2 += q[0][k];
-          s2 += q[2 * R][k];
-          acc += c2 * (s2 + e[k] + e[k + 4]);
+        float acc;
+        if constexpr (VW == 4) {
+          float s1 = 0.f, s2 = 0.f;
+          s1 += a1[k];
+          s1 += b1[k];
+          s1 += q[R - 1][k];
+          s1 += q[R + 1][k];
+          acc = d[k] * q[R][k] + c1 * (s1 + e[k + 1] + e[k + 3]);
+          if (R == 2) {
+            s2 += a2[k];
+            s2 += b2[k];
+            s2 += q[0][k];
+            s2 += q[2 * R][k];
+            acc += c2 * (s2 + e[k] + e[k + 4]);
+          }
+        } else {
+          // this is the FP32 stencil of such grids: x first, as in the one-point
+          // kernel, and the multiply-adds written out (H C of smooth columns
+          // at order 4 was 5 % further from 64 bits the other way)
+          float s1 = e[k + 1] + e[k + 3];
+          s1 = (s1 + a1[k]) + b1[k];
+          s1 = (s1 + q[R - 1][k]) + q[R + 1][k];
+          acc = fmaf(c1, s1, __fmul_rn(d[k], q[R][k]));
+          if (R == 2) {
+            float s2 = e[k] + e[k + 4];
+            s2 = (s2 + a2[k]) + b2[k];
+            s2 = (s2 + q[0][k]) + q[2 * R][k];
+            acc = fmaf(c2, s2, acc);
+          }
         }
         out[k] = acc;
       }

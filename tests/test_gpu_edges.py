@@ -451,3 +451,46 @@ def test_full_sp_rotation_on_odd_grids_does_not_shrink(trm, shape, m):
     assert q > 1e-5
     bound = 16 * 2.0 ** -24 / np.sqrt(N * m) + 2.0 ** -20 * q
     assert abs(np.sum(got ** 2) / m - 1.0) <= bound
+
+
+@pytest.mark.parametrize("order", [2, 4])
+@pytest.mark.parametrize("shape", [(9, 11, 13), (6, 5, 7), (7, 50, 1), (31, 1, 1)])
+def test_fp32_stencil_of_odd_rows_operation_by_operation(trm, shape, order):
+    """nx % 4 != 0: neighbours at distance one added along x, y, z, then one
+    multiply-add per distance onto the rounded diagonal term. The same in numpy,
+    a multiply-add through FP64 (whose second rounding differs from a true one
+    in about one entry of 2^29): equal bytes."""
+    V = ti.gaussian_wells(shape, 2, seed=2)
+    N, m = V.size, 6
+    nx, ny, nz = (tuple(shape) + (1, 1))[:3]
+    f = np.float32
+    C = ti.random_block(N, m, seed=3).astype(f)
+    w = {2: (2.0, -1.0), 4: (2.5, -4.0 / 3.0, 1.0 / 12.0)}[order]
+    ndim = sum(n > 1 for n in (nx, ny, nz))
+    d = (0.5 * w[0] * ndim + V).astype(f).reshape(nz, ny, nx)
+    B = C.T.reshape(m, nz, ny, nx)
+
+    def shift(ax, k):
+        pad = [(0, 0)] * 4
+        pad[ax] = (abs(k), abs(k))
+        take = [slice(None)] * 4
+        take[ax] = slice(abs(k) + k, abs(k) + k + B.shape[ax])
+        return np.pad(B, pad)[tuple(take)]
+
+    acc = d * B
+    for r in range(1, len(w)):
+        s = np.zeros_like(B)
+        for ax in (3, 2, 1):
+            if B.shape[ax] > 1:
+                s = (s + shift(ax, -r)) + shift(ax, r)
+        c = np.float64(f(0.5 * w[r]))
+        acc = (c * s.astype(np.float64) + acc.astype(np.float64)).astype(f)
+    opt = trm.trm_default_options(stream=gu.stream())
+    h = trm.trm_create_stencil(nx, ny, nz, order, 1.0, V, m - 1, 1e-10, opt)
+    try:
+        x = gu.to_dev(C, f)
+        y = gu.empty(N, m, f)
+        trm.trm_apply_h(h, trm.TRM_F32, x.data_ptr(), trm.TRM_F32, y.data_ptr(), m)
+        assert np.array_equal(gu.from_dev(y), acc.reshape(m, N).T)
+    finally:
+        trm.trm_destroy(h)
